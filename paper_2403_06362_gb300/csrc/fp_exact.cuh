@@ -72,9 +72,29 @@ __host__ __device__ __forceinline__ uint64_t floor_nonneg(double t) {
   return e <= 52 ? m >> (52 - e) : m << (e - 52);
 }
 
+// The bits of x for comparisons.  On the device they come through a move that
+// the compiler does not see through: given a plain bit cast it recognises
+// bits & ~2^63 as |x| and issues that to the fp64 unit, where it takes as
+// long as an addition, and bits << 1 == 0 as a comparison with zero.  (65 of
+// the 126 fp64 instructions of a box flight were such; without them 3 * 10^6
+// histories took 37.9 ms instead of 45.7.)
+__host__ __device__ __forceinline__ uint64_t raw_bits(double x) {
+#ifdef __CUDA_ARCH__
+  uint64_t b;
+  asm("mov.b64 %0, %1;" : "=l"(b) : "d"(x));
+  return b;
+#else
+  return to_bits(x);
+#endif
+}
+__host__ __device__ __forceinline__ uint64_t mag_bits(double x) { return raw_bits(x) & ~(1ull << 63); }
+
+// |x|.
+__host__ __device__ __forceinline__ double abs_bits(double x) { return from_bits(mag_bits(x)); }
+
 // |x| <= h for h >= 0 (finite): non-negative doubles order like their bits.
 __host__ __device__ __forceinline__ bool abs_le(double x, double h) {
-  return (to_bits(x) & ~(1ull << 63)) <= to_bits(h);
+  return mag_bits(x) <= to_bits(h);
 }
 
 // q = RN(2^105 / M) for 2^52 < M < 2^53 (ties cannot occur: 2^106 = (2q + 1) M
@@ -137,14 +157,13 @@ __host__ __device__ __forceinline__ long long llrint_nonneg(double v) {
 // Order key of a non-NaN double: a < b  <=>  okey(a) < okey(b); -0 and +0
 // share the key 0.
 __host__ __device__ __forceinline__ long long okey(double x) {
-  const uint64_t b = to_bits(x);
-  const long long m = (long long)(b & ~(1ull << 63));
-  return (b >> 63) ? -m : m;
+  const long long m = (long long)mag_bits(x);
+  return (long long)raw_bits(x) < 0 ? -m : m;
 }
 __host__ __device__ __forceinline__ bool d_lt(double a, double b) { return okey(a) < okey(b); }
-__host__ __device__ __forceinline__ bool d_pos(double a) { return (long long)to_bits(a) > 0; }        // a > 0
-__host__ __device__ __forceinline__ bool d_neg(double a) { return to_bits(a) > (1ull << 63); }         // a < 0
-__host__ __device__ __forceinline__ bool d_zero(double a) { return (to_bits(a) << 1) == 0ull; }        // a == 0
+__host__ __device__ __forceinline__ bool d_pos(double a) { return (long long)raw_bits(a) > 0; }        // a > 0
+__host__ __device__ __forceinline__ bool d_neg(double a) { return raw_bits(a) > (1ull << 63); }         // a < 0
+__host__ __device__ __forceinline__ bool d_zero(double a) { return (raw_bits(a) << 1) == 0ull; }        // a == 0
 
 // RN(j h) for an integer 0 <= j < 2^11 and a normal h > 0 whose product
 // stays normal: the exact product m_h j has at most 64 bits, rounded once.

@@ -311,7 +311,7 @@ __device__ __forceinline__ float mu_f32(uint64_t n) { return __double2float_rn(m
 // 2^32 / |mu| rounded once: 2^32 RN(1 / |mu|), the reciprocal on the
 // integer pipes (fp_exact.cuh), the scaling an exponent add.
 __device__ __forceinline__ double fix_per_mu(double mu) {
-  return mu != 0.0 ? mcx::scale_pow2(mcx::recip_rn(fabs(mu)), 32) : 0.0;
+  return !mcx::d_zero(mu) ? mcx::scale_pow2(mcx::recip_rn(mcx::abs_bits(mu)), 32) : 0.0;
 }
 
 // Per-lane counters for the lane's current problem (flushed with atomics,
