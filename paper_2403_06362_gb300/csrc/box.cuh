@@ -38,6 +38,7 @@ struct BoxDev {
   int ih_s;
   float side_f, lo_f, hi_f, h_f, inv_h_f;
   float inv_st_f[2], c_f[2], wl_f[2], wh_f[2], ws_f[2];
+  uint64_t cdf_n[2][kMaxG][kMaxG];  // u < cdf  <=>  n < cdf_n for u = n 2^-53
   uint64_t seed_hash, hist_begin;
 };
 
@@ -61,9 +62,12 @@ struct ChildRec {
 
 enum BoxOutcome : int { kBoxCollide = 0, kBoxCross = 1, kBoxLeak = 2, kBoxContinue = 3, kBoxKilled = 4 };
 
-template <typename T> __device__ __forceinline__ T from_u(double u);
-template <> __device__ __forceinline__ double from_u<double>(double u) { return u; }
-template <> __device__ __forceinline__ float from_u<float>(double u) { return (float)u; }
+// The uniform u = n 2^-53 in T (fp32: rounded once).
+template <typename T> __device__ __forceinline__ T from_n(uint64_t n);
+template <> __device__ __forceinline__ double from_n<double>(uint64_t n) {
+  return mcd::u53_to_double((uint32_t)(n >> 32), (uint32_t)n);
+}
+template <> __device__ __forceinline__ float from_n<float>(uint64_t n) { return mcs::u53_to_float(n); }
 
 template <typename T> __device__ __forceinline__ T sel(const double& d, const float& f);
 template <> __device__ __forceinline__ double sel<double>(const double& d, const float&) { return d; }
@@ -84,14 +88,30 @@ __device__ __forceinline__ bool is0(float a) { return a == 0.0f; }
 
 template <typename T> __device__ __forceinline__ T recip(T v);
 template <> __device__ __forceinline__ double recip<double>(double v) { return mcx::recip_rn(v); }
-template <> __device__ __forceinline__ float recip<float>(float v) { return 1.0f / v; }
+template <> __device__ __forceinline__ float recip<float>(float v) { return __frcp_rn(v); }
 
 // Componentwise inverse of the direction (fp64: the correctly rounded
-// reciprocal on the integer pipes, fp_exact.cuh).
+// reciprocal on the integer pipes, fp_exact.cuh); 0 for a zero component.
+// One copy of the reciprocal's code, run three times with the components
+// rotated through it: an indexed loop would put the direction in local
+// memory, three inlined copies cost instruction-cache misses (the fp64
+// kernel's largest stall).
 template <typename T>
 __device__ __forceinline__ void set_inv(Part<T>& q) {
+  T u0 = q.u[0], u1 = q.u[1], u2 = q.u[2], i0 = T(0), i1 = T(0), i2 = T(0);
 #pragma unroll 1
-  for (int a = 0; a < 3; ++a) q.inv[a] = !is0(q.u[a]) ? recip<T>(q.u[a]) : T(0);
+  for (int a = 0; a < 3; ++a) {
+    const T v = !is0(u0) ? recip<T>(u0) : T(0), r = u0;
+    u0 = u1;
+    u1 = u2;
+    u2 = r;
+    i0 = i1;
+    i1 = i2;
+    i2 = v;
+  }
+  q.inv[0] = i0;
+  q.inv[1] = i1;
+  q.inv[2] = i2;
 }
 
 // Marsaglia (1972): v1, v2 uniform on [-1,1)^2 until v1^2 + v2^2 < 1.
@@ -103,8 +123,8 @@ __device__ __forceinline__ void iso_dir(mcs::Rng<M>& r, const mcd::Lcg& l, T u[3
       v1 = mcx::two_u_minus_1(r.next_n(l));
       v2 = mcx::two_u_minus_1(r.next_n(l));
     } else {
-      v1 = T(2) * from_u<T>(r.next(l)) - T(1);
-      v2 = T(2) * from_u<T>(r.next(l)) - T(1);
+      v1 = T(2) * from_n<T>(r.next_n(l)) - T(1);
+      v2 = T(2) * from_n<T>(r.next_n(l)) - T(1);
     }
     s = v1 * v1 + v2 * v2;
   } while (!lt(s, T(1)));
@@ -125,51 +145,57 @@ __device__ __forceinline__ uint32_t region_of(const BoxDev& b, const T p[3], con
   return 1u;
 }
 
+// Distance to the way out of [lo, hi]^3 from inside: per axis the face ahead
+// is picked first, so that lanes flying in different directions take one
+// subtraction and one product together.
 template <typename T>
 __device__ __forceinline__ T exit_dist(const Part<T>& q, T lo, T hi) {
   T t = T(INFINITY);
+#pragma unroll
   for (int a = 0; a < 3; ++a) {
-    T ta;
-    if (gt0(q.u[a])) ta = (hi - q.p[a]) * q.inv[a];
-    else if (lt0(q.u[a])) ta = (lo - q.p[a]) * q.inv[a];
-    else continue;
-    if (lt(ta, t)) t = ta;
+    const T ta = ((gt0(q.u[a]) ? hi : lo) - q.p[a]) * q.inv[a];
+    if (!is0(q.u[a]) && lt(ta, t)) t = ta;
   }
   return lt0(t) ? T(0) : t;
 }
 
+// Distance to the way into [lo, hi]^3 from outside (infinite: it misses).
+// Rounding is monotone, so the face on the side the particle comes from has
+// the smaller of an axis's two distances.
 template <typename T>
 __device__ __forceinline__ T entry_dist(const Part<T>& q, T lo, T hi) {
   T tn = T(-INFINITY), tf = T(INFINITY);
+  bool miss = false;
+#pragma unroll
   for (int a = 0; a < 3; ++a) {
+    const bool neg = lt0(q.u[a]);
+    const T tmin = ((neg ? hi : lo) - q.p[a]) * q.inv[a], tmax = ((neg ? lo : hi) - q.p[a]) * q.inv[a];
     if (!is0(q.u[a])) {
-      const T t1 = (lo - q.p[a]) * q.inv[a], t2 = (hi - q.p[a]) * q.inv[a];
-      const bool o = lt(t1, t2);
-      const T tmin = o ? t1 : t2, tmax = o ? t2 : t1;
       if (lt(tn, tmin)) tn = tmin;
       if (lt(tmax, tf)) tf = tmax;
     } else if (!lt(lo, q.p[a]) || !lt(q.p[a], hi)) {
-      return T(INFINITY);
+      miss = true;
     }
   }
-  if (!lt0(tn) && lt(tn, tf)) return tn;
-  return T(INFINITY);
+  return !miss && !lt0(tn) && lt(tn, tf) ? tn : T(INFINITY);
 }
 
 // Distance to the region surface and its kind (1: into the other region,
-// 2: out of the box).
+// 2: out of the box).  Both regions share the code of the way out.
 template <typename T>
 __device__ __forceinline__ T surface(const BoxDev& b, const Part<T>& q, int& kind) {
   const T lo = sel<T>(b.lo, b.lo_f), hi = sel<T>(b.hi, b.hi_f), side = sel<T>(b.side, b.side_f);
-  if (q.region == 1u) {
-    kind = 1;
-    return exit_dist(q, lo, hi);
+  const bool inner = q.region == 1u;
+  T ds = exit_dist(q, inner ? lo : T(0), inner ? hi : side);
+  kind = inner ? 1 : 2;
+  if (!inner) {
+    const T de = entry_dist(q, lo, hi);
+    if (lt(de, ds)) {
+      ds = de;
+      kind = 1;
+    }
   }
-  const T de = entry_dist(q, lo, hi);
-  const T dx = exit_dist(q, T(0), side);
-  const bool in = lt(de, dx);
-  kind = in ? 1 : 2;
-  return in ? de : dx;
+  return ds;
 }
 
 __device__ __forceinline__ long long fix_of(double wl) { return mcx::fix32_nonneg(wl); }
@@ -198,70 +224,156 @@ template <> __device__ __forceinline__ int voxel_guess<float>(const BoxDev& b, f
   return (int)floorf(p * b.inv_h_f);
 }
 
-// Track-length tally of p + t u, 0 <= t <= L, by a voxel walk: the next
-// crossing on each axis is computed from the segment start directly,
-// t = (plane - p) / u, so every piece has the length the clipping definition
-// gives it.  base: this history's [mesh^3] slot row.
+// The walk of a segment p + t u, 0 <= t <= L, through the mesh: t, the start
+// of the current piece; per axis the distance tn to its next plane and that
+// plane's index j; the voxel's slot.  A lane can leave the walk after any
+// step and take it up again (the history kernel walks in chunks).  The axes
+// are scalars picked by selects: arrays indexed by the crossed axis would
+// live in local memory.
 template <typename T>
-__device__ void trace(const BoxDev& b, const Part<T>& q, T L, unsigned long long* base, const double* tab,
-                      bool agg) {
+struct Walk {
+  T t, L, tn0, tn1, tn2;
+  int j0, j1, j2;
+  uint32_t slot;
+};
+
+// The voxel of coordinate p on one axis and, as seen by direction u, the
+// next plane j and its distance tn.  The looked-up voxel is within one of the
+// right one; the exact plane comparisons correct it, and put a particle on a plane on
+// the side it flies to, in a rarely taken branch.
+template <typename T>
+__device__ __forceinline__ int walk_axis(const BoxDev& b, const double* tab, int nm, T p, T u, T inv, int& j, T& tn) {
+  int i = voxel_guess<T>(b, p);
+  i = i < 0 ? 0 : (i >= nm ? nm - 1 : i);
+  T lo = plane<T>(b, tab, i), hi = plane<T>(b, tab, i + 1);
+  const bool neg = lt0(u);
+  if ((i > 0 && !lt(lo, p)) || (i + 1 < nm && !lt(p, hi))) {
+    while (i > 0 && lt(p, lo)) { hi = lo; lo = plane<T>(b, tab, --i); }
+    while (i + 1 < nm && !lt(p, hi)) { lo = hi; hi = plane<T>(b, tab, ++i + 1); }
+    if (neg && i > 0 && eq(p, lo)) lo = plane<T>(b, tab, --i);
+  }
+  j = neg ? i : i + 1;
+  tn = is0(u) ? T(INFINITY) : ((neg ? lo : hi) - p) * inv;
+  return i;
+}
+
+template <typename T>
+__device__ __forceinline__ void walk_begin(const BoxDev& b, const Part<T>& q, T L, const double* tab, Walk<T>& k) {
   const int nm = (int)b.mesh;
-  const T h = sel<T>(b.h, b.h_f), inv_h = sel<T>(b.inv_h, b.inv_h_f);
-  int idx[3];
-  T tn[3];
-  for (int a = 0; a < 3; ++a) {
-    int i = voxel_guess<T>(b, q.p[a]);
-    i = i < 0 ? 0 : (i >= nm ? nm - 1 : i);
-    while (i > 0 && lt(q.p[a], plane<T>(b, tab, i))) --i;
-    while (i + 1 < nm && !lt(q.p[a], plane<T>(b, tab, i + 1))) ++i;
-    if (lt0(q.u[a]) && i > 0 && eq(q.p[a], plane<T>(b, tab, i))) --i;
-    idx[a] = i;
-    if (gt0(q.u[a])) tn[a] = (plane<T>(b, tab, i + 1) - q.p[a]) * q.inv[a];
-    else if (lt0(q.u[a])) tn[a] = (plane<T>(b, tab, i) - q.p[a]) * q.inv[a];
-    else tn[a] = T(INFINITY);
+  const int i0 = walk_axis<T>(b, tab, nm, q.p[0], q.u[0], q.inv[0], k.j0, k.tn0);
+  const int i1 = walk_axis<T>(b, tab, nm, q.p[1], q.u[1], q.inv[1], k.j1, k.tn1);
+  const int i2 = walk_axis<T>(b, tab, nm, q.p[2], q.u[2], q.inv[2], k.j2, k.tn2);
+  k.slot = (uint32_t)((i2 * nm + i1) * nm + i0);  // mesh <= 1024: below 2^30
+  k.t = T(0);
+  k.L = L;
+}
+
+// One piece of the walk: its track length into the voxel (t to the next
+// plane or to L), then across the plane.  The next crossing on an axis is
+// computed from the segment start directly, t = (plane - p) / u, so every
+// piece has the length the clipping definition gives it.  Returns true when
+// the walk has ended (L reached, or the mesh left).  base: this history's
+// [mesh^3] slot row.
+template <typename T>
+__device__ __forceinline__ bool walk_step(const BoxDev& b, const Part<T>& q, Walk<T>& k, unsigned long long* base,
+                                          const double* tab, bool agg) {
+  const bool y = lt(k.tn1, k.tn0);
+  const T t01 = y ? k.tn1 : k.tn0;
+  const bool z = lt(k.tn2, t01);
+  const T ta = z ? k.tn2 : t01;
+  const bool inside = lt(ta, k.L);
+  const T tend = inside ? ta : k.L;
+  const unsigned long long v = (unsigned long long)fix_of(q.w * (tend - k.t));
+  if (lt(k.t, tend)) {
+    if (agg) mcd::warp_agg_add(base + k.slot, v);
+    else atomicAdd(base + k.slot, v);
+    k.t = tend;
   }
-  (void)h;
-  (void)inv_h;
-  T t = T(0);
-  const T w = q.w;
-  for (int guard = 0; guard < 3 * nm + 8; ++guard) {
-    int a = 0;
-    if (lt(tn[1], tn[a])) a = 1;
-    if (lt(tn[2], tn[a])) a = 2;
-    const bool inside = lt(tn[a], L);
-    const T tend = inside ? tn[a] : L;
-    if (lt(t, tend)) {
-      const long long v = fix_of(w * (tend - t));
-      if (v != 0) {
-        const uint64_t slot = ((uint64_t)idx[2] * nm + idx[1]) * nm + idx[0];
-        if (agg) mcd::warp_agg_add(base + slot, (unsigned long long)v);
-        else atomicAdd(base + slot, (unsigned long long)v);
-      }
-      t = tend;
-    }
-    if (!inside) break;
-    // step across the plane on axis a
-    if (gt0(q.u[a])) {
-      idx[a] += 1;
-      if (idx[a] >= nm) break;
-      tn[a] = (plane<T>(b, tab, idx[a] + 1) - q.p[a]) * q.inv[a];
-    } else {
-      idx[a] -= 1;
-      if (idx[a] < 0) break;
-      tn[a] = (plane<T>(b, tab, idx[a]) - q.p[a]) * q.inv[a];
-    }
-  }
+  if (!inside) return true;
+  const uint32_t nm = b.mesh;
+  const T p = z ? q.p[2] : (y ? q.p[1] : q.p[0]), inv = z ? q.inv[2] : (y ? q.inv[1] : q.inv[0]);
+  const int s = lt0(inv) ? -1 : 1;
+  const int j = (z ? k.j2 : (y ? k.j1 : k.j0)) + s;
+  k.slot += (uint32_t)s * (z ? nm * nm : (y ? nm : 1u));
+  if ((uint32_t)j > nm) return true;  // the plane crossed was the mesh's face
+  const T tn = (plane<T>(b, tab, j) - p) * inv;
+  if (z) { k.j2 = j; k.tn2 = tn; }
+  else if (y) { k.j1 = j; k.tn1 = tn; }
+  else { k.j0 = j; k.tn0 = tn; }
+  return false;
+}
+
+// The source up to its direction (three draws): position, weight, group.
+template <int M, typename T>
+__device__ __forceinline__ void source_position(const BoxDev& b, mcs::Rng<M>& r, const mcd::Lcg& l, Part<T>& q) {
+  const T side = sel<T>(b.side, b.side_f);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) q.p[a] = side * from_n<T>(r.next_n(l));
+  q.w = T(1);
+  q.g = 0u;
 }
 
 template <int M, typename T>
 __device__ __forceinline__ void box_source(const BoxDev& b, mcs::Rng<M>& r, const mcd::Lcg& l, Part<T>& q) {
-  const T side = sel<T>(b.side, b.side_f);
-  for (int a = 0; a < 3; ++a) q.p[a] = side * from_u<T>(r.next(l));
+  source_position<M, T>(b, r, l, q);
   iso_dir<M, T>(r, l, q.u);
   set_inv(q);
-  q.w = T(1);
-  q.g = 0u;
   q.region = region_of<T>(b, q.p, q.u);
+}
+
+// The fp32 path's decision near the surface, made again in fp64 from the
+// flight's uniform: bit 0 collide, the upper bits the surface's kind.  Out
+// of line: about one flight in 2^15 takes it.
+static __device__ __noinline__ int decide_f64(const BoxDev* b, float p0, float p1, float p2, float u0, float u1,
+                                              float u2, uint32_t region, uint64_t n) {
+  Part<double> q;
+  q.p[0] = p0;
+  q.p[1] = p1;
+  q.p[2] = p2;
+  q.u[0] = u0;
+  q.u[1] = u1;
+  q.u[2] = u2;
+  for (int a = 0; a < 3; ++a) q.inv[a] = q.u[a] != 0.0 ? mcx::recip_rn(q.u[a]) : 0.0;
+  q.region = region;
+  int kind = 0;
+  const double ds = surface<double>(*b, q, kind);
+  const double d = -mclog::log1m_n(n) * b->inv_st[region];
+  return (d < ds ? 1 : 0) | (kind << 1);
+}
+
+// The length of the next flight and how it ends (kBoxCollide, kBoxCross or
+// kBoxLeak): the sampled distance against the region surface.
+template <int M, typename T>
+__device__ __forceinline__ int flight_length(const BoxDev& b, mcs::Rng<M>& r, const mcd::Lcg& l, const Part<T>& q,
+                                             T& len) {
+  int kind = 0;
+  const T ds = surface<T>(b, q, kind);
+  bool collide;
+  T d;
+  if constexpr (sizeof(T) == 8) {
+    d = -mclog::log1m_n(r.next_n(l)) * b.inv_st[q.region];
+    collide = lt(d, ds);
+  } else {
+    const uint64_t n = r.next_n(l);
+    d = mcs::flight_f32(n) * b.inv_st_f[q.region];
+    collide = d < ds;
+    if (fabsf(d - ds) <= 0x1p-16f * fmaxf(d, ds)) {  // near the surface: decide in fp64
+      const int k = decide_f64(&b, q.p[0], q.p[1], q.p[2], q.u[0], q.u[1], q.u[2], q.region, n);
+      collide = (k & 1) != 0;
+      kind = k >> 1;
+    }
+  }
+  len = collide ? d : ds;
+  return collide ? kBoxCollide : (kind == 2 ? kBoxLeak : kBoxCross);
+}
+
+// The end of a flight of length len: the particle at its end point, in the
+// region it crossed into.
+template <typename T>
+__device__ __forceinline__ void arrive(Part<T>& q, T len, int outcome) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) q.p[a] = q.p[a] + len * q.u[a];
+  if (outcome == kBoxCross) q.region ^= 1u;
 }
 
 // One flight: collide (position moved to the site), cross into the other
@@ -269,64 +381,54 @@ __device__ __forceinline__ void box_source(const BoxDev& b, mcs::Rng<M>& r, cons
 template <int M, typename T>
 __device__ __forceinline__ int box_flight(const BoxDev& b, mcs::Rng<M>& r, const mcd::Lcg& l, Part<T>& q,
                                           unsigned long long* base, const double* tab, bool agg) {
-  int kind = 0;
-  T ds = surface<T>(b, q, kind);
-  bool collide;
-  T d;
-  if constexpr (sizeof(T) == 8) {
-    d = -mclog::log1m_n(r.next_n(l)) * b.inv_st[q.region];
-    collide = lt(d, ds);
-  } else {
-    const double u = r.next(l);
-    d = mcs::flight_f32(u) * b.inv_st_f[q.region];
-    collide = d < ds;
-    if (fabsf(d - ds) <= 0x1p-16f * fmaxf(d, ds)) {  // near the surface: decide in fp64
-      Part<double> q64;
-      for (int a = 0; a < 3; ++a) {
-        q64.p[a] = q.p[a];
-        q64.u[a] = q.u[a];
-        q64.inv[a] = q.inv[a] != 0.0f ? mcx::recip_rn((double)q.u[a]) : 0.0;
-      }
-      q64.region = q.region;
-      int k64 = 0;
-      const double ds64 = surface<double>(b, q64, k64);
-      const double d64 = -mclog::log1m(u) * b.inv_st[q.region];
-      collide = d64 < ds64;
-      kind = k64;
-    }
-  }
-  const T len = collide ? d : ds;
-  trace<T>(b, q, len, base, tab, agg);
-  for (int a = 0; a < 3; ++a) q.p[a] = q.p[a] + len * q.u[a];
-  if (collide) return kBoxCollide;
-  if (kind == 2) return kBoxLeak;
-  q.region ^= 1u;
-  return kBoxCross;
+  T len;
+  const int o = flight_length<M, T>(b, r, l, q, len);
+  Walk<T> k;
+  walk_begin<T>(b, q, len, tab, k);
+  while (!walk_step<T>(b, q, k, base, tab, agg)) {}
+  arrive<T>(q, len, o);
+  return o;
 }
 
-// One collision: implicit capture, group, direction, weight window.
-// Returns kBoxContinue, kBoxKilled (roulette), or the number n >= 2 of
-// particles of a split (the parent keeps weight w/n; the caller creates the
-// n-1 children from the parent's state after this call).
+// The integer form of u < v over u = n 2^-53, n < 2^53: n < threshold.  The
+// comparison is that of the bit patterns read as signed integers (a value
+// with its sign bit set is below every uniform, one of 1 or more, or a NaN,
+// above).
+__device__ __forceinline__ uint64_t cdf_threshold(double v) {
+  const long long bits = __double_as_longlong(v);
+  if (bits < 0) return 0ull;
+  if (bits >= 0x3ff0000000000000ll) return 1ull << 53;
+  return (uint64_t)ceil(v * 0x1p53);
+}
+
+// A collision up to the new direction: implicit capture and the group.
 template <int M, typename T>
-__device__ __forceinline__ int box_collide(const BoxDev& b, mcs::Rng<M>& r, const mcd::Lcg& l, Part<T>& q) {
+__device__ __forceinline__ void collide_group(const BoxDev& b, mcs::Rng<M>& r, const mcd::Lcg& l, Part<T>& q) {
   const uint32_t rg = q.region;
   q.w = q.w * sel<T>(b.c[rg], b.c_f[rg]);
-  const double ug = r.next(l);
+  const uint64_t ug = r.next_n(l);
   uint32_t g2 = q.g;
   for (uint32_t k = q.g; k < b.ng; ++k) {
-    if (mcs::nn_lt(ug, b.cdf[rg][q.g][k])) {  // both non-negative
+    if (ug < b.cdf_n[rg][q.g][k]) {
       g2 = k;
       break;
     }
   }
   q.g = g2;
-  iso_dir<M, T>(r, l, q.u);
-  set_inv(q);
+}
+
+// The weight window after a collision's new direction: kBoxContinue,
+// kBoxKilled (roulette), or kSplitBase + n for a split into n >= 2 (the
+// parent keeps weight w/n; the caller creates the n-1 children from the
+// parent's state after this call).
+constexpr int kSplitBase = 8;
+template <int M, typename T>
+__device__ __forceinline__ int weight_window(const BoxDev& b, mcs::Rng<M>& r, const mcd::Lcg& l, Part<T>& q) {
+  const uint32_t rg = q.region;
   const T wl = sel<T>(b.wl[rg], b.wl_f[rg]), wh = sel<T>(b.wh[rg], b.wh_f[rg]);
   if (lt(q.w, wl)) {
     const T ws = sel<T>(b.ws[rg], b.ws_f[rg]);
-    if (lt(from_u<T>(r.next(l)), q.w / ws)) {
+    if (lt(from_n<T>(r.next_n(l)), q.w / ws)) {
       q.w = ws;
       return kBoxContinue;
     }
@@ -337,10 +439,19 @@ __device__ __forceinline__ int box_collide(const BoxDev& b, mcs::Rng<M>& r, cons
     const uint32_t ns = nd > (T)b.max_split ? b.max_split : (uint32_t)nd;
     if (ns > 1u) {
       q.w = q.w / (T)ns;
-      return (int)ns + 8;  // encoded: n + 8 (> every other outcome)
+      return kSplitBase + (int)ns;  // (> every other outcome)
     }
   }
   return kBoxContinue;
+}
+
+// One collision: implicit capture, group, direction, weight window.
+template <int M, typename T>
+__device__ __forceinline__ int box_collide(const BoxDev& b, mcs::Rng<M>& r, const mcd::Lcg& l, Part<T>& q) {
+  collide_group<M, T>(b, r, l, q);
+  iso_dir<M, T>(r, l, q.u);
+  set_inv(q);
+  return weight_window<M, T>(b, r, l, q);
 }
 
 // Per-lane counters of one problem, flushed with atomics (lane by lane, or
@@ -405,8 +516,6 @@ struct BoxCounts {
   }
 };
 
-constexpr int kSplitBase = 8;
-
 // Child k of a split: Eq. (5), S_c = hash(k, S_p) mod 2^m.
 __device__ __forceinline__ uint64_t child_seed(uint32_t k, uint64_t parent_state, uint64_t mask) {
   return mcd::hash64((uint64_t)k, parent_state & mask) & mask;
@@ -428,8 +537,11 @@ __device__ __forceinline__ void store_child(ChildRec& c, const Part<T>& q, uint6
   c.pad = 0;
 }
 
+// A child's record but for the inverse of its direction (child_state), and
+// the whole of it.
 template <typename T>
-__device__ __forceinline__ void load_child(const ChildRec& c, Part<T>& q) {
+__device__ __forceinline__ void child_state(const ChildRec& c, Part<T>& q) {
+#pragma unroll
   for (int a = 0; a < 3; ++a) {
     q.p[a] = (T)c.p[a];
     q.u[a] = (T)c.u[a];
@@ -437,6 +549,11 @@ __device__ __forceinline__ void load_child(const ChildRec& c, Part<T>& q) {
   q.w = (T)c.w;
   q.g = c.g;
   q.region = c.region;
+}
+
+template <typename T>
+__device__ __forceinline__ void load_child(const ChildRec& c, Part<T>& q) {
+  child_state(c, q);
   set_inv(q);
 }
 

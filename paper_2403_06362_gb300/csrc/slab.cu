@@ -363,7 +363,7 @@ __device__ __noinline__ void coop_draws(const CoopArgs* c, const mcd::Affine* ta
       float d = 0.0f;
       if (e < E) {
         const uint64_t sd = mcd::lcg_step(xs, l.g, l.c);
-        d = mcs::flight_f32(mcd::u01<M>(sd, l.m)) * p.inv_st_f;
+        d = mcs::flight_f32(mcd::u53<M>(sd, l.m)) * p.inv_st_f;
         const float pr = __fmul_rn(d, muf);
         R.p[e] = pack2(pr, __fmaf_rn(d, muf, -pr));
         R.m[e] = sd;
@@ -461,7 +461,7 @@ __device__ __noinline__ void coop_walk(const CoopArgs* c, const mcd::Affine* tab
       const unsigned long long pc = R.p[e];
       float xn, xnlo;
       const int f = mcs::advance32(p, xf, xlo, hi_of(R.d[e]), lo_of(pc), hi_of(pc),
-                                   [&] { return mcd::u01<M>(R.m[e], m); }, xn, xnlo);
+                                   [&] { return mcd::u53<M>(R.m[e], m); }, xn, xnlo);
       if (f != mcs::kCollide) { out = f; ++e; break; }
       xf = xn;
       xlo = xnlo;

@@ -213,10 +213,10 @@ __device__ __forceinline__ void point64(const SlabDev& p, double x, double d, co
   s.add(j, mcx::fix32_nonneg(d));
 }
 
-// Exact llrint((double)v * 2^32) for a finite float v >= 0, in integer
-// arithmetic (scaling by 2^32 is exact; only values below 2^-9 need a
-// rounding of the shifted-out bits, done half-to-even).
-__device__ __forceinline__ long long fix32_from_float(float v) {
+// Exact llrint((double)v * 2^32) for a finite float v >= 0 (scaling by 2^32
+// is exact; bits below the last are rounded half to even).
+// On integers, for any v.  Out of line: tracks below 2^22 cm take the other way.
+static __device__ __noinline__ long long fix32_any(float v) {
   const uint32_t b = __float_as_uint(v);
   const int e = (int)(b >> 23) & 0xff;
   if (e == 0) return 0;  // zero or subnormal: below 2^-126, rounds to 0 at scale 2^32
@@ -228,6 +228,22 @@ __device__ __forceinline__ long long fix32_from_float(float v) {
   const uint64_t q = mant >> r, rem = mant & ((1ull << r) - 1ull), half = 1ull << (r - 1);
   const uint64_t up = (rem > half) || (rem == half && (q & 1ull));
   return (long long)(q + up);
+}
+
+// For v < 2^22 on the fp32 pipe, without branches: adding 2^23 rounded down
+// leaves floor(v) in the low bits; the fraction (exact) gives its next 16
+// bits the same way, and the last 16 by an addition rounded to nearest even,
+// whose parity is that of the whole.  (A fraction has at most 24 bits, so
+// the last step never carries out of its 16.)
+__device__ __forceinline__ long long fix32_from_float(float v) {
+  if (v >= 4194304.0f) return fix32_any(v);
+  constexpr float kM = 8388608.0f;  // 2^23, bit pattern 0x4b000000
+  const float m1 = __fadd_rz(v, kM);
+  const float g = __fmul_rn(__fsub_rn(v, __fsub_rn(m1, kM)), 65536.0f);
+  const float m2 = __fadd_rz(g, kM);
+  const float m3 = __fadd_rn(__fmul_rn(__fsub_rn(g, __fsub_rn(m2, kM)), 65536.0f), kM);
+  const uint32_t lo = __float_as_uint(m2) * 65536u + (__float_as_uint(m3) - 0x4b000000u);
+  return (long long)(((uint64_t)(__float_as_uint(m1) - 0x4b000000u) << 32) | lo);
 }
 
 __device__ __forceinline__ float slab_edge_f(const SlabDev& p, int j) {
@@ -295,18 +311,39 @@ __device__ __forceinline__ void two_sum_f(float a, float b, float& s, float& t) 
   t = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bv)), __fsub_rn(b, bv));
 }
 
-// -ln(1 - u) in fp32 for u in [0, 1): log1pf(-u) below 1/2 (no
-// cancellation for small u), else logf of 1 - u, which is exact in fp64 and
-// at least 2^-53, so it rounds to a positive float and the result is finite
-// (log1pf of -(float)u would meet -1 and give an infinite distance for u
-// within 2^-25 of 1).
-__device__ __forceinline__ float flight_f32(double u) {
-  return u < 0.5 ? -log1pf(-(float)u) : -logf(__double2float_rn(__dsub_rn(1.0, u)));
+// z 2^-64 rounded once to fp32, for z != 0 with its low 10 bits zero: the
+// leading 32 bits of z, with a sticky bit for the rest, through the 32-bit
+// conversion.  The same value as rounding the exact double (which costs the
+// fp64 unit 16 cycles per SM and warp); z below 2^32 takes that way.
+__device__ __forceinline__ float top_bits_to_float(uint64_t z) {
+  const uint32_t hi = (uint32_t)(z >> 32), lo = (uint32_t)z;
+  if (hi == 0u) return __uint2float_rn(lo) * 0x1p-64f;  // at most 22 bits: exact
+  const int lz = __clz((int)hi);
+  const uint32_t t = __funnelshift_l(lo, hi, lz) | ((lo << lz) != 0u ? 1u : 0u);
+  return __int_as_float(__float_as_int(__uint2float_rn(t)) - ((32 + lz) << 23));
 }
 
-// The fp32 direction 2u - 1 for u = n 2^-53: the exact fp64 value rounded
-// once to fp32.
-__device__ __forceinline__ float mu_f32(uint64_t n) { return __double2float_rn(mcx::two_u_minus_1(n)); }
+// The uniform u = n 2^-53 (n < 2^53) rounded once to fp32.
+__device__ __forceinline__ float u53_to_float(uint64_t n) { return top_bits_to_float(n << 11); }
+
+// -ln(1 - u) in fp32 for u = n 2^-53: log1pf(-u) below 1/2 (no
+// cancellation for small u), else logf of 1 - u, which is exact as an
+// integer and at least 2^-53, so it rounds to a positive float and the result
+// is finite (log1pf of -(float)u would meet -1 and give an infinite distance
+// for u within 2^-25 of 1).
+__device__ __forceinline__ float flight_f32(uint64_t n) {
+  const bool low = n < (1ull << 52);
+  const float v = u53_to_float(low ? n : (1ull << 53) - n);
+  return low ? -log1pf(-v) : -logf(v);
+}
+
+// The fp32 direction 2u - 1 for u = n 2^-53, rounded once.
+__device__ __forceinline__ float mu_f32(uint64_t n) {
+  const long long w = (long long)(n << 1) - (1ll << 53);
+  if (w == 0) return 0.0f;
+  const float a = 2.0f * top_bits_to_float((uint64_t)(w < 0 ? -w : w) << 10);
+  return w < 0 ? -a : a;
+}
 
 // 2^32 / |mu| rounded once: 2^32 RN(1 / |mu|), the reciprocal on the
 // integer pipes (fp_exact.cuh), the scaling an exponent add.
@@ -451,10 +488,10 @@ __device__ __forceinline__ bool plain_collision32(const SlabDev& p, float muf, f
 
 // The end of a flight of the fp32 path by pair_step, and whether it leaves
 // the slab; near a face the leak-or-collide decision is made again in fp64
-// from the flight's uniform, uf() (called only there).
+// from the flight's uniform nf() 2^-53 (called only there).
 template <class UF>
 __device__ __forceinline__ int advance32(const SlabDev& p, float xf, float xlo, float muf, float pr, float pe,
-                                         UF uf, float& xn, float& xnlo) {
+                                         UF nf, float& xn, float& xnlo) {
   pair_step(xf, xlo, pr, pe, xn, xnlo);
   // Guard band: re-decide leak vs collide in fp64 near a face.
   const bool near_hi = muf > 0.0f && fabsf(xn - p.L_f) <= p.guard_f;
@@ -463,7 +500,7 @@ __device__ __forceinline__ int advance32(const SlabDev& p, float xf, float xlo, 
   bool leak_hi = muf > 0.0f && (xn > p.L_f || (xn == p.L_f && xnlo >= 0.0f));
   bool leak_lo = muf < 0.0f && (xn < 0.0f || (xn == 0.0f && xnlo <= 0.0f));
   if (near_hi || near_lo) {
-    const double d64 = __dmul_rn(-mclog::log1m(uf()), p.inv_st);
+    const double d64 = __dmul_rn(-mclog::log1m_n(nf()), p.inv_st);
     const double x64 = __dadd_rn((double)xf, (double)xlo);
     const double xn64 = __dadd_rn(x64, __dmul_rn(d64, (double)muf));
     leak_hi = muf > 0.0f && xn64 >= p.L;
@@ -503,12 +540,12 @@ __device__ __forceinline__ int slab_flight(const SlabDev& p, Rng<M>& r, const mc
     if (f == kCollide) q.x = xn;
     return f;
   } else {
-    const double u = r.next(l);
-    const float d = flight_f32(u) * p.inv_st_f;
+    const uint64_t n = r.next_n(l);
+    const float d = flight_f32(n) * p.inv_st_f;
     const float pr = __fmul_rn(d, q.muf);
     const float pe = __fmaf_rn(d, q.muf, -pr);
     float xn, xnlo;
-    const int f = advance32(p, q.xf, q.xlo, q.muf, pr, pe, [u] { return u; }, xn, xnlo);
+    const int f = advance32(p, q.xf, q.xlo, q.muf, pr, pe, [n] { return n; }, xn, xnlo);
     tally32(p, q.xf, q.xlo, xn, xnlo, q.muf, d, q.wf, f, s);
     if (f == kCollide) {
       q.xf = xn;
