@@ -34,7 +34,10 @@ __global__ void box_prep_kernel(BoxDev* __restrict__ p, uint32_t n) {
     b.hi_f = (float)b.hi;
     b.h_f = b.side_f / (float)b.mesh;
     b.inv_h_f = (float)b.mesh / b.side_f;
+    bool ok = b.side >= 0x1p-40 && b.side <= 0x1p40;
     for (int r = 0; r < 2; ++r) {
+      ok = ok && b.ws[r] >= 0x1p-60 && b.ws[r] <= 0x1p60;
+      b.inv_ws_f[r] = 1.0f / (float)b.ws[r];
       b.inv_st[r] = 1.0 / b.st[r];
       b.inv_st_f[r] = 1.0f / (float)b.st[r];
       b.c_f[r] = (float)b.c[r];
@@ -44,6 +47,7 @@ __global__ void box_prep_kernel(BoxDev* __restrict__ p, uint32_t n) {
       for (int g = 0; g < mcb::kMaxG; ++g)
         for (int k = 0; k < mcb::kMaxG; ++k) b.cdf_n[r][g][k] = mcb::cdf_threshold(b.cdf[r][g][k]);
     }
+    b.f32_ok = ok ? 1u : 0u;
     const uint64_t parent = b.seeding == MC_SEED_HASH_HIER ? mcd::hash64(b.key, b.seed) : b.seed;
     b.seed_hash = mcd::seed_hash_of(parent);
   }
@@ -112,8 +116,8 @@ constexpr uint32_t kCountProbs = 16;  // problems whose counters a block keeps i
 // warp.  Particle, walk and axis state are scalars in registers (no local
 // memory); a particle's counts go to its block's counters in shared memory
 // when it ends.  Four blocks per SM in fp32 (64 registers: 17.1 ms for 10^7
-// histories against 17.9 with three), three in fp64 (80: 21.0 ms for
-// 3 * 10^6 against 22.1 with four).
+// histories against 17.9 with three), three in fp64 (80: 16.0 ms for
+// 3 * 10^6 against 16.2 with four).
 template <int M, typename T, bool AGG>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) box_history_kernel(const BoxArgs a) {
   __shared__ mcd::Affine tab[64];

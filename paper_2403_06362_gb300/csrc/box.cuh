@@ -38,6 +38,8 @@ struct BoxDev {
   int ih_s;
   float side_f, lo_f, hi_f, h_f, inv_h_f;
   float inv_st_f[2], c_f[2], wl_f[2], wh_f[2], ws_f[2];
+  float inv_ws_f[2];
+  uint32_t f32_ok;  // extents and windows lie in the range of the fp32 decisions of the fp64 path
   uint64_t cdf_n[2][kMaxG][kMaxG];  // u < cdf  <=>  n < cdf_n for u = n 2^-53
   uint64_t seed_hash, hist_begin;
 };
@@ -77,6 +79,9 @@ template <> __device__ __forceinline__ float sel<float>(const double&, const flo
 // the fp64 comparisons for non-NaN values), fp32 native.
 __device__ __forceinline__ bool lt(double a, double b) { return mcx::d_lt(a, b); }
 __device__ __forceinline__ bool lt(float a, float b) { return a < b; }
+// the same for non-negative values (fp64: the bits order them)
+__device__ __forceinline__ bool ltn(double a, double b) { return mcs::nn_lt(a, b); }
+__device__ __forceinline__ bool ltn(float a, float b) { return a < b; }
 __device__ __forceinline__ bool eq(double a, double b) { return mcx::okey(a) == mcx::okey(b); }
 __device__ __forceinline__ bool eq(float a, float b) { return a == b; }
 __device__ __forceinline__ bool gt0(double a) { return mcx::d_pos(a); }
@@ -115,23 +120,41 @@ __device__ __forceinline__ void set_inv(Part<T>& q) {
 }
 
 // Marsaglia (1972): v1, v2 uniform on [-1,1)^2 until v1^2 + v2^2 < 1.
+// fp64: a try is decided in fp32 where v1^2 + v2^2 is not within 2^-19 of 1
+// (its fp32 value is off by less than 2^-21), so the fp64 unit forms s for
+// the accepted try alone; the square root is the integer pipes'.
 template <int M, typename T>
 __device__ __forceinline__ void iso_dir(mcs::Rng<M>& r, const mcd::Lcg& l, T u[3]) {
-  T v1, v2, s;
-  do {
-    if constexpr (sizeof(T) == 8) {  // 2u - 1 exactly, on the integer pipes
-      v1 = mcx::two_u_minus_1(r.next_n(l));
-      v2 = mcx::two_u_minus_1(r.next_n(l));
-    } else {
+  if constexpr (sizeof(T) == 8) {
+    uint64_t n1, n2;
+    for (;;) {
+      n1 = r.next_n(l);
+      n2 = r.next_n(l);
+      const float f1 = mcs::mu_f32(n1), f2 = mcs::mu_f32(n2);
+      const float s = f1 * f1 + f2 * f2 - 1.0f;
+      if (s < -0x1p-19f) break;
+      if (s > 0x1p-19f) continue;
+      const double v1 = mcx::two_u_minus_1(n1), v2 = mcx::two_u_minus_1(n2);
+      if (lt(v1 * v1 + v2 * v2, 1.0)) break;
+    }
+    const double v1 = mcx::two_u_minus_1(n1), v2 = mcx::two_u_minus_1(n2);
+    const double s = v1 * v1 + v2 * v2;
+    const double t = mcx::scale_pow2(mcx::sqrt_rn(1.0 - s), 1);  // (2 v) t = v (2 t): doubling is exact
+    u[0] = v1 * t;
+    u[1] = v2 * t;
+    u[2] = __fma_rn(-2.0, s, 1.0);  // 2 s is exact: one rounding either way
+  } else {
+    T v1, v2, s;
+    do {
       v1 = T(2) * from_n<T>(r.next_n(l)) - T(1);
       v2 = T(2) * from_n<T>(r.next_n(l)) - T(1);
-    }
-    s = v1 * v1 + v2 * v2;
-  } while (!lt(s, T(1)));
-  const T t = sqrt(T(1) - s);
-  u[0] = T(2) * v1 * t;
-  u[1] = T(2) * v2 * t;
-  u[2] = T(1) - T(2) * s;
+      s = v1 * v1 + v2 * v2;
+    } while (!lt(s, T(1)));
+    const T t = sqrt(T(1) - s);
+    u[0] = T(2) * v1 * t;
+    u[1] = T(2) * v2 * t;
+    u[2] = T(1) - T(2) * s;
+  }
 }
 
 template <typename T>
@@ -183,7 +206,7 @@ __device__ __forceinline__ T entry_dist(const Part<T>& q, T lo, T hi) {
 // Distance to the region surface and its kind (1: into the other region,
 // 2: out of the box).  Both regions share the code of the way out.
 template <typename T>
-__device__ __forceinline__ T surface(const BoxDev& b, const Part<T>& q, int& kind) {
+__device__ __forceinline__ T surface_of(const BoxDev& b, const Part<T>& q, int& kind) {
   const T lo = sel<T>(b.lo, b.lo_f), hi = sel<T>(b.hi, b.hi_f), side = sel<T>(b.side, b.side_f);
   const bool inner = q.region == 1u;
   T ds = exit_dist(q, inner ? lo : T(0), inner ? hi : side);
@@ -198,6 +221,85 @@ __device__ __forceinline__ T surface(const BoxDev& b, const Part<T>& q, int& kin
   return ds;
 }
 
+// surface_of in fp64, out of line: for the few flights that pass an edge too
+// closely for surface<double>'s fp32 decision.
+static __device__ __noinline__ double surface_exact(const BoxDev* b, const Part<double>* q, int* kind) {
+  return surface_of<double>(*b, *q, *kind);
+}
+
+template <typename T> __device__ __forceinline__ T surface(const BoxDev& b, const Part<T>& q, int& kind);
+template <> __device__ __forceinline__ float surface<float>(const BoxDev& b, const Part<float>& q, int& kind) {
+  return surface_of<float>(b, q, kind);
+}
+
+// fp64: which face the flight meets is decided in fp32, and only that face's
+// distance is formed in fp64 (2 operations instead of 18).  The fp32 distance
+// to a face ahead on axis a is off by less than e_a = |1/u_a| side 2^-20:
+// position (truncated), face and their difference are off by less than
+// 2^-22 side together, 1/u_a and the product by less than 2^-22 of a distance
+// that is at most |1/u_a| side.  Distances closer to each other than their
+// e's, a direction with a zero component and boxes outside the fp32 range go
+// to surface_exact.
+template <> __device__ __forceinline__ double surface<double>(const BoxDev& b, const Part<double>& q, int& kind) {
+  const bool inner = q.region == 1u;
+  const float xl = inner ? b.lo_f : 0.0f, xh = inner ? b.hi_f : b.side_f, eps = b.side_f * 0x1p-20f;
+  bool sure = b.f32_ok != 0u;
+  float t[3], e[3], p[3], inv[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    sure = sure && mcx::f32_range(q.inv[a]);
+    p[a] = mcx::f32_range(q.p[a]) ? mcx::f32_trunc(q.p[a]) : 0.0f;  // (out of the range: below 2^-120)
+    inv[a] = mcx::f32_trunc(q.inv[a]);
+    e[a] = fabsf(inv[a]) * eps;
+    t[a] = ((inv[a] < 0.0f ? xl : xh) - p[a]) * inv[a];
+  }
+  // the nearest face ahead, and the least the other two can be
+  const bool s1 = t[1] < t[0];
+  const float m1 = s1 ? t[1] : t[0], f1 = s1 ? e[1] : e[0], o1 = s1 ? t[0] - e[0] : t[1] - e[1];
+  const bool s2 = t[2] < m1;
+  const float m = s2 ? t[2] : m1, f = s2 ? e[2] : f1;
+  const float others = fminf(o1, s2 ? m1 - f1 : t[2] - e[2]);
+  int ax = s2 ? 2 : (s1 ? 1 : 0);
+  bool into = false;
+  bool clear = others > m + f;
+  if (!inner) {
+    float n[3], lo_far = INFINITY, hi_far = INFINITY;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const bool neg = inv[a] < 0.0f;
+      n[a] = ((neg ? b.hi_f : b.lo_f) - p[a]) * inv[a];
+      const float far = ((neg ? b.lo_f : b.hi_f) - p[a]) * inv[a];
+      lo_far = fminf(lo_far, far - e[a]);
+      hi_far = fminf(hi_far, far + e[a]);
+    }
+    // the last near face, and the most the other two can be
+    const bool r1 = n[1] > n[0];
+    const float k1 = r1 ? n[1] : n[0], g1 = r1 ? e[1] : e[0], h1 = r1 ? n[0] + e[0] : n[1] + e[1];
+    const bool r2 = n[2] > k1;
+    const float k = r2 ? n[2] : k1, g = r2 ? e[2] : g1;
+    const float rest = fmaxf(h1, r2 ? k1 + g1 : n[2] + e[2]);
+    const float hi_near = fmaxf(rest, k + g), lo_near = k - g;
+    const bool miss = hi_near < 0.0f || lo_near > hi_far;
+    const bool hit = lo_near > 0.0f && rest < lo_near && hi_near < lo_far && hi_near < fminf(others, m - f);
+    into = hit;
+    clear = hit || (miss && clear);
+    if (hit) ax = r2 ? 2 : (r1 ? 1 : 0);
+  }
+  if (!(sure && clear)) {
+    const Part<double> c = q;
+    return surface_exact(&b, &c, &kind);
+  }
+  kind = inner || into ? 1 : 2;
+  const double pa = ax == 2 ? q.p[2] : (ax == 1 ? q.p[1] : q.p[0]);
+  const double ia = ax == 2 ? q.inv[2] : (ax == 1 ? q.inv[1] : q.inv[0]);
+  // the face ahead of the particle (the near one of the inner cube, the far
+  // one of the region it is in)
+  const bool low = lt0(ia) != into;
+  const double face = inner || into ? (low ? b.lo : b.hi) : (low ? 0.0 : b.side);
+  const double ds = (face - pa) * ia;
+  return lt0(ds) ? 0.0 : ds;
+}
+
 __device__ __forceinline__ long long fix_of(double wl) { return mcx::fix32_nonneg(wl); }
 __device__ __forceinline__ long long fix_of(float wl) { return mcs::fix32_from_float(wl); }
 
@@ -208,9 +310,10 @@ constexpr int kMaxPlanes = MC_BOX_MAX_MESH + 1;
 __device__ __forceinline__ double plane_of(const BoxDev& b, int j) {
   return j >= (int)b.mesh ? b.side : mcx::mul_small((uint32_t)j, b.h);
 }
+static __device__ __noinline__ double plane_call(const BoxDev* b, int j) { return plane_of(*b, j); }
 template <typename T> __device__ __forceinline__ T plane(const BoxDev& b, const double* tab, int j);
 template <> __device__ __forceinline__ double plane<double>(const BoxDev& b, const double* tab, int j) {
-  return tab ? tab[j] : plane_of(b, j);
+  return tab ? tab[j] : plane_call(&b, j);
 }
 template <> __device__ __forceinline__ float plane<float>(const BoxDev& b, const double*, int j) {
   return j >= (int)b.mesh ? b.side_f : (float)j * b.h_f;
@@ -247,13 +350,15 @@ __device__ __forceinline__ int walk_axis(const BoxDev& b, const double* tab, int
   i = i < 0 ? 0 : (i >= nm ? nm - 1 : i);
   T lo = plane<T>(b, tab, i), hi = plane<T>(b, tab, i + 1);
   const bool neg = lt0(u);
-  if ((i > 0 && !lt(lo, p)) || (i + 1 < nm && !lt(p, hi))) {
+  if ((i > 0 && !ltn(lo, p)) || (i + 1 < nm && !ltn(p, hi))) {
     while (i > 0 && lt(p, lo)) { hi = lo; lo = plane<T>(b, tab, --i); }
     while (i + 1 < nm && !lt(p, hi)) { lo = hi; hi = plane<T>(b, tab, ++i + 1); }
     if (neg && i > 0 && eq(p, lo)) lo = plane<T>(b, tab, --i);
   }
   j = neg ? i : i + 1;
-  tn = is0(u) ? T(INFINITY) : ((neg ? lo : hi) - p) * inv;
+  tn = ((neg ? lo : hi) - p) * inv;
+  if (lt0(tn)) tn = T(0);  // p beyond the plane by a rounding: an empty piece either way
+  if (is0(u)) tn = T(INFINITY);
   return i;
 }
 
@@ -277,14 +382,14 @@ __device__ __forceinline__ void walk_begin(const BoxDev& b, const Part<T>& q, T 
 template <typename T>
 __device__ __forceinline__ bool walk_step(const BoxDev& b, const Part<T>& q, Walk<T>& k, unsigned long long* base,
                                           const double* tab, bool agg) {
-  const bool y = lt(k.tn1, k.tn0);
+  const bool y = ltn(k.tn1, k.tn0);
   const T t01 = y ? k.tn1 : k.tn0;
-  const bool z = lt(k.tn2, t01);
+  const bool z = ltn(k.tn2, t01);
   const T ta = z ? k.tn2 : t01;
-  const bool inside = lt(ta, k.L);
+  const bool inside = ltn(ta, k.L);
   const T tend = inside ? ta : k.L;
   const unsigned long long v = (unsigned long long)fix_of(q.w * (tend - k.t));
-  if (lt(k.t, tend)) {
+  if (ltn(k.t, tend)) {
     if (agg) mcd::warp_agg_add(base + k.slot, v);
     else atomicAdd(base + k.slot, v);
     k.t = tend;
@@ -336,7 +441,7 @@ static __device__ __noinline__ int decide_f64(const BoxDev* b, float p0, float p
   for (int a = 0; a < 3; ++a) q.inv[a] = q.u[a] != 0.0 ? mcx::recip_rn(q.u[a]) : 0.0;
   q.region = region;
   int kind = 0;
-  const double ds = surface<double>(*b, q, kind);
+  const double ds = surface_of<double>(*b, q, kind);
   const double d = -mclog::log1m_n(n) * b->inv_st[region];
   return (d < ds ? 1 : 0) | (kind << 1);
 }
@@ -428,7 +533,19 @@ __device__ __forceinline__ int weight_window(const BoxDev& b, mcs::Rng<M>& r, co
   const T wl = sel<T>(b.wl[rg], b.wl_f[rg]), wh = sel<T>(b.wh[rg], b.wh_f[rg]);
   if (lt(q.w, wl)) {
     const T ws = sel<T>(b.ws[rg], b.ws_f[rg]);
-    if (lt(from_n<T>(r.next_n(l)), q.w / ws)) {
+    const uint64_t n = r.next_n(l);
+    bool survives;
+    if constexpr (sizeof(T) == 8) {
+      // u < w / ws, decided in fp32 (each side off by less than a relative
+      // 2^-21) unless the two are within a relative 2^-20
+      const float u = mcs::u53_to_float(n), v = mcx::f32_trunc(q.w) * b.inv_ws_f[rg];
+      survives = u < v * (1.0f - 0x1p-20f);
+      if (!b.f32_ok || !mcx::f32_range(q.w) || (!survives && !(u > v * (1.0f + 0x1p-20f))))
+        survives = lt(from_n<T>(n), q.w / ws);
+    } else {
+      survives = from_n<T>(n) < q.w / ws;
+    }
+    if (survives) {
       q.w = ws;
       return kBoxContinue;
     }

@@ -10,6 +10,7 @@
 //   floor_nonneg   floor(t) for 0 <= t < 2^63
 //   abs_le         |x| <= h for h >= 0
 //   recip_rn       1/y correctly rounded (IEEE round to nearest even)
+//   sqrt_rn        sqrt(x) correctly rounded
 //   llrint_nonneg  llrint(v) for 0 <= v < 2^62
 //   okey, d_lt ..  comparisons of doubles (sign-magnitude order keys)
 //   mul_small      RN(j h) for a small integer j
@@ -140,6 +141,55 @@ __host__ __device__ __forceinline__ double recip_rn(double y) {
   if (frac == 0ull) return from_bits(sign | ((uint64_t)(2046u - E) << 52));  // a power of two
   const uint64_t q = recip_mantissa(frac | (1ull << 52));  // in [2^52, 2^53)
   return from_bits(sign | (((uint64_t)(2045u - E) << 52) + (q - (1ull << 52))));
+}
+
+// RN(sqrt(x)) for a positive normal x.  With x = A 2^(2k - 64), A in
+// [2^62, 2^64), the result is RN(sqrt(N)) 2^(k - 53), N = A 2^42.  An fp32
+// reciprocal square root y (relative error below 2^-20) gives sqrt(A) with
+// scale 2^63, and two steps s += (x - s^2) y / 2 on 64-bit products, each
+// shrinking the error by y's own, leave it below 2^-59; rounded to 53 bits
+// it is within one unit, and the exact remainder N - q^2 (its low word: it is
+// far below 2^63) rounds it.  A tie cannot occur: (q + 1/2)^2 is no integer.
+// About 75 integer instructions; the fp64 unit's square root is a dozen of
+// its own, 16 cycles per SM and warp each.
+__host__ __device__ __forceinline__ double sqrt_rn(double x) {
+  const uint64_t b = to_bits(x);
+  const int E = (int)(b >> 52);  // positive: no sign
+  const uint64_t m = (b & ((1ull << 52) - 1ull)) | (1ull << 52);
+  const int odd = (E + 1) & 1;   // E - 1023 odd: one more doubling
+  const uint64_t A = m << (10 + odd);
+  const int k = (E - 1023 - odd) / 2 + 1;  // x = A 2^(2k - 64), E - 1023 - odd even
+  const uint32_t ah = (uint32_t)(A >> 32);
+#ifdef __CUDA_ARCH__
+  const float y0 = rsqrtf(__uint2float_rn(ah) * 0x1p-32f);
+  const uint32_t y = __float2uint_rz(fminf(y0 * 0x1p31f, 4294967040.0f));
+#else
+  const float y0 = 1.0f / std::sqrt((float)ah * 0x1p-32f);
+  const uint32_t y = y0 * 0x1p31f < 4294967040.0f ? (uint32_t)(y0 * 0x1p31f) : 4294967040u;
+#endif
+  uint64_t s = mulhi64(A, (uint64_t)y << 32);  // sqrt(x) 2^63
+  long long d = (long long)((A >> 2) - mulhi64(s, s));  // (x - s^2) 2^62, below 2^44
+  s += (uint64_t)(((d >> 13) * (long long)y) >> 18);
+  d = (long long)((A >> 2) - mulhi64(s, s));  // below 2^24
+  s += (uint64_t)((d * (long long)y) >> 31);
+  uint64_t q = (s + 512ull) >> 10;
+  const long long rem = (long long)((A << 42) - q * q);
+  if (rem > (long long)q) ++q;
+  else if (rem <= -(long long)q) --q;
+  // q in [2^52, 2^53]: the leading 1 (or the carry) adds into the exponent
+  return from_bits(((uint64_t)(k + 1021) << 52) + q);
+}
+
+// A double's leading bits as an fp32 (truncated: relative error below 2^-23),
+// |x| in [2^-120, 2^120], and whether x is in that range.
+__host__ __device__ __forceinline__ bool f32_range(double x) {
+  const uint32_t e = (uint32_t)(raw_bits(x) >> 52) & 0x7ffu;
+  return e - 903u <= 240u;
+}
+__device__ __forceinline__ float f32_trunc(double x) {
+  const uint64_t b = raw_bits(x);
+  const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
+  return __uint_as_float((hi & 0x80000000u) | ((((hi & 0x7fffffffu) << 3) | (lo >> 29)) - (896u << 23)));
 }
 
 // llrint(v) (round half to even) for 0 <= v < 2^62, from the bits.
