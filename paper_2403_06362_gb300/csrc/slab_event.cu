@@ -545,9 +545,10 @@ int slab_event_run_t(const mci::SlabLaunch& L, void* d_bank, uint32_t cap, unsig
   a.hist_draws = L.tally->d_hist_draws;
   a.lcg = mcd::Lcg{L.lcg.g, L.lcg.c, mcd::mask_of(L.lcg.m), L.lcg.m};
   a.event_cap = L.event_cap;
-  // One problem with at most 4095 bins: its edge and width tables in shared
-  // memory; otherwise each problem's tables in global memory.
-  a.smem_edges = (L.n_problems == 1 && L.single_n_bins + 1 <= 4096) ? L.single_n_bins + 1 : 0u;
+  // One problem with at most 3071 bins: its edge and width tables in shared
+  // memory (48 KiB, what a launch may ask for without opting in); otherwise
+  // each problem's tables in global memory.
+  a.smem_edges = (L.n_problems == 1 && L.single_n_bins + 1 <= 3072) ? L.single_n_bins + 1 : 0u;
   a.tables = a.smem_edges ? nullptr : static_cast<const double*>(L.d_tables);
   a.smem_counts = (L.n_problems > 1 && L.n_problems <= kSmemCountProblems) ? 1u : 0u;
   a.order = mcs::Order{L.d_order, L.d_order_begin};
