@@ -92,7 +92,7 @@ __device__ __forceinline__ bool is0(double a) { return mcx::d_zero(a); }
 __device__ __forceinline__ bool is0(float a) { return a == 0.0f; }
 
 template <typename T> __device__ __forceinline__ T recip(T v);
-template <> __device__ __forceinline__ double recip<double>(double v) { return mcx::recip_rn(v); }
+template <> __device__ __forceinline__ double recip<double>(double v) { return mcx::recip_normal(v); }
 template <> __device__ __forceinline__ float recip<float>(float v) { return __frcp_rn(v); }
 
 // Componentwise inverse of the direction (fp64: the correctly rounded
@@ -106,7 +106,7 @@ __device__ __forceinline__ void set_inv(Part<T>& q) {
   T u0 = q.u[0], u1 = q.u[1], u2 = q.u[2], i0 = T(0), i1 = T(0), i2 = T(0);
 #pragma unroll 1
   for (int a = 0; a < 3; ++a) {
-    const T v = !is0(u0) ? recip<T>(u0) : T(0), r = u0;
+    const T i = recip<T>(u0), v = is0(u0) ? T(0) : i, r = u0;  // |u0| >= 2^-78 otherwise
     u0 = u1;
     u1 = u2;
     u2 = r;
@@ -442,7 +442,7 @@ static __device__ __noinline__ int decide_f64(const BoxDev* b, float p0, float p
   q.region = region;
   int kind = 0;
   const double ds = surface_of<double>(*b, q, kind);
-  const double d = -mclog::log1m_n(n) * b->inv_st[region];
+  const double d = mclog::neglog1m_n(n) * b->inv_st[region];
   return (d < ds ? 1 : 0) | (kind << 1);
 }
 
@@ -456,7 +456,7 @@ __device__ __forceinline__ int flight_length(const BoxDev& b, mcs::Rng<M>& r, co
   bool collide;
   T d;
   if constexpr (sizeof(T) == 8) {
-    d = -mclog::log1m_n(r.next_n(l)) * b.inv_st[q.region];
+    d = mclog::neglog1m_n(r.next_n(l)) * b.inv_st[q.region];
     collide = lt(d, ds);
   } else {
     const uint64_t n = r.next_n(l);

@@ -54,14 +54,20 @@ __host__ __device__ __forceinline__ float rcp_f32(float x) {
 // exact (|2n - 2^53| <= 2^53), +0 for n = 2^52.
 __host__ __device__ __forceinline__ double two_u_minus_1(uint64_t n) {
   const long long w = (long long)(n << 1) - (1ll << 53);
-  if (w == 0) return 0.0;
-  const uint64_t sign = w < 0 ? (1ull << 63) : 0ull;
-  const uint64_t a = w < 0 ? (uint64_t)(-w) : (uint64_t)w;  // 2 .. 2^53
-  if (a == (1ull << 53)) return -1.0;
-  const int lz = clz64(a);  // 11 .. 62
-  // leading 1 moved to bit 52; it carries into the exponent field, so the
-  // word to add is (biased exponent - 1) << 52 with biased = 1033 - lz
-  return from_bits(sign | ((a << (lz - 11)) + ((uint64_t)(1032 - lz) << 52)));
+  const uint64_t sign = (uint64_t)w & (1ull << 63);
+  const uint64_t z = (uint64_t)(w < 0 ? -w : w) << 10;  // |w|, at most 2^53, at the top of the word
+  const uint32_t zh = (uint32_t)(z >> 32), zl = (uint32_t)z;
+  if (zh == 0u) {  // |2u - 1| < 2^-31 (or 0)
+    if (z == 0ull) return 0.0;
+    const int lz = clz64(z);
+    return from_bits(sign | (((z << lz) >> 11) + ((uint64_t)(1022 - lz) << 52)));
+  }
+  // the leading 1 moved to bit 63, then to bit 52, where it adds one to the
+  // exponent field
+  const uint32_t lz = mclog::clz32_(zh);
+  const uint32_t mh = mclog::fsr32_(zl, zh, 32u - lz), ml = zl << lz;
+  const uint64_t m = (((uint64_t)mh << 32) | ml) >> 11;
+  return from_bits(sign | (m + ((uint64_t)(1022u - lz) << 52)));
 }
 
 // floor(t) for 0 <= t < 2^63 (t finite, not negative zero excluded).
@@ -98,8 +104,8 @@ __host__ __device__ __forceinline__ bool abs_le(double x, double h) {
   return mag_bits(x) <= to_bits(h);
 }
 
-// q = RN(2^105 / M) for 2^52 < M < 2^53 (ties cannot occur: 2^106 = (2q + 1) M
-// would make M a power of two).  With m = M 2^-52 = F (1 + r), F = 1 + j/1024
+// q = RN(2^105 / M) for 2^52 <= M < 2^53 (ties cannot occur: 2^106 = (2q + 1) M
+// would make M a power of two, and M = 2^52 divides exactly).  With m = M 2^-52 = F (1 + r), F = 1 + j/1024
 // the left end of m's cell (the table of 2^63 / F that the logarithm uses)
 // and 0 <= r < 2^-10,
 //   2^53 / m = (2^53 / F) (1 - r (1 - r (1 - r (1 - r (1 - r))))) + O(r^6 < 2^-60)
@@ -123,8 +129,10 @@ __host__ __device__ __forceinline__ uint64_t recip_mantissa(uint64_t M) {
   uint64_t q = mclog::umulhi_(inv, S) >> 9;                                // ~ 2^53 / m
   // exact remainder r = 2^105 - q M (|r| < 2^63: the low words decide), then round
   long long rem = (long long)(0ull - q * M);
-  for (int i = 0; i < 4 && rem < 0; ++i) { --q; rem += (long long)M; }
-  for (int i = 0; i < 4 && rem >= (long long)M; ++i) { ++q; rem -= (long long)M; }
+  // (q's error: its truncation and below 2^-6 of a unit before it, so one
+  // correction either way is enough)
+  if (rem < 0) { --q; rem += (long long)M; }
+  if (rem >= (long long)M) { ++q; rem -= (long long)M; }
   if ((uint64_t)rem * 2ull > M) ++q;
   return q;
 }
@@ -192,15 +200,25 @@ __device__ __forceinline__ float f32_trunc(double x) {
   return __uint_as_float((hi & 0x80000000u) | ((((hi & 0x7fffffffu) << 3) | (lo >> 29)) - (896u << 23)));
 }
 
+// RN(1 / y) for a normal y with a normal reciprocal, biased exponent
+// 1..2044 (a flight direction's component, say), without branches.
+__host__ __device__ __forceinline__ double recip_normal(double y) {
+  const uint64_t b = to_bits(y);
+  const uint64_t q = recip_mantissa((b & ((1ull << 52) - 1ull)) | (1ull << 52));  // in [2^52, 2^53]
+  const uint32_t E = (uint32_t)(b >> 52) & 0x7FFu;
+  return from_bits((b & (1ull << 63)) + ((uint64_t)(2044u - E) << 52) + q);
+}
+
 // llrint(v) (round half to even) for 0 <= v < 2^62, from the bits.
 __host__ __device__ __forceinline__ long long llrint_nonneg(double v) {
   const uint64_t b = to_bits(v);
-  const int e = (int)(b >> 52) - 1023;
-  if (e < -1) return 0;  // v < 1/2
+  const int E = (int)(b >> 52);  // biased exponent: v = m 2^(E - 1075)
   const uint64_t m = (b & ((1ull << 52) - 1ull)) | (1ull << 52);
-  if (e >= 52) return (long long)(m << (e - 52));
-  const int sh = 52 - e;  // 1..53
-  const uint64_t q = m >> sh, rem = m & ((1ull << sh) - 1ull), half = 1ull << (sh - 1);
+  if (E >= 1075) return (long long)(m << (E - 1075));
+  // at most 63: below 1/2 (and zero) everything is shifted out, less than a half
+  const int sh = 1075 - E < 63 ? 1075 - E : 63;
+  const uint64_t q = m >> sh, rem = m << (64 - sh);  // rem: the bits shifted out, at the top
+  const uint64_t half = 1ull << 63;
   return (long long)(q + ((rem > half || (rem == half && (q & 1ull))) ? 1ull : 0ull));
 }
 

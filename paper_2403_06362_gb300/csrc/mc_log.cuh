@@ -14,7 +14,7 @@
 // 64-bit reciprocal of F (scale 2^73), ln(1 + r) comes from its series
 // through r^6 by Horner's rule on non-negative fixed point (the inner terms
 // on 32 bits, the outer two on 64), and the sum is
-// accumulated on 128 bits with scale 2^90 (ln 2 and ln F from 128-bit
+// accumulated on 96 bits with scale 2^90 (ln 2 and ln F from 128-bit
 // tables).  For u < 2^-8 (x so close to 1 that e ln 2 + ln F would cancel)
 // -ln(1 - u) = u (1 + u/2 + ... + u^8/9) is used instead, relative to u.
 // The absolute error before the final rounding is below 2^-66 while the
@@ -96,41 +96,12 @@ struct W128 {
   uint64_t lo, hi;
 };
 
-__host__ __device__ __forceinline__ W128 add128(W128 a, W128 b) {
-  W128 r;
-  r.lo = a.lo + b.lo;
-  r.hi = a.hi + b.hi + (r.lo < a.lo ? 1ull : 0ull);
-  return r;
-}
-
-__host__ __device__ __forceinline__ W128 sub128(W128 a, W128 b) {
-  W128 r;
-  r.lo = a.lo - b.lo;
-  r.hi = a.hi - b.hi - (a.lo < b.lo ? 1ull : 0ull);
-  return r;
-}
-
-__host__ __device__ __forceinline__ int mulhi32_(int a, int b) {
-#ifdef __CUDA_ARCH__
-  return __mulhi(a, b);
-#else
-  return (int)(((long long)a * b) >> 32);
-#endif
-}
-
 __host__ __device__ __forceinline__ uint32_t umulhi32_(uint32_t a, uint32_t b) {
 #ifdef __CUDA_ARCH__
   return __umulhi(a, b);
 #else
   return (uint32_t)(((uint64_t)a * b) >> 32);
 #endif
-}
-
-__host__ __device__ __forceinline__ W128 neg128(W128 a) {
-  W128 r;
-  r.lo = 0ull - a.lo;
-  r.hi = ~a.hi + (a.lo == 0ull ? 1ull : 0ull);
-  return r;
 }
 
 // a 2^-scale as the nearest double (round half to even), a > 0, the result
@@ -163,8 +134,6 @@ __host__ __device__ __forceinline__ double w128_to_double(W128 a, int scale) {
   return from_bits(((biased - 1ull) << 52) + m53);  // the leading 1 adds one to the exponent
 }
 
-// The same for 2^82 <= a < 2^96, on the three low 32-bit words (the high
-// word is below 2^32), without branches.
 __host__ __device__ __forceinline__ uint32_t clz32_(uint32_t x) {
 #ifdef __CUDA_ARCH__
   return (uint32_t)__clz((int)x);
@@ -180,71 +149,112 @@ __host__ __device__ __forceinline__ uint32_t fsr32_(uint32_t lo, uint32_t hi, ui
   return (uint32_t)((((uint64_t)hi << 32) | lo) >> s);
 #endif
 }
-__host__ __device__ __forceinline__ double w128_to_double_hi(W128 a, int scale) {
-  const uint32_t h = (uint32_t)a.hi, l1 = (uint32_t)(a.lo >> 32), l0 = (uint32_t)a.lo;
-  const int top = 95 - (int)clz32_(h);  // 82..95
-  const uint32_t sh = (uint32_t)(top - 63);  // 19..32
-  const uint64_t m64 = ((uint64_t)fsr32_(l1, h, sh) << 32) | fsr32_(l0, l1, sh);  // bits sh..sh+63
-  const bool sticky = (l0 << (32u - sh)) != 0u;  // any of the bits below sh
-  uint64_t m53 = m64 >> 11;
-  const uint64_t rest = m64 & 0x7FFull;
-  if (rest > 0x400ull || (rest == 0x400ull && (sticky || (m53 & 1ull)))) ++m53;
-  return from_bits(((uint64_t)(top - scale + 1022) << 52) + m53);
+
+// A 96-bit integer on three words (a carry chain of three instructions per
+// subtraction; pairs of 64-bit words would compare for each borrow).
+struct W96 {
+  uint32_t w0, w1, w2;
+};
+__host__ __device__ __forceinline__ W96 sub96(W96 a, W96 b) {
+  W96 r;
+#ifdef __CUDA_ARCH__
+  asm("sub.cc.u32 %0, %3, %6;\n\tsubc.cc.u32 %1, %4, %7;\n\tsubc.u32 %2, %5, %8;"
+      : "=r"(r.w0), "=r"(r.w1), "=r"(r.w2)
+      : "r"(a.w0), "r"(a.w1), "r"(a.w2), "r"(b.w0), "r"(b.w1), "r"(b.w2));
+#else
+  const uint64_t lo = (((uint64_t)a.w1 << 32) | a.w0), bl = (((uint64_t)b.w1 << 32) | b.w0), d = lo - bl;
+  r.w0 = (uint32_t)d;
+  r.w1 = (uint32_t)(d >> 32);
+  r.w2 = a.w2 - b.w2 - (lo < bl ? 1u : 0u);
+#endif
+  return r;
 }
 
-// ln(1 - u) for u = n 2^-53, 0 <= n < 2^53: a double <= 0 (+0 for n = 0).
-__host__ __device__ __forceinline__ double log1m_n(uint64_t n) {
+// a 2^-scale as the nearest double (round half to even) for
+// 2^82 <= a < 2^96, without branches.
+__host__ __device__ __forceinline__ double w96_to_double(W96 a, int scale) {
+  const int top = 95 - (int)clz32_(a.w2);  // 82..95
+  const uint32_t sh = (uint32_t)(top - 63);  // 19..32
+  const uint32_t mh = fsr32_(a.w1, a.w2, sh), ml = fsr32_(a.w0, a.w1, sh);  // bits sh..sh+63, leading 1 at the top
+  const uint32_t sticky = (a.w0 << (32u - sh)) != 0u ? 1u : 0u;  // any of the bits below sh
+  const uint64_t m53 = (((uint64_t)mh << 32) | ml) >> 11;
+  // the 11 bits below the last, with the sticky bit: up above a half, and at
+  // a half when the last bit is odd
+  const uint32_t up = (((ml & 0x7ffu) | sticky) + 0x3ffu + ((uint32_t)m53 & 1u)) >> 11;
+  return from_bits(((uint64_t)(uint32_t)(top - scale + 1022) << 52) + m53 + up);
+}
+
 #ifdef __CUDA_ARCH__
-  using namespace dev;
-#define MC_LOG_LD(a, i) __ldg(&(a)[(i)])
+#define MC_LOG_NS dev
+#define MC_LOG_LD(a, i) __ldg(&MC_LOG_NS::a[(i)])
 #else
-  using namespace host;
-#define MC_LOG_LD(a, i) (a)[(i)]
+#define MC_LOG_NS host
+#define MC_LOG_LD(a, i) MC_LOG_NS::a[(i)]
 #endif
-  if (n < (1ull << 45)) {  // u < 2^-8: -u (1 + u/2 + ... + u^8/9)
-    if (n == 0ull) return 0.0;
-    const long long U = (long long)(n << 18);  // u 2^71
-    long long t = kLn1mB[8];
+
+// -ln(1 - u) where the straight-line form below does not hold: u < 2^-8, by
+// u (1 + u/2 + ... + u^8/9) (0 for u = 0), and 1 - u < 2^-21, through the
+// same table form with its normalisation on 64 bits.
+__host__ __device__ __forceinline__ double neglog1m_small(uint64_t n) {
+  if (n == 0ull) return 0.0;
+  const long long U = (long long)(n << 18);  // u 2^71
+  long long t = MC_LOG_NS::kLn1mB[8];
 #pragma unroll
-    for (int k = 7; k >= 0; --k) t = kLn1mB[k] + (smulhi_(U, t) >> 7);  // scale 2^62
-    W128 p;
-    p.lo = n * (uint64_t)t;
-    p.hi = umulhi_(n, (uint64_t)t);  // n t = -ln(1 - u) 2^115
-    return -w128_to_double(p, 115);
-  }
-  const uint64_t K = (1ull << 53) - n;  // x = K 2^-53, 1 <= K < 2^53 - 2^45
-  const int lz = clz64_(K);             // 12..63
-  const int e = 10 - lz;                // x = 2^e m
-  const uint64_t mant = K << (lz - 11);  // m 2^52, leading 1 at bit 52
-  const int j = (int)((mant >> 42) & (uint64_t)(kLogCells - 1));  // m in [F_j, F_j + 2^-10)
+  for (int k = 7; k >= 0; --k) t = MC_LOG_NS::kLn1mB[k] + (smulhi_(U, t) >> 7);  // scale 2^62
+  W128 p;
+  p.lo = n * (uint64_t)t;
+  p.hi = umulhi_(n, (uint64_t)t);  // n t = -ln(1 - u) 2^115
+  return w128_to_double(p, 115);
+}
+
+// The table form: -ln x for x = 2^-ae mant 2^-52, ae >= 1, mant's leading 1 at
+// bit 52 (and x < 1 - 2^-8, or the result is not used).
+__host__ __device__ __forceinline__ double neglog1m_table(uint64_t mant, uint32_t ae) {
+  const int j = (int)((mant >> 42) & (uint64_t)(MC_LOG_NS::kLogCells - 1));  // m in [F_j, F_j + 2^-10)
   const uint64_t D = mant & ((1ull << 42) - 1ull);                // (m - F_j) 2^52, exact
   const uint64_t R = umulhi_(D << 22, MC_LOG_LD(kInvF, j));       // r 2^73 (2^63 / F_j in the table)
   // ln(1 + r) = r P, P = 1 - r Q0, Q0 = 1/2 - r Q1, Q1 = 1/3 - r Q2, Q2 = 1/4 - r Q3,
   // Q3 = 1/5 - r/6 (the r^7 term is below 2^-72): r and Q3, Q2 and Q1 - 85/256
   // on 32 bits, Q0 and P on 64 (scale 2^63); every quantity is non-negative.
   const uint32_t r32 = (uint32_t)(R >> 31);                        // r 2^42
-  uint32_t q = kQ3 - (umulhi32_(r32, kQ4) >> 10);                  // Q3 2^32
+  uint32_t q = MC_LOG_NS::kQ3 - (umulhi32_(r32, MC_LOG_NS::kQ4) >> 10);  // Q3 2^32
   q = (1u << 30) - (umulhi32_(r32, q) >> 10);                      // Q2 2^32
-  q = kQ1B - (umulhi32_(r32, q) >> 1);                             // (Q1 - 85/256) 2^41
+  q = MC_LOG_NS::kQ1B - (umulhi32_(r32, q) >> 1);                  // (Q1 - 85/256) 2^41
   const uint64_t rq = ((uint64_t)(uint32_t)(R >> 32) * q + (((uint64_t)(uint32_t)R * q) >> 32)) >> 19;
   const uint64_t q0 = (1ull << 62) - (((R >> 10) * 85ull) >> 8) - rq;  // Q0 2^63
   const uint64_t P = (1ull << 63) - (umulhi_(R, q0) >> 9);            // P 2^63
   const uint64_t p72 = umulhi_(R, P);                                 // ln(1 + r) 2^72
-  W128 p;
-  p.lo = p72 << 18;
-  p.hi = p72 >> 46;
-  // -ln x = |e| ln 2 - ln F - ln(1 + r) > 2^-8, on 128 bits with scale 2^90
-  const uint64_t ae = (uint64_t)(-e);
-  W128 a;
-  a.lo = ae * kLn2Lo;
-  a.hi = umulhi_(ae, kLn2Lo) + ae * kLn2Hi;
-  W128 f;
-  f.lo = MC_LOG_LD(kLnFLo, j);
-  f.hi = MC_LOG_LD(kLnFHi, j);
-  a = sub128(sub128(a, f), p);
-#undef MC_LOG_LD
-  return -w128_to_double_hi(a, 90);
+  const W96 p{(uint32_t)p72 << 18, (uint32_t)(p72 >> 14), (uint32_t)(p72 >> 46)};
+  // -ln x = ae ln 2 - ln F - ln(1 + r) > 2^-8, on 96 bits with scale 2^90
+  const uint64_t a0 = (uint64_t)ae * (uint32_t)MC_LOG_NS::kLn2Lo;
+  const uint64_t a1 = (uint64_t)ae * (uint32_t)(MC_LOG_NS::kLn2Lo >> 32) + (a0 >> 32);
+  const W96 a{(uint32_t)a0, (uint32_t)a1, ae * (uint32_t)MC_LOG_NS::kLn2Hi + (uint32_t)(a1 >> 32)};
+  const uint64_t fl = MC_LOG_LD(kLnFLo, j);
+  const W96 f{(uint32_t)fl, (uint32_t)(fl >> 32), (uint32_t)MC_LOG_LD(kLnFHi, j)};
+  return w96_to_double(sub96(sub96(a, f), p), 90);
 }
+
+// -ln(1 - u) for u = n 2^-53, 0 <= n < 2^53: a double >= 0 (the sign is the
+// flight distance's, so that no negation is left for the fp64 unit).
+// The table form runs for every lane without a branch, so that its chain can
+// be interleaved with independent work of the caller; the arguments it does
+// not cover (one in 256) are done again after it.
+__host__ __device__ __forceinline__ double neglog1m_n(uint64_t n) {
+  const uint64_t K = (1ull << 53) - n;  // x = K 2^-53, 1 <= K <= 2^53
+  const uint32_t kh = (uint32_t)(K >> 32), kl = (uint32_t)K;
+  const uint32_t lz = clz32_(kh);       // 11..31 where used
+  const uint32_t s = (lz - 11u) & 31u;
+  double v = neglog1m_table(((uint64_t)fsr32_(kl, kh, 32u - s) << 32) | (uint32_t)(kl << s), lz - 10u);
+  if (n < (1ull << 45)) {
+    v = neglog1m_small(n);
+  } else if (kh == 0u) {
+    const int z = clz64_(K);  // 32..63
+    v = neglog1m_table(K << (z - 11), (uint32_t)(z - 10));
+  }
+  return v;
+}
+#undef MC_LOG_LD
+#undef MC_LOG_NS
 
 // ln(1 - u) for a double u = n 2^-53 in [0, 1) (every uniform of the library).
 __host__ __device__ __forceinline__ double log1m(double u) {
@@ -252,7 +262,7 @@ __host__ __device__ __forceinline__ double log1m(double u) {
   if (b == 0ull) return 0.0;
   const int e = (int)(b >> 52) - 1023;  // u = (1.f) 2^e, e in [-53, -1]
   const uint64_t m = (b & ((1ull << 52) - 1ull)) | (1ull << 52);
-  return log1m_n(m >> (-e - 1));  // n = u 2^53 = m 2^(e + 1)
+  return -neglog1m_n(m >> (-e - 1));  // n = u 2^53 = m 2^(e + 1)
 }
 
 }  // namespace mclog

@@ -281,7 +281,7 @@ __global__ void __maxnreg__(96) pulse_census_kernel(const CensusArgs a) {
     } else {
       ++events;
       ++lc.flights;
-      const double d = -mclog::log1m_n(r.next_n(l)) * P.inv_st;
+      const double d = mclog::neglog1m_n(r.next_n(l)) * P.inv_st;
       const double tn = t + d;
       if (!mcs::nn_lt(tn, a.tp)) {  // tn >= T_p, both non-negative
         ended = true;

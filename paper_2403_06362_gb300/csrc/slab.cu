@@ -151,12 +151,10 @@ __device__ __forceinline__ void pool_unlock(int* lk) {
   atomicExch(lk, 0);
 }
 
-template <int M>
-__device__ __forceinline__ void pool_put(unsigned long long* e, const mcs::Rng<M>& r,
-                                         const mcs::SlabParticle& q, uint64_t gi, uint64_t events,
-                                         uint32_t pi) {
-  e[0] = r.x;
-  e[1] = r.draws;
+__device__ __forceinline__ void pool_put(unsigned long long* e, uint64_t x, const mcs::SlabParticle& q, uint64_t gi,
+                                         uint64_t events, uint32_t pi) {
+  e[0] = x;
+  e[1] = (unsigned long long)(uint32_t)q.j;
   e[2] = (unsigned long long)__double_as_longlong(q.x);
   e[3] = (unsigned long long)__double_as_longlong(q.mu);
   e[4] = (unsigned long long)__double_as_longlong(q.w_mu);
@@ -167,11 +165,10 @@ __device__ __forceinline__ void pool_put(unsigned long long* e, const mcs::Rng<M
   e[9] = __float_as_uint(q.xlo);
 }
 
-template <int M>
-__device__ __forceinline__ uint32_t pool_get(const unsigned long long* e, mcs::Rng<M>& r, mcs::SlabParticle& q,
+__device__ __forceinline__ uint32_t pool_get(const unsigned long long* e, uint64_t& x, mcs::SlabParticle& q,
                                              uint64_t& gi, uint64_t& events) {
-  r.x = e[0];
-  r.draws = e[1];
+  x = e[0];
+  q.j = (int)(uint32_t)e[1];
   q.x = __longlong_as_double((long long)e[2]);
   q.mu = __longlong_as_double((long long)e[3]);
   q.w_mu = __longlong_as_double((long long)e[4]);
@@ -199,17 +196,91 @@ struct CoopArgs {
   const SlabDev* probs;
 };
 
-// End of a history: its draws into the lane's counters, its final state and
-// draw count where the caller asked for them.
-template <int M>
-__device__ __forceinline__ void end_history(const TailArgs& t, const mcs::Rng<M>& r, const SlabDev* P, uint64_t gi,
-                                            mcs::LaneCounts& lc) {
-  lc.draws += r.draws;
-  if (r.draws > lc.maxd) lc.maxd = r.draws;
-  if (P->stride_q != 0 && r.draws > P->stride_q) { ++lc.exh; lc.exd += r.draws - P->stride_q; }
-  if (t.hist_state) t.hist_state[gi] = r.x & t.lcg.mask;
-  if (t.hist_draws) t.hist_draws[gi] = r.draws;
-  if (lc.draws > (1ull << 31)) lc.flush(t.counts);
+// All counts of one ended history, straight to its problem's counters (but
+// for its source).
+__device__ __noinline__ void count_history(unsigned long long* c, uint64_t events, uint64_t draws, int outcome,
+                                           uint64_t stride_q) {
+  const bool leaked = outcome == mcs::kLeakLo || outcome == mcs::kLeakHi;
+  atomicAdd(c + MC_C_FLIGHTS, (unsigned long long)events);
+  atomicAdd(c + MC_C_COLLISIONS, (unsigned long long)(events - (leaked ? 1u : 0u)));
+  atomicAdd(c + MC_C_SCATTERS, (unsigned long long)(events - (leaked || outcome == mcs::kAbsorbed ? 1u : 0u)));
+  atomicAdd(c + (outcome == mcs::kAbsorbed ? MC_C_ABSORPTIONS : outcome == mcs::kLeakLo ? MC_C_LEAK_LO
+                 : outcome == mcs::kLeakHi ? MC_C_LEAK_HI : MC_C_CAPPED), 1ull);
+  atomicAdd(c + MC_C_DRAWS, (unsigned long long)draws);
+  atomicMax(c + MC_C_MAX_DRAWS, (unsigned long long)draws);
+  if (stride_q != 0 && draws > stride_q) {
+    atomicAdd(c + MC_C_EXCEED_HIST, 1ull);
+    atomicAdd(c + MC_C_EXCEED_DRAWS, (unsigned long long)(draws - stride_q));
+  }
+}
+
+// A lane's counts for its current problem, few enough to stay in registers
+// beside the particle: how many histories started and how they ended, and
+// their flights.  Collisions, scatterings and draws follow from these (every
+// flight but a leaking one collides, every collision but an absorbing one
+// scatters; three draws per event, slab_draws).  Histories that the sums do
+// not fit (capped ones, 2^30 flights or more) are counted straight away, and
+// exceedances in the block's shared memory (one problem) or straight away.  Flushed with atomics, lane by lane or summed over a
+// converged warp first: a problem's counters share a cache line.
+struct HistCounts {
+  int prob;
+  uint32_t src, flights, absn, llo, lhi, maxd;
+  __device__ void clear() { src = flights = absn = llo = lhi = maxd = 0u; }
+  __device__ static void add(unsigned long long* c, const SlabDev& p, unsigned long long so, unsigned long long fl,
+                             unsigned long long ab, unsigned long long lo, unsigned long long hi,
+                             unsigned long long mx) {
+    const unsigned long long lk = lo + hi, co = fl - lk;
+    if (so) atomicAdd(c + MC_C_SOURCE, so);
+    if (fl == 0ull) return;  // no history ended
+    atomicAdd(c + MC_C_FLIGHTS, fl);
+    if (co) atomicAdd(c + MC_C_COLLISIONS, co);
+    if (ab) atomicAdd(c + MC_C_ABSORPTIONS, ab);
+    if (co != ab) atomicAdd(c + MC_C_SCATTERS, co - ab);
+    if (lo) atomicAdd(c + MC_C_LEAK_LO, lo);
+    if (hi) atomicAdd(c + MC_C_LEAK_HI, hi);
+    atomicAdd(c + MC_C_DRAWS, 3ull * fl - 2ull * lk - ab + (p.source == MC_SRC_BEAM ? 0ull : 2ull * (lk + ab)));
+    atomicMax(c + MC_C_MAX_DRAWS, mx);
+  }
+  __device__ void flush(unsigned long long* counts, const SlabDev* probs) {
+    if (prob < 0) return;
+    add(counts + (size_t)prob * MC_NCOUNT, probs[prob], src, flights, absn, llo, lhi, maxd);
+    clear();
+  }
+  __device__ void flush_warp(unsigned long long* counts, const SlabDev* probs) {
+    const int p = mcd::warp_common_prob(prob);
+    if (p == -2) { flush(counts, probs); return; }
+    if (p < 0) return;
+    const unsigned long long so = mcd::warp_sum64(src), fl = mcd::warp_sum64(flights), ab = mcd::warp_sum64(absn),
+                             lo = mcd::warp_sum64(llo), hi = mcd::warp_sum64(lhi), mx = mcd::warp_max64(maxd);
+    if ((threadIdx.x & 31u) == 0u) add(counts + (size_t)p * MC_NCOUNT, probs[p], so, fl, ab, lo, hi, mx);
+    clear();
+  }
+};
+
+// End of a history after `events` flights: its counts, its final state and
+// draw count where the caller asked for them.  exceed: the block's
+// exceedance counts (nullptr: straight to the problem's).
+__device__ __forceinline__ void end_history(const TailArgs& t, const SlabDev* probs, uint64_t x, const SlabDev& p,
+                                            uint64_t gi, uint64_t events, int outcome, unsigned long long* exceed,
+                                            HistCounts& lc) {
+  const uint64_t draws = mcs::slab_draws(p, events, outcome);
+  if (t.hist_state) t.hist_state[gi] = x & t.lcg.mask;
+  if (t.hist_draws) t.hist_draws[gi] = draws;
+  unsigned long long* const c = t.counts + (size_t)lc.prob * MC_NCOUNT;
+  if (outcome < 0 || events >= (1ull << 30)) {
+    count_history(c, events, draws, outcome, p.stride_q);
+    return;
+  }
+  if (p.stride_q != 0 && draws > p.stride_q) {
+    atomicAdd(exceed ? exceed : c + MC_C_EXCEED_HIST, 1ull);
+    atomicAdd(exceed ? exceed + 1 : c + MC_C_EXCEED_DRAWS, (unsigned long long)(draws - p.stride_q));
+  }
+  lc.flights += (uint32_t)events;
+  lc.absn += outcome == mcs::kAbsorbed ? 1u : 0u;
+  lc.llo += outcome == mcs::kLeakLo ? 1u : 0u;
+  lc.lhi += outcome == mcs::kLeakHi ? 1u : 0u;
+  lc.maxd = max(lc.maxd, (uint32_t)draws);  // below 3 * 2^30 + 2
+  if (lc.flights > (1u << 30)) lc.flush(t.counts, probs);
 }
 
 // Cooperative tail.  When the ticket has run out, the block's pool is empty
@@ -240,7 +311,7 @@ __device__ __forceinline__ void end_history(const TailArgs& t, const mcs::Rng<M>
 // there: the main loop has ended, and almost nothing stays in registers
 // across the calls.
 constexpr int kCoopMax = 4;            // live histories at most
-constexpr int kCoopHistWords = 16;     // 8-byte words per history record
+constexpr int kCoopHistWords = 12;     // 8-byte words per history record
 constexpr int kCoopWords = 6;          // 8-byte words per event record
 constexpr uint32_t kCoopEvents = 128;  // events per history and round at most
 constexpr uint32_t kCoopMinEvents = 8;
@@ -285,7 +356,6 @@ struct CoopHist {
   unsigned long long* w;
   enum {
     kX = 0,      // stream state
-    kDraws,      // draws taken
     kPos,        // fp64 x (fp32: xf, xlo)
     kDir,        // fp64 mu (fp32: muf, wf)
     kW,          // fp64 2^32 / |mu|
@@ -295,11 +365,7 @@ struct CoopHist {
     kBase,       // tally row
     kEdges,      // edge and width tables (null: computed)
     kWidths,
-    kFlights,    // counts of the tail's events
-    kColl,
-    kScat,
-    kEnd,        // last round: events run (low half) and how the last one ended (high half)
-    kSpare
+    kEnd         // last round: events run (low half) and how the last one ended (high half)
   };
   __device__ __forceinline__ explicit CoopHist(unsigned long long* p) : w(p) {}
   __device__ __forceinline__ bool live() const { return (w[kProb] >> 32) != 0ull; }
@@ -348,7 +414,7 @@ __device__ __noinline__ void coop_draws(const CoopArgs* c, const mcd::Affine* ta
       R.w[e] = dbits(w);
       if (e < E) {
         const uint64_t sd = mcd::lcg_step(xs, l.g, l.c);
-        const double d = __dmul_rn(-mclog::log1m_n(mcd::u53<M>(sd, l.m)), p.inv_st);
+        const double d = __dmul_rn(mclog::neglog1m_n(mcd::u53<M>(sd, l.m)), p.inv_st);
         R.d[e] = dbits(d);
         R.p[e] = dbits(__dmul_rn(d, mu));
         R.f[e] = mcd::u53<M>(mcd::lcg_step(sd, l.g, l.c), l.m) < p.p_abs_n ? 1ull : 0ull;
@@ -472,40 +538,21 @@ __device__ __noinline__ void coop_walk(const CoopArgs* c, const mcd::Affine* tab
     H.w[CoopHist::kPos] = pack2(xf, xlo);
     if (out == mcs::kContinue) H.w[CoopHist::kDir] = pack2(hi_of(R.d[E]), lo_of(R.w[E]));
   }
-  // every event run is a flight; a collision unless it leaked; then an
-  // absorption or a scattering
-  const bool leaked = out == mcs::kLeakLo || out == mcs::kLeakHi;
-  H.w[CoopHist::kEvents] = events + e;
-  H.w[CoopHist::kFlights] += e;
-  H.w[CoopHist::kColl] += e - (leaked ? 1u : 0u);
-  H.w[CoopHist::kScat] += e - (leaked || out == mcs::kAbsorbed ? 1u : 0u);
+  const uint64_t total = events + e;
+  H.w[CoopHist::kEvents] = total;
   H.w[CoopHist::kEnd] = (unsigned long long)e | ((unsigned long long)(uint32_t)out << 32);
-  // draws taken: three per completed event, one for a leaking flight, two
-  // for an absorbed one, none for a capped event
+  // draws the round took: three per completed event, one for a leaking
+  // flight, two for an absorbed one, none for a capped event
   const uint64_t used = out == mcs::kContinue ? 3ull * E
                       : out == -1 ? 3ull * e
                       : out == mcs::kAbsorbed ? 3ull * e - 1ull : 3ull * e - 2ull;
   const uint64_t x = mcs::skip_tab(tab, H.w[CoopHist::kX], used);
-  const uint64_t draws = H.w[CoopHist::kDraws] + used;
   H.w[CoopHist::kX] = x;
-  H.w[CoopHist::kDraws] = draws;
   if (out == mcs::kContinue) return;
-  // the history's end: its counts as the one-lane path would flush them
+  // the history's end
+  const uint64_t draws = mcs::slab_draws(p, total, out);
   const uint32_t pi = (uint32_t)H.w[CoopHist::kProb];
-  unsigned long long* cnt = c->t.counts + (size_t)pi * MC_NCOUNT;
-  atomicAdd(cnt + MC_C_FLIGHTS, H.w[CoopHist::kFlights]);
-  if (H.w[CoopHist::kColl]) atomicAdd(cnt + MC_C_COLLISIONS, H.w[CoopHist::kColl]);
-  if (H.w[CoopHist::kScat]) atomicAdd(cnt + MC_C_SCATTERS, H.w[CoopHist::kScat]);
-  if (out == mcs::kAbsorbed) atomicAdd(cnt + MC_C_ABSORPTIONS, 1ull);
-  else if (out == mcs::kLeakLo) atomicAdd(cnt + MC_C_LEAK_LO, 1ull);
-  else if (out == mcs::kLeakHi) atomicAdd(cnt + MC_C_LEAK_HI, 1ull);
-  else atomicAdd(cnt + MC_C_CAPPED, 1ull);
-  atomicAdd(cnt + MC_C_DRAWS, draws);
-  atomicMax(cnt + MC_C_MAX_DRAWS, draws);
-  if (p.stride_q != 0 && draws > p.stride_q) {
-    atomicAdd(cnt + MC_C_EXCEED_HIST, 1ull);
-    atomicAdd(cnt + MC_C_EXCEED_DRAWS, draws - p.stride_q);
-  }
+  count_history(c->t.counts + (size_t)pi * MC_NCOUNT, total, draws, out, p.stride_q);
   const uint64_t gi = H.w[CoopHist::kGi];
   if (c->t.hist_state) c->t.hist_state[gi] = x & c->t.lcg.mask;
   if (c->t.hist_draws) c->t.hist_draws[gi] = draws;
@@ -532,12 +579,14 @@ __device__ __noinline__ void coop_tally(const CoopArgs* c, uint32_t hist_off, ui
     if constexpr (!F32) {
       const double xe = dval(R.x[e]);
       const double xn = f == mcs::kCollide ? dval(R.x[e + 1]) : 0.0;
-      mcs::tally64(p, xe, xn, dval(R.m[e]), dval(R.d[e]), dval(R.w[e]), f, sk);
+      int j = mcs::bin_of(p, sk, xe);
+      mcs::tally64(p, xe, xn, dval(R.m[e]), dval(R.d[e]), dval(R.w[e]), f, sk, j);
     } else {
       const unsigned long long xa = R.x[e];
       const unsigned long long xb = f == mcs::kCollide ? R.x[e + 1] : 0ull;
       const unsigned long long dw = R.d[e];
-      mcs::tally32(p, lo_of(xa), hi_of(xa), lo_of(xb), hi_of(xb), hi_of(dw), lo_of(dw), lo_of(R.w[e]), f, sk);
+      int j = mcs::bin_of_pair(p, lo_of(xa), hi_of(xa));
+      mcs::tally32(p, lo_of(xa), hi_of(xa), lo_of(xb), hi_of(xb), hi_of(dw), lo_of(dw), lo_of(R.w[e]), f, sk, j);
     }
   }
 }
@@ -590,7 +639,9 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
   // the particle pool after the tally and the edge tables
   unsigned long long* s_pool = s_tally + (SMEM ? a.smem_slots : 0u) + 2u * a.smem_edges;
   __shared__ PoolCtl ctl;
+  __shared__ unsigned long long s_exceed[2];  // one problem: exceeding histories, and their draws beyond Q
   if (threadIdx.x == 0) {
+    s_exceed[0] = s_exceed[1] = 0ull;
     ctl.lock = 0;
     ctl.n = 0;
     ctl.active = (int)(blockDim.x >> 5);
@@ -615,12 +666,12 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
   uint64_t pool_next = 0, pool_end = 0;
   bool more = true;
   bool alive = false;
-  mcs::LaneCounts lc;
+  HistCounts lc;
   lc.prob = -1;
   lc.clear();
 
   const SlabDev* P = a.probs;
-  mcs::Rng<M> r{0ull, 0ull};
+  uint64_t x = 0;  // stream state
   mcs::SlabParticle q{};
   mcs::Sink sink{nullptr, s_edges, s_widths, AGG};
   uint64_t gi = 0, events = 0;
@@ -642,7 +693,7 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
       if (!alive && rank < avail) {
         uint32_t pi;
         mcs::ticket_history(a.probs, a.nprob, a.range_begin, a.order, pool_next + rank, pi, gi);
-        if ((int)pi != lc.prob) { lc.flush(a.counts); lc.prob = (int)pi; }
+        if ((int)pi != lc.prob) { lc.flush(a.counts, a.probs); lc.prob = (int)pi; }
         P = a.probs + pi;
         const uint64_t id = gi - P->hist_begin;
         const uint64_t batch = mcs::batch_of(id, P->n_hist, P->n_batches);
@@ -651,9 +702,10 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
           sink.edges = a.tables + P->tab_off;
           sink.widths = sink.edges + P->n_bins + 1;
         }
-        r.x = mcs::slab_seed(*P, id, tab, l.mask);
-        r.draws = 0;
+        mcs::Rng<M> r{mcs::slab_seed(*P, id, tab, l.mask), 0ull};
         mcs::slab_source<M, F32>(*P, r, l, q);
+        x = r.x;
+        q.j = mcs::locate<F32>(*P, q, sink);
         events = 0;
         ++lc.src;
         alive = true;
@@ -685,8 +737,8 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
         __syncwarp();
         const unsigned rank = __popc(dead & lt_mask);
         if (!alive && (int)rank < k) {
-          const uint32_t pi = pool_get<M>(s_pool + (size_t)(n - k + (int)rank) * kPoolWords, r, q, gi, events);
-          if ((int)pi != lc.prob) { lc.flush(a.counts); lc.prob = (int)pi; }
+          const uint32_t pi = pool_get(s_pool + (size_t)(n - k + (int)rank) * kPoolWords, x, q, gi, events);
+          if ((int)pi != lc.prob) { lc.flush(a.counts, a.probs); lc.prob = (int)pi; }
           P = a.probs + pi;
           const uint64_t id = gi - P->hist_begin;
           sink.base = (SMEM ? s_tally : a.tally) + P->tally_offset + mcs::batch_of(id, P->n_hist, P->n_batches) * P->n_bins;
@@ -713,11 +765,10 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
           pool_unlock(&ctl.lock);
         }
         if (__shfl_sync(kFull, ok, 0)) {
-          lc.flush_warp(a.counts);
+          lc.flush_warp(a.counts, a.probs);
           if (alive) {
             CoopHist H(s_pool + (size_t)__popc(live & lt_mask) * kCoopHistWords);
-            H.w[CoopHist::kX] = r.x;
-            H.w[CoopHist::kDraws] = r.draws;
+            H.w[CoopHist::kX] = x;
             H.w[CoopHist::kPos] = F32 ? pack2(q.xf, q.xlo) : dbits(q.x);
             H.w[CoopHist::kDir] = F32 ? pack2(q.muf, q.wf) : dbits(q.mu);
             H.w[CoopHist::kW] = dbits(q.w_mu);
@@ -727,7 +778,6 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
             H.w[CoopHist::kBase] = reinterpret_cast<unsigned long long>(sink.base);
             H.w[CoopHist::kEdges] = reinterpret_cast<unsigned long long>(sink.edges);
             H.w[CoopHist::kWidths] = reinterpret_cast<unsigned long long>(sink.widths);
-            H.w[CoopHist::kFlights] = H.w[CoopHist::kColl] = H.w[CoopHist::kScat] = 0ull;
           }
           coop_n = nlive;
           alive = false;
@@ -757,7 +807,7 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
           if (nlive != 0) {
             const uint32_t slot = (uint32_t)n + (uint32_t)__popc(live & lt_mask);
             if (alive && slot < a.pool_cap)  // always, by the count taken under the lock
-              pool_put<M>(s_pool + (size_t)slot * kPoolWords, r, q, gi, events, (uint32_t)(P - a.probs));
+              pool_put(s_pool + (size_t)slot * kPoolWords, x, q, gi, events, (uint32_t)(P - a.probs));
             else if (alive)
               atomicAdd(a.counts + MC_C_DROPPED, 1ull);
             __syncwarp();
@@ -772,20 +822,14 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
       break;
     }
     if (alive) {
-      int outcome;
-      if (events == a.event_cap) {
-        ++lc.capped;
-        outcome = -1;
-      } else {
+      int outcome = -1;  // event cap
+      if (events != a.event_cap) {
         ++events;
-        ++lc.flights;
-        outcome = mcs::slab_event<M, F32>(*P, r, l, q, sink, lc.coll, lc.scat);
-        if (outcome == mcs::kAbsorbed) ++lc.absn;
-        else if (outcome == mcs::kLeakLo) ++lc.llo;
-        else if (outcome == mcs::kLeakHi) ++lc.lhi;
+        outcome = mcs::slab_event<M, F32>(*P, x, l, q, sink);
       }
       if (outcome != mcs::kContinue) {
-        end_history<M>(TailArgs{a.hist_state, a.hist_draws, a.counts, a.lcg, a.event_cap}, r, P, gi, lc);
+        end_history(TailArgs{a.hist_state, a.hist_draws, a.counts, a.lcg, a.event_cap}, a.probs, x, *P, gi, events, outcome,
+                    a.nprob == 1 ? s_exceed : nullptr, lc);
         alive = false;
       }
     }
@@ -798,10 +842,14 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
     __syncwarp();
     coop_tail<M, F32>(&s_coop, tab, (uint32_t)(s_pool - s_tally), a.coop_slots, coop_n);
   }
-  lc.flush_warp(a.counts);
+  lc.flush_warp(a.counts, a.probs);
 
+  __syncthreads();
+  if (threadIdx.x == 0 && s_exceed[0] != 0ull) {
+    atomicAdd(a.counts + MC_C_EXCEED_HIST, s_exceed[0]);
+    atomicAdd(a.counts + MC_C_EXCEED_DRAWS, s_exceed[1]);
+  }
   if constexpr (SMEM) {
-    __syncthreads();
     for (uint32_t s = threadIdx.x; s < a.smem_slots; s += blockDim.x) {
       const unsigned long long v = s_tally[s];
       if (v != 0ull) atomicAdd(a.tally + s, v);

@@ -147,7 +147,6 @@ struct Sink {
   const double* widths;  // with edges: widths[j] = e_{j+1} - e_j (the same fp64 difference)
   bool agg;              // warp-aggregated atomics (mcd::warp_agg_add) instead of one per lane
   __device__ __forceinline__ void add(int j, long long v) const {
-    if (v == 0) return;
     if (agg) mcd::warp_agg_add(base + j, (unsigned long long)v);
     else atomicAdd(base + j, (unsigned long long)v);
   }
@@ -164,53 +163,43 @@ __device__ __forceinline__ double edge_of(const SlabDev& p, const Sink& s, int j
   return s.edges ? s.edges[j] : slab_edge(p, j);
 }
 
-// Track length in every bin met by the segment [a, b] (0 <= a <= b <= L):
-// |[a,b] & [e_j, e_{j+1}]| / |mu|, to fixed point.  w_fix = 2^32 / |mu|,
-// rounded once; since scaling by 2^32 commutes with rounding,
-// (hi - lo) * w_fix rounds to exactly 2^32 times the rounded
-// (hi - lo) * (1/|mu|).  The walk visits only the bins the segment
-// overlaps, starting from the one that holds a.
-__device__ __forceinline__ void seg64(const SlabDev& p, double a, double b, double w_fix, const Sink& s) {
-  const int nb = (int)p.n_bins;
-  int j = clamp_bin(bin_guess(p, a), nb);
-  while (j > 0 && nn_lt(a, edge_of(p, s, j))) --j;
-  while (j + 1 < nb && !nn_lt(a, edge_of(p, s, j + 1))) ++j;
-  if (s.widths) {
-    // The same walk with the interior bins' lengths from the width table:
-    // the first bin [a, min(b, e_{j+1})], the whole bins while e_{j+1} <= b,
-    // the last [e_j, b]; only the ends take an fp64 difference.
-    double e1 = s.edges[j + 1];
-    const double hi = nn_lt(b, e1) ? b : e1;
-    if (nn_lt(a, hi)) s.add(j, mcx::llrint_nonneg(__dmul_rn(__dsub_rn(hi, a), w_fix)));
-    if (!nn_lt(e1, b) || j + 1 >= nb) return;
-    for (++j;; ++j) {
-      e1 = s.edges[j + 1];
-      if (nn_lt(b, e1)) break;
-      s.add(j, mcx::llrint_nonneg(__dmul_rn(s.widths[j], w_fix)));
-      if (!nn_lt(e1, b) || j + 1 >= nb) return;
-    }
-    const double ej = s.edges[j];
-    if (nn_lt(ej, b)) s.add(j, mcx::llrint_nonneg(__dmul_rn(__dsub_rn(b, ej), w_fix)));
-    return;
-  }
-  double lo = a;
-  for (;;) {
-    const double e1 = edge_of(p, s, j + 1);
-    const double hi = nn_lt(b, e1) ? b : e1;
-    if (nn_lt(lo, hi)) s.add(j, mcx::llrint_nonneg(__dmul_rn(__dsub_rn(hi, lo), w_fix)));
-    if (!nn_lt(e1, b) || j + 1 >= nb) break;
-    lo = e1;
-    ++j;
-  }
-}
-
-// mu == 0: the whole flight d lies in the bin holding x.
-__device__ __forceinline__ void point64(const SlabDev& p, double x, double d, const Sink& s) {
+// The bin of a position x in [0, L]: the largest j with e_j <= x (the last
+// bin for x = L).
+__device__ __forceinline__ int bin_of(const SlabDev& p, const Sink& s, double x) {
   const int nb = (int)p.n_bins;
   int j = clamp_bin(bin_guess(p, x), nb);
-  while (j > 0 && nn_lt(x, slab_edge(p, j))) --j;
-  while (j + 1 < nb && !nn_lt(x, slab_edge(p, j + 1))) ++j;
-  s.add(j, mcx::fix32_nonneg(d));
+  while (j > 0 && nn_lt(x, edge_of(p, s, j))) --j;
+  while (j + 1 < nb && !nn_lt(x, edge_of(p, s, j + 1))) ++j;
+  return j;
+}
+
+// Track length in every bin met by a flight from x to xe (both in [0, L];
+// forward: xe >= x, else xe <= x): |[x, xe] & [e_j, e_{j+1}]| / |mu|, to fixed
+// point.  w_fix = 2^32 / |mu|, rounded once; since scaling by 2^32 commutes
+// with rounding, (hi - lo) * w_fix rounds to exactly 2^32 times the rounded
+// (hi - lo) * (1/|mu|).  The walk starts from x's bin j, goes the way the
+// particle flies and leaves j at the bin of xe, where the next flight starts:
+// no bin is ever looked up.  (At an edge either neighbour will do for j: the
+// piece in the other one has length zero and adds nothing.)  The first piece,
+// to xe or to the first edge, and the last, from the last edge to xe, take an
+// fp64 difference; whole bins take their length from the width table.
+__device__ __forceinline__ void walk64(const SlabDev& p, double x, double xe, bool fwd, double w_fix, const Sink& s,
+                                       int& j) {
+  const int up = fwd ? 1 : 0, dj = fwd ? 1 : -1;
+  double e = edge_of(p, s, j + up);
+  bool last = fwd ? !nn_lt(e, xe) : !nn_lt(xe, e);
+  s.add(j, mcx::llrint_nonneg(__dmul_rn(mcx::abs_bits(__dsub_rn(last ? xe : e, x)), w_fix)));
+  if (last) return;
+  for (;;) {
+    j += dj;
+    const double e2 = edge_of(p, s, j + up);
+    last = fwd ? !nn_lt(e2, xe) : !nn_lt(xe, e2);
+    if (last) break;
+    const double w = s.widths ? s.widths[j] : mcx::abs_bits(__dsub_rn(e2, e));
+    s.add(j, mcx::llrint_nonneg(__dmul_rn(w, w_fix)));
+    e = e2;
+  }
+  s.add(j, mcx::llrint_nonneg(__dmul_rn(mcx::abs_bits(__dsub_rn(xe, e)), w_fix)));
 }
 
 // Exact llrint((double)v * 2^32) for a finite float v >= 0 (scaling by 2^32
@@ -250,8 +239,7 @@ __device__ __forceinline__ float slab_edge_f(const SlabDev& p, int j) {
   return j >= (int)p.n_bins ? p.L_f : (float)j * p.h_f;
 }
 
-// Track length of the segment [a, b] in every bin it meets, the ends given
-// as pairs (ah + al, bh + bl) of the fp32 path.  Each bin's length is taken
+// The fp32 path's positions are pairs of floats.  Each bin's length is taken
 // from the pairs, (hi_h - lo_h) + (hi_l - lo_l), so a flight whose
 // displacement is far below an ulp of its position (a direction nearly
 // parallel to the faces, where 1 / |mu| is large) keeps its true length
@@ -271,17 +259,21 @@ __device__ __forceinline__ int bin_of_pair(const SlabDev& p, float h, float l) {
   return j;
 }
 
-__device__ __forceinline__ void seg32(const SlabDev& p, float ah, float al, float bh, float bl, float w_mu,
-                                      const Sink& s) {
-  const int j0 = bin_of_pair(p, ah, al), j1 = bin_of_pair(p, bh, bl);
-  for (int j = j0; j <= j1; ++j) {
-    const float lo_e = slab_edge_f(p, j), hi_e = slab_edge_f(p, j + 1);
-    // max(a, lo_e) and min(b, hi_e) as pairs (an edge's low part is zero)
-    float loh = lo_e, lol = 0.0f, hih = hi_e, hil = 0.0f;
-    if (ah > lo_e || (ah == lo_e && al > 0.0f)) { loh = ah; lol = al; }
-    if (bh < hi_e || (bh == hi_e && bl < 0.0f)) { hih = bh; hil = bl; }
-    const float len = __fadd_rn(__fsub_rn(hih, loh), __fsub_rn(hil, lol));
+// walk64's counterpart: from the pair (xh + xl) in bin j to (eh + el).
+__device__ __forceinline__ void walk32(const SlabDev& p, float xh, float xl, float eh, float el, bool fwd, float w_mu,
+                                       const Sink& s, int& j) {
+  const int up = fwd ? 1 : 0, dj = fwd ? 1 : -1;
+  for (;;) {
+    const float e = slab_edge_f(p, j + up);
+    // (eh, el) lies beyond the edge?
+    const bool last = fwd ? !(eh > e || (eh == e && el > 0.0f)) : !(eh < e || (eh == e && el < 0.0f));
+    const float th = last ? eh : e, tl = last ? el : 0.0f;
+    const float d = __fadd_rn(__fsub_rn(th, xh), __fsub_rn(tl, xl)), len = fwd ? d : -d;
     if (len > 0.0f) s.add(j, fix32_from_float(__fmul_rn(len, w_mu)));
+    if (last) break;
+    xh = e;
+    xl = 0.0f;
+    j += dj;
   }
 }
 
@@ -297,10 +289,11 @@ __device__ __forceinline__ void point32(const SlabDev& p, float x, float d, cons
 // holds 2^32 / |mu| (0 for mu = 0); the fp32 path keeps its geometry in
 // fp32: the position as an unevaluated sum xf + xlo of two floats (so that
 // it does not drift from the fp64 trajectory by one rounding per flight),
-// muf and wf = 1 / |muf|.
+// muf and wf = 1 / |muf|.  Both keep the bin of the position.
 struct SlabParticle {
   double x, mu, w_mu;
   float xf, xlo, muf, wf;
+  int j;  // the bin of the position
 };
 
 // s + t = a + b exactly (Knuth's TwoSum; six fp32 operations, no fused
@@ -348,7 +341,8 @@ __device__ __forceinline__ float mu_f32(uint64_t n) {
 // 2^32 / |mu| rounded once: 2^32 RN(1 / |mu|), the reciprocal on the
 // integer pipes (fp_exact.cuh), the scaling an exponent add.
 __device__ __forceinline__ double fix_per_mu(double mu) {
-  return !mcx::d_zero(mu) ? mcx::scale_pow2(mcx::recip_rn(mcx::abs_bits(mu)), 32) : 0.0;
+  const double w = mcx::scale_pow2(mcx::recip_normal(mcx::abs_bits(mu)), 32);
+  return mcx::d_zero(mu) ? 0.0 : w;
 }
 
 // Per-lane counters for the lane's current problem (flushed with atomics,
@@ -410,6 +404,18 @@ struct LaneCounts {
 // Outcome of a flight or a collision.
 enum Outcome : int { kContinue = 0, kAbsorbed = 1, kLeakLo = 2, kLeakHi = 3, kCollide = 4 };
 
+// A new direction from its draw: mu and 2^32 / |mu|, or the fp32 pair.
+template <bool F32>
+__device__ __forceinline__ void set_direction(SlabParticle& q, uint64_t n) {
+  if constexpr (!F32) {
+    q.mu = mcx::two_u_minus_1(n);
+    q.w_mu = fix_per_mu(q.mu);
+  } else {
+    q.muf = mu_f32(n);
+    q.wf = q.muf != 0.0f ? __frcp_rn(fabsf(q.muf)) : 0.0f;
+  }
+}
+
 // Source of a history (isotropic uniform in [0, L], or a beam at x = 0).
 template <int M, bool F32>
 __device__ __forceinline__ void slab_source(const SlabDev& p, Rng<M>& r, const mcd::Lcg& l, SlabParticle& q) {
@@ -421,16 +427,13 @@ __device__ __forceinline__ void slab_source(const SlabDev& p, Rng<M>& r, const m
   const double u1 = r.next(l);
   if constexpr (!F32) {
     q.x = __dmul_rn(p.L, u1);
-    q.mu = mcx::two_u_minus_1(r.next_n(l));
-    q.w_mu = fix_per_mu(q.mu);
   } else {
     // x = L u as the fp64 path has it, split into two floats
     const double x64 = __dmul_rn(p.L, u1);
     q.xf = __double2float_rn(x64);
     q.xlo = __double2float_rn(__dsub_rn(x64, (double)q.xf));
-    q.muf = mu_f32(r.next_n(l));
-    q.wf = q.muf != 0.0f ? __frcp_rn(fabsf(q.muf)) : 0.0f;
   }
+  set_direction<F32>(q, r.next_n(l));
 }
 
 // The end of a flight of the fp64 path: xn = x + pm (pm = d mu, rounded
@@ -451,20 +454,20 @@ __device__ __forceinline__ bool leaves64(const SlabDev& p, long long mb, double 
   return (mb > 0 && !nn_lt(xn, p.L)) || (mb < 0 && __double_as_longlong(xn) <= 0);
 }
 
-// The tally of that flight: the track from x to xn, to the face it leaves
-// through, or (mu = 0) the whole distance d in the bin holding x.  Every
-// kind of flight ends in the one call of the bin walk, with its ends chosen
-// first, so that the lanes of a warp whose flights differ in kind still walk
-// the bins together.
+// The tally of that flight, from x's bin j (left at the bin of xn): the track
+// from x to xn, to the face it leaves through, or (mu = 0) the whole distance
+// d in the bin holding x.  Every kind of flight ends in the one call of the
+// bin walk, with its end chosen first, so that the lanes of a warp whose
+// flights differ in kind still walk the bins together.
 __device__ __forceinline__ void tally64(const SlabDev& p, double x, double xn, double mu, double d, double w_mu,
-                                        int outcome, const Sink& s) {
+                                        int outcome, const Sink& s, int& j) {
   const long long mb = __double_as_longlong(mu);
-  if (outcome == kCollide && mb == 0) { point64(p, x, d, s); return; }
-  double a = x, b = xn;                          // forward flight
-  if (outcome == kLeakHi) b = p.L;
-  else if (outcome == kLeakLo) { a = 0.0; b = x; }
-  else if (mb < 0) { a = xn; b = x; }            // backward flight
-  seg64(p, a, b, w_mu, s);
+  if (outcome == kCollide && mb == 0) {
+    s.add(bin_of(p, s, x), mcx::fix32_nonneg(d));
+    return;
+  }
+  const double xe = outcome == kLeakHi ? p.L : (outcome == kLeakLo ? 0.0 : xn);
+  walk64(p, x, xe, mb > 0, w_mu, s, j);
 }
 
 // The fp32 path's position step: xn + xnlo = (xf + xlo) + d muf, with pr =
@@ -500,7 +503,7 @@ __device__ __forceinline__ int advance32(const SlabDev& p, float xf, float xlo, 
   bool leak_hi = muf > 0.0f && (xn > p.L_f || (xn == p.L_f && xnlo >= 0.0f));
   bool leak_lo = muf < 0.0f && (xn < 0.0f || (xn == 0.0f && xnlo <= 0.0f));
   if (near_hi || near_lo) {
-    const double d64 = __dmul_rn(-mclog::log1m_n(nf()), p.inv_st);
+    const double d64 = __dmul_rn(mclog::neglog1m_n(nf()), p.inv_st);
     const double x64 = __dadd_rn((double)xf, (double)xlo);
     const double xn64 = __dadd_rn(x64, __dmul_rn(d64, (double)muf));
     leak_hi = muf > 0.0f && xn64 >= p.L;
@@ -516,27 +519,39 @@ __device__ __forceinline__ int advance32(const SlabDev& p, float xf, float xlo, 
   return leak_hi ? kLeakHi : (leak_lo ? kLeakLo : kCollide);
 }
 
-// tally64's counterpart for the fp32 path, on position pairs.
+// tally64's counterpart for the fp32 path, on position pairs.  A pair's
+// last rounding can move a flight of next to no length backwards; its bin is
+// then looked up again.
 __device__ __forceinline__ void tally32(const SlabDev& p, float xf, float xlo, float xn, float xnlo, float muf,
-                                        float d, float wf, int outcome, const Sink& s) {
+                                        float d, float wf, int outcome, const Sink& s, int& j) {
   if (outcome == kCollide && muf == 0.0f) { point32(p, xf, d, s); return; }
-  float ah = xf, al = xlo, bh = xn, bl = xnlo;   // forward flight
-  if (outcome == kLeakHi) { bh = p.L_f; bl = 0.0f; }
-  else if (outcome == kLeakLo) { ah = 0.0f; al = 0.0f; bh = xf; bl = xlo; }
-  else if (muf < 0.0f) { ah = xn; al = xnlo; bh = xf; bl = xlo; }  // backward flight
-  seg32(p, ah, al, bh, bl, wf, s);
+  float eh = xn, el = xnlo;
+  if (outcome == kLeakHi) { eh = p.L_f; el = 0.0f; }
+  else if (outcome == kLeakLo) { eh = 0.0f; el = 0.0f; }
+  const bool fwd = muf > 0.0f;
+  walk32(p, xf, xlo, eh, el, fwd, wf, s, j);
+  const bool less = xn < xf || (xn == xf && xnlo < xlo), more = xn > xf || (xn == xf && xnlo > xlo);
+  if (outcome == kCollide && (fwd ? less : more)) j = bin_of_pair(p, xn, xnlo);
 }
 
-// One flight: sample the distance, tally the track, and either leak
-// (kLeakLo / kLeakHi) or stop at the collision site (kCollide).
+// The bin of the particle's position, where none is known from a flight.
+template <bool F32>
+__device__ __forceinline__ int locate(const SlabDev& p, const SlabParticle& q, const Sink& s) {
+  if constexpr (F32) return bin_of_pair(p, q.xf, q.xlo);
+  else return bin_of(p, s, q.x);
+}
+
+// One flight from the particle's bin q.j: sample the distance, tally the
+// track, and either leak (kLeakLo / kLeakHi) or stop at the collision site
+// (kCollide).
 template <int M, bool F32>
 __device__ __forceinline__ int slab_flight(const SlabDev& p, Rng<M>& r, const mcd::Lcg& l, SlabParticle& q,
                                            const Sink& s) {
   if constexpr (!F32) {
-    const double d = __dmul_rn(-mclog::log1m_n(r.next_n(l)), p.inv_st);
+    const double d = __dmul_rn(mclog::neglog1m_n(r.next_n(l)), p.inv_st);
     double xn;
     const int f = advance64(p, q.x, q.mu, __dmul_rn(d, q.mu), xn);
-    tally64(p, q.x, xn, q.mu, d, q.w_mu, f, s);
+    tally64(p, q.x, xn, q.mu, d, q.w_mu, f, s, q.j);
     if (f == kCollide) q.x = xn;
     return f;
   } else {
@@ -546,7 +561,7 @@ __device__ __forceinline__ int slab_flight(const SlabDev& p, Rng<M>& r, const mc
     const float pe = __fmaf_rn(d, q.muf, -pr);
     float xn, xnlo;
     const int f = advance32(p, q.xf, q.xlo, q.muf, pr, pe, [n] { return n; }, xn, xnlo);
-    tally32(p, q.xf, q.xlo, xn, xnlo, q.muf, d, q.wf, f, s);
+    tally32(p, q.xf, q.xlo, xn, xnlo, q.muf, d, q.wf, f, s, q.j);
     if (f == kCollide) {
       q.xf = xn;
       q.xlo = xnlo;
@@ -560,27 +575,56 @@ __device__ __forceinline__ int slab_flight(const SlabDev& p, Rng<M>& r, const mc
 template <int M, bool F32>
 __device__ __forceinline__ int slab_collide(const SlabDev& p, Rng<M>& r, const mcd::Lcg& l, SlabParticle& q) {
   if (r.next_n(l) < p.p_abs_n) return kAbsorbed;  // u < 1 - c
-  if constexpr (!F32) {
-    q.mu = mcx::two_u_minus_1(r.next_n(l));
-    q.w_mu = fix_per_mu(q.mu);
-  } else {
-    q.muf = mu_f32(r.next_n(l));
-    q.wf = q.muf != 0.0f ? __frcp_rn(fabsf(q.muf)) : 0.0f;
-  }
+  set_direction<F32>(q, r.next_n(l));
   return kContinue;
 }
 
-// One flight and, if the particle stays in the slab, one collision (the
-// history-based step).  Counts collisions and scatters into *coll, *scat.
+// One event of the history schedule on the stream state x: a flight and, if
+// the particle stays in the slab, a collision.  The event's three draws have
+// fixed roles (distance, absorption test, new direction), so the new
+// direction and its tally weight are computed beside the distance whether or
+// not the event comes to use them: the two chains of integer operations
+// (the logarithm, the reciprocal) are independent and fill each other's
+// latencies.  x moves on by the draws the event takes.
 template <int M, bool F32>
-__device__ __forceinline__ int slab_event(const SlabDev& p, Rng<M>& r, const mcd::Lcg& l, SlabParticle& q,
-                                          const Sink& s, uint32_t& coll, uint32_t& scat) {
-  const int f = slab_flight<M, F32>(p, r, l, q, s);
-  if (f != kCollide) return f;
-  ++coll;
-  const int c = slab_collide<M, F32>(p, r, l, q);
-  if (c == kContinue) ++scat;
-  return c;
+__device__ __forceinline__ int slab_event(const SlabDev& p, uint64_t& x, const mcd::Lcg& l, SlabParticle& q,
+                                          const Sink& s) {
+  const uint64_t x1 = mcd::lcg_step(x, l.g, l.c), x2 = mcd::lcg_step(x1, l.g, l.c), x3 = mcd::lcg_step(x2, l.g, l.c);
+  const uint64_t n = mcd::u53<M>(x1, l.m);
+  SlabParticle nq = q;
+  set_direction<F32>(nq, mcd::u53<M>(x3, l.m));
+  int f;
+  if constexpr (!F32) {
+    asm volatile("" : "+d"(nq.mu), "+d"(nq.w_mu));  // not moved to its use after the tally
+    const double d = __dmul_rn(mclog::neglog1m_n(n), p.inv_st);
+    f = advance64(p, q.x, q.mu, __dmul_rn(d, q.mu), nq.x);
+    tally64(p, q.x, nq.x, q.mu, d, q.w_mu, f, s, nq.j);
+  } else {
+    asm volatile("" : "+f"(nq.muf), "+f"(nq.wf));
+    const float d = flight_f32(n) * p.inv_st_f;
+    const float pr = __fmul_rn(d, q.muf);
+    const float pe = __fmaf_rn(d, q.muf, -pr);
+    f = advance32(p, q.xf, q.xlo, q.muf, pr, pe, [n] { return n; }, nq.xf, nq.xlo);
+    tally32(p, q.xf, q.xlo, nq.xf, nq.xlo, q.muf, d, q.wf, f, s, nq.j);
+  }
+  if (f != kCollide) {
+    x = x1;
+    return f;
+  }
+  if (mcd::u53<M>(x2, l.m) < p.p_abs_n) {  // u < 1 - c
+    x = x2;
+    return kAbsorbed;
+  }
+  x = x3;
+  q = nq;
+  return kContinue;
+}
+
+// Draws of a history of the slab: the source's (none for a beam), three per
+// event, less those its last event did not take (event cap: whole events).
+__device__ __forceinline__ uint64_t slab_draws(const SlabDev& p, uint64_t events, int outcome) {
+  const uint64_t unused = outcome == kLeakLo || outcome == kLeakHi ? 2u : (outcome == kAbsorbed ? 1u : 0u);
+  return (p.source == MC_SRC_BEAM ? 0u : 2u) + 3ull * events - unused;
 }
 
 }  // namespace mcs

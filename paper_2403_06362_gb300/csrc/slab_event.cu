@@ -378,7 +378,9 @@ __global__ void __launch_bounds__(256) ev_step_kernel(EvArgs<F32> a) {
         if ((int)v.prob != ec.prob) { ec.flush(cnt); ec.prob = (int)v.prob; }
         ++ec.flights;
       }
-      outcome = mcs::slab_flight<M, F32>(P, r, a.lcg, v.q, sink_of<F32>(a, P, v, s_edges));
+      const mcs::Sink sink = sink_of<F32>(a, P, v, s_edges);
+      v.q.j = mcs::locate<F32>(P, v.q, sink);
+      outcome = mcs::slab_flight<M, F32>(P, r, a.lcg, v.q, sink);
       if (outcome == mcs::kCollide) {
         ++v.coll;
         outcome = mcs::slab_collide<M, F32>(P, r, a.lcg, v.q);
@@ -443,6 +445,7 @@ __global__ void __launch_bounds__(256) ev_tail_kernel(EvArgs<F32> a) {
     const SlabDev& P = a.probs[v.prob];
     mcs::Rng<M> r{v.rng, v.draws};
     const mcs::Sink sink = sink_of<F32>(a, P, v, s_edges);
+    v.q.j = mcs::locate<F32>(P, v.q, sink);
     const uint64_t ev0 = v.events, co0 = v.coll, sc0 = v.scat;
     int outcome;
     for (;;) {
