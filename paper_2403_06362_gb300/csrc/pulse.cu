@@ -71,214 +71,313 @@ __global__ void pulse_prep_kernel(PulseDev* p) {
   }
 }
 
+// A lane's counts, few enough to stay in registers beside the particle.
+// Collisions, absorptions and the rest follow from them: a flight ends at the
+// census or collides, a collision scatters or absorbs.  Event caps, dropped
+// secondaries and exceedances go to the block's counters in shared memory.
 struct PulseCounts {
-  uint64_t src, flights, coll, absn, scat, census, children, capped, dropped, draws, exh, exd, maxd;
+  uint32_t src, flights, census, scat, children;
+  uint64_t draws, maxd;
   __device__ void flush(unsigned long long* c) {
     if (src) atomicAdd(c + MC_C_SOURCE, (unsigned long long)src);
     if (flights) atomicAdd(c + MC_C_FLIGHTS, (unsigned long long)flights);
+    const uint32_t coll = flights - census;
     if (coll) atomicAdd(c + MC_C_COLLISIONS, (unsigned long long)coll);
-    if (absn) atomicAdd(c + MC_C_ABSORPTIONS, (unsigned long long)absn);
+    if (coll != scat) atomicAdd(c + MC_C_ABSORPTIONS, (unsigned long long)(coll - scat));
     if (scat) atomicAdd(c + MC_C_SCATTERS, (unsigned long long)scat);
     if (census) atomicAdd(c + MC_C_LEAK_HI, (unsigned long long)census);
     if (children) atomicAdd(c + MC_C_CHILDREN, (unsigned long long)children);
-    if (capped) atomicAdd(c + MC_C_CAPPED, (unsigned long long)capped);
-    if (dropped) atomicAdd(c + MC_C_DROPPED, (unsigned long long)dropped);
     if (draws) atomicAdd(c + MC_C_DRAWS, (unsigned long long)draws);
-    if (exh) atomicAdd(c + MC_C_EXCEED_HIST, (unsigned long long)exh);
-    if (exd) atomicAdd(c + MC_C_EXCEED_DRAWS, (unsigned long long)exd);
     if (maxd) atomicMax(c + MC_C_MAX_DRAWS, (unsigned long long)maxd);
-  }
-  // The same for a whole converged warp: the counters share a cache line, so
-  // the warp's totals go out through one lane.
-  __device__ void flush_warp(unsigned long long* c) {
-    src = mcd::warp_sum64(src);
-    flights = mcd::warp_sum64(flights);
-    coll = mcd::warp_sum64(coll);
-    absn = mcd::warp_sum64(absn);
-    scat = mcd::warp_sum64(scat);
-    census = mcd::warp_sum64(census);
-    children = mcd::warp_sum64(children);
-    capped = mcd::warp_sum64(capped);
-    dropped = mcd::warp_sum64(dropped);
-    draws = mcd::warp_sum64(draws);
-    exh = mcd::warp_sum64(exh);
-    exd = mcd::warp_sum64(exd);
-    maxd = mcd::warp_max64(maxd);
-    if ((threadIdx.x & 31u) == 0u) flush(c);
+    src = flights = census = scat = children = 0u;
+    draws = maxd = 0ull;
   }
 };
 
+// Lanes that wait for a source before a warp refills (its seeds, three
+// hashes each, cost the warp the same for one lane as for many), and, once
+// the sources have run out, before it hands pending secondaries to them.
+constexpr int kRefillMin = 3;
+constexpr int kShareMin = 8;
+
+// Bound by integer issue (the logarithm, 59 % of the slots at 21 lanes per
+// instruction).  A lane follows a source particle and its family depth first.  Hash seeds: the secondaries of a collision are one record,
+// the newest of which stays in registers (their seeds are hashed one by one
+// as they are taken), so most collisions touch no memory; and when the
+// sources have run out, lanes with nothing left take records from the lanes
+// of their warp that still hold some -- a stream depends on its seed alone,
+// so who follows it changes nothing.  (Stride: the family shares one stream
+// in depth-first order, so its secondaries stay with their lane.)  Against
+// one record per secondary, all in memory, and no sharing: 58.0 -> 40.4 ms for
+// 3 * 10^7 sources (29.7 -> 16.7 warp instructions per flight at 12.2 -> 20.7
+// lanes; 52.0 ms without the sharing), 3.4 -> 0.5 ms for 5000.  Hash at 64
+// registers (40.4 ms; 46.6 at 84), stride at 72 (15.5 ms for 6 * 10^6; 15.9).
 template <int M, bool HASH, bool AGG>
-__global__ void __launch_bounds__(256) pulse_kernel(const PulseArgs a) {
+__global__ void __launch_bounds__(256, HASH ? 4 : 1) pulse_kernel(const PulseArgs a) {
   __shared__ mcd::Affine tab[64];
   __shared__ PulseDev sP;
+  __shared__ unsigned long long s_counts[MC_NCOUNT];
   if (threadIdx.x == 0) {
-    mcd::Affine sq{a.lcg.g, a.lcg.c};
-    for (int j = 0; j < 64; ++j) { tab[j] = sq; sq = mcd::compose(sq, sq); }
+    if constexpr (!HASH) {
+      mcd::Affine sq{a.lcg.g, a.lcg.c};
+      for (int j = 0; j < 64; ++j) { tab[j] = sq; sq = mcd::compose(sq, sq); }
+    }
     sP = *a.prob;
   }
+  for (uint32_t i = threadIdx.x; i < MC_NCOUNT; i += blockDim.x) s_counts[i] = 0ull;
   __syncthreads();
   const PulseDev& P = sP;
   const mcd::Lcg l = a.lcg;
-  constexpr bool hash_mode = HASH;  // (P.seeding != MC_SEED_STRIDE, chosen by the host)
   const unsigned kFull = 0xffffffffu;
   const unsigned lane = threadIdx.x & 31u;
   const unsigned lt_mask = (1u << lane) - 1u;
 
   const uint64_t nthreads = (uint64_t)gridDim.x * blockDim.x;
   mcp::StackRec* const my_stack = a.stack + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  uint32_t sp = 0;
+  // the lane's records in memory: sp of them, from the lo-th of its
+  // stack_depth entries on, round the end (at most pend - left, so they fit)
+  uint32_t lo = 0, sp = 0;
+  auto entry = [&](uint32_t k) {
+    const uint32_t i = lo + k;
+    return my_stack + (uint64_t)(i >= a.stack_depth ? i - a.stack_depth : i) * nthreads;
+  };
+  // hash: the newest record, in registers; `left` secondaries of it are not
+  // yet taken, `pend` wait in all
+  double tx = 0.0, tt = 0.0;
+  uint64_t ts = 0;
+  uint32_t left = 0, pend = 0;
   uint64_t pool_next = 0, pool_end = 0;
   bool more = true, alive = false, primary = false;
   PulseCounts lc{};
   mcs::Rng<M> r{0ull, 0ull};
   double x = 0.0, t = 0.0, mu = 0.0;
-  uint64_t gi = 0, events = 0, fam_draws = 0;
+  uint64_t gi = 0, events = 0;
   uint32_t grp = 0;
-  unsigned long long* row = nullptr;
   const uint64_t total = a.ovf_in ? min((uint64_t)*a.ovf_in_count, a.ovf_cap) : a.total;
 
   for (;;) {
     unsigned dead = __ballot_sync(kFull, !alive);
-    while (dead != 0u && more) {
-      if (pool_next >= pool_end) {
-        unsigned long long b0 = 0;
-        if (lane == 0) b0 = atomicAdd(a.ticket, (unsigned long long)a.chunk);
-        b0 = __shfl_sync(kFull, b0, 0);
-        if (b0 >= total) { more = false; break; }
-        pool_next = b0;
-        pool_end = min((uint64_t)b0 + (uint64_t)a.chunk, total);
+    if (more && (__popc(dead) >= kRefillMin || dead == kFull)) {
+      while (dead != 0u && more) {
+        if (pool_next >= pool_end) {
+          unsigned long long b0 = 0;
+          if (lane == 0) b0 = atomicAdd(a.ticket, (unsigned long long)a.chunk);
+          b0 = __shfl_sync(kFull, b0, 0);
+          if (b0 >= total) { more = false; break; }
+          pool_next = b0;
+          pool_end = min((uint64_t)b0 + (uint64_t)a.chunk, total);
+        }
+        const uint64_t avail = pool_end - pool_next;
+        const unsigned rank = __popc(dead & lt_mask);
+        if (!alive && rank < avail) {
+          if (a.ovf_in) {
+            // an overflowed secondary: hash seeded, it starts a family of its own
+            const Overflow e = a.ovf_in[pool_next + rank];
+            grp = e.group;
+            r = mcs::Rng<M>{e.seed, 0ull};
+            x = e.x;
+            t = e.t;
+            primary = false;
+          } else {
+            gi = a.range_begin + pool_next + rank;
+            grp = mcp::pulse_group(P, gi);
+            r = mcs::Rng<M>{pulse_seed(P, gi, grp, tab, l.mask), 0ull};
+            x = 0.0;
+            t = 0.0;
+            primary = true;
+            ++lc.src;
+          }
+          mu = mcx::two_u_minus_1(r.next_n(l));
+          events = 0;
+          alive = true;
+        }
+        pool_next += min((uint64_t)__popc(dead), avail);
+        dead = __ballot_sync(kFull, !alive);
       }
-      const uint64_t avail = pool_end - pool_next;
-      const unsigned rank = __popc(dead & lt_mask);
-      if (!alive && rank < avail && a.ovf_in) {
-        // an overflowed secondary: hash seeded, it starts a family of its own
-        const Overflow e = a.ovf_in[pool_next + rank];
-        grp = e.group;
-        row = a.tally + P.tally_offset + (uint64_t)grp * P.n_time_bins;
-        r = mcs::Rng<M>{e.seed, 0ull};
-        x = e.x;
-        t = e.t;
-        mu = mcx::two_u_minus_1(r.next_n(l));
-        events = 0;
-        fam_draws = 0;
-        sp = 0;
-        primary = false;
-        alive = true;
-      } else if (!alive && rank < avail) {
-        gi = a.range_begin + pool_next + rank;
-        grp = (uint32_t)(gi / P.per_batch);
-        row = a.tally + P.tally_offset + (uint64_t)grp * P.n_time_bins;
-        r = mcs::Rng<M>{pulse_seed(P, gi, tab, l.mask), 0ull};
-        x = 0.0;
-        t = 0.0;
-        mu = mcx::two_u_minus_1(r.next_n(l));
-        events = 0;
-        fam_draws = 0;
-        sp = 0;
-        primary = true;
-        ++lc.src;
-        alive = true;
-      }
-      pool_next += min((uint64_t)__popc(dead), avail);
-      dead = __ballot_sync(kFull, !alive);
     }
-    if (__ballot_sync(kFull, alive) == 0u) break;
-    if (!alive) continue;
+    if (dead == kFull) break;  // (while there are sources, the refill leaves some lane alive)
+    bool take = false;  // the lane's next particle is the newest record's next secondary
+    if constexpr (HASH) {
+      if (!more && __popc(dead) >= kShareMin) {
+        // the r-th lane without a particle takes a record of the r-th lane that has one to spare
+        const unsigned donors = __ballot_sync(kFull, alive && pend != 0u);
+        if (donors != 0u) {
+          const unsigned rank = __popc((alive ? donors : dead) & lt_mask);
+          const bool give = alive && pend != 0u && rank < (unsigned)__popc(dead);
+          double rx = tx, rt = tt;
+          uint64_t rs = ts;
+          uint32_t rl = left;
+          if (give) {
+            if (sp != 0u) {  // its oldest
+              mcp::stack_get(entry(0u), rx, rt, rs, rl);
+              --sp;
+              lo = lo + 1u == a.stack_depth ? 0u : lo + 1u;
+            } else {
+              left = 0u;
+            }
+            pend -= rl;
+          }
+          const bool get = !alive && rank < (unsigned)__popc(donors);
+          unsigned m = donors;
+          for (unsigned i = 0; get && i < rank; ++i) m &= m - 1u;
+          const int from = get ? __ffs((int)m) - 1 : (int)lane;
+          rx = __shfl_sync(kFull, rx, from);
+          rt = __shfl_sync(kFull, rt, from);
+          rs = __shfl_sync(kFull, rs, from);
+          rl = __shfl_sync(kFull, rl, from);
+          const uint32_t rg = __shfl_sync(kFull, grp, from);
+          if (get) {
+            tx = rx;
+            tt = rt;
+            ts = rs;
+            left = pend = rl;
+            grp = rg;
+            take = alive = true;
+            primary = false;
+          }
+        }
+      }
+    }
 
-    bool ended = false, redraw = false;
-    if (events == a.event_cap) {
-      ++lc.capped;
-      ended = true;
-    } else {
-      ++events;
-      ++lc.flights;
-      const double d = mclog::neglog1m_n(r.next_n(l)) * P.inv_st;
-      const double tn = t + d;
-      if (!mcs::nn_lt(tn, P.t_end)) {  // tn >= t_end, both non-negative
-        ++lc.census;
+    bool redraw = take;
+    if (alive && !take) {
+      bool ended = false;
+      if (events == a.event_cap) {
+        atomicAdd(s_counts + MC_C_CAPPED, 1ull);
         ended = true;
       } else {
-        const double xn = x + d * mu;
-        ++lc.coll;
-        if (mcx::abs_le(xn, P.x_half)) {
-          const uint64_t jf = mcx::floor_nonneg(tn);
-          const uint32_t j = jf < P.n_time_bins ? (uint32_t)jf : P.n_time_bins - 1;
-          if constexpr (AGG) mcd::warp_agg_add(row + j, (unsigned long long)P.unit);
-          else atomicAdd(row + j, (unsigned long long)P.unit);
-        }
-        x = xn;
-        t = tn;
-        if (r.next_n(l) < P.c_n) {  // u < c
-          ++lc.scat;
-          const uint32_t n = P.nu_floor + (r.next_n(l) >= P.nu_n ? 1u : 0u);  // floor(nu + u)
-          for (uint32_t k = 0; k + 1 < n; ++k) {
-            const uint64_t seed = hash_mode ? (mcd::hash64((uint64_t)k, r.x & l.mask) & l.mask) : 0ull;
-            if (sp < a.stack_depth) {
-              mcp::stack_put(my_stack + sp * nthreads, x, t, seed);
-              ++sp;
-              ++lc.children;
-            } else if (a.ovf_out) {  // hash modes only
-              const unsigned long long idx = atomicAdd(a.ovf_out_count, 1ull);
-              if (idx < a.ovf_cap) {
-                a.ovf_out[idx] = Overflow{x, t, seed, grp, 0u};
-                ++lc.children;
-              } else {
-                ++lc.dropped;
+        ++events;
+        ++lc.flights;
+        const double d = mclog::neglog1m_n(r.next_n(l)) * P.inv_st;
+        const double tn = t + d;
+        if (!mcs::nn_lt(tn, P.t_end)) {  // tn >= t_end, both non-negative
+          ++lc.census;
+          ended = true;
+        } else {
+          const double xn = x + d * mu;
+          if (mcx::abs_le(xn, P.x_half)) {
+            const uint64_t jf = mcx::floor_nonneg(tn);
+            const uint32_t j = jf < P.n_time_bins ? (uint32_t)jf : P.n_time_bins - 1;
+            unsigned long long* const slot = a.tally + P.tally_offset + (uint64_t)grp * P.n_time_bins + j;
+            if constexpr (AGG) mcd::warp_agg_add(slot, (unsigned long long)P.unit);
+            else atomicAdd(slot, (unsigned long long)P.unit);
+          }
+          x = xn;
+          t = tn;
+          if (r.next_n(l) < P.c_n) {  // u < c
+            ++lc.scat;
+            const uint32_t n = P.nu_floor + (r.next_n(l) >= P.nu_n ? 1u : 0u);  // floor(nu + u)
+            if constexpr (HASH) {
+              const uint32_t kids = n - 1u, room = a.stack_depth - pend, fit = min(kids, room);
+              if (fit != 0u) {
+                if (left != 0u) {
+                  mcp::stack_put(entry(sp), tx, tt, ts, left);
+                  ++sp;
+                }
+                tx = x;
+                tt = t;
+                ts = r.x & l.mask;
+                left = fit;
+                pend += fit;
               }
+              for (uint32_t k = fit; k < kids; ++k) {  // a full stack: to the overflow bank
+                const unsigned long long idx = atomicAdd(a.ovf_out_count, 1ull);
+                if (idx < a.ovf_cap) a.ovf_out[idx] = Overflow{x, t, mcd::hash64(k, r.x & l.mask) & l.mask, grp, 0u};
+                else atomicAdd(s_counts + MC_C_DROPPED, 1ull);  // reported as MC_ERR_CAPACITY by mc_tally_read
+                lc.children += idx < a.ovf_cap ? 1u : 0u;
+              }
+              lc.children += fit;
             } else {
-              ++lc.dropped;  // reported as MC_ERR_CAPACITY by mc_tally_read
+              for (uint32_t k = 0; k + 1 < n; ++k) {
+                if (sp < a.stack_depth) {
+                  mcp::stack_put(entry(sp), x, t, 0ull, 1u);
+                  ++sp;
+                  ++lc.children;
+                } else {
+                  atomicAdd(s_counts + MC_C_DROPPED, 1ull);
+                }
+              }
+            }
+            redraw = true;
+          } else {
+            ended = true;
+          }
+        }
+      }
+      if (ended) {  // the current particle ended
+        if (HASH || sp == 0u) {  // and with it its stream
+          lc.draws += r.draws;
+          if (r.draws > lc.maxd) lc.maxd = r.draws;
+          if (!HASH || primary) {
+            if (a.hist_state) a.hist_state[gi] = r.x & l.mask;
+            if (a.hist_draws) a.hist_draws[gi] = r.draws;
+            if (P.stride_q != 0 && r.draws > P.stride_q) {
+              atomicAdd(s_counts + MC_C_EXCEED_HIST, 1ull);
+              atomicAdd(s_counts + MC_C_EXCEED_DRAWS, (unsigned long long)(r.draws - P.stride_q));
             }
           }
-          // its new direction: drawn in place (hash) or below, on the code path the
-          // pop shares (stride; measured faster for each variant)
-          if constexpr (HASH) mu = mcx::two_u_minus_1(r.next_n(l));
-          else redraw = true;
-        } else {
-          ++lc.absn;
-          ended = true;
         }
-      }
-    }
-    if (ended) {  // the current particle ended
-      if (hash_mode) {
-        fam_draws += r.draws;
-        if (r.draws > lc.maxd) lc.maxd = r.draws;
-        if (primary) {
-          if (a.hist_state) a.hist_state[gi] = r.x & l.mask;
-          if (a.hist_draws) a.hist_draws[gi] = r.draws;
-          if (P.stride_q != 0 && r.draws > P.stride_q) { ++lc.exh; lc.exd += r.draws - P.stride_q; }
-        }
-      }
-      primary = false;
-      events = 0;
-      if (sp > 0) {  // the next secondary of the family; its direction below
-        --sp;
-        uint64_t seed;
-        mcp::stack_get(my_stack + sp * nthreads, x, t, seed);
+        primary = false;
+        events = 0;
         if constexpr (HASH) {
-          r = mcs::Rng<M>{seed, 0ull};
-          mu = mcx::two_u_minus_1(r.next_n(l));
+          take = pend != 0u;
+          alive = take;
         } else {
-          redraw = true;
+          alive = sp != 0u;
+          if (alive) {  // the next secondary of the family, on the family's stream
+            --sp;
+            uint64_t s;
+            uint32_t n;
+            mcp::stack_get(entry(sp), x, t, s, n);
+          }
         }
-      } else {
-        if (!hash_mode) {
-          fam_draws = r.draws;
-          if (r.draws > lc.maxd) lc.maxd = r.draws;
-          if (a.hist_state) a.hist_state[gi] = r.x & l.mask;
-          if (a.hist_draws) a.hist_draws[gi] = r.draws;
-          if (P.stride_q != 0 && r.draws > P.stride_q) { ++lc.exh; lc.exd += r.draws - P.stride_q; }
-        }
-        lc.draws += fam_draws;
-        alive = false;
+        redraw = alive;
+        if (lc.flights > (1u << 24)) lc.flush(a.counts);  // (up to 63 secondaries each)
       }
     }
-    // stride: one code path draws the direction of a scattered or a popped
-    // particle (the same draw, in the same stream order, as drawing it in place)
+    if constexpr (HASH) {
+      if (take) {  // Eq. (5)
+        --pend;
+        --left;
+        x = tx;
+        t = tt;
+        r = mcs::Rng<M>{mcd::hash64((uint64_t)left, ts) & l.mask, 0ull};
+        events = 0;
+        if (left == 0u && sp != 0u) {
+          --sp;
+          mcp::stack_get(entry(sp), tx, tt, ts, left);
+        }
+      }
+    }
+    // one code path draws the direction of a scattered and of a new particle
+    // (the same draw, in the same stream order, as drawing it in place)
     if (redraw) mu = mcx::two_u_minus_1(r.next_n(l));
   }
-  lc.flush_warp(a.counts);
+  // the lanes' counts, summed over the warp (they share a cache line)
+  {
+    const unsigned long long so = mcd::warp_sum64(lc.src), fl = mcd::warp_sum64(lc.flights),
+                             ce = mcd::warp_sum64(lc.census), sc = mcd::warp_sum64(lc.scat),
+                             ch = mcd::warp_sum64(lc.children), dr = mcd::warp_sum64(lc.draws),
+                             mx = mcd::warp_max64(lc.maxd);
+    if (lane == 0) {
+      atomicAdd(s_counts + MC_C_SOURCE, so);
+      atomicAdd(s_counts + MC_C_FLIGHTS, fl);
+      atomicAdd(s_counts + MC_C_COLLISIONS, fl - ce);
+      atomicAdd(s_counts + MC_C_ABSORPTIONS, fl - ce - sc);
+      atomicAdd(s_counts + MC_C_SCATTERS, sc);
+      atomicAdd(s_counts + MC_C_LEAK_HI, ce);
+      atomicAdd(s_counts + MC_C_CHILDREN, ch);
+      atomicAdd(s_counts + MC_C_DRAWS, dr);
+      atomicMax(s_counts + MC_C_MAX_DRAWS, mx);
+    }
+  }
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < MC_NCOUNT; i += blockDim.x) {
+    const unsigned long long v = s_counts[i];
+    if (v == 0ull) continue;
+    if (i == MC_C_MAX_DRAWS) atomicMax(a.counts + i, v);
+    else atomicAdd(a.counts + i, v);
+  }
 }
 
 }  // namespace

@@ -26,30 +26,36 @@ struct PulseDev {
 
 constexpr int kStack = 256;  // most pending secondaries a lane keeps (run config stack_depth)
 
-// A pending secondary on a lane's local stack (census phases: shallow
-// families, where the L1-resident local stack measured faster).
+// Pending secondaries of one collision on a lane's local stack (census
+// phases: shallow families, where the L1-resident local stack measured
+// faster); the fields are StackRec's.
 struct Pending {
   double x, t;
-  uint64_t seed;
+  uint64_t s;
+  uint32_t left, pad;
 };
 
-// A pending secondary in device memory (one 32-byte sector): the stacks of
+// Pending secondaries in device memory (one 32-byte sector): the stacks of
 // all lanes of a launch, depth-major (entry j of every lane together), so a
 // push writes one whole sector and the shallow entries, the busy ones, stay
-// together in L2.
+// together in L2.  Hash seeds: one record holds all secondaries of a
+// collision (its point, the parent's state S_p and how many are left; the
+// k-th is seeded hash(k, S_p) when it is taken).  Stride: one record each.
 struct __align__(32) StackRec {
   double x, t;
-  uint64_t seed, pad;
+  uint64_t s, left;
 };
-__device__ __forceinline__ void stack_put(StackRec* e, double x, double t, uint64_t seed) {
+__device__ __forceinline__ void stack_put(StackRec* e, double x, double t, uint64_t s, uint32_t left) {
   reinterpret_cast<double2*>(e)[0] = make_double2(x, t);
-  reinterpret_cast<ulonglong2*>(e)[1] = make_ulonglong2(seed, 0ull);
+  reinterpret_cast<ulonglong2*>(e)[1] = make_ulonglong2(s, left);
 }
-__device__ __forceinline__ void stack_get(const StackRec* e, double& x, double& t, uint64_t& seed) {
+__device__ __forceinline__ void stack_get(const StackRec* e, double& x, double& t, uint64_t& s, uint32_t& left) {
   const double2 v = reinterpret_cast<const double2*>(e)[0];
+  const ulonglong2 w = reinterpret_cast<const ulonglong2*>(e)[1];
   x = v.x;
   t = v.y;
-  seed = reinterpret_cast<const ulonglong2*>(e)[1].x;
+  s = w.x;
+  left = (uint32_t)w.y;
 }
 
 // A hash-seeded secondary that did not fit on its lane's stack (32 bytes):
@@ -61,12 +67,19 @@ struct Overflow {
   uint32_t pad;
 };
 
-__device__ __forceinline__ uint64_t pulse_seed(const PulseDev& P, uint64_t g, const mcd::Affine* tab,
+// The (rep, batch) group of history g (on 32 bits where they hold g: a
+// 64-bit division takes five times as long).
+__device__ __forceinline__ uint32_t pulse_group(const PulseDev& P, uint64_t g) {
+  return (g >> 32) == 0ull ? (uint32_t)g / P.per_batch : (uint32_t)(g / P.per_batch);
+}
+
+// The seed of history g of group grp (Eqs. 2-4).
+__device__ __forceinline__ uint64_t pulse_seed(const PulseDev& P, uint64_t g, uint32_t grp, const mcd::Affine* tab,
                                                uint64_t mask) {
   if (P.seeding == MC_SEED_STRIDE) return mcs::skip_tab(tab, P.seed, P.stride_q * (P.id_offset + g)) & mask;
   if (P.seeding == MC_SEED_HASH) return mcd::hash_with(g, P.seed_hash) & mask;
-  const uint64_t pb = P.per_batch, nb = P.n_batches;
-  const uint64_t rep = g / (pb * nb), batch = (g / pb) % nb, part = g % pb;
+  const uint32_t rep = grp / P.n_batches, batch = grp - rep * P.n_batches;
+  const uint64_t part = g - (uint64_t)grp * P.per_batch;
   const uint64_t h_rep = mcd::hash64(rep, P.seed);
   return mcd::hash64(part, mcd::hash64(batch, h_rep)) & mask;
 }
