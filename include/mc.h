@@ -85,13 +85,12 @@ MC_API void mc_ctx_destroy(mc_ctx* ctx);
  * would not end into an error status instead of a hang; the defaults are
  * far above anything a valid run needs, and lowering them exists to test
  * the give-up paths.  Every field is taken literally (0 is a bound of 0).
- *   pool_lock_attempts  slab history kernel: attempts a warp makes at its
- *                       block's compaction-pool lock before it gives up
- *                       (default 2^20).  A warp that gives up skips the
- *                       hand-over; one that is leaving counts what the pool
- *                       may still hold in MC_C_DROPPED, which mc_tally_read
- *                       reports as MC_ERR_CAPACITY.  0: no warp ever takes
- *                       the lock, so no particle moves (tallies unchanged).
+ *   pool_lock_attempts  slab history kernel: 0 keeps every history on the
+ *                       lane that started it; otherwise (default 2^20) the
+ *                       warps of a block hand their last, long histories to
+ *                       the block's cooperative tail once the work has run
+ *                       out.  Nothing waits for a lock any more, so any other
+ *                       value means the same.  The tallies do not depend on it.
  *   box_generations     generations of weight-window children the host
  *                       follows before MC_ERR_TIMEOUT (default 10000).
  *   pulse_generations   generations of overflowed pulse secondaries (hash

@@ -5,13 +5,15 @@
 // direction stay in registers.  Each loop iteration every live lane flies
 // one flight (and collides once); a lane whose history ended refills from
 // its warp's chunk of history indices, and the warp leader takes a new chunk
-// from a global ticket when the chunk runs dry.  So a warp keeps all 32
-// lanes busy until the ticket is exhausted, however uneven the histories.
+// from a global ticket when the chunk runs dry.  So a warp keeps its lanes
+// busy until the ticket is exhausted, however uneven the histories; the long
+// ones that are left then are finished by the whole block together.
 //
 // Tallies are int64 fixed point (2^32), staged in shared memory when the
 // whole tally fits and flushed with one global atomic per nonzero slot per
-// block; otherwise contributions go straight to global atomics.  Counters
-// are accumulated per lane and flushed when a lane changes problem.
+// block; otherwise each warp caches the tally row most of its lanes are on,
+// and other contributions go to global atomics.  Counters are accumulated
+// per lane and flushed when a lane changes problem.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -116,70 +118,13 @@ struct RunArgs {
   uint32_t smem_slots;
   uint32_t smem_edges;  // single-problem launches: n_bins + 1 edges in shared memory (0: none)
   const double* tables; // else per-problem edge and width tables in global memory (nullable)
-  uint32_t donate_max;  // a warp with 1..donate_max live lanes after the ticket ran out donates them
-  uint32_t pool_cap;    // particles the block's shared pool holds (0: no compaction)
-  uint32_t lock_attempts;  // attempts at the pool lock before a warp gives up
-  uint32_t coop_slots;     // event records of the cooperative tail the pool's memory holds
+  uint32_t grab_shift;  // a warp takes at most 2^-grab_shift of the histories left at once,
+  uint32_t min_grab;    // but at least min_grab
+  uint32_t row_bins;    // bins of a warp's row cache (0: none; all problems fit it otherwise)
+  uint32_t coop_hist;   // histories the block's cooperative tail takes over (0: none)
+  uint32_t coop_slots;  // its event records, a power of two
   mcs::Order order;        // processing order of several problems (empty: id order)
 };
-
-// In-block compaction of the long-chain tail.  Once the ticket runs out,
-// lanes whose histories end are no longer refilled and warps thin out (the
-// fp64 slab ran at 4 live lanes of 32).  A warp left with few live lanes
-// hands them to a shared-memory pool of its block and leaves the loop; warps
-// with dead lanes take them from the pool.  A particle carries its whole
-// state (stream, position, direction, history index, flight count), so the
-// move changes no draw and no result.  The pool is guarded by a lock taken
-// by one lane per warp, with bounded attempts; a warp that cannot take it
-// skips the hand-over (or, leaving, counts the stranded particles in
-// MC_C_DROPPED, the error the host reports).
-constexpr int kPoolWords = 10;
-struct PoolCtl {
-  int lock, n, active, pad;
-};
-
-__device__ __forceinline__ bool pool_lock(int* lk, uint32_t attempts) {
-  for (uint32_t i = 0; i < attempts; ++i)
-    if (atomicCAS(lk, 0, 1) == 0) {
-      __threadfence_block();
-      return true;
-    }
-  return false;
-}
-__device__ __forceinline__ void pool_unlock(int* lk) {
-  __threadfence_block();
-  atomicExch(lk, 0);
-}
-
-__device__ __forceinline__ void pool_put(unsigned long long* e, uint64_t x, const mcs::SlabParticle& q, uint64_t gi,
-                                         uint64_t events, uint32_t pi) {
-  e[0] = x;
-  e[1] = (unsigned long long)(uint32_t)q.j;
-  e[2] = (unsigned long long)__double_as_longlong(q.x);
-  e[3] = (unsigned long long)__double_as_longlong(q.mu);
-  e[4] = (unsigned long long)__double_as_longlong(q.w_mu);
-  e[5] = ((unsigned long long)__float_as_uint(q.muf) << 32) | __float_as_uint(q.xf);
-  e[6] = ((unsigned long long)pi << 32) | __float_as_uint(q.wf);
-  e[7] = gi;
-  e[8] = events;
-  e[9] = __float_as_uint(q.xlo);
-}
-
-__device__ __forceinline__ uint32_t pool_get(const unsigned long long* e, uint64_t& x, mcs::SlabParticle& q,
-                                             uint64_t& gi, uint64_t& events) {
-  x = e[0];
-  q.j = (int)(uint32_t)e[1];
-  q.x = __longlong_as_double((long long)e[2]);
-  q.mu = __longlong_as_double((long long)e[3]);
-  q.w_mu = __longlong_as_double((long long)e[4]);
-  q.xf = __uint_as_float((uint32_t)e[5]);
-  q.muf = __uint_as_float((uint32_t)(e[5] >> 32));
-  q.wf = __uint_as_float((uint32_t)e[6]);
-  gi = e[7];
-  events = e[8];
-  q.xlo = __uint_as_float((uint32_t)e[9]);
-  return (uint32_t)(e[6] >> 32);
-}
 
 // What the end of a history and the cooperative tail need of the launch.
 struct TailArgs {
@@ -283,54 +228,38 @@ __device__ __forceinline__ void end_history(const TailArgs& t, const SlabDev* pr
   if (lc.flights > (1u << 30)) lc.flush(t.counts, probs);
 }
 
-// Cooperative tail.  When the ticket has run out, the block's pool is empty
-// and its last warp holds at most kCoopMax live histories, the rest of the
-// launch is the latency of those few chains: one lane runs each, and a
-// flight's dependent instructions (the logarithm of its uniform, its product
-// with the direction, the absorption test, the next direction and its
-// reciprocal) leave the other lanes idle.  But a history's draws have fixed
-// roles -- each event takes one draw for the distance, one for the
+// Cooperative tail.  Once the ticket has run out, a block's lanes are no
+// longer refilled: what is left is a heavy tail of long histories, and one
+// lane runs each of them at the latency of a flight's dependent instructions
+// (3600 cycles) while the rest of the block idles.  But a history's draws have
+// fixed roles -- each event takes one draw for the distance, one for the
 // absorption test and one for the new direction, until the history ends --
-// so everything that depends on the draws alone can be computed ahead.  The
-// warp splits into one group of 32 / kp lanes per live history (kp: the live
-// count rounded up to a power of two) and advances every history by rounds
-// of E events:
-//   1. the group's lanes compute, for each event e of the round, the
-//      distance d_e, the product p_e = d_e mu_e, the absorption test and the
-//      direction mu_{e+1} with its tally weight, jumping the stream to draw
-//      3e with the maps of 2^j steps;
-//   2. one lane runs the chain of positions alone, x_{e+1} = x_e + p_e and
-//      the face tests, until the round ends or the history does (an event
-//      cap, a leak, an absorption);
-//   3. the group's lanes make the tally contributions of the round's events.
-// Every value comes from the same function, with the same operands, as in
-// the one-lane path, so the draws, tallies and counters are the same bits.
-// The histories' state and the rounds' event records sit in the (then
-// empty) pool's shared memory, the launch's arguments in a small shared
-// record, and each phase is a function of its own that takes them from
-// there: the main loop has ended, and almost nothing stays in registers
-// across the calls.
-constexpr int kCoopMax = 4;            // live histories at most
-constexpr int kCoopHistWords = 12;     // 8-byte words per history record
-constexpr int kCoopWords = 6;          // 8-byte words per event record
-constexpr uint32_t kCoopEvents = 128;  // events per history and round at most
-constexpr uint32_t kCoopMinEvents = 8;
-// shared memory the tail's records get at least (words): room for rounds of
-// kCoopEvents events with one history
-constexpr size_t kCoopAreaWords = (size_t)kCoopMax * kCoopHistWords + (size_t)kCoopWords * (kCoopEvents + 1u);
-
-__device__ __forceinline__ int coop_groups(int nlive) { return nlive <= 1 ? 1 : nlive <= 2 ? 2 : nlive <= 4 ? 4 : 8; }
-
-__device__ __forceinline__ uint32_t coop_events(uint32_t slots, int kp) {
-  const uint32_t per = slots / (uint32_t)kp;  // records per history: E events and the direction after them
-  return per > 1u ? min(kCoopEvents, per - 1u) : 0u;
-}
-
-// Event records the pool's memory holds beside the history records.
-__host__ __device__ __forceinline__ uint32_t coop_slots_of(uint32_t pool_words) {
-  const uint32_t h = (uint32_t)(kCoopMax * kCoopHistWords);
-  return pool_words > h ? (pool_words - h) / (uint32_t)kCoopWords : 0u;
-}
+// so everything that depends on the draws alone can be computed ahead, by any
+// thread.  When a block's live histories are down to a quarter of its threads
+// (and have shown that they are long ones), its warps put them into records in
+// shared memory and the whole block advances all of them by rounds of E
+// events:
+//   1. every thread computes events of the round: the product p_e = d_e mu_e,
+//      the absorption test and the tally weight, jumping the history's stream
+//      to draw 3e with the maps of 2^j steps;
+//   2. one thread per history runs the chain of positions alone,
+//      x_{e+1} = x_e + p_e and the face tests, until the round ends or the
+//      history does (an event cap, a leak, an absorption);
+//   3. every thread tallies events of the round.
+// E grows as histories end, so that a round always fills the block.  Every
+// value comes from the same function, with the same operands, as in the
+// one-lane path, so the draws, tallies and counters are the same bits.
+//
+// An event's record is two words.  fp64: p_e, which the walk replaces by
+// x_{e+1}, and the tally weight with the absorption test in its sign bit.
+// fp32: the pair (pr, pe), replaced by the position pair, and (wf, muf) with
+// the test in wf's sign bit.
+constexpr int kCoopHistWords = 14;    // 8-byte words per history record
+constexpr int kCoopWords = 2;         // per event record
+constexpr int kCoopMaxLog = 8;        // at most 2^8 records per history and round
+constexpr int kCoopMinLog = 3;        // at least 2^3: E = 7 events
+constexpr uint32_t kCoopAfter = 32;   // passes of a warp after the ticket ran out before it offers its histories
+constexpr uint32_t kCoopMaxHist = 256;
 
 __device__ __forceinline__ mcd::Affine affine_steps(const mcd::Affine* tab, uint64_t k) {
   mcd::Affine acc{1ull, 0ull};
@@ -350,22 +279,24 @@ __device__ __forceinline__ float hi_of(unsigned long long w) { return __uint_as_
 __device__ __forceinline__ unsigned long long dbits(double v) { return (unsigned long long)__double_as_longlong(v); }
 __device__ __forceinline__ double dval(unsigned long long w) { return __longlong_as_double((long long)w); }
 
-// A history's record: its stream, particle, ids, tally sink and the counts
-// of its events in the tail.
+// A history's record: its stream, particle, ids and tally sink, and the last
+// round it ran.
 struct CoopHist {
   unsigned long long* w;
   enum {
     kX = 0,      // stream state
     kPos,        // fp64 x (fp32: xf, xlo)
-    kDir,        // fp64 mu (fp32: muf, wf)
-    kW,          // fp64 2^32 / |mu|
+    kDir,        // fp64 mu (fp32: muf in the high half)
+    kW,          // fp64 2^32 / |mu| (fp32: wf in the low half)
     kGi,         // global history index
     kEvents,     // flights flown
     kProb,       // problem index; bit 32: live
     kBase,       // tally row
     kEdges,      // edge and width tables (null: computed)
     kWidths,
-    kEnd         // last round: events run (low half) and how the last one ended (high half)
+    kEnd,        // last round: events run (low half) and how the last one ended (high half)
+    kX0,         // stream state and position at its start
+    kPos0
   };
   __device__ __forceinline__ explicit CoopHist(unsigned long long* p) : w(p) {}
   __device__ __forceinline__ bool live() const { return (w[kProb] >> 32) != 0ull; }
@@ -376,108 +307,71 @@ struct CoopHist {
   }
 };
 
-// The records of one history's round, six arrays of E + 1 words.
-struct CoopRec {
-  unsigned long long* p;  // p_e = d_e mu_e (fp32: pr and pe, the product and its error)
-  unsigned long long* d;  // d_e (fp32: d_e and muf_e)
-  unsigned long long* m;  // mu_e (fp32: the state of event e's distance draw)
-  unsigned long long* w;  // tally weight of event e's flight
-  unsigned long long* x;  // position at the start of event e
-  unsigned long long* f;  // absorption test of event e
-  __device__ __forceinline__ CoopRec(unsigned long long* r, uint32_t E)
-      : p(r), d(r + (E + 1u)), m(r + 2u * (E + 1u)), w(r + 3u * (E + 1u)), x(r + 4u * (E + 1u)),
-        f(r + 5u * (E + 1u)) {}
-};
+constexpr unsigned long long kAbsBit = 1ull << 63;  // fp64 weight word: the event's absorption test
 
-// Phase 1, on lane hl of the G lanes of a history's group: the draw-only
-// values of the events e = hl, hl + G, ... <= E.
+// Phase 1 for event e of E of the history in H, whose stream is xs after the
+// 3e draws before it: the event's record, or (e = E) the direction after the
+// round.
 template <int M, bool F32>
-__device__ __noinline__ void coop_draws(const CoopArgs* c, const mcd::Affine* tab, uint32_t hist_off,
-                                        uint32_t rec_off, uint32_t E, int G, int hl) {
-  extern __shared__ unsigned long long s_dyn[];
-  const CoopHist H(s_dyn + hist_off);
-  const CoopRec R(s_dyn + rec_off, E);
-  const mcd::Lcg l = c->t.lcg;
-  const SlabDev& p = *H.prob(c->probs);
-  const uint64_t x0 = H.w[CoopHist::kX];
-  const unsigned long long dir0 = H.w[CoopHist::kDir], w0 = H.w[CoopHist::kW];
-  const mcd::Affine step3g = affine_steps(tab, 3ull * (uint64_t)G);
-  uint64_t xs = mcs::skip_tab(tab, x0, 3ull * (uint64_t)hl);  // the state after 3e draws
-  for (uint32_t e = (uint32_t)hl; e <= E; e += (uint32_t)G) {
-    if constexpr (!F32) {
-      double mu = dval(dir0), w = dval(w0);
-      if (e != 0u) {
-        mu = mcx::two_u_minus_1(mcd::u53<M>(xs, l.m));
-        w = mcs::fix_per_mu(mu);
-      }
-      R.m[e] = dbits(mu);
-      R.w[e] = dbits(w);
-      if (e < E) {
-        const uint64_t sd = mcd::lcg_step(xs, l.g, l.c);
-        const double d = __dmul_rn(mclog::neglog1m_n(mcd::u53<M>(sd, l.m)), p.inv_st);
-        R.d[e] = dbits(d);
-        R.p[e] = dbits(__dmul_rn(d, mu));
-        R.f[e] = mcd::u53<M>(mcd::lcg_step(sd, l.g, l.c), l.m) < p.p_abs_n ? 1ull : 0ull;
-      }
-    } else {
-      float muf = lo_of(dir0), wf = hi_of(dir0);
-      if (e != 0u) {
-        muf = mcs::mu_f32(mcd::u53<M>(xs, l.m));
-        wf = muf != 0.0f ? __frcp_rn(fabsf(muf)) : 0.0f;
-      }
-      R.w[e] = pack2(wf, 0.0f);
-      float d = 0.0f;
-      if (e < E) {
-        const uint64_t sd = mcd::lcg_step(xs, l.g, l.c);
-        d = mcs::flight_f32(mcd::u53<M>(sd, l.m)) * p.inv_st_f;
-        const float pr = __fmul_rn(d, muf);
-        R.p[e] = pack2(pr, __fmaf_rn(d, muf, -pr));
-        R.m[e] = sd;
-        R.f[e] = mcd::u53<M>(mcd::lcg_step(sd, l.g, l.c), l.m) < p.p_abs_n ? 1ull : 0ull;
-      }
-      R.d[e] = pack2(d, muf);
-    }
-    xs = mcd::apply(step3g, xs);
+__device__ __forceinline__ void coop_draw(const CoopHist& H, const SlabDev& p, const mcd::Lcg& l, uint64_t xs,
+                                          uint32_t e, uint32_t E, unsigned long long* rec) {
+  const uint64_t sd = mcd::lcg_step(xs, l.g, l.c);
+  const bool absorbed = mcd::u53<M>(mcd::lcg_step(sd, l.g, l.c), l.m) < p.p_abs_n;
+  mcs::SlabParticle q;
+  mcs::set_direction<F32>(q, mcd::u53<M>(xs, l.m));
+  if constexpr (!F32) {
+    const double d = __dmul_rn(mclog::neglog1m_n(mcd::u53<M>(sd, l.m)), p.inv_st);
+    const double mu = e == 0u ? dval(H.w[CoopHist::kDir]) : q.mu, w = e == 0u ? dval(H.w[CoopHist::kW]) : q.w_mu;
+    rec[0] = dbits(e == E ? mu : __dmul_rn(d, mu));
+    rec[1] = dbits(w) | (absorbed && e != E ? kAbsBit : 0ull);
+  } else {
+    const float d = mcs::flight_f32(mcd::u53<M>(sd, l.m)) * p.inv_st_f;
+    const float muf = e == 0u ? hi_of(H.w[CoopHist::kDir]) : q.muf, wf = e == 0u ? lo_of(H.w[CoopHist::kW]) : q.wf;
+    const float pr = __fmul_rn(d, muf);
+    rec[0] = pack2(pr, __fmaf_rn(d, muf, -pr));
+    rec[1] = pack2(__uint_as_float(__float_as_uint(wf) | (absorbed && e != E ? 0x80000000u : 0u)), muf);
   }
 }
 
-// Phase 2, on one lane: the chain of positions through the round's events,
+// Phase 2, on one thread: the chain of positions through the round's events,
 // until the round ends (kContinue), an event would pass the cap (-1), or the
 // history leaks or is absorbed.  Then the history's record moves on by the
 // events run, and a history that ended is counted and written out.
 template <int M, bool F32>
-__device__ __noinline__ void coop_walk(const CoopArgs* c, const mcd::Affine* tab, uint32_t hist_off,
-                                       uint32_t rec_off, uint32_t E) {
-  extern __shared__ unsigned long long s_dyn[];
-  const CoopHist H(s_dyn + hist_off);
-  const CoopRec R(s_dyn + rec_off, E);
-  const SlabDev* P = H.prob(c->probs);
-  const SlabDev p = *P;
-  const uint64_t events = H.w[CoopHist::kEvents];
-  const uint64_t left = c->t.event_cap - events;  // events never pass the cap
-  const uint32_t ok = left < E ? (uint32_t)left : E;
+__device__ __noinline__ void coop_walk(const CoopArgs* c, const mcd::Affine* tab, unsigned long long* hist,
+                                       unsigned long long* rec, uint32_t E) {
+  const CoopHist H(hist);
+  const SlabDev& p = *H.prob(c->probs);
+  const uint64_t events = H.w[CoopHist::kEvents], x0 = H.w[CoopHist::kX];
+  const uint64_t cap_left = c->t.event_cap - events;  // events never pass the cap
+  const uint32_t ok = cap_left < E ? (uint32_t)cap_left : E;
   int out = mcs::kContinue;
   uint32_t e = 0;
+  H.w[CoopHist::kX0] = x0;
+  H.w[CoopHist::kPos0] = H.w[CoopHist::kPos];
   // Four events at a time while none of them can end the history (no
   // leak, no absorption, no cap, and in fp32 no guard band): the chain of
   // additions runs back to back and one branch takes the four.  Otherwise
-  // one event at a time, with the same operations.
+  // one event at a time, with the same operations.  (p_e = d_e mu_e has the
+  // sign of mu_e, or is zero: the face tests take it for mu_e.)
   if constexpr (!F32) {
     double x = dval(H.w[CoopHist::kPos]);
-    R.x[0] = dbits(x);
+    const double L = p.L;
+    auto leaves = [&](unsigned long long pb, double xn) {
+      return ((long long)pb > 0 && !mcs::nn_lt(xn, L)) || ((long long)pb < 0 && __double_as_longlong(xn) <= 0);
+    };
     for (;;) {
+      unsigned long long* const r = rec + kCoopWords * e;
       if (e + 4u <= ok) {
-        const double p0 = dval(R.p[e]), p1 = dval(R.p[e + 1u]), p2 = dval(R.p[e + 2u]), p3 = dval(R.p[e + 3u]);
-        const long long m0 = (long long)R.m[e], m1 = (long long)R.m[e + 1u], m2 = (long long)R.m[e + 2u],
-                        m3 = (long long)R.m[e + 3u];
-        const unsigned long long a = R.f[e] | R.f[e + 1u] | R.f[e + 2u] | R.f[e + 3u];
-        const double x1 = __dadd_rn(x, p0), x2 = __dadd_rn(x1, p1), x3 = __dadd_rn(x2, p2), x4 = __dadd_rn(x3, p3);
-        if (!(a | mcs::leaves64(p, m0, x1) | mcs::leaves64(p, m1, x2) | mcs::leaves64(p, m2, x3) |
-              mcs::leaves64(p, m3, x4))) {
-          R.x[e + 1u] = dbits(x1);
-          R.x[e + 2u] = dbits(x2);
-          R.x[e + 3u] = dbits(x3);
-          R.x[e + 4u] = dbits(x4);
+        const unsigned long long b0 = r[0], b1 = r[2], b2 = r[4], b3 = r[6];
+        const unsigned long long a = r[1] | r[3] | r[5] | r[7];
+        const double x1 = __dadd_rn(x, dval(b0)), x2 = __dadd_rn(x1, dval(b1)), x3 = __dadd_rn(x2, dval(b2)),
+                     x4 = __dadd_rn(x3, dval(b3));
+        if (!((a & kAbsBit) != 0ull || leaves(b0, x1) || leaves(b1, x2) || leaves(b2, x3) || leaves(b3, x4))) {
+          r[0] = dbits(x1);
+          r[2] = dbits(x2);
+          r[4] = dbits(x3);
+          r[6] = dbits(x4);
           x = x4;
           e += 4u;
           continue;
@@ -486,36 +380,39 @@ __device__ __noinline__ void coop_walk(const CoopArgs* c, const mcd::Affine* tab
       if (e == E) break;
       if (e == ok) { out = -1; break; }
       double xn;
-      const int f = mcs::advance64(p, x, dval(R.m[e]), dval(R.p[e]), xn);
+      const int f = mcs::advance64(p, x, dval(r[0]), dval(r[0]), xn);
       if (f != mcs::kCollide) { out = f; ++e; break; }
       x = xn;
-      R.x[e + 1u] = dbits(x);
-      if (R.f[e]) { out = mcs::kAbsorbed; ++e; break; }
+      r[0] = dbits(x);
       ++e;
+      if (r[1] & kAbsBit) { out = mcs::kAbsorbed; break; }
     }
     H.w[CoopHist::kPos] = dbits(x);
-    if (out == mcs::kContinue) { H.w[CoopHist::kDir] = R.m[E]; H.w[CoopHist::kW] = R.w[E]; }
+    if (out == mcs::kContinue) {
+      H.w[CoopHist::kDir] = rec[kCoopWords * E];
+      H.w[CoopHist::kW] = rec[kCoopWords * E + 1u];
+    }
   } else {
     const unsigned long long pos = H.w[CoopHist::kPos];
     float xf = lo_of(pos), xlo = hi_of(pos);
-    R.x[0] = pos;
-    const uint32_t m = c->t.lcg.m;
+    const mcd::Lcg l = c->t.lcg;
     for (;;) {
+      unsigned long long* const r = rec + kCoopWords * e;
       if (e + 4u <= ok) {
-        const unsigned long long q0 = R.p[e], q1 = R.p[e + 1u], q2 = R.p[e + 2u], q3 = R.p[e + 3u];
-        const float u0 = hi_of(R.d[e]), u1 = hi_of(R.d[e + 1u]), u2 = hi_of(R.d[e + 2u]), u3 = hi_of(R.d[e + 3u]);
-        const unsigned long long a = R.f[e] | R.f[e + 1u] | R.f[e + 2u] | R.f[e + 3u];
+        const unsigned long long q0 = r[0], q1 = r[2], q2 = r[4], q3 = r[6];
+        const unsigned long long w0 = r[1], w1 = r[3], w2 = r[5], w3 = r[7];
         float h1, l1, h2, l2, h3, l3, h4, l4;
         mcs::pair_step(xf, xlo, lo_of(q0), hi_of(q0), h1, l1);
         mcs::pair_step(h1, l1, lo_of(q1), hi_of(q1), h2, l2);
         mcs::pair_step(h2, l2, lo_of(q2), hi_of(q2), h3, l3);
         mcs::pair_step(h3, l3, lo_of(q3), hi_of(q3), h4, l4);
-        if (a == 0ull && mcs::plain_collision32(p, u0, h1, l1) && mcs::plain_collision32(p, u1, h2, l2) &&
-            mcs::plain_collision32(p, u2, h3, l3) && mcs::plain_collision32(p, u3, h4, l4)) {
-          R.x[e + 1u] = pack2(h1, l1);
-          R.x[e + 2u] = pack2(h2, l2);
-          R.x[e + 3u] = pack2(h3, l3);
-          R.x[e + 4u] = pack2(h4, l4);
+        if (((w0 | w1 | w2 | w3) & 0x80000000ull) == 0ull && mcs::plain_collision32(p, hi_of(w0), h1, l1) &&
+            mcs::plain_collision32(p, hi_of(w1), h2, l2) && mcs::plain_collision32(p, hi_of(w2), h3, l3) &&
+            mcs::plain_collision32(p, hi_of(w3), h4, l4)) {
+          r[0] = pack2(h1, l1);
+          r[2] = pack2(h2, l2);
+          r[4] = pack2(h3, l3);
+          r[6] = pack2(h4, l4);
           xf = h4;
           xlo = l4;
           e += 4u;
@@ -524,19 +421,21 @@ __device__ __noinline__ void coop_walk(const CoopArgs* c, const mcd::Affine* tab
       }
       if (e == E) break;
       if (e == ok) { out = -1; break; }
-      const unsigned long long pc = R.p[e];
       float xn, xnlo;
-      const int f = mcs::advance32(p, xf, xlo, hi_of(R.d[e]), lo_of(pc), hi_of(pc),
-                                   [&] { return mcd::u53<M>(R.m[e], m); }, xn, xnlo);
+      const int f = mcs::advance32(p, xf, xlo, hi_of(r[1]), lo_of(r[0]), hi_of(r[0]),
+                                   [&] { return mcd::u53<M>(mcs::skip_tab(tab, x0, 3ull * e + 1ull), l.m); }, xn, xnlo);
       if (f != mcs::kCollide) { out = f; ++e; break; }
       xf = xn;
       xlo = xnlo;
-      R.x[e + 1u] = pack2(xf, xlo);
-      if (R.f[e]) { out = mcs::kAbsorbed; ++e; break; }
+      r[0] = pack2(xf, xlo);
       ++e;
+      if (r[1] & 0x80000000ull) { out = mcs::kAbsorbed; break; }
     }
     H.w[CoopHist::kPos] = pack2(xf, xlo);
-    if (out == mcs::kContinue) H.w[CoopHist::kDir] = pack2(hi_of(R.d[E]), lo_of(R.w[E]));
+    if (out == mcs::kContinue) {
+      H.w[CoopHist::kDir] = rec[kCoopWords * E + 1u];
+      H.w[CoopHist::kW] = rec[kCoopWords * E + 1u];
+    }
   }
   const uint64_t total = events + e;
   H.w[CoopHist::kEvents] = total;
@@ -546,7 +445,7 @@ __device__ __noinline__ void coop_walk(const CoopArgs* c, const mcd::Affine* tab
   const uint64_t used = out == mcs::kContinue ? 3ull * E
                       : out == -1 ? 3ull * e
                       : out == mcs::kAbsorbed ? 3ull * e - 1ull : 3ull * e - 2ull;
-  const uint64_t x = mcs::skip_tab(tab, H.w[CoopHist::kX], used);
+  const uint64_t x = mcs::skip_tab(tab, x0, used);
   H.w[CoopHist::kX] = x;
   if (out == mcs::kContinue) return;
   // the history's end
@@ -559,73 +458,116 @@ __device__ __noinline__ void coop_walk(const CoopArgs* c, const mcd::Affine* tab
   H.w[CoopHist::kProb] = pi;  // no longer live
 }
 
-// Phase 3, on lane hl of the group: the tally contributions of the round's
-// events e = hl, hl + G, ... of those the history ran, with warp-aggregated
-// atomics whatever the launch's setting (the bits are the same either way):
-// the lanes of a group tally consecutive events of one history, mostly in
-// the same bins.
-template <bool F32>
-__device__ __noinline__ void coop_tally(const CoopArgs* c, uint32_t hist_off, uint32_t rec_off, uint32_t E, int G,
-                                        int hl) {
-  extern __shared__ unsigned long long s_dyn[];
-  const CoopHist H(s_dyn + hist_off);
-  const CoopRec R(s_dyn + rec_off, E);
-  const SlabDev& p = *H.prob(c->probs);
+// Phase 3 for event e of those the history in H ran (nev, the last one
+// ending as out): its tally, from its positions x_e and x_{e+1}.  With
+// warp-aggregated atomics whatever the launch's setting (the bits are the
+// same either way): neighbouring threads tally neighbouring events of one
+// history, mostly in the same bins.  A direction of exactly zero (weight 0)
+// needs the flight's distance, drawn again.
+template <int M, bool F32>
+__device__ __forceinline__ void coop_tally(const CoopHist& H, const SlabDev& p, const mcd::Lcg& l,
+                                           const mcd::Affine* tab, uint32_t e, uint32_t nev, int out,
+                                           const unsigned long long* rec) {
   const mcs::Sink sk = H.sink(true);
-  const unsigned long long end = H.w[CoopHist::kEnd];
-  const int nev = (int)(uint32_t)end, out = (int)(uint32_t)(end >> 32);
-  for (int e = hl; e < nev; e += G) {
-    const int f = (e == nev - 1 && (out == mcs::kLeakLo || out == mcs::kLeakHi)) ? out : mcs::kCollide;
-    if constexpr (!F32) {
-      const double xe = dval(R.x[e]);
-      const double xn = f == mcs::kCollide ? dval(R.x[e + 1]) : 0.0;
-      int j = mcs::bin_of(p, sk, xe);
-      mcs::tally64(p, xe, xn, dval(R.m[e]), dval(R.d[e]), dval(R.w[e]), f, sk, j);
-    } else {
-      const unsigned long long xa = R.x[e];
-      const unsigned long long xb = f == mcs::kCollide ? R.x[e + 1] : 0ull;
-      const unsigned long long dw = R.d[e];
-      int j = mcs::bin_of_pair(p, lo_of(xa), hi_of(xa));
-      mcs::tally32(p, lo_of(xa), hi_of(xa), lo_of(xb), hi_of(xb), hi_of(dw), lo_of(dw), lo_of(R.w[e]), f, sk, j);
+  const int f = e == nev - 1u && (out == mcs::kLeakLo || out == mcs::kLeakHi) ? out : mcs::kCollide;
+  const unsigned long long from = e == 0u ? H.w[CoopHist::kPos0] : rec[-kCoopWords];
+  auto n_dist = [&] { return mcd::u53<M>(mcs::skip_tab(tab, H.w[CoopHist::kX0], 3ull * e + 1ull), l.m); };
+  if constexpr (!F32) {
+    const double x = dval(from), w = dval(rec[1] & ~kAbsBit);
+    int j = mcs::bin_of(p, sk, x);
+    if (f == mcs::kCollide && mcx::d_zero(w)) {
+      sk.add(j, mcx::fix32_nonneg(__dmul_rn(mclog::neglog1m_n(n_dist()), p.inv_st)));
+      return;
+    }
+    const double xe = f == mcs::kLeakHi ? p.L : (f == mcs::kLeakLo ? 0.0 : dval(rec[0]));
+    mcs::walk64(p, x, xe, !mcs::nn_lt(xe, x), w, sk, j);
+  } else {
+    const unsigned long long to = rec[0];
+    const float xf = lo_of(from), xlo = hi_of(from), muf = hi_of(rec[1]);
+    const float wf = __uint_as_float((uint32_t)rec[1] & 0x7fffffffu);
+    int j = mcs::bin_of_pair(p, xf, xlo);
+    const float d = muf == 0.0f ? mcs::flight_f32(n_dist()) * p.inv_st_f : 0.0f;  // (used for a zero direction alone)
+    mcs::tally32(p, xf, xlo, lo_of(to), hi_of(to), muf, d, wf, f, sk, j);
+  }
+}
+
+// The rounds, by the whole block, over the n history records at hist, with
+// `slots` event records after them.
+template <int M, bool F32>
+__device__ __noinline__ void coop_tail(const CoopArgs* c, const mcd::Affine* tab, unsigned long long* hist,
+                                       unsigned long long* recs, uint32_t slots, uint32_t n) {
+  __shared__ uint16_t s_list[kCoopMaxHist];  // the live histories' records
+  __shared__ uint32_t s_live;
+  const uint32_t t = threadIdx.x, T = blockDim.x;
+  __syncthreads();  // the arguments are in place
+  const mcd::Lcg l = c->t.lcg;
+  uint32_t map_e = ~0u;
+  mcd::Affine map{1ull, 0ull};
+  for (;;) {
+    __syncthreads();
+    if (t < 32u) {
+      uint32_t cnt = 0;
+      for (uint32_t b = 0; b < n; b += 32u) {
+        const bool live = b + t < n && CoopHist(hist + (size_t)(b + t) * kCoopHistWords).live();
+        const unsigned m = __ballot_sync(0xffffffffu, live);
+        if (live) s_list[cnt + __popc(m & ((1u << t) - 1u))] = (uint16_t)(b + t);
+        cnt += __popc(m);
+      }
+      if (t == 0u) s_live = cnt;
+    }
+    __syncthreads();
+    const uint32_t H = s_live;
+    if (H == 0u) break;
+    int k = kCoopMaxLog;
+    while (k > kCoopMinLog && (H << k) > slots) --k;
+    const uint32_t S = 1u << k, E = S - 1u;
+    for (uint32_t s = t; s < H << k; s += T) {
+      const uint32_t e = s & (S - 1u);
+      if (e != map_e) {  // (the same for all of a thread's events when S divides the block)
+        map = affine_steps(tab, 3ull * e);
+        map_e = e;
+      }
+      const CoopHist h(hist + (size_t)s_list[s >> k] * kCoopHistWords);
+      coop_draw<M, F32>(h, *h.prob(c->probs), l, mcd::apply(map, h.w[CoopHist::kX]), e, E, recs + (size_t)kCoopWords * s);
+    }
+    __syncthreads();
+    for (uint32_t i = t; i < H; i += T)
+      coop_walk<M, F32>(c, tab, hist + (size_t)s_list[i] * kCoopHistWords, recs + ((size_t)kCoopWords * i << k), E);
+    __syncthreads();
+    for (uint32_t s = t; s < H << k; s += T) {
+      const CoopHist h(hist + (size_t)s_list[s >> k] * kCoopHistWords);
+      const uint32_t e = s & (S - 1u), nev = (uint32_t)h.w[CoopHist::kEnd];
+      if (e < nev)
+        coop_tally<M, F32>(h, *h.prob(c->probs), l, tab, e, nev, (int)(uint32_t)(h.w[CoopHist::kEnd] >> 32),
+                           recs + (size_t)kCoopWords * s);
     }
   }
 }
 
-// The rounds, warp-uniform, over the n_in history records at area_off.
-template <int M, bool F32>
-__device__ __noinline__ void coop_tail(const CoopArgs* c, const mcd::Affine* tab, uint32_t area_off,
-                                       uint32_t slots, int n_in) {
+constexpr uint32_t kMaxRowBins = 256;  // of a warp's row cache (2 KiB)
+
+// Lane-passes of waiting after which a warp refills (8 to 32 measure within 2 %
+// of each other; refilling at every pass that finds a dead lane: 256 problems
+// fp32 10.9 ms against 10.6, fp64 17.3 against 15.0).
+constexpr uint32_t kIdle = 16;
+
+// Adds a warp's row cache to its tally row in global memory and clears it.
+__device__ __forceinline__ void flush_row(unsigned long long* global_row, uint32_t row, uint32_t n_bins) {
   extern __shared__ unsigned long long s_dyn[];
-  const unsigned lane = threadIdx.x & 31u;
-  const uint32_t rec_base = area_off + (uint32_t)(kCoopMax * kCoopHistWords);
-  for (;;) {
-    __syncwarp();
-    unsigned live = 0u;
-    for (int h = 0; h < n_in; ++h)
-      if (CoopHist(s_dyn + area_off + (uint32_t)h * kCoopHistWords).live()) live |= 1u << h;
-    if (live == 0u) break;
-    const int nl = __popc(live);
-    const int kp = coop_groups(nl);
-    const int G = 32 / kp;
-    const int grp = (int)lane / G, hl = (int)lane % G;
-    unsigned m = live;
-    for (int i = 0; i < grp && m != 0u; ++i) m &= m - 1u;
-    const int h = (grp < nl && m != 0u) ? __ffs(m) - 1 : -1;
-    const uint32_t E = coop_events(slots, kp);
-    const uint32_t hist_off = area_off + (uint32_t)(h < 0 ? 0 : h) * kCoopHistWords;
-    const uint32_t rec_off = rec_base + (uint32_t)grp * (E + 1u) * kCoopWords;
-    __syncwarp();
-    if (h >= 0) coop_draws<M, F32>(c, tab, hist_off, rec_off, E, G, hl);
-    __syncwarp();
-    if (h >= 0 && hl == 0) coop_walk<M, F32>(c, tab, hist_off, rec_off, E);
-    __syncwarp();
-    if (h >= 0) coop_tally<F32>(c, hist_off, rec_off, E, G, hl);
+  __syncwarp();
+  for (uint32_t j = threadIdx.x & 31u; j < n_bins; j += 32u) {
+    const unsigned long long v = s_dyn[row + j];
+    if (v == 0ull) continue;
+    s_dyn[row + j] = 0ull;
+    atomicAdd(global_row + j, v);
   }
+  __syncwarp();
 }
 
 template <int M, bool F32, bool SMEM, bool AGG>
 __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
-  extern __shared__ unsigned long long s_tally[];
+  extern __shared__ unsigned long long s_dyn[];
+  unsigned long long* const s_tally = s_dyn;
   __shared__ mcd::Affine tab[64];
   if (threadIdx.x == 0) {
     mcd::Affine sq{a.lcg.g, a.lcg.c};
@@ -636,17 +578,20 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
   }
   double* s_edges = a.smem_edges ? reinterpret_cast<double*>(s_tally + (SMEM ? a.smem_slots : 0u)) : nullptr;
   double* s_widths = s_edges ? s_edges + a.smem_edges : nullptr;  // n_bins widths after the edges
-  // the particle pool after the tally and the edge tables
-  unsigned long long* s_pool = s_tally + (SMEM ? a.smem_slots : 0u) + 2u * a.smem_edges;
-  __shared__ PoolCtl ctl;
+  // the cooperative tail's records after the tally and the edge tables
+  unsigned long long* s_coop = s_tally + (SMEM ? a.smem_slots : 0u) + 2u * a.smem_edges;
+  __shared__ uint32_t s_live[16];   // per warp: an upper bound on its live histories
+  __shared__ uint32_t s_go, s_n;    // the tail has begun; histories in its records
   __shared__ unsigned long long s_exceed[2];  // one problem: exceeding histories, and their draws beyond Q
   if (threadIdx.x == 0) {
     s_exceed[0] = s_exceed[1] = 0ull;
-    ctl.lock = 0;
-    ctl.n = 0;
-    ctl.active = (int)(blockDim.x >> 5);
-    ctl.pad = 0;
+    s_go = s_n = 0u;
   }
+  // the warps' row caches after those
+  const uint32_t row0 = (SMEM ? a.smem_slots : 0u) + 2u * a.smem_edges + a.coop_hist * kCoopHistWords + a.coop_slots * kCoopWords;
+  if constexpr (!SMEM)
+    for (uint32_t i = threadIdx.x; i < (blockDim.x >> 5) * a.row_bins; i += blockDim.x) s_dyn[row0 + i] = 0ull;
+  if (threadIdx.x < 16u) s_live[threadIdx.x] = threadIdx.x < (blockDim.x >> 5) ? kCoopMaxHist : 0u;
   if (s_edges) {
     const SlabDev& p0 = a.probs[0];
     for (uint32_t j = threadIdx.x; j + 1 < a.smem_edges; j += blockDim.x)
@@ -664,6 +609,7 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
   const mcd::Lcg l = a.lcg;
 
   uint64_t pool_next = 0, pool_end = 0;
+  uint32_t grab = a.chunk, idle = 0;
   bool more = true;
   bool alive = false;
   HistCounts lc;
@@ -675,18 +621,30 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
   mcs::SlabParticle q{};
   mcs::Sink sink{nullptr, s_edges, s_widths, AGG};
   uint64_t gi = 0, events = 0;
-  int coop_n = 0;  // histories handed to the cooperative tail (warp-uniform)
+  uint32_t after = 0;  // passes since the ticket ran out
+  const uint32_t my_row = row0 + (threadIdx.x >> 5) * a.row_bins;
+  unsigned long long* row_of = nullptr;  // the tally row the warp's cache accumulates
+  uint32_t row_n = 0;                    // its bins
 
   for (;;) {
     unsigned dead = __ballot_sync(kFull, !alive);
-    while (dead != 0u && more) {
+    const unsigned waiting = dead;
+    // A refill (seed, source draws, the problem's lookup) costs the warp the
+    // same for one lane as for many, about what kIdle lanes lose by waiting
+    // a pass.
+    idle += (uint32_t)__popc(dead);
+    const bool refill = idle >= kIdle || dead == kFull;
+    if (refill) idle = 0u;
+    while (refill && dead != 0u && more) {
       if (pool_next >= pool_end) {
         unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(a.ticket, (unsigned long long)a.chunk);
+        if (lane == 0) base = atomicAdd(a.ticket, (unsigned long long)grab);
         base = __shfl_sync(kFull, base, 0);
         if (base >= a.total) { more = false; break; }
         pool_next = base;
-        pool_end = min((uint64_t)base + (uint64_t)a.chunk, (uint64_t)a.total);
+        pool_end = min((uint64_t)base + (uint64_t)grab, (uint64_t)a.total);
+        // smaller chunks towards the end, so that the warps run out together
+        grab = (uint32_t)min((uint64_t)a.chunk, max((uint64_t)a.min_grab, (a.total - pool_next) >> a.grab_shift));
       }
       const uint64_t avail = pool_end - pool_next;
       const unsigned rank = __popc(dead & lt_mask);
@@ -713,113 +671,62 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
       pool_next += min((uint64_t)__popc(dead), avail);
       dead = __ballot_sync(kFull, !alive);
     }
-    if (!more && a.pool_cap != 0u) {
-      // ticket exhausted: take particles from the block's pool into dead
-      // lanes, hand this warp's few over, or leave
-      // the pool's count and active warps as lane 0 reads them: every branch
-      // below must be taken by the whole warp (full-mask shuffles inside)
-      volatile PoolCtl& vc = ctl;
-      const int hint_n = __shfl_sync(kFull, lane == 0 ? vc.n : 0, 0);
-      const int hint_active = __shfl_sync(kFull, lane == 0 ? vc.active : 0, 0);
-      if (dead != 0u && hint_n > 0) {
-        int k = 0, n = 0, ok = 0;
-        if (lane == 0) {
-          ok = pool_lock(&ctl.lock, a.lock_attempts);
-          if (ok) {
-            n = vc.n;
-            k = min(n, __popc(dead));
-            vc.n = n - k;
-          }
-        }
-        k = __shfl_sync(kFull, k, 0);
-        n = __shfl_sync(kFull, n, 0);
-        if (k < 0 || n > (int)a.pool_cap || k > n) k = 0;  // never outside the pool
-        __syncwarp();
-        const unsigned rank = __popc(dead & lt_mask);
-        if (!alive && (int)rank < k) {
-          const uint32_t pi = pool_get(s_pool + (size_t)(n - k + (int)rank) * kPoolWords, x, q, gi, events);
-          if ((int)pi != lc.prob) { lc.flush(a.counts, a.probs); lc.prob = (int)pi; }
-          P = a.probs + pi;
-          const uint64_t id = gi - P->hist_begin;
-          sink.base = (SMEM ? s_tally : a.tally) + P->tally_offset + mcs::batch_of(id, P->n_hist, P->n_batches) * P->n_bins;
-          if (a.tables) {
-            sink.edges = a.tables + P->tab_off;
-            sink.widths = sink.edges + P->n_bins + 1;
-          }
-          alive = true;
-        }
-        __syncwarp();
-        if (lane == 0 && ok) pool_unlock(&ctl.lock);
-        dead = __ballot_sync(kFull, !alive);
-      }
-      const unsigned live = ~dead;
-      const int nlive = __popc(live);
-      if (nlive != 0 && nlive <= kCoopMax && hint_active == 1 && hint_n == 0 &&
-          coop_events(a.coop_slots, coop_groups(nlive)) >= kCoopMinEvents) {
-        // the block's last warp with a few long histories: confirm under the
-        // lock that no warp is left to fill the pool, then finish them
-        // together
-        int ok = 0;
-        if (lane == 0 && pool_lock(&ctl.lock, a.lock_attempts)) {
-          ok = (vc.n == 0 && vc.active == 1) ? 1 : 0;
-          pool_unlock(&ctl.lock);
-        }
-        if (__shfl_sync(kFull, ok, 0)) {
-          lc.flush_warp(a.counts, a.probs);
-          if (alive) {
-            CoopHist H(s_pool + (size_t)__popc(live & lt_mask) * kCoopHistWords);
-            H.w[CoopHist::kX] = x;
-            H.w[CoopHist::kPos] = F32 ? pack2(q.xf, q.xlo) : dbits(q.x);
-            H.w[CoopHist::kDir] = F32 ? pack2(q.muf, q.wf) : dbits(q.mu);
-            H.w[CoopHist::kW] = dbits(q.w_mu);
-            H.w[CoopHist::kGi] = gi;
-            H.w[CoopHist::kEvents] = events;
-            H.w[CoopHist::kProb] = (uint64_t)(uint32_t)(P - a.probs) | (1ull << 32);
-            H.w[CoopHist::kBase] = reinterpret_cast<unsigned long long>(sink.base);
-            H.w[CoopHist::kEdges] = reinterpret_cast<unsigned long long>(sink.edges);
-            H.w[CoopHist::kWidths] = reinterpret_cast<unsigned long long>(sink.widths);
-          }
-          coop_n = nlive;
-          alive = false;
-          break;
+    if (!SMEM && a.row_bins != 0u && dead != waiting) {
+      // new histories: the row most lanes are on is the one the warp caches
+      if (waiting & (1u << lane)) sink.row = mcs::kNoRow;
+      unsigned out = __ballot_sync(kFull, alive && sink.base != row_of) & waiting;
+      if (out != 0u) {
+        const int who = 31 - __clz((int)out);
+        unsigned long long* const cand = reinterpret_cast<unsigned long long*>(
+            __shfl_sync(kFull, reinterpret_cast<unsigned long long>(sink.base), who));
+        const uint32_t n = __shfl_sync(kFull, alive ? P->n_bins : 0u, who);
+        if (__popc(__ballot_sync(kFull, alive && sink.base == cand)) >
+            __popc(__ballot_sync(kFull, alive && sink.base == row_of))) {
+          if (row_of) flush_row(row_of, my_row, row_n);
+          row_of = cand;
+          row_n = n;
         }
       }
-      if (nlive == 0 || (nlive <= (int)a.donate_max && hint_active > 1 && hint_n + nlive <= (int)a.pool_cap)) {
-        int go = 0, n = 0;
-        if (lane == 0) {
-          if (pool_lock(&ctl.lock, a.lock_attempts)) {
-            n = vc.n;
-            if (nlive == 0 ? n == 0 : (vc.active > 1 && n + nlive <= (int)a.pool_cap)) {
-              vc.n = n + nlive;
-              vc.active = vc.active - 1;
-              go = 1;
-            }
-            if (!go || nlive == 0) pool_unlock(&ctl.lock);
-          } else if (nlive == 0) {
-            // cannot see the pool: leave, counting what may be stranded
-            atomicAdd(a.counts + MC_C_DROPPED, (unsigned long long)max(vc.n, 0));
-            go = 1;
-          }
-        }
-        go = __shfl_sync(kFull, go, 0);
-        n = __shfl_sync(kFull, n, 0);
-        if (go) {
-          if (nlive != 0) {
-            const uint32_t slot = (uint32_t)n + (uint32_t)__popc(live & lt_mask);
-            if (alive && slot < a.pool_cap)  // always, by the count taken under the lock
-              pool_put(s_pool + (size_t)slot * kPoolWords, x, q, gi, events, (uint32_t)(P - a.probs));
-            else if (alive)
-              atomicAdd(a.counts + MC_C_DROPPED, 1ull);
-            __syncwarp();
-            if (lane == 0) pool_unlock(&ctl.lock);
-            alive = false;
-          }
-          break;
-        }
-        if (nlive == 0) continue;  // the pool holds particles: take them on the next pass
-      }
-    } else if (__ballot_sync(kFull, alive) == 0u) {
+      sink.row = alive && sink.base == row_of ? my_row : mcs::kNoRow;
+    }
+    if (dead == kFull) {
+      if (lane == 0) s_live[threadIdx.x >> 5] = 0u;
       break;
+    }
+    if (!more && a.coop_hist != 0u && ++after >= kCoopAfter) {
+      // The block's live histories, from each warp's own count (a warp that
+      // still refills, or has not run kCoopAfter passes since, counts as
+      // full).  Counts only fall, so a sum read while they change is an upper
+      // bound, and whoever finds it small enough starts the tail for all.
+      volatile uint32_t* const vl = s_live;
+      if (lane == 0) vl[threadIdx.x >> 5] = (uint32_t)__popc(~dead);
+      const uint32_t mine = lane < 16u ? vl[lane] : 0u;
+      const bool go = __reduce_add_sync(kFull, mine) <= a.coop_hist || *(volatile uint32_t*)&s_go != 0u;
+      if (__any_sync(kFull, go)) {
+        uint32_t base = 0;
+        if (lane == 0) {
+          *(volatile uint32_t*)&s_go = 1u;
+          base = atomicAdd(&s_n, (uint32_t)__popc(~dead));
+        }
+        base = __shfl_sync(kFull, base, 0);
+        const uint32_t at = base + (uint32_t)__popc(~dead & lt_mask);
+        if (alive && at < a.coop_hist) {  // always, by the bound
+          unsigned long long* const w = s_coop + (size_t)at * kCoopHistWords;
+          w[CoopHist::kX] = x;
+          w[CoopHist::kPos] = F32 ? pack2(q.xf, q.xlo) : dbits(q.x);
+          w[CoopHist::kDir] = F32 ? pack2(0.0f, q.muf) : dbits(q.mu);
+          w[CoopHist::kW] = F32 ? pack2(q.wf, 0.0f) : dbits(q.w_mu);
+          w[CoopHist::kGi] = gi;
+          w[CoopHist::kEvents] = events;
+          w[CoopHist::kProb] = (uint64_t)(uint32_t)(P - a.probs) | (1ull << 32);
+          w[CoopHist::kBase] = reinterpret_cast<unsigned long long>(sink.base);
+          w[CoopHist::kEdges] = reinterpret_cast<unsigned long long>(sink.edges);
+          w[CoopHist::kWidths] = reinterpret_cast<unsigned long long>(sink.widths);
+        } else if (alive) {
+          atomicAdd(a.counts + MC_C_DROPPED, 1ull);
+        }
+        break;
+      }
     }
     if (alive) {
       int outcome = -1;  // event cap
@@ -834,17 +741,18 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
       }
     }
   }
-  if (coop_n != 0) {
-    // the arguments through shared memory too: a call with them by value
-    // would put them on the stack of the whole kernel
-    __shared__ CoopArgs s_coop;
-    if (lane == 0) s_coop = CoopArgs{TailArgs{a.hist_state, a.hist_draws, a.counts, a.lcg, a.event_cap}, a.probs};
-    __syncwarp();
-    coop_tail<M, F32>(&s_coop, tab, (uint32_t)(s_pool - s_tally), a.coop_slots, coop_n);
-  }
   lc.flush_warp(a.counts, a.probs);
+  if (!SMEM && row_of) flush_row(row_of, my_row, row_n);
 
   __syncthreads();
+  if (s_n != 0u) {
+    // the arguments through shared memory: a call with them by value would
+    // put them on the stack of the whole kernel
+    __shared__ CoopArgs s_args;
+    if (threadIdx.x == 0) s_args = CoopArgs{TailArgs{a.hist_state, a.hist_draws, a.counts, a.lcg, a.event_cap}, a.probs};
+    coop_tail<M, F32>(&s_args, tab, s_coop, s_coop + (size_t)a.coop_hist * kCoopHistWords, a.coop_slots,
+                      min(s_n, a.coop_hist));
+  }
   if (threadIdx.x == 0 && s_exceed[0] != 0ull) {
     atomicAdd(a.counts + MC_C_EXCEED_HIST, s_exceed[0]);
     atomicAdd(a.counts + MC_C_EXCEED_DRAWS, s_exceed[1]);
@@ -882,8 +790,8 @@ int launch_history(const RunArgs& a0, int block, int blocks_per_sm, int num_sms,
   auto k = history_kernel_of<M, F32, SMEM, AGG>();
   RunArgs a = a0;
   // Static shared memory of this instantiation (read once) and the device's
-  // opt-in limit: what does not fit beside them is given up, the compaction
-  // pool first and then the edge tables (both only save time).
+  // opt-in limit: what does not fit beside them is given up, the cooperative
+  // tail first and then the edge tables (both only save time).
   static size_t static_smem = ~(size_t)0;
   if (static_smem == ~(size_t)0) {
     cudaFuncAttributes fa{};
@@ -894,18 +802,15 @@ int launch_history(const RunArgs& a0, int block, int blocks_per_sm, int num_sms,
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  // the pool's memory, which the cooperative tail reuses: at least
-  // kCoopAreaWords when there is a pool
-  auto pool_words = [&a]() {
-    return a.pool_cap ? std::max<size_t>((size_t)a.pool_cap * kPoolWords, kCoopAreaWords) : (size_t)0;
-  };
-  auto dynamic_smem = [&a, &pool_words]() {
+  auto dynamic_smem = [&a, block]() {
     return (SMEM ? (size_t)a.smem_slots * 8u : 0u) + (size_t)a.smem_edges * 16u +  // edges + widths
-           pool_words() * 8u;
+           ((size_t)a.coop_hist * kCoopHistWords + (size_t)a.coop_slots * kCoopWords) * 8u +
+           (size_t)(block / 32) * a.row_bins * 8u;
   };
-  if (static_smem + dynamic_smem() > (size_t)optin) a.pool_cap = 0;
+  if (SMEM || a.row_bins > kMaxRowBins) a.row_bins = 0;
+  if (static_smem + dynamic_smem() > (size_t)optin) a.row_bins = 0;
+  if (static_smem + dynamic_smem() > (size_t)optin) a.coop_hist = a.coop_slots = 0;
   if (static_smem + dynamic_smem() > (size_t)optin) a.smem_edges = 0;
-  a.coop_slots = coop_slots_of((uint32_t)pool_words());
   const size_t smem = dynamic_smem();
   if (static_smem + smem > (size_t)optin) {
     mci::set_error("slab_history_kernel: %u tally slots do not fit in shared memory", a.smem_slots);
@@ -928,6 +833,8 @@ int launch_history(const RunArgs& a0, int block, int blocks_per_sm, int num_sms,
   const uint64_t blocks_needed = (warps_needed * 32 + block - 1) / block;
   const uint64_t full = (uint64_t)num_sms * (uint64_t)per_sm;
   const int grid = (int)std::max<uint64_t>(1, std::min(full, blocks_needed));
+  a.grab_shift = 1u;  // twice the launch's warps, rounded up to a power of two
+  while ((1ull << a.grab_shift) < 2ull * (uint64_t)grid * (uint64_t)(block / 32)) ++a.grab_shift;
   k<<<grid, block, smem, s>>>(a);
   return mci::cuda_status(cudaGetLastError(), "slab_history_kernel launch");
 }
@@ -1012,11 +919,27 @@ int slab_history_launch(const SlabLaunch& L, cudaStream_t s) {
   }
   // otherwise each problem's tables in global memory, where staged
   a.tables = a.smem_edges ? nullptr : static_cast<const double*>(L.d_tables);
-  // compaction: a warp with at most 12 live lanes hands them over; the pool
-  // holds what every other warp of the block could hand over
-  a.donate_max = 12;
-  a.pool_cap = L.block >= 64 ? (uint32_t)((L.block >> 5) - 1) * a.donate_max : 0u;
-  a.lock_attempts = L.pool_lock_attempts;
+  // One problem: chunks down to 8 histories at the end, so that the warps run
+  // out together (300 000 histories of 9 flights: 321 -> 312 us).  Several: a
+  // chunk that spans few problems is worth more (256 problems fp32: 11.0 ms
+  // with whole chunks, 11.6 with chunks down to 8 or 32).
+  a.min_grab = L.n_problems == 1 ? 8u : a.chunk;
+  // The cooperative tail takes over when a quarter of a block's threads still
+  // carry a history, with four event records per thread in fp64 and two in
+  // fp32 (a power of two).  slab_long, 10^6 histories: fp64 154 ms, against 164
+  // with half the threads and 157 with two records; fp32 107 ms, against 114
+  // with four records; without the tail 244 and 160 ms.
+  if (L.pool_lock_attempts != 0u && L.block >= 64) {
+    a.coop_slots = 128u;
+    while (a.coop_slots * 2u <= (uint32_t)L.block * (L.f32 ? 2u : 4u)) a.coop_slots *= 2u;
+    // (a round's records, at least 2^kCoopMinLog per history, must fit)
+    a.coop_hist = std::min((uint32_t)L.block / 4u, a.coop_slots >> kCoopMinLog);
+  }
+  // Without the whole tally in shared memory each warp accumulates the row
+  // most of its lanes are on in a cache of its own: all warps work through the
+  // problems in one order, and their atomics met at a few lines of L2 (256
+  // problems: fp32 16.6 -> 11.0 ms, fp64 21.2 -> 17.0 ms).
+  a.row_bins = L.max_n_bins;
   a.order = mcs::Order{L.d_order, L.d_order_begin};
   if (L.tally_agg) {
     if (L.lcg.m == 63) return launch_history_m<63, true>(a, L.f32, L.block, L.blocks_per_sm, L.num_sms, s);

@@ -138,17 +138,27 @@ __device__ __forceinline__ int bin_guess(const SlabDev& p, double x) {
 
 __device__ __forceinline__ int clamp_bin(int j, int nb) { return j < 0 ? 0 : (j >= nb ? nb - 1 : j); }
 
-// Tally sink: shared-memory staging or direct global atomics, and an
-// optional table of the bin edges e_0..e_nb (shared memory; nullptr: each
-// edge is computed as j * h).
+// Tally sink: this history's [bin] row in shared memory (the whole tally
+// staged) or global memory, the offset of its warp's row cache in dynamic
+// shared memory (kNoRow: none) where the warp accumulates that row, and an
+// optional table of the bin edges e_0..e_nb (nullptr: each edge is computed
+// as j * h).
+constexpr uint32_t kNoRow = ~0u;
 struct Sink {
-  unsigned long long* base;  // this history's [bin] row (smem or global)
+  unsigned long long* base;
   const double* edges;
   const double* widths;  // with edges: widths[j] = e_{j+1} - e_j (the same fp64 difference)
   bool agg;              // warp-aggregated atomics (mcd::warp_agg_add) instead of one per lane
+  uint32_t row = kNoRow;
   __device__ __forceinline__ void add(int j, long long v) const {
-    if (agg) mcd::warp_agg_add(base + j, (unsigned long long)v);
-    else atomicAdd(base + j, (unsigned long long)v);
+    if (row != kNoRow) {
+      extern __shared__ unsigned long long s_dyn[];
+      atomicAdd(s_dyn + row + j, (unsigned long long)v);
+    } else if (agg) {
+      mcd::warp_agg_add(base + j, (unsigned long long)v);
+    } else {
+      atomicAdd(base + j, (unsigned long long)v);
+    }
   }
 };
 

@@ -21,6 +21,7 @@ struct SlabLaunch {
   uint64_t event_cap;
   uint32_t smem_slots;         // 0 = global atomics; else slots staged in smem
   uint32_t single_n_bins;      // n_bins of the problem when n_problems == 1
+  uint32_t max_n_bins = 0;     // the most bins of any problem
   const void* d_tables = nullptr;  // per-problem edge and width tables (nullable; see slab_prep)
   bool f32;
   int block, blocks_per_sm, num_sms;

@@ -78,3 +78,22 @@ def test_exceedances_of_several_problems(env):
     assert np.array_equal(together[0], np.concatenate([r[0] for r in one]))
     assert np.array_equal(together[1], np.concatenate([r[1] for r in one]))
     assert np.all(together[1][:, 8] > 0)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("block", [64, 96, 160, 256, 512])
+def test_cooperative_tail_of_any_block(env, block, precision):
+    """Long chains of several problems through the tail (blocks of 64 threads
+    and more), with and without row caches, against single-warp blocks, which
+    have none."""
+    probs, off = [], 0
+    for i, (bins, batches) in enumerate([(7, 3), (200, 20), (300, 20)]):
+        probs.append(W.slab_problem(60.0, 1.0, 0.999, 150, bins, batches, W.SEED_HASH_HIER, key=i, tally_offset=off))
+        off += bins * batches
+    for some in (probs, probs[:2]):  # with 300 bins no row is cached
+        ref = run(env, some, precision=precision, block=32)
+        for cfg in (dict(), dict(tally_mode=2), dict(blocks_per_sm=1, chunk=8), dict(event_cap=40)):
+            want = ref if "event_cap" not in cfg else run(env, some, precision=precision, block=32, **cfg)
+            got = run(env, some, precision=precision, block=block, **cfg)
+            for x, y in zip(want, got):
+                assert np.array_equal(x, y), cfg
