@@ -77,6 +77,7 @@ struct BoxArgs {
   uint64_t* hist_draws;
   mcd::Lcg lcg;
   uint64_t event_cap;
+  mcd::Pow2Maps pow2;
 };
 
 __device__ __forceinline__ uint32_t find_box(const BoxDev* p, uint32_t n, uint64_t gi) {
@@ -126,10 +127,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) box_history_kerne
   // fp64, one problem: its mesh planes, read on every voxel crossing
   __shared__ double s_planes[sizeof(T) == 8 ? mcb::kMaxPlanes : 1];
   __shared__ unsigned long long s_counts[kCountProbs * MC_NCOUNT];
-  if (threadIdx.x == 0) {
-    mcd::Affine sq{a.lcg.g, a.lcg.c};
-    for (int j = 0; j < 64; ++j) { tab[j] = sq; sq = mcd::compose(sq, sq); }
-  }
+  mcd::load_maps(a.pow2, tab);
   const bool block_counts = a.nprob <= kCountProbs;
   if (block_counts)
     for (uint32_t i = threadIdx.x; i < a.nprob * MC_NCOUNT; i += blockDim.x) s_counts[i] = 0ull;
@@ -334,6 +332,7 @@ int run_box_history(const mci::BoxLaunch& L, cudaStream_t s) {
   a.hist_draws = L.tally->d_hist_draws;
   a.lcg = mcd::Lcg{L.lcg.g, L.lcg.c, mcd::mask_of(L.lcg.m), L.lcg.m};
   a.event_cap = L.event_cap;
+  a.pow2 = mcd::pow2_maps(L.lcg.g, L.lcg.c);
   a.ticket = L.d_ticket;
   a.child_cap = L.child_cap;
   ChildRec* bank[2] = {static_cast<ChildRec*>(L.d_child[0]), static_cast<ChildRec*>(L.d_child[1])};

@@ -56,6 +56,26 @@ __host__ __device__ __forceinline__ Affine skip_map(uint64_t g, uint64_t c, uint
   return acc;
 }
 
+// The maps of 2^j steps, j = 0..63 (Brown's squares), computed on the host and
+// handed to a kernel with its arguments: a thread that squares its way through
+// them takes 1.3 us, which every block of the launch would wait for.
+struct Pow2Maps {
+  Affine m[64];
+};
+inline __host__ Pow2Maps pow2_maps(uint64_t g, uint64_t c) {
+  Pow2Maps p;
+  Affine sq{g, c};
+  for (int j = 0; j < 64; ++j) {
+    p.m[j] = sq;
+    sq = compose(sq, sq);
+  }
+  return p;
+}
+// The block's copy in shared memory (complete at the next barrier).
+__device__ __forceinline__ void load_maps(const Pow2Maps& p, Affine* tab) {
+  for (uint32_t j = threadIdx.x; j < 64u; j += blockDim.x) tab[j] = p.m[j];
+}
+
 // Section 4, Listing 1 and Eq. 3: one mixing step multiplies by the murmur
 // constant (mod 2^64) and folds the product's top 17 bits into its low bits;
 // the hash mixes the key, multiplies it by the constant again, combines it by

@@ -48,6 +48,7 @@ struct PulseArgs {
   Overflow* ovf_out;               // non-null (hash modes): where secondaries beyond the stack go
   unsigned long long* ovf_out_count;
   uint64_t ovf_cap;
+  mcd::Pow2Maps pow2;              // stride
 };
 
 __global__ void pulse_prep_kernel(PulseDev* p) {
@@ -117,13 +118,8 @@ __global__ void __launch_bounds__(256, HASH ? 4 : 1) pulse_kernel(const PulseArg
   __shared__ mcd::Affine tab[64];
   __shared__ PulseDev sP;
   __shared__ unsigned long long s_counts[MC_NCOUNT];
-  if (threadIdx.x == 0) {
-    if constexpr (!HASH) {
-      mcd::Affine sq{a.lcg.g, a.lcg.c};
-      for (int j = 0; j < 64; ++j) { tab[j] = sq; sq = mcd::compose(sq, sq); }
-    }
-    sP = *a.prob;
-  }
+  if constexpr (!HASH) mcd::load_maps(a.pow2, tab);
+  if (threadIdx.x == 0) sP = *a.prob;
   for (uint32_t i = threadIdx.x; i < MC_NCOUNT; i += blockDim.x) s_counts[i] = 0ull;
   __syncthreads();
   const PulseDev& P = sP;
@@ -458,6 +454,7 @@ int pulse_run(const PulseLaunch& L, cudaStream_t s) {
   a.hist_draws = L.tally->d_hist_draws;
   a.lcg = mcd::Lcg{L.lcg.g, L.lcg.c, mcd::mask_of(L.lcg.m), L.lcg.m};
   a.event_cap = L.event_cap;
+  a.pow2 = mcd::pow2_maps(L.lcg.g, L.lcg.c);
   a.stack_depth = L.stack_depth;
   a.stack = static_cast<mcp::StackRec*>(L.d_stack);
   const bool hash = L.seeding != MC_SEED_STRIDE;

@@ -4,8 +4,8 @@
 // Seeding (Section 3, Eq. 2 and Section 4, Listing 1 / Eq. 3) is bound by
 // the HBM store of 8 bytes per stream: each thread produces two adjacent
 // states and writes them with one 16-byte store.  Stride seeds use Brown's
-// binary skip-ahead only once per thread, from a per-block table of the
-// maps of 2^j steps; after that a thread advances to its next pair with
+// binary skip-ahead only once per thread, from a table of maps that comes
+// with the arguments; after that a thread advances to its next pair with
 // one precomputed affine map (Q * pairs-per-sweep * 2 steps).
 //
 // Draws (Eq. 1) are bound by integer issue: the 64-bit state stays in
@@ -16,6 +16,7 @@
 
 #include <atomic>
 #include <cstdint>
+#include <type_traits>
 
 #include "internal.h"
 #include "mc_device.cuh"
@@ -27,37 +28,42 @@ using mcd::Affine;
 constexpr int kSeedBlock = 256;
 constexpr int kDrawBlock = 256;
 
-// Per-block table of the maps of 2^j LCG steps, j = 0..63 (Brown's squares).
-__device__ void build_pow2_table(Affine* tab, uint64_t g, uint64_t c) {
-  if (threadIdx.x == 0) {
-    Affine sq{g, c};
-    for (int j = 0; j < 64; ++j) {
-      tab[j] = sq;
-      sq = mcd::compose(sq, sq);
-    }
+// Stride seeding shares between threads what does not depend on the thread:
+// the state X_{Q id_begin} of the first unit and the maps of u, 2u, 4u, ...
+// steps for threads u = Q (or 2Q, in pairs) apart, all computed on the host.
+// Thread t then composes one map per set bit of t.  (The maps of 2^j steps
+// alone, squared by one thread of each block, cost every block 1.3 us, and the
+// bits of Q t are more than the bits of t: 2^26 seeds took 90.0 us, now 85.8.)
+constexpr int kThreadBits = 32;  // a grid has fewer than 2^32 threads
+struct ThreadMaps {
+  Affine m[kThreadBits];
+  uint64_t first;
+};
+
+ThreadMaps thread_maps(uint64_t g, uint64_t c, uint64_t x0, uint64_t q, uint64_t id_begin, uint64_t unit) {
+  ThreadMaps t;
+  Affine sq = mcd::skip_map(g, c, unit);
+  for (int j = 0; j < kThreadBits; ++j) {
+    t.m[j] = sq;
+    sq = mcd::compose(sq, sq);
   }
+  t.first = mcd::apply(mcd::skip_map(g, c, q * id_begin), x0);
+  return t;
+}
+
+__device__ __forceinline__ void load_maps(const ThreadMaps& t, Affine* tab) {
+  for (uint32_t j = threadIdx.x; j < (uint32_t)kThreadBits; j += blockDim.x) tab[j] = t.m[j];
   __syncthreads();
 }
 
-// The state k steps after x, walking the set bits of k through the table.
-__device__ __forceinline__ uint64_t skip_by_table(const Affine* tab, uint64_t x, uint64_t k) {
-  while (k) {
-    const int j = __ffsll((long long)k) - 1;
-    x = mcd::apply(tab[j], x);
-    k &= k - 1;
+// The state of thread `tid`: units tid after the first.
+__device__ __forceinline__ uint64_t thread_state(const ThreadMaps& t, const Affine* tab, uint32_t tid) {
+  uint64_t x = t.first;
+  while (tid) {
+    x = mcd::apply(tab[__ffs((int)tid) - 1], x);
+    tid &= tid - 1u;
   }
   return x;
-}
-
-// The map of k steps, composed from the table.
-__device__ __forceinline__ Affine map_by_table(const Affine* tab, uint64_t k) {
-  Affine acc{1ull, 0ull};
-  while (k) {
-    const int j = __ffsll((long long)k) - 1;
-    acc = mcd::compose(tab[j], acc);
-    k &= k - 1;
-  }
-  return acc;
 }
 
 // ------------------------------------------------------------ hash seeding
@@ -84,39 +90,39 @@ __global__ void __launch_bounds__(kSeedBlock) seed_hash_kernel(uint64_t parent_s
 }
 
 // ---------------------------------------------------------- stride seeding
+struct StrideArgs {
+  ThreadMaps t;
+  Affine step_q, sweep;  // Q steps, and a whole sweep of the grid
+  uint64_t last;         // the last unit's state
+  uint64_t count, mask;
+};
+
 template <bool VEC>
-__global__ void __launch_bounds__(kSeedBlock) seed_stride_kernel(uint64_t g, uint64_t c, uint64_t x0,
-                                                                 uint64_t q, uint64_t id_begin,
-                                                                 uint64_t count, uint64_t mask,
-                                                                 uint64_t* __restrict__ out) {
-  __shared__ Affine tab[64];
-  build_pow2_table(tab, g, c);
+__global__ void __launch_bounds__(kSeedBlock) seed_stride_kernel(const StrideArgs a, uint64_t* __restrict__ out) {
+  __shared__ Affine tab[kThreadBits];
+  load_maps(a.t, tab);
   const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const uint64_t nthreads = (uint64_t)gridDim.x * blockDim.x;
   if constexpr (VEC) {
-    const uint64_t npairs = count >> 1;
+    const uint64_t npairs = a.count >> 1;
     if (tid < npairs) {
       // Unit k = id_begin + 2p gets X_{Qk}; its neighbour is one map of Q steps on.
-      const Affine step_q = map_by_table(tab, q);
-      const Affine sweep = map_by_table(tab, q * 2ull * nthreads);
-      uint64_t x = skip_by_table(tab, x0, q * (id_begin + 2ull * tid));
+      uint64_t x = thread_state(a.t, tab, (uint32_t)tid);
       for (uint64_t p = tid; p < npairs; p += nthreads) {
         ulonglong2 v;
-        v.x = x & mask;
-        v.y = mcd::apply(step_q, x) & mask;
+        v.x = x & a.mask;
+        v.y = mcd::apply(a.step_q, x) & a.mask;
         reinterpret_cast<ulonglong2*>(out)[p] = v;
-        x = mcd::apply(sweep, x);
+        x = mcd::apply(a.sweep, x);
       }
     }
-    if ((count & 1) && tid == 0)
-      out[count - 1] = skip_by_table(tab, x0, q * (id_begin + count - 1)) & mask;
+    if ((a.count & 1) && tid == 0) out[a.count - 1] = a.last & a.mask;
   } else {
-    if (tid < count) {
-      const Affine sweep = map_by_table(tab, q * nthreads);
-      uint64_t x = skip_by_table(tab, x0, q * (id_begin + tid));
-      for (uint64_t i = tid; i < count; i += nthreads) {
-        out[i] = x & mask;
-        x = mcd::apply(sweep, x);
+    if (tid < a.count) {
+      uint64_t x = thread_state(a.t, tab, (uint32_t)tid);
+      for (uint64_t i = tid; i < a.count; i += nthreads) {
+        out[i] = x & a.mask;
+        x = mcd::apply(a.sweep, x);
       }
     }
   }
@@ -136,26 +142,27 @@ struct DrawArgs {
   uint64_t* states;    // kLoad: in/out; else nullable out
   double* u;           // nullable, [draws][n]
   uint64_t* digest;    // nullable, [n]
-  // kStride digest kernel: the maps of Q T and 2 Q T steps (T = threads in
-  // the grid), the same for every thread; set by the launcher so that they
-  // stay in the parameter bank instead of registers
+};
+// kStride: the threads' maps, and (the same for every thread, in the
+// parameter bank instead of registers) the maps of Q T steps and, digest
+// kernel, of 2 Q T steps, T = threads in the grid; set by the launcher.
+struct DrawArgsStride : DrawArgs {
+  ThreadMaps t;
   Affine half, sweep;
 };
+template <int SEED>
+using DrawArgsOf = std::conditional_t<SEED == kStride, DrawArgsStride, DrawArgs>;
 
 template <int M, int SEED, bool WANT_U, bool WANT_DIGEST>
-__global__ void __launch_bounds__(kDrawBlock) draw_kernel(const DrawArgs a) {
-  __shared__ Affine tab[64];
-  if constexpr (SEED == kStride) build_pow2_table(tab, a.g, a.c);
+__global__ void __launch_bounds__(kDrawBlock) draw_kernel(const DrawArgsOf<SEED> a) {
+  __shared__ Affine tab[kThreadBits];
+  if constexpr (SEED == kStride) load_maps(a.t, tab);
   const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const uint64_t nthreads = (uint64_t)gridDim.x * blockDim.x;
   if (tid >= a.n) return;
-  Affine sweep{1ull, 0ull};
   uint64_t xs = 0, seed_hash = 0;
   if constexpr (SEED == kHash) seed_hash = mcd::seed_hash_of(a.hier ? mcd::hash64(a.key, a.seed) : a.seed);
-  if constexpr (SEED == kStride) {
-    sweep = map_by_table(tab, a.q * nthreads);
-    xs = skip_by_table(tab, a.x0, a.q * (a.id_begin + tid));
-  }
+  if constexpr (SEED == kStride) xs = thread_state(a.t, tab, (uint32_t)tid);
   const uint64_t g = a.g, c = a.c;
   for (uint64_t i = tid; i < a.n; i += nthreads) {
     uint64_t x;
@@ -165,7 +172,7 @@ __global__ void __launch_bounds__(kDrawBlock) draw_kernel(const DrawArgs a) {
       x = mcd::hash_with(a.id_begin + i, seed_hash) & a.mask;
     } else {
       x = xs & a.mask;
-      xs = mcd::apply(sweep, xs);
+      xs = mcd::apply(a.half, xs);
     }
     uint64_t dg = 0;
     double* up = WANT_U ? a.u + i : nullptr;
@@ -216,17 +223,17 @@ __global__ void __launch_bounds__(kDrawBlock) draw_kernel(const DrawArgs a) {
 // 1.73 / 1.80 ms per launch (hash / stride) against 1.78 / 1.87 ms with
 // the bare block size.
 template <int SEED, int DRAWS>
-__global__ void __launch_bounds__(kDrawBlock, SEED == kStride ? 4 : 1) draw_digest_m63_kernel(const DrawArgs a) {
+__global__ void __launch_bounds__(kDrawBlock, SEED == kStride ? 4 : 1) draw_digest_m63_kernel(const DrawArgsOf<SEED> a) {
   static_assert(DRAWS % 2 == 0 && DRAWS * 31 < (1 << 24), "count sum must stay exact");
-  __shared__ Affine tab[64];
-  if constexpr (SEED == kStride) build_pow2_table(tab, a.g, a.c);
+  __shared__ Affine tab[kThreadBits];
+  if constexpr (SEED == kStride) load_maps(a.t, tab);
   const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const uint64_t nthreads = (uint64_t)gridDim.x * blockDim.x;
   if (tid >= a.n) return;
   const uint32_t draws = DRAWS > 0 ? (uint32_t)DRAWS : a.draws;
   uint64_t xs = 0, seed_hash = 0;
   if constexpr (SEED == kHash) seed_hash = mcd::seed_hash_of(a.hier ? mcd::hash64(a.key, a.seed) : a.seed);
-  if constexpr (SEED == kStride) xs = skip_by_table(tab, a.x0, a.q * (a.id_begin + tid));
+  if constexpr (SEED == kStride) xs = thread_state(a.t, tab, (uint32_t)tid);
   const uint64_t g = a.g, c2 = 2ull * a.c;
   for (uint64_t i = tid; i < a.n; i += 2 * nthreads) {
     const uint64_t i2 = i + nthreads;
@@ -330,36 +337,48 @@ __global__ void __launch_bounds__(kDrawBlock, SEED == kStride ? 4 : 1) draw_dige
 }
 
 // Persistent grid: every SM filled to its occupancy limit, never more
-// blocks than the work needs.
-template <typename K>
-int persistent_grid(K kernel, int block, size_t smem, uint64_t work_items) {
-  static std::atomic<int> cached[64];  // SM count per device ordinal (0: not read yet)
+// blocks than the work needs.  The limit of each kernel is asked for once per
+// device.
+template <auto Kernel, int Block>
+int persistent_grid(uint64_t work_items) {
+  static std::atomic<int> cached[64];  // blocks that fill the device, per ordinal (0: not known yet)
   int dev = 0;
   cudaGetDevice(&dev);
-  int sms = dev >= 0 && dev < 64 ? cached[dev].load(std::memory_order_relaxed) : 0;
-  if (sms == 0) {
+  int full = dev >= 0 && dev < 64 ? cached[dev].load(std::memory_order_relaxed) : 0;
+  if (full == 0) {
+    int sms = 0, per_sm = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (dev >= 0 && dev < 64) cached[dev].store(sms, std::memory_order_relaxed);
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, Kernel, Block, 0);
+    full = sms * (per_sm < 1 ? 1 : per_sm);
+    if (e == cudaSuccess && dev >= 0 && dev < 64) cached[dev].store(full, std::memory_order_relaxed);
   }
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem);
-  if (per_sm < 1) per_sm = 1;
-  uint64_t want = (work_items + block - 1) / block;
-  uint64_t full = (uint64_t)sms * per_sm;
-  if (want < 1) want = 1;
-  return (int)(want < full ? want : full);
+  const uint64_t want = work_items ? (work_items + Block - 1) / Block : 1;
+  return (int)(want < (uint64_t)full ? want : (uint64_t)full);
+}
+
+// The launch's arguments: with the maps of a grid of `grid` blocks for stride
+// seeds.
+template <int SEED>
+DrawArgsOf<SEED> args_of(const DrawArgs& a, int grid) {
+  if constexpr (SEED == kStride) {
+    DrawArgsStride b{};
+    static_cast<DrawArgs&>(b) = a;
+    const uint64_t nthreads = (uint64_t)grid * kDrawBlock;
+    b.t = thread_maps(a.g, a.c, a.x0, a.q, a.id_begin, a.q);
+    b.half = mcd::skip_map(a.g, a.c, a.q * nthreads);
+    b.sweep = mcd::compose(b.half, b.half);
+    return b;
+  } else {
+    (void)grid;
+    return a;
+  }
 }
 
 template <int SEED, int DRAWS>
-void launch_digest_k(DrawArgs a, cudaStream_t s) {
-  auto k = draw_digest_m63_kernel<SEED, DRAWS>;
-  const int grid = persistent_grid(k, kDrawBlock, 0, (a.n + 1) / 2);
-  if constexpr (SEED == kStride) {
-    const uint64_t nthreads = (uint64_t)grid * kDrawBlock;
-    a.half = mcd::skip_map(a.g, a.c, a.q * nthreads);
-    a.sweep = mcd::skip_map(a.g, a.c, a.q * 2ull * nthreads);
-  }
-  k<<<grid, kDrawBlock, 0, s>>>(a);
+void launch_digest_k(const DrawArgs& a, cudaStream_t s) {
+  constexpr auto k = draw_digest_m63_kernel<SEED, DRAWS>;
+  const int grid = persistent_grid<k, kDrawBlock>((a.n + 1) / 2);
+  k<<<grid, kDrawBlock, 0, s>>>(args_of<SEED>(a, grid));
 }
 
 template <int SEED>
@@ -369,23 +388,18 @@ int launch_digest_m63(const DrawArgs& a, cudaStream_t s) {
   return mci::cuda_status(cudaGetLastError(), "draw_digest_m63_kernel launch");
 }
 
+template <int M, int SEED, bool WANT_U, bool WANT_DIGEST>
+int launch_draw_k(const DrawArgs& a, cudaStream_t s) {
+  constexpr auto k = draw_kernel<M, SEED, WANT_U, WANT_DIGEST>;
+  const int grid = persistent_grid<k, kDrawBlock>(a.n);
+  k<<<grid, kDrawBlock, 0, s>>>(args_of<SEED>(a, grid));
+  return mci::cuda_status(cudaGetLastError(), "draw_kernel launch");
+}
+
 template <int M, int SEED>
 int launch_draw(const DrawArgs& a, cudaStream_t s) {
-  const bool wu = a.u != nullptr, wd = a.digest != nullptr;
-  if (wu && wd) {
-    auto k = draw_kernel<M, SEED, true, true>;
-    k<<<persistent_grid(k, kDrawBlock, 0, a.n), kDrawBlock, 0, s>>>(a);
-  } else if (wu) {
-    auto k = draw_kernel<M, SEED, true, false>;
-    k<<<persistent_grid(k, kDrawBlock, 0, a.n), kDrawBlock, 0, s>>>(a);
-  } else if (wd) {
-    auto k = draw_kernel<M, SEED, false, true>;
-    k<<<persistent_grid(k, kDrawBlock, 0, a.n), kDrawBlock, 0, s>>>(a);
-  } else {
-    auto k = draw_kernel<M, SEED, false, false>;
-    k<<<persistent_grid(k, kDrawBlock, 0, a.n), kDrawBlock, 0, s>>>(a);
-  }
-  return mci::cuda_status(cudaGetLastError(), "draw_kernel launch");
+  if (a.u) return a.digest ? launch_draw_k<M, SEED, true, true>(a, s) : launch_draw_k<M, SEED, true, false>(a, s);
+  return a.digest ? launch_draw_k<M, SEED, false, true>(a, s) : launch_draw_k<M, SEED, false, false>(a, s);
 }
 
 template <int M>
@@ -414,12 +428,11 @@ MC_API int mc_seed_hash(mc_ctx* ctx, const mc_lcg* lcg, uint64_t parent_seed, ui
   cudaStream_t s = (cudaStream_t)stream;
   const uint64_t sh = parent_seed, mask = mcd::mask_of(lcg->m);
   if (((uintptr_t)d_states & 15u) == 0) {
-    auto k = seed_hash_kernel<true>;
-    k<<<persistent_grid(k, kSeedBlock, 0, (count + 1) / 2), kSeedBlock, 0, s>>>(sh, key_begin, count, mask,
-                                                                                  d_states);
+    constexpr auto k = seed_hash_kernel<true>;
+    k<<<persistent_grid<k, kSeedBlock>((count + 1) / 2), kSeedBlock, 0, s>>>(sh, key_begin, count, mask, d_states);
   } else {
-    auto k = seed_hash_kernel<false>;
-    k<<<persistent_grid(k, kSeedBlock, 0, count), kSeedBlock, 0, s>>>(sh, key_begin, count, mask, d_states);
+    constexpr auto k = seed_hash_kernel<false>;
+    k<<<persistent_grid<k, kSeedBlock>(count), kSeedBlock, 0, s>>>(sh, key_begin, count, mask, d_states);
   }
   return mci::cuda_status(cudaGetLastError(), "seed_hash_kernel launch");
 }
@@ -435,15 +448,23 @@ MC_API int mc_seed_stride(mc_ctx* ctx, const mc_lcg* lcg, uint64_t x0, uint64_t 
     return MC_ERR_ARG;
   }
   cudaStream_t s = (cudaStream_t)stream;
-  const uint64_t mask = mcd::mask_of(lcg->m);
-  if (((uintptr_t)d_states & 15u) == 0) {
-    auto k = seed_stride_kernel<true>;
-    k<<<persistent_grid(k, kSeedBlock, 0, (count + 1) / 2), kSeedBlock, 0, s>>>(lcg->g, lcg->c, x0, stride_q,
-                                                                                  id_begin, count, mask, d_states);
+  const bool vec = ((uintptr_t)d_states & 15u) == 0;
+  StrideArgs a{};
+  a.t = thread_maps(lcg->g, lcg->c, x0, stride_q, id_begin, vec ? 2ull * stride_q : stride_q);
+  a.step_q = mcd::skip_map(lcg->g, lcg->c, stride_q);
+  a.last = mcd::apply(mcd::skip_map(lcg->g, lcg->c, stride_q * (id_begin + count - 1)), x0);
+  a.count = count;
+  a.mask = mcd::mask_of(lcg->m);
+  if (vec) {
+    constexpr auto k = seed_stride_kernel<true>;
+    const int grid = persistent_grid<k, kSeedBlock>((count + 1) / 2);
+    a.sweep = mcd::skip_map(lcg->g, lcg->c, stride_q * 2ull * (uint64_t)grid * kSeedBlock);
+    k<<<grid, kSeedBlock, 0, s>>>(a, d_states);
   } else {
-    auto k = seed_stride_kernel<false>;
-    k<<<persistent_grid(k, kSeedBlock, 0, count), kSeedBlock, 0, s>>>(lcg->g, lcg->c, x0, stride_q, id_begin,
-                                                                        count, mask, d_states);
+    constexpr auto k = seed_stride_kernel<false>;
+    const int grid = persistent_grid<k, kSeedBlock>(count);
+    a.sweep = mcd::skip_map(lcg->g, lcg->c, stride_q * (uint64_t)grid * kSeedBlock);
+    k<<<grid, kSeedBlock, 0, s>>>(a, d_states);
   }
   return mci::cuda_status(cudaGetLastError(), "seed_stride_kernel launch");
 }

@@ -124,6 +124,7 @@ struct RunArgs {
   uint32_t coop_hist;   // histories the block's cooperative tail takes over (0: none)
   uint32_t coop_slots;  // its event records, a power of two
   mcs::Order order;        // processing order of several problems (empty: id order)
+  mcd::Pow2Maps pow2;
 };
 
 // What the end of a history and the cooperative tail need of the launch.
@@ -569,10 +570,7 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
   extern __shared__ unsigned long long s_dyn[];
   unsigned long long* const s_tally = s_dyn;
   __shared__ mcd::Affine tab[64];
-  if (threadIdx.x == 0) {
-    mcd::Affine sq{a.lcg.g, a.lcg.c};
-    for (int j = 0; j < 64; ++j) { tab[j] = sq; sq = mcd::compose(sq, sq); }
-  }
+  mcd::load_maps(a.pow2, tab);
   if constexpr (SMEM) {
     for (uint32_t s = threadIdx.x; s < a.smem_slots; s += blockDim.x) s_tally[s] = 0ull;
   }
@@ -910,6 +908,7 @@ int slab_history_launch(const SlabLaunch& L, cudaStream_t s) {
   a.hist_draws = L.tally->d_hist_draws;
   a.lcg = mcd::Lcg{L.lcg.g, L.lcg.c, mcd::mask_of(L.lcg.m), L.lcg.m};
   a.event_cap = L.event_cap;
+  a.pow2 = mcd::pow2_maps(L.lcg.g, L.lcg.c);
   a.smem_slots = L.smem_slots;
   a.smem_edges = 0;
   if (L.n_problems == 1) {
