@@ -614,14 +614,26 @@ int transport_run_impl(mc_ctx* ctx, const mc_lcg* lcg, const mc_problem* problem
   if (cfg->use_graph && cfg->schedule == MC_SCHED_HISTORY && problems[0].geometry == MC_GEOM_SLAB && re > rb)
     return run_slab_graph(ctx, lcg, problems, n_problems, cfg, tally, rb, re, s);
 
-  st = stage_problems(ctx, problems, n_problems, s);
-  if (st != MC_OK) return st;
-  if (!cfg->accumulate) {
-    MC_TRY_CUDA(cudaMemsetAsync(tally->d_bins, 0, tally->n_slots * sizeof(int64_t), s));
-    MC_TRY_CUDA(cudaMemsetAsync(tally->d_counts, 0, (size_t)n_problems * MC_NCOUNT * sizeof(uint64_t), s));
-  }
   auto* ticket = reinterpret_cast<unsigned long long*>(static_cast<char*>(ctx->scratch.ptr) + kTicketOff);
-  MC_TRY_CUDA(cudaMemsetAsync(ticket, 0, sizeof(unsigned long long), s));
+  if (problems[0].geometry == MC_GEOM_SLAB && n_problems <= mci::kInitProblems &&
+      tally->n_slots <= mci::kInitSlots) {
+    ctx->staged_kind = -1;  // these records do not pass through the staging image
+    st = ctx->problems.reserve(slab_stage_bytes(problems, n_problems));
+    if (st != MC_OK) return st;
+    // (one problem of up to 3071 bins has its tables in shared memory)
+    void* const tables = n_problems == 1 && problems[0].n_bins < 3072u ? nullptr : slab_tables_of(ctx, n_problems);
+    st = mci::slab_init(problems, n_problems, ctx->problems.ptr, tables,
+                        slab_order_of(ctx, problems, n_problems), tally, !cfg->accumulate, ticket, s);
+    if (st != MC_OK) return st;
+  } else {
+    st = stage_problems(ctx, problems, n_problems, s);
+    if (st != MC_OK) return st;
+    if (!cfg->accumulate) {
+      MC_TRY_CUDA(cudaMemsetAsync(tally->d_bins, 0, tally->n_slots * sizeof(int64_t), s));
+      MC_TRY_CUDA(cudaMemsetAsync(tally->d_counts, 0, (size_t)n_problems * MC_NCOUNT * sizeof(uint64_t), s));
+    }
+    MC_TRY_CUDA(cudaMemsetAsync(ticket, 0, sizeof(unsigned long long), s));
+  }
   if (re == rb) return MC_OK;
 
   if (problems[0].geometry == MC_GEOM_BOX) return run_box(ctx, lcg, n_problems, cfg, tally, rb, re, ticket, s);

@@ -29,17 +29,19 @@ namespace {
 
 using mcs::SlabDev;
 
+// Bin edge and width tables of one problem, by the threads of a block.
+__device__ __forceinline__ void write_tables(const SlabDev& q, double* __restrict__ tables) {
+  double* e = tables + q.tab_off;
+  double* w = e + q.n_bins + 1;
+  for (uint32_t j = threadIdx.x; j <= q.n_bins; j += blockDim.x) e[j] = mcs::slab_edge(q, (int)j);
+  for (uint32_t j = threadIdx.x; j < q.n_bins; j += blockDim.x)
+    w[j] = __dsub_rn(mcs::slab_edge(q, (int)j + 1), mcs::slab_edge(q, (int)j));
+}
+
 // Bin edge and width tables of every problem, after the records (`tables`
 // may be null: no tables).
 __global__ void slab_tables_kernel(const SlabDev* __restrict__ p, uint32_t n, double* __restrict__ tables) {
-  for (uint32_t i = blockIdx.x; i < n; i += gridDim.x) {
-    const SlabDev& q = p[i];
-    double* e = tables + q.tab_off;
-    double* w = e + q.n_bins + 1;
-    for (uint32_t j = threadIdx.x; j <= q.n_bins; j += blockDim.x) e[j] = mcs::slab_edge(q, (int)j);
-    for (uint32_t j = threadIdx.x; j < q.n_bins; j += blockDim.x)
-      w[j] = __dsub_rn(mcs::slab_edge(q, (int)j + 1), mcs::slab_edge(q, (int)j));
-  }
+  for (uint32_t i = blockIdx.x; i < n; i += gridDim.x) write_tables(p[i], tables);
 }
 
 // Expected flights per history of a slab problem with a uniform isotropic
@@ -55,25 +57,27 @@ __device__ __forceinline__ float expected_flights(const SlabDev& q) {
   return 1.0f / fmaxf(1e-6f, 1.0f - (float)q.c * (1.0f - p_esc));
 }
 
-__global__ void slab_prep_kernel(SlabDev* __restrict__ p, uint32_t n, uint32_t* __restrict__ order,
-                                 uint64_t* __restrict__ order_begin) {
-  for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
-    SlabDev& q = p[i];
-    q.h = q.L / (double)q.n_bins;
-    q.inv_h = (double)q.n_bins / q.L;
-    mcx::fixed_of(q.inv_h, q.ih_q, q.ih_s);
-    q.inv_st = 1.0 / q.sigma_t;
-    q.p_abs = 1.0 - q.c;
-    q.p_abs_n = (uint64_t)ceil(q.p_abs * 0x1p53);
-    q.L_f = (float)q.L;
-    q.h_f = q.L_f / (float)q.n_bins;
-    q.inv_h_f = (float)q.n_bins / q.L_f;
-    q.inv_st_f = 1.0f / (float)q.sigma_t;
-    q.guard_f = q.L_f * 0x1p-18f;
-    const uint64_t parent = q.seeding == MC_SEED_HASH_HIER ? mcd::hash64(q.key, q.seed) : q.seed;
-    q.seed_hash = mcd::seed_hash_of(parent);
-  }
-  __syncthreads();
+// The fields of a record that follow from the others (but hist_begin).
+__device__ __forceinline__ void derive(SlabDev& q) {
+  q.h = q.L / (double)q.n_bins;
+  q.inv_h = (double)q.n_bins / q.L;
+  mcx::fixed_of(q.inv_h, q.ih_q, q.ih_s);
+  q.inv_st = 1.0 / q.sigma_t;
+  q.p_abs = 1.0 - q.c;
+  q.p_abs_n = (uint64_t)ceil(q.p_abs * 0x1p53);
+  q.L_f = (float)q.L;
+  q.h_f = q.L_f / (float)q.n_bins;
+  q.inv_h_f = (float)q.n_bins / q.L_f;
+  q.inv_st_f = 1.0f / (float)q.sigma_t;
+  q.guard_f = q.L_f * 0x1p-18f;
+  const uint64_t parent = q.seeding == MC_SEED_HASH_HIER ? mcd::hash64(q.key, q.seed) : q.seed;
+  q.seed_hash = mcd::seed_hash_of(parent);
+}
+
+// hist_begin of every record and (order non-null) the processing order, by
+// one block, from records whose other fields are complete.
+__device__ __forceinline__ void chain_records(SlabDev* __restrict__ p, uint32_t n, uint32_t* __restrict__ order,
+                                              uint64_t* __restrict__ order_begin) {
   if (threadIdx.x == 0) {
     uint64_t acc = 0;
     for (uint32_t i = 0; i < n; ++i) {
@@ -103,6 +107,58 @@ __global__ void slab_prep_kernel(SlabDev* __restrict__ p, uint32_t n, uint32_t* 
   }
 }
 
+__global__ void slab_prep_kernel(SlabDev* __restrict__ p, uint32_t n, uint32_t* __restrict__ order,
+                                 uint64_t* __restrict__ order_begin) {
+  for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) derive(p[i]);
+  __syncthreads();
+  chain_records(p, n, order, order_begin);
+}
+
+// A whole call's set-up in one launch, for few problems (their records travel
+// with the launch's arguments): records, order and tables as slab_prep has
+// them, the ticket, and a fresh tally's zeros.  Against an upload from pinned
+// memory, two prep kernels and three memsets, a call of 10^4 histories whose
+// problem differs from the last one's took 59 us and takes 38 (6 of them by
+// slab_history_kernel_few).
+struct InitArgs {
+  SlabDev src[mci::kInitProblems];
+  uint32_t n;
+  SlabDev* dst;
+  uint32_t* order;          // nullable
+  uint64_t* order_begin;
+  double* tables;           // nullable
+  unsigned long long* ticket;
+  unsigned long long* bins;    // nullable: accumulating
+  unsigned long long* counts;
+  uint64_t n_slots;
+};
+
+__global__ void __launch_bounds__(128) slab_init_kernel(const InitArgs a) {
+  const uint32_t tblocks = a.tables ? a.n : 0u;
+  if (blockIdx.x == 0u) {
+    for (uint32_t i = threadIdx.x; i < a.n; i += blockDim.x) {
+      SlabDev q = a.src[i];
+      derive(q);
+      a.dst[i] = q;
+    }
+    if (threadIdx.x == 0) *a.ticket = 0ull;
+    if (a.bins)
+      for (uint32_t i = threadIdx.x; i < a.n * MC_NCOUNT; i += blockDim.x) a.counts[i] = 0ull;
+    __syncthreads();
+    chain_records(a.dst, a.n, a.order, a.order_begin);
+    return;
+  }
+  if (blockIdx.x <= tblocks) {
+    SlabDev q = a.src[blockIdx.x - 1u];
+    derive(q);
+    write_tables(q, a.tables);
+    return;
+  }
+  const uint64_t nz = (uint64_t)(gridDim.x - 1u - tblocks) * blockDim.x;
+  for (uint64_t i = (uint64_t)(blockIdx.x - 1u - tblocks) * blockDim.x + threadIdx.x; i < a.n_slots; i += nz)
+    a.bins[i] = 0ull;
+}
+
 struct RunArgs {
   const SlabDev* probs;
   uint32_t nprob;
@@ -123,6 +179,7 @@ struct RunArgs {
   uint32_t row_bins;    // bins of a warp's row cache (0: none; all problems fit it otherwise)
   uint32_t coop_hist;   // histories the block's cooperative tail takes over (0: none)
   uint32_t coop_slots;  // its event records, a power of two
+  uint32_t coop_after;  // passes of a warp after the ticket ran out before it offers its histories
   mcs::Order order;        // processing order of several problems (empty: id order)
   mcd::Pow2Maps pow2;
 };
@@ -259,7 +316,6 @@ constexpr int kCoopHistWords = 14;    // 8-byte words per history record
 constexpr int kCoopWords = 2;         // per event record
 constexpr int kCoopMaxLog = 8;        // at most 2^8 records per history and round
 constexpr int kCoopMinLog = 3;        // at least 2^3: E = 7 events
-constexpr uint32_t kCoopAfter = 32;   // passes of a warp after the ticket ran out before it offers its histories
 constexpr uint32_t kCoopMaxHist = 256;
 
 __device__ __forceinline__ mcd::Affine affine_steps(const mcd::Affine* tab, uint64_t k) {
@@ -691,9 +747,9 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
       if (lane == 0) s_live[threadIdx.x >> 5] = 0u;
       break;
     }
-    if (!more && a.coop_hist != 0u && ++after >= kCoopAfter) {
+    if (!more && a.coop_hist != 0u && ++after >= a.coop_after) {
       // The block's live histories, from each warp's own count (a warp that
-      // still refills, or has not run kCoopAfter passes since, counts as
+      // still refills, or has not run coop_after passes since, counts as
       // full).  Counts only fall, so a sum read while they change is an upper
       // bound, and whoever finds it small enough starts the tail for all.
       volatile uint32_t* const vl = s_live;
@@ -777,58 +833,90 @@ __global__ void __maxnreg__(80) slab_history_kernel_f64(const RunArgs a) {
   slab_history_body<M, F32, SMEM, AGG>(a);
 }
 
+// A run of at most a few warps per SM waits for its longest histories, not for
+// issue slots: registers to interleave an event's chains are worth more than
+// warps that are not there (10^4 histories, fp64: 53 us a call at 96 registers
+// and more against 59 at 80).
 template <int M, bool F32, bool SMEM, bool AGG>
-auto history_kernel_of() {
+__global__ void __maxnreg__(128) slab_history_kernel_few(const RunArgs a) {
+  slab_history_body<M, F32, SMEM, AGG>(a);
+}
+
+constexpr uint64_t kFewThreads = 128;  // per SM, at most, for the kernel of small runs
+
+template <int M, bool F32, bool SMEM, bool AGG>
+auto history_kernel_of(bool few) {
+  if constexpr (M == 63 && !AGG) {
+    if (few) return slab_history_kernel_few<M, F32, SMEM, AGG>;
+  }
   if constexpr (F32) return slab_history_kernel_f32<M, F32, SMEM, AGG>;
   else return slab_history_kernel_f64<M, F32, SMEM, AGG>;
 }
 
 template <int M, bool F32, bool SMEM, bool AGG>
 int launch_history(const RunArgs& a0, int block, int blocks_per_sm, int num_sms, cudaStream_t s) {
-  auto k = history_kernel_of<M, F32, SMEM, AGG>();
   RunArgs a = a0;
-  // Static shared memory of this instantiation (read once) and the device's
-  // opt-in limit: what does not fit beside them is given up, the cooperative
-  // tail first and then the edge tables (both only save time).
-  static size_t static_smem = ~(size_t)0;
-  if (static_smem == ~(size_t)0) {
-    cudaFuncAttributes fa{};
-    const int st = mci::cuda_status(cudaFuncGetAttributes(&fa, k), "cudaFuncGetAttributes(slab_history_kernel)");
-    if (st != MC_OK) return st;
-    static_smem = fa.sharedSizeBytes;
-  }
-  int dev = 0, optin = 0;
+  // Enough warps for every chunk, never more than fill the GPU.
+  const uint64_t warps_needed = (a.total + a.chunk - 1) / a.chunk;
+  const uint64_t blocks_needed = (warps_needed * 32 + block - 1) / block;
+  const bool few = blocks_needed * (uint64_t)block <= (uint64_t)num_sms * kFewThreads;
+  auto k = history_kernel_of<M, F32, SMEM, AGG>(few);
+  // What the driver says about this kernel on this device, asked for once: its
+  // static shared memory, the opt-in limit, and after the request for all of
+  // that, the blocks per SM of the last launch shape.
+  struct Known {
+    int dev = -1, optin = 0, block = 0, per_sm = 0;
+    size_t static_smem = 0, smem = 0;
+  };
+  static thread_local Known known[2];
+  Known& kn = known[few ? 1 : 0];
+  int dev = 0;
   cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (kn.dev != dev) {
+    cudaFuncAttributes fa{};
+    int st = mci::cuda_status(cudaFuncGetAttributes(&fa, k), "cudaFuncGetAttributes(slab_history_kernel)");
+    if (st != MC_OK) return st;
+    Known n;
+    st = mci::cuda_status(cudaDeviceGetAttribute(&n.optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev),
+                          "cudaDeviceGetAttribute(shared memory)");
+    if (st != MC_OK) return st;
+    n.static_smem = fa.sharedSizeBytes;
+    st = mci::cuda_status(
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, n.optin - (int)n.static_smem),
+        "cudaFuncSetAttribute(slab_history_kernel)");
+    if (st != MC_OK) return st;
+    n.dev = dev;
+    kn = n;
+  }
+  const size_t optin = (size_t)kn.optin, static_smem = kn.static_smem;
+  // What does not fit beside the static part is given up, the row caches first,
+  // then the cooperative tail and the edge tables (all only save time).
   auto dynamic_smem = [&a, block]() {
     return (SMEM ? (size_t)a.smem_slots * 8u : 0u) + (size_t)a.smem_edges * 16u +  // edges + widths
            ((size_t)a.coop_hist * kCoopHistWords + (size_t)a.coop_slots * kCoopWords) * 8u +
            (size_t)(block / 32) * a.row_bins * 8u;
   };
   if (SMEM || a.row_bins > kMaxRowBins) a.row_bins = 0;
-  if (static_smem + dynamic_smem() > (size_t)optin) a.row_bins = 0;
-  if (static_smem + dynamic_smem() > (size_t)optin) a.coop_hist = a.coop_slots = 0;
-  if (static_smem + dynamic_smem() > (size_t)optin) a.smem_edges = 0;
+  if (static_smem + dynamic_smem() > optin) a.row_bins = 0;
+  if (static_smem + dynamic_smem() > optin) a.coop_hist = a.coop_slots = 0;
+  if (static_smem + dynamic_smem() > optin) a.smem_edges = 0;
   const size_t smem = dynamic_smem();
-  if (static_smem + smem > (size_t)optin) {
+  if (static_smem + smem > optin) {
     mci::set_error("slab_history_kernel: %u tally slots do not fit in shared memory", a.smem_slots);
     return MC_ERR_ARG;
   }
-  if (static_smem + smem > 48u * 1024u) {
-    int st = mci::cuda_status(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                              "cudaFuncSetAttribute(slab_history_kernel)");
-    if (st != MC_OK) return st;
-  }
   int per_sm = blocks_per_sm;
   if (per_sm <= 0) {
-    int st = mci::cuda_status(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem),
-                              "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
-    if (st != MC_OK) return st;
-    if (per_sm < 1) per_sm = 1;
+    if (kn.per_sm == 0 || kn.block != block || kn.smem != smem) {
+      int st = mci::cuda_status(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem),
+                                "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
+      if (st != MC_OK) return st;
+      kn.per_sm = std::max(per_sm, 1);
+      kn.block = block;
+      kn.smem = smem;
+    }
+    per_sm = kn.per_sm;
   }
-  // Enough warps for every chunk, never more than fill the GPU.
-  const uint64_t warps_needed = (a.total + a.chunk - 1) / a.chunk;
-  const uint64_t blocks_needed = (warps_needed * 32 + block - 1) / block;
   const uint64_t full = (uint64_t)num_sms * (uint64_t)per_sm;
   const int grid = (int)std::max<uint64_t>(1, std::min(full, blocks_needed));
   a.grab_shift = 1u;  // twice the launch's warps, rounded up to a power of two
@@ -888,6 +976,24 @@ int slab_prep(void* d_probs, uint32_t n, cudaStream_t s, void* d_tables, void* d
   return cuda_status(cudaGetLastError(), "slab_tables_kernel launch");
 }
 
+int slab_init(const mc_problem* src, uint32_t n, void* d_probs, void* d_tables, void* d_order, const mc_tally* tally,
+              bool zero, unsigned long long* d_ticket, cudaStream_t s) {
+  InitArgs a;
+  slab_fill_host(src, n, a.src);
+  a.n = n;
+  a.dst = static_cast<SlabDev*>(d_probs);
+  a.order = n >= 2 ? static_cast<uint32_t*>(d_order) : nullptr;
+  a.order_begin = a.order ? reinterpret_cast<uint64_t*>(a.order + ((n + 1u) & ~1u)) : nullptr;
+  a.tables = static_cast<double*>(d_tables);
+  a.ticket = d_ticket;
+  a.bins = zero ? reinterpret_cast<unsigned long long*>(tally->d_bins) : nullptr;
+  a.counts = reinterpret_cast<unsigned long long*>(tally->d_counts);
+  a.n_slots = zero ? tally->n_slots : 0u;
+  const uint32_t zblocks = (uint32_t)std::min<uint64_t>((a.n_slots + 511u) / 512u, 1024u);
+  slab_init_kernel<<<1u + (a.tables ? n : 0u) + zblocks, 128, 0, s>>>(a);
+  return cuda_status(cudaGetLastError(), "slab_init_kernel launch");
+}
+
 uint64_t slab_table_doubles(const mc_problem* src, uint32_t n) {
   uint64_t t = 0;
   for (uint32_t i = 0; i < n; ++i) t += 2ull * src[i].n_bins + 1ull;
@@ -928,6 +1034,9 @@ int slab_history_launch(const SlabLaunch& L, cudaStream_t s) {
   // fp32 (a power of two).  slab_long, 10^6 histories: fp64 154 ms, against 164
   // with half the threads and 157 with two records; fp32 107 ms, against 114
   // with four records; without the tail 244 and 160 ms.
+  // passes after which what is left counts as long (16: 298 us instead of 292
+  // for 300 000 histories of 9 flights, 4: 329; long chains do not care)
+  a.coop_after = 32u;
   if (L.pool_lock_attempts != 0u && L.block >= 64) {
     a.coop_slots = 128u;
     while (a.coop_slots * 2u <= (uint32_t)L.block * (L.f32 ? 2u : 4u)) a.coop_slots *= 2u;
