@@ -1,6 +1,6 @@
 // host_io.cu -- mc_lcg_draw_host: fused seeding and draws on host buffers.
 //
-// The id range is cut into slices of kSlice streams.  Two device slots
+// The id range is cut into slices.  Two device slots
 // (context-owned) alternate: while the draw kernel of slice j runs on the
 // caller's stream, a private copy stream returns slice j - 1's final states
 // and digests to the host, and a slot is reused only after its last copy
@@ -15,7 +15,18 @@
 
 namespace {
 
-constexpr uint64_t kSlice = 1ull << 22;  // streams per slice (32 MiB per array)
+constexpr uint64_t kSlice = 1ull << 20;     // streams per slice at most (8 MiB per array)
+constexpr uint64_t kMinSlice = 1ull << 17;  // and at least
+
+// A quarter of the range, so that all but the first slice's kernel runs behind
+// a copy; a slice costs some 5 us of its own, so not more of them than that
+// until a slice is long against it.  (64 draws: 3 * 10^6 streams in slices of
+// up to 2^22 took 361 us, an 80 us kernel and then the copy, now 312; in
+// sixteenths 341.  8 * 10^6 streams 805, now 744.)
+uint64_t slice_of(uint64_t n) {
+  const uint64_t s = (n / 4 + 31) & ~(uint64_t)31;
+  return std::min(kSlice, std::max(kMinSlice, s));
+}
 
 int io_setup(mc_ctx* ctx) {
   if (!ctx->io_stream) MC_TRY_CUDA(cudaStreamCreateWithFlags(&ctx->io_stream, cudaStreamNonBlocking));
@@ -51,10 +62,10 @@ extern "C" MC_API int mc_lcg_draw_host(mc_ctx* ctx, const mc_lcg* lcg, const mc_
   if (st != MC_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
   uint64_t* base = static_cast<uint64_t*>(ctx->host_io.ptr);
-  const uint64_t nslices = (n_streams + kSlice - 1) / kSlice;
+  const uint64_t slice = slice_of(n_streams), nslices = (n_streams + slice - 1) / slice;
   for (uint64_t j = 0; j < nslices; ++j) {
     const int k = (int)(j & 1u);
-    const uint64_t lo = j * kSlice, cnt = std::min<uint64_t>(kSlice, n_streams - lo);
+    const uint64_t lo = j * slice, cnt = std::min<uint64_t>(slice, n_streams - lo);
     uint64_t* d_st = base + (size_t)k * 2 * kSlice;
     uint64_t* d_dg = d_st + kSlice;
     if (j >= 2) MC_TRY_CUDA(cudaStreamWaitEvent(s, ctx->io_copied[k], 0));  // slot free again
