@@ -21,7 +21,6 @@
 // secondaries overflowed the lane stacks in a phase, and launches the
 // generations of those before the phase's control.
 // The fp64 arithmetic is rounded once per operation (--fmad=false).
-#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -34,8 +33,6 @@
 #include "slab.cuh"
 #include "transport.h"
 
-namespace cg = cooperative_groups;
-
 namespace {
 
 using mcp::kStack;
@@ -43,8 +40,8 @@ using mcp::Overflow;
 using mcp::Pending;
 using mcp::PulseDev;
 
-// A particle waiting at a census (48 bytes).
-struct BankRec {
+// A particle waiting at a census (48 bytes, moved as three 16-byte words).
+struct __align__(16) BankRec {
   double x, mu, w;
   uint64_t s;      // LCG state, masked to m bits
   uint64_t draws;  // draws made from this stream so far
@@ -57,7 +54,7 @@ constexpr uint64_t kOneOffKey = 1ull << 63;  // keys of one-off values: 2^63 + p
 // Per group, derived from the group's exact weight total W after a phase:
 // the factor N / (W 2^-32) of the copy counts (0 when W = 0: no copies),
 // the copies' weight W 2^-32 / N, its collision score and its fixed point.
-struct GroupCtl {
+struct __align__(16) GroupCtl {
   double ratio, w;
   long long unit, wfix;
 };
@@ -128,9 +125,9 @@ struct StagedItem {
   GroupCtl gc;
 };
 
-// Held at 96 registers: 3 * 10^6 sources in 20 phases take 7.33 ms, against
+// Held at 96 registers: 3 * 10^6 sources in 20 phases take 7.24 ms, against
 // 7.76 / 7.86 / 8.06 ms at 80 / 72 / 64 (more warps, but spills and a smaller
-// share of the L1 for each).
+// share of the L1 for each) and 8.1 at 112 and 128.
 template <int M, bool AGG>
 __global__ void __maxnreg__(96) pulse_census_kernel(const CensusArgs a) {
   extern __shared__ StagedItem s_items[];
@@ -284,17 +281,19 @@ __global__ void __maxnreg__(96) pulse_census_kernel(const CensusArgs a) {
           e.draws = r.draws;
           e.group = grp;
           e.pad = 0;
-          cg::coalesced_group cgp = cg::coalesced_threads();
+          // one slot claim for the lanes that bank together
+          const unsigned act = __activemask();
+          const int leader = __ffs((int)act) - 1;
           unsigned long long base = 0;
-          if (cgp.thread_rank() == 0) base = atomicAdd(a.out_count, (unsigned long long)cgp.size());
-          base = cgp.shfl(base, 0);
-          const uint64_t idx = base + cgp.thread_rank();
+          if ((int)lane == leader) base = atomicAdd(a.out_count, (unsigned long long)__popc(act));
+          base = __shfl_sync(act, base, leader);
+          const uint64_t idx = base + __popc(act & lt_mask);
           if (idx < a.cap) a.out[idx] = e;
           else atomicAdd(s_counts + MC_C_DROPPED, 1ull);  // reported as MC_ERR_CAPACITY by mc_tally_read
           // lanes of one group carry one weight in a phase: one atomic per group
-          cg::coalesced_group same = cg::labeled_partition(cgp, grp);
-          if (same.thread_rank() == 0)
-            atomicAdd(a.w_out + (grp - a.group_begin), (unsigned long long)(wfix * (long long)same.size()));
+          const unsigned same = __match_any_sync(act, grp);
+          if ((int)lane == __ffs((int)same) - 1)
+            atomicAdd(a.w_out + (grp - a.group_begin), (unsigned long long)(wfix * (long long)__popc(same)));
         }
       } else {
         const double xn = x + d * mu;
