@@ -608,6 +608,12 @@ constexpr uint32_t kMaxRowBins = 256;  // of a warp's row cache (2 KiB)
 // fp32 10.9 ms against 10.6, fp64 17.3 against 15.0).
 constexpr uint32_t kIdle = 16;
 
+// The ticket positions of one problem: begin + id for its history id.
+struct Span {
+  uint64_t begin;
+  uint32_t prob;
+};
+
 // Adds a warp's row cache to its tally row in global memory and clears it.
 __device__ __forceinline__ void flush_row(unsigned long long* global_row, uint32_t row, uint32_t n_bins) {
   extern __shared__ unsigned long long s_dyn[];
@@ -645,6 +651,8 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
   const uint32_t row0 = (SMEM ? a.smem_slots : 0u) + 2u * a.smem_edges + a.coop_hist * kCoopHistWords + a.coop_slots * kCoopWords;
   if constexpr (!SMEM)
     for (uint32_t i = threadIdx.x; i < (blockDim.x >> 5) * a.row_bins; i += blockDim.x) s_dyn[row0 + i] = 0ull;
+  __shared__ Span s_span[16];
+  if (threadIdx.x < 16u) s_span[threadIdx.x] = Span{1ull << 63, 0u};
   if (threadIdx.x < 16u) s_live[threadIdx.x] = threadIdx.x < (blockDim.x >> 5) ? kCoopMaxHist : 0u;
   if (s_edges) {
     const SlabDev& p0 = a.probs[0];
@@ -703,12 +711,21 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
       const uint64_t avail = pool_end - pool_next;
       const unsigned rank = __popc(dead & lt_mask);
       if (!alive && rank < avail) {
-        uint32_t pi;
-        mcs::ticket_history(a.probs, a.nprob, a.range_begin, a.order, pool_next + rank, pi, gi);
+        uint32_t pi = 0;
+        const uint64_t t = pool_next + rank;
+        uint64_t id = 0;
+        if (a.nprob != 1u) {  // mostly the problem the warp's last history was of
+          pi = s_span[threadIdx.x >> 5].prob;
+          id = t - s_span[threadIdx.x >> 5].begin;
+        }
+        if (a.nprob == 1u || id >= a.probs[pi].n_hist) {
+          mcs::ticket_history(a.probs, a.nprob, a.range_begin, a.order, t, pi, gi);
+          id = gi - a.probs[pi].hist_begin;
+        }
         if ((int)pi != lc.prob) { lc.flush(a.counts, a.probs); lc.prob = (int)pi; }
         P = a.probs + pi;
-        const uint64_t id = gi - P->hist_begin;
-        const uint64_t batch = mcs::batch_of(id, P->n_hist, P->n_batches);
+        gi = P->hist_begin + id;
+        const uint64_t batch = P->n_batches > 1u ? mcs::batch_of(id, P->n_hist, P->n_batches) : 0ull;
         sink.base = (SMEM ? s_tally : a.tally) + P->tally_offset + batch * P->n_bins;
         if (a.tables) {
           sink.edges = a.tables + P->tab_off;
@@ -721,6 +738,12 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
         events = 0;
         ++lc.src;
         alive = true;
+      }
+      if (a.nprob != 1u) {  // the last position taken: its problem's span of positions
+        __syncwarp();
+        if ((dead & (1u << lane)) != 0u && rank + 1u == min((uint64_t)__popc(dead), avail))
+          s_span[threadIdx.x >> 5] = Span{pool_next + rank - (gi - P->hist_begin), (uint32_t)(P - a.probs)};
+        __syncwarp();
       }
       pool_next += min((uint64_t)__popc(dead), avail);
       dead = __ballot_sync(kFull, !alive);
