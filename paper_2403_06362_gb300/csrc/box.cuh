@@ -103,6 +103,11 @@ template <> __device__ __forceinline__ float recip<float>(float v) { return __fr
 // kernel's largest stall).
 template <typename T>
 __device__ __forceinline__ void set_inv(Part<T>& q) {
+  if constexpr (sizeof(T) == 4) {  // short enough three times over
+#pragma unroll
+    for (int a = 0; a < 3; ++a) q.inv[a] = q.u[a] != T(0) ? recip<T>(q.u[a]) : T(0);
+    return;
+  }
   T u0 = q.u[0], u1 = q.u[1], u2 = q.u[2], i0 = T(0), i1 = T(0), i2 = T(0);
 #pragma unroll 1
   for (int a = 0; a < 3; ++a) {
@@ -119,10 +124,20 @@ __device__ __forceinline__ void set_inv(Part<T>& q) {
   q.inv[2] = i2;
 }
 
+// v1^2 + v2^2 - 1 of a direction try in fp32, off by less than 2^-20: from
+// the leading 24 bits of each draw (exact in fp32; |v| off by less than
+// 2^-23).
+__device__ __forceinline__ float try_s(uint64_t n1, uint64_t n2) {
+  const float a = __uint2float_rn((uint32_t)(n1 >> 29)) * 0x1p-23f - 1.0f;
+  const float b = __uint2float_rn((uint32_t)(n2 >> 29)) * 0x1p-23f - 1.0f;
+  return a * a + b * b - 1.0f;
+}
+
 // Marsaglia (1972): v1, v2 uniform on [-1,1)^2 until v1^2 + v2^2 < 1.
-// fp64: a try is decided in fp32 where v1^2 + v2^2 is not within 2^-19 of 1
-// (its fp32 value is off by less than 2^-21), so the fp64 unit forms s for
-// the accepted try alone; the square root is the integer pipes'.
+// A try is decided by try_s where that is not within 2^-19 of the circle, so
+// that only the accepted one's v1 and v2 are formed as the path has them
+// (fp32: 2 RN(u) - 1; fp64: exact, and the fp64 unit forms s once); fp64's
+// square root is the integer pipes'.
 template <int M, typename T>
 __device__ __forceinline__ void iso_dir(mcs::Rng<M>& r, const mcd::Lcg& l, T u[3]) {
   if constexpr (sizeof(T) == 8) {
@@ -130,8 +145,7 @@ __device__ __forceinline__ void iso_dir(mcs::Rng<M>& r, const mcd::Lcg& l, T u[3
     for (;;) {
       n1 = r.next_n(l);
       n2 = r.next_n(l);
-      const float f1 = mcs::mu_f32(n1), f2 = mcs::mu_f32(n2);
-      const float s = f1 * f1 + f2 * f2 - 1.0f;
+      const float s = try_s(n1, n2);
       if (s < -0x1p-19f) break;
       if (s > 0x1p-19f) continue;
       const double v1 = mcx::two_u_minus_1(n1), v2 = mcx::two_u_minus_1(n2);
@@ -144,12 +158,18 @@ __device__ __forceinline__ void iso_dir(mcs::Rng<M>& r, const mcd::Lcg& l, T u[3
     u[1] = v2 * t;
     u[2] = __fma_rn(-2.0, s, 1.0);  // 2 s is exact: one rounding either way
   } else {
+    uint64_t n1, n2;
     T v1, v2, s;
-    do {
-      v1 = T(2) * from_n<T>(r.next_n(l)) - T(1);
-      v2 = T(2) * from_n<T>(r.next_n(l)) - T(1);
+    for (;;) {
+      n1 = r.next_n(l);
+      n2 = r.next_n(l);
+      const float c = try_s(n1, n2);
+      if (c > 0x1p-19f) continue;
+      v1 = T(2) * from_n<T>(n1) - T(1);
+      v2 = T(2) * from_n<T>(n2) - T(1);
       s = v1 * v1 + v2 * v2;
-    } while (!lt(s, T(1)));
+      if (c < -0x1p-19f || lt(s, T(1))) break;
+    }
     const T t = sqrt(T(1) - s);
     u[0] = T(2) * v1 * t;
     u[1] = T(2) * v2 * t;

@@ -105,32 +105,30 @@ __host__ __device__ __forceinline__ bool abs_le(double x, double h) {
 }
 
 // q = RN(2^105 / M) for 2^52 <= M < 2^53 (ties cannot occur: 2^106 = (2q + 1) M
-// would make M a power of two, and M = 2^52 divides exactly).  With m = M 2^-52 = F (1 + r), F = 1 + j/1024
-// the left end of m's cell (the table of 2^63 / F that the logarithm uses)
-// and 0 <= r < 2^-10,
-//   2^53 / m = (2^53 / F) (1 - r (1 - r (1 - r (1 - r (1 - r))))) + O(r^6 < 2^-60)
-// by Horner's rule on non-negative fixed point (the inner terms on 32 bits)
-// puts q within a unit; an exact remainder fixes it and rounds.
+// would make M a power of two, and M = 2^52 divides exactly).  An fp32
+// reciprocal of m = M 2^-52 gives Q = 2^32 / m (1 - e) with |e| < 2^-22, and
+// 2^84 e = 2^84 - M Q exactly from the low words.  Then
+//   2^53 / m = 2^21 Q (1 + e + e^2) + O(2^53 e^3 < 2^-13)
+// puts q within a unit, and the exact remainder fixes and rounds it.  (Half
+// the instructions of a table reduction with a polynomial.)
 __host__ __device__ __forceinline__ uint64_t recip_mantissa(uint64_t M) {
-  const int j = (int)((M >> 42) & 1023ull);
+  const uint32_t m32 = (uint32_t)(M >> 21);  // m 2^31
 #ifdef __CUDA_ARCH__
-  const uint64_t inv = __ldg(&mclog::dev::kInvF[j]);  // 2^63 / F
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__uint2float_rn(m32) * 0x1p-31f));
+  const uint32_t Q = __float2uint_rz(fminf(y * 0x1p32f, 4294967040.0f));
 #else
-  const uint64_t inv = mclog::host::kInvF[j];
+  const float y = 1.0f / ((float)m32 * 0x1p-31f) * 0x1p32f;
+  const uint32_t Q = y < 4294967040.0f ? (uint32_t)y : 4294967040u;
 #endif
-  const uint64_t R = mclog::umulhi_((M & ((1ull << 42) - 1ull)) << 22, inv);  // r 2^73
-  const uint32_t r32 = (uint32_t)(R >> 31);                                     // r 2^42
-  uint32_t t = (1u << 31) - (r32 >> 11);                       // T3 = 1 - r, scale 2^31
-  t = (1u << 31) - (mclog::umulhi32_(r32, t) >> 10);           // T2 = 1 - r T3, scale 2^31
-  t = (1u << 31) - mclog::umulhi32_(r32, t);                   // T1 - (1 - 2^-10), scale 2^41
-  const uint64_t rt = ((uint64_t)(uint32_t)(R >> 32) * t + (((uint64_t)(uint32_t)R * t) >> 32)) >> 19;
-  const uint64_t t0 = (1ull << 63) - ((R >> 10) - (R >> 20)) - rt;         // T0 = 1 - r T1, scale 2^63
-  const uint64_t S = (1ull << 63) - (mclog::umulhi_(R, t0) >> 9);          // 1 / (1 + r), scale 2^63
-  uint64_t q = mclog::umulhi_(inv, S) >> 9;                                // ~ 2^53 / m
-  // exact remainder r = 2^105 - q M (|r| < 2^63: the low words decide), then round
-  long long rem = (long long)(0ull - q * M);
-  // (q's error: its truncation and below 2^-6 of a unit before it, so one
-  // correction either way is enough)
+  const long long e = (long long)(0ull - M * (uint64_t)Q);  // 2^84 (1 - M Q 2^-84), below 2^62 in magnitude
+  const int eh = (int)(e >> 32);                             // e 2^52
+  // 2^21 Q e = Q (e 2^84) 2^-63, and 2^21 Q e^2 from e's high word
+  const long long t1 = ((long long)eh * (long long)Q + (long long)(((uint64_t)(uint32_t)e * Q) >> 32)) >> 31;
+  const uint32_t e2 = (uint32_t)(((long long)eh * eh) >> 32);  // e^2 2^72, below 2^30
+  const uint32_t t2 = (uint32_t)(((uint64_t)e2 * Q) >> 51);    // Q e^2 2^21
+  uint64_t q = ((uint64_t)Q << 21) + (uint64_t)t1 + t2 + 1ull;  // (1: half of what the truncations take)
+  long long rem = (long long)(0ull - q * M);  // 2^105 - q M (its low word: |rem| < 2^63)
   if (rem < 0) { --q; rem += (long long)M; }
   if (rem >= (long long)M) { ++q; rem -= (long long)M; }
   if ((uint64_t)rem * 2ull > M) ++q;
