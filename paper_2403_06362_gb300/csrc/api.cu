@@ -437,6 +437,7 @@ MC_API void mc_ctx_destroy(mc_ctx* ctx) {
   if (ctx->h_problems) cudaFreeHost(ctx->h_problems);
   if (ctx->h_done) cudaFreeHost(ctx->h_done);
   if (ctx->h_count) cudaFreeHost(ctx->h_count);
+  if (ctx->h_read) cudaFreeHost(ctx->h_read);
   ctx->children.release();
   ctx->census.release();
   delete ctx->staged_image;
@@ -923,11 +924,25 @@ MC_API int mc_tally_read(mc_ctx* ctx, const mc_problem* problems, uint32_t probl
   MC_TRY_CUDA(cudaSetDevice(ctx->device));
   std::vector<int64_t> raw(slots);
   std::vector<uint64_t> cnt(MC_NCOUNT);
-  MC_TRY_CUDA(cudaMemcpyAsync(raw.data(), tally->d_bins + p.tally_offset, slots * sizeof(int64_t),
+  // A small tally comes back through page-locked memory of the context: a copy
+  // into pageable memory waits for the stream by itself and is staged by the
+  // driver, 10 us each (10^4 histories run and read: 78 -> 67 us).
+  int64_t* bins_to = raw.data();
+  uint64_t* cnt_to = cnt.data();
+  if (slots <= mci::kReadSlots) {
+    if (!ctx->h_read) MC_TRY_CUDA(cudaMallocHost(&ctx->h_read, (mci::kReadSlots + MC_NCOUNT) * sizeof(uint64_t)));
+    cnt_to = ctx->h_read;
+    bins_to = reinterpret_cast<int64_t*>(ctx->h_read + MC_NCOUNT);
+  }
+  MC_TRY_CUDA(cudaMemcpyAsync(bins_to, tally->d_bins + p.tally_offset, slots * sizeof(int64_t),
                               cudaMemcpyDeviceToHost, s));
-  MC_TRY_CUDA(cudaMemcpyAsync(cnt.data(), tally->d_counts + (size_t)problem * MC_NCOUNT,
-                              MC_NCOUNT * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+  MC_TRY_CUDA(cudaMemcpyAsync(cnt_to, tally->d_counts + (size_t)problem * MC_NCOUNT, MC_NCOUNT * sizeof(uint64_t),
+                              cudaMemcpyDeviceToHost, s));
   MC_TRY_CUDA(cudaStreamSynchronize(s));
+  if (bins_to != raw.data()) {
+    std::memcpy(raw.data(), bins_to, slots * sizeof(int64_t));
+    std::memcpy(cnt.data(), cnt_to, MC_NCOUNT * sizeof(uint64_t));
+  }
   if (h_raw) std::memcpy(h_raw, raw.data(), slots * sizeof(int64_t));
   if (h_counts) std::memcpy(h_counts, cnt.data(), MC_NCOUNT * sizeof(uint64_t));
 

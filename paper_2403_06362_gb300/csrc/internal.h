@@ -72,6 +72,8 @@ constexpr bool kSlabAggDefault = false;
 constexpr bool kBoxAggDefault = false;
 constexpr bool kPulseAggDefault = false;
 
+constexpr uint64_t kReadSlots = 1u << 16;  // tally slots mc_tally_read stages in page-locked memory (512 KiB)
+
 // Instantiated launch graphs of the history schedule, keyed by launch shape.
 struct GraphCache {
   std::unordered_map<uint64_t, cudaGraphExec_t> m;
@@ -102,6 +104,8 @@ struct mc_ctx {
   // Event-based schedule: particle bank and a pinned completion flag.
   mci::DeviceBuf bank;
   unsigned int* h_done = nullptr;
+  // mc_tally_read: pinned counts and slots of a small tally.
+  uint64_t* h_read = nullptr;
   // Box transport: two banks of split children and a pinned count.
   mci::DeviceBuf children;
   unsigned long long* h_count = nullptr;
