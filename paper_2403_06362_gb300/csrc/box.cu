@@ -105,8 +105,8 @@ enum LaneState : int {
 // makes per pass.  (Flat around these values: 3 to 8 lanes and 4 to 8 pieces
 // are within 5 %; a pass makes 25.5 flights of 2.8 pieces each, at 12.7 lanes
 // per piece, and refills every sixth time.)
-constexpr int kRefillMin = 3;
-constexpr int kWalkSteps = 5;
+template <typename T> constexpr int kRefillMin = sizeof(T) == 4 ? 3 : 4;
+template <typename T> constexpr int kWalkSteps = sizeof(T) == 4 ? 5 : 4;
 constexpr uint32_t kCountProbs = 16;  // problems whose counters a block keeps in shared memory
 
 // Bound by integer issue (fp32: 70 % of the issue slots at 15 lanes per
@@ -119,30 +119,29 @@ constexpr uint32_t kCountProbs = 16;  // problems whose counters a block keeps i
 // when it ends.  Four blocks per SM in fp32 (64 registers: 17.1 ms for 10^7
 // histories against 17.9 with three), three in fp64 (80: 16.0 ms for
 // 3 * 10^6 against 16.2 with four).
-template <int M, typename T, bool AGG>
+template <int M, typename T, bool AGG, bool ONE>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) box_history_kernel(const BoxArgs a) {
   __shared__ mcd::Affine tab[64];
   // A single problem's record is read on every flight: keep it in shared memory.
-  __shared__ __align__(16) unsigned char s_prob[sizeof(BoxDev)];
+  __shared__ __align__(16) unsigned char s_prob[ONE ? sizeof(BoxDev) : 16];
   // fp64, one problem: its mesh planes, read on every voxel crossing
-  __shared__ double s_planes[sizeof(T) == 8 ? mcb::kMaxPlanes : 1];
+  __shared__ double s_planes[ONE && sizeof(T) == 8 ? mcb::kMaxPlanes : 1];
   __shared__ unsigned long long s_counts[kCountProbs * MC_NCOUNT];
   mcd::load_maps(a.pow2, tab);
-  const bool block_counts = a.nprob <= kCountProbs;
+  const bool block_counts = ONE || a.nprob <= kCountProbs;
   if (block_counts)
     for (uint32_t i = threadIdx.x; i < a.nprob * MC_NCOUNT; i += blockDim.x) s_counts[i] = 0ull;
-  if (a.nprob == 1) {
+  if constexpr (ONE) {
     const uint64_t* src = reinterpret_cast<const uint64_t*>(a.probs);
     uint64_t* dst = reinterpret_cast<uint64_t*>(s_prob);
     for (uint32_t i = threadIdx.x; i < sizeof(BoxDev) / 8; i += blockDim.x) dst[i] = src[i];
   }
   __syncthreads();
-  const BoxDev* probs = a.nprob == 1 ? reinterpret_cast<const BoxDev*>(s_prob) : a.probs;
-  const double* planes = nullptr;
-  if (sizeof(T) == 8 && a.nprob == 1) {
+  const BoxDev* const probs = ONE ? reinterpret_cast<const BoxDev*>(s_prob) : a.probs;
+  const double* const planes = ONE && sizeof(T) == 8 ? s_planes : nullptr;
+  if constexpr (ONE && sizeof(T) == 8) {
     for (uint32_t j = threadIdx.x; j <= probs->mesh; j += blockDim.x) s_planes[j] = mcb::plane_of(*probs, (int)j);
     __syncthreads();
-    planes = s_planes;
   }
   unsigned long long* const counts = block_counts ? s_counts : a.counts;
   const unsigned kFull = 0xffffffffu;
@@ -153,7 +152,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) box_history_kerne
   uint64_t pool_next = 0, pool_end = 0;
   bool more = true, primary = false;
   int state = kDead, outcome = 0;
-  const BoxDev* P = probs;
+  const BoxDev* P = probs;  // (ONE: never changes, nor does pi)
   uint32_t pi = 0, ncoll = 0;
   mcs::Rng<M> r{0ull, 0ull};
   mcb::Part<T> q{};
@@ -164,7 +163,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) box_history_kerne
     // New items once enough lanes wait for one: a refill (seed, source draws,
     // record loads) costs the warp the same for one lane as for many.
     unsigned dead = __ballot_sync(kFull, state == kDead);
-    if (more && (__popc(dead) >= kRefillMin || dead == kFull)) {
+    if (more && (__popc(dead) >= kRefillMin<T> || dead == kFull)) {
       while (dead != 0u && more) {
         if (pool_next >= pool_end) {
           unsigned long long b0 = 0;
@@ -180,8 +179,10 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) box_history_kerne
           const uint64_t item = pool_next + rank;
           if (a.child_in == nullptr) {
             gi = a.range_begin + item;
-            pi = a.nprob == 1 ? 0u : find_box(a.probs, a.nprob, gi);
-            P = probs + pi;
+            if constexpr (!ONE) {
+              pi = find_box(a.probs, a.nprob, gi);
+              P = probs + pi;
+            }
             const uint64_t id = gi - P->hist_begin;
             const uint64_t nvox = (uint64_t)P->mesh * P->mesh * P->mesh;
             tbase = P->tally_offset;
@@ -196,14 +197,17 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) box_history_kerne
             state = kSource;
           } else {
             const ChildRec& c = a.child_in[item];
-            pi = c.prob;
-            P = probs + pi;
+            if constexpr (!ONE) {
+              pi = c.prob;
+              P = probs + pi;
+            }
             tbase = c.tbase;
             r = mcs::Rng<M>{c.rng, 0ull};
             mcb::child_state<T>(c, q);
             primary = false;
             state = kInverse;
           }
+          mcb::walk_locate<T>(*P, q, k);
           events = 0;
           ncoll = 0;
         }
@@ -258,11 +262,12 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) box_history_kerne
     // The tallies, at most kWalkSteps pieces per lane: the number of pieces
     // varies from lane to lane, and a lane with many goes on in the next
     // pass while the others take their next flight.
-    for (int i = 0; i < kWalkSteps; ++i) {
+    for (int i = 0; i < kWalkSteps<T>; ++i) {
       if (__ballot_sync(kFull, state == kWalking) == 0u) break;
       if (state == kWalking && mcb::walk_step<T>(*P, q, k, a.tally + tbase, planes, AGG)) state = kArrived;
     }
     if (state == kArrived) {
+      mcb::walk_leave<T>(*P, q, k);
       mcb::arrive<T>(q, k.L, outcome);
       state = outcome == mcb::kBoxCollide ? kCollided : (outcome == mcb::kBoxLeak ? kEnded : kReady);
     }
@@ -302,9 +307,20 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) box_history_kerne
 
 namespace {
 
+// One problem, as most launches have (an instantiation of its own: the record
+// and the planes at fixed places in shared memory), or several.
+template <int M, typename T, bool AGG>
+void (*box_kernel_for(bool one))(const BoxArgs) {
+  if constexpr (M == 63 && !AGG) {
+    if (one) return box_history_kernel<M, T, AGG, true>;
+  }
+  (void)one;
+  return box_history_kernel<M, T, AGG, false>;
+}
+
 template <int M, typename T, bool AGG>
 int launch_box_gen(const BoxArgs& a, int block, int bps, int num_sms, cudaStream_t s) {
-  auto k = box_history_kernel<M, T, AGG>;
+  auto k = box_kernel_for<M, T, AGG>(a.nprob == 1);
   int per_sm = bps;
   if (per_sm <= 0) {
     int st = mci::cuda_status(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, 0),

@@ -360,14 +360,14 @@ struct Walk {
   uint32_t slot;
 };
 
-// The voxel of coordinate p on one axis and, as seen by direction u, the
-// next plane j and its distance tn.  The looked-up voxel is within one of the
-// right one; the exact plane comparisons correct it, and put a particle on a plane on
+// The voxel of coordinate p on one axis, from a guess i in [0, nm), and, as
+// seen by direction u, the next plane j and its distance tn.  A looked-up guess
+// is within one of the right voxel, the voxel the last flight ended in mostly
+// right; the exact plane comparisons correct it, and put a particle on a plane on
 // the side it flies to, in a rarely taken branch.
 template <typename T>
-__device__ __forceinline__ int walk_axis(const BoxDev& b, const double* tab, int nm, T p, T u, T inv, int& j, T& tn) {
-  int i = voxel_guess<T>(b, p);
-  i = i < 0 ? 0 : (i >= nm ? nm - 1 : i);
+__device__ __forceinline__ int walk_axis(const BoxDev& b, const double* tab, int nm, int i, T p, T u, T inv, int& j,
+                                         T& tn) {
   T lo = plane<T>(b, tab, i), hi = plane<T>(b, tab, i + 1);
   const bool neg = lt0(u);
   if ((i > 0 && !ltn(lo, p)) || (i + 1 < nm && !ltn(p, hi))) {
@@ -383,11 +383,35 @@ __device__ __forceinline__ int walk_axis(const BoxDev& b, const double* tab, int
 }
 
 template <typename T>
+__device__ __forceinline__ int guess_axis(const BoxDev& b, int nm, T p) {
+  const int i = voxel_guess<T>(b, p);
+  return i < 0 ? 0 : (i >= nm ? nm - 1 : i);
+}
+
+// k.j0 .. k.j2: guesses of the particle's voxel, from its position ...
+template <typename T>
+__device__ __forceinline__ void walk_locate(const BoxDev& b, const Part<T>& q, Walk<T>& k) {
+  const int nm = (int)b.mesh;
+  k.j0 = guess_axis<T>(b, nm, q.p[0]);
+  k.j1 = guess_axis<T>(b, nm, q.p[1]);
+  k.j2 = guess_axis<T>(b, nm, q.p[2]);
+}
+
+// ... or, at the end of a walk in direction u, from its next planes.
+template <typename T>
+__device__ __forceinline__ void walk_leave(const BoxDev& b, const Part<T>& q, Walk<T>& k) {
+  const int top = (int)b.mesh - 1;
+  k.j0 = max(0, min(top, k.j0 - (lt0(q.u[0]) ? 0 : 1)));
+  k.j1 = max(0, min(top, k.j1 - (lt0(q.u[1]) ? 0 : 1)));
+  k.j2 = max(0, min(top, k.j2 - (lt0(q.u[2]) ? 0 : 1)));
+}
+
+template <typename T>
 __device__ __forceinline__ void walk_begin(const BoxDev& b, const Part<T>& q, T L, const double* tab, Walk<T>& k) {
   const int nm = (int)b.mesh;
-  const int i0 = walk_axis<T>(b, tab, nm, q.p[0], q.u[0], q.inv[0], k.j0, k.tn0);
-  const int i1 = walk_axis<T>(b, tab, nm, q.p[1], q.u[1], q.inv[1], k.j1, k.tn1);
-  const int i2 = walk_axis<T>(b, tab, nm, q.p[2], q.u[2], q.inv[2], k.j2, k.tn2);
+  const int i0 = walk_axis<T>(b, tab, nm, k.j0, q.p[0], q.u[0], q.inv[0], k.j0, k.tn0);
+  const int i1 = walk_axis<T>(b, tab, nm, k.j1, q.p[1], q.u[1], q.inv[1], k.j1, k.tn1);
+  const int i2 = walk_axis<T>(b, tab, nm, k.j2, q.p[2], q.u[2], q.inv[2], k.j2, k.tn2);
   k.slot = (uint32_t)((i2 * nm + i1) * nm + i0);  // mesh <= 1024: below 2^30
   k.t = T(0);
   k.L = L;
@@ -509,6 +533,7 @@ __device__ __forceinline__ int box_flight(const BoxDev& b, mcs::Rng<M>& r, const
   T len;
   const int o = flight_length<M, T>(b, r, l, q, len);
   Walk<T> k;
+  walk_locate<T>(b, q, k);
   walk_begin<T>(b, q, len, tab, k);
   while (!walk_step<T>(b, q, k, base, tab, agg)) {}
   arrive<T>(q, len, o);
