@@ -505,6 +505,7 @@ int make_slab_launch(mc_ctx* ctx, const mc_lcg* lcg, const mc_problem* problems,
   mci::SlabLaunch L{};
   L.single_n_bins = n_problems == 1 ? problems[0].n_bins : 0u;
   for (uint32_t i = 0; i < n_problems; ++i) L.max_n_bins = std::max(L.max_n_bins, problems[i].n_bins);
+  L.walk_pieces = mci::slab_walk_pieces(problems, n_problems);
   L.d_probs = ctx->problems.ptr;
   L.d_tables = slab_tables_of(ctx, n_problems);
   L.n_problems = n_problems;
@@ -567,6 +568,7 @@ int run_slab_graph(mc_ctx* ctx, const mc_lcg* lcg, const mc_problem* problems, u
   key = fnv(key, &L.block, sizeof L.block);
   key = fnv(key, &L.single_n_bins, sizeof L.single_n_bins);
   key = fnv(key, &L.max_n_bins, sizeof L.max_n_bins);
+  key = fnv(key, &L.walk_pieces, sizeof L.walk_pieces);
   if (!ctx->graphs) ctx->graphs = new mci::GraphCache();
   auto it = ctx->graphs->m.find(key);
   cudaGraphExec_t exec = nullptr;

@@ -168,6 +168,7 @@ extern "C" MC_API int mc_transport_run_static(const mc_lcg* lcg, const mc_proble
   L.smem_slots = slots;
   L.single_n_bins = n_problems == 1 ? problems[0].n_bins : 0u;
   for (uint32_t i = 0; i < n_problems; ++i) L.max_n_bins = std::max(L.max_n_bins, problems[i].n_bins);
+  L.walk_pieces = mci::slab_walk_pieces(problems, n_problems);
   L.f32 = cfg->precision == MC_FP32_GUARDED;
   L.block = cfg->block ? (int)cfg->block : mci::slab_default_block(L.total, L.chunk, slot->num_sms);
   L.blocks_per_sm = (int)cfg->blocks_per_sm;

@@ -177,6 +177,7 @@ struct RunArgs {
   uint32_t grab_shift;  // a warp takes at most 2^-grab_shift of the histories left at once,
   uint32_t min_grab;    // but at least min_grab
   uint32_t row_bins;    // bins of a warp's row cache (0: none; all problems fit it otherwise)
+  uint32_t walk_pieces; // of a flight's tally a lane adds per pass, after the first
   uint32_t coop_hist;   // histories the block's cooperative tail takes over (0: none)
   uint32_t coop_slots;  // its event records, a power of two
   uint32_t coop_after;  // passes of a warp after the ticket ran out before it offers its histories
@@ -537,7 +538,9 @@ __device__ __forceinline__ void coop_tally(const CoopHist& H, const SlabDev& p, 
       return;
     }
     const double xe = f == mcs::kLeakHi ? p.L : (f == mcs::kLeakLo ? 0.0 : dval(rec[0]));
-    mcs::walk64(p, x, xe, !mcs::nn_lt(xe, x), w, sk, j);
+    const mcs::Walk64 k{xe, w, !mcs::nn_lt(xe, x)};
+    if (mcs::walk_first(p, x, k, sk, j))
+      while (mcs::walk_next(p, k, sk, j)) {}
   } else {
     const unsigned long long to = rec[0];
     const float xf = lo_of(from), xlo = hi_of(from), muf = hi_of(rec[1]);
@@ -683,6 +686,9 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
   mcs::SlabParticle q{};
   mcs::Sink sink{nullptr, s_edges, s_widths, AGG};
   uint64_t gi = 0, events = 0;
+  typename mcs::WalkOf<F32>::type wk{};  // the rest of the current flight's tally, while `walking`
+  bool walking = false;
+  int outcome = mcs::kContinue;          // of the history's last event
   uint32_t after = 0;  // passes since the ticket ran out
   const uint32_t my_row = row0 + (threadIdx.x >> 5) * a.row_bins;
   unsigned long long* row_of = nullptr;  // the tally row the warp's cache accumulates
@@ -736,6 +742,7 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
         x = r.x;
         q.j = mcs::locate<F32>(*P, q, sink);
         events = 0;
+        outcome = mcs::kContinue;
         ++lc.src;
         alive = true;
       }
@@ -780,6 +787,15 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
       const uint32_t mine = lane < 16u ? vl[lane] : 0u;
       const bool go = __reduce_add_sync(kFull, mine) <= a.coop_hist || *(volatile uint32_t*)&s_go != 0u;
       if (__any_sync(kFull, go)) {
+        // between two events: tallies under way are completed first, and the
+        // histories that they were the end of
+        while (walking) walking = mcs::walk_next(*P, wk, sink, q.j);
+        if (alive && outcome != mcs::kContinue) {
+          end_history(TailArgs{a.hist_state, a.hist_draws, a.counts, a.lcg, a.event_cap}, a.probs, x, *P, gi, events,
+                      outcome, a.nprob == 1 ? s_exceed : nullptr, lc);
+          alive = false;
+        }
+        dead = __ballot_sync(kFull, !alive);
         uint32_t base = 0;
         if (lane == 0) {
           *(volatile uint32_t*)&s_go = 1u;
@@ -805,17 +821,24 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
         break;
       }
     }
-    if (alive) {
-      int outcome = -1;  // event cap
+    if (alive && !walking) {
+      outcome = -1;  // event cap
       if (events != a.event_cap) {
         ++events;
-        outcome = mcs::slab_event<M, F32>(*P, x, l, q, sink);
+        outcome = mcs::slab_event<M, F32>(*P, x, l, q, sink, wk, walking);
       }
-      if (outcome != mcs::kContinue) {
-        end_history(TailArgs{a.hist_state, a.hist_draws, a.counts, a.lcg, a.event_cap}, a.probs, x, *P, gi, events, outcome,
-                    a.nprob == 1 ? s_exceed : nullptr, lc);
-        alive = false;
-      }
+    }
+    // The other pieces of the tallies, walk_pieces per lane at most: a lane
+    // whose flight crosses more bins goes on in the next pass, while the others
+    // take their next event.
+    for (uint32_t i = 0; i < a.walk_pieces; ++i) {
+      if (__ballot_sync(kFull, walking) == 0u) break;
+      if (walking) walking = mcs::walk_next(*P, wk, sink, q.j);
+    }
+    if (alive && !walking && outcome != mcs::kContinue) {
+      end_history(TailArgs{a.hist_state, a.hist_draws, a.counts, a.lcg, a.event_cap}, a.probs, x, *P, gi, events, outcome,
+                  a.nprob == 1 ? s_exceed : nullptr, lc);
+      alive = false;
     }
   }
   lc.flush_warp(a.counts, a.probs);
@@ -1023,6 +1046,20 @@ uint64_t slab_table_doubles(const mc_problem* src, uint32_t n) {
   return t;
 }
 
+// Pieces per pass from the edges an average flight crosses, (1/2) bins per
+// mean free path (averaged over the histories): as many as most flights need.
+// slab_long (1/2): 1 / 2 / 3 / all of them 141 / 148 / 159 / 163 ms; 256
+// problems (1.0), fp32: 9.4 / 8.7 / 9.0 / 10.0 ms.
+uint32_t slab_walk_pieces(const mc_problem* src, uint32_t n) {
+  double bins = 0.0, paths = 0.0;
+  for (uint32_t i = 0; i < n; ++i) {
+    bins += (double)src[i].n_histories * src[i].n_bins;
+    paths += (double)src[i].n_histories * src[i].L * src[i].sigma_t;
+  }
+  const double crossed = 0.5 * bins / std::max(paths, 1e-300);
+  return crossed < 0.75 ? 1u : crossed < 2.0 ? 2u : crossed < 6.0 ? 3u : 4u;
+}
+
 int slab_history_launch(const SlabLaunch& L, cudaStream_t s) {
   RunArgs a{};
   a.probs = static_cast<const SlabDev*>(L.d_probs);
@@ -1071,6 +1108,7 @@ int slab_history_launch(const SlabLaunch& L, cudaStream_t s) {
   // problems in one order, and their atomics met at a few lines of L2 (256
   // problems: fp32 16.6 -> 11.0 ms, fp64 21.2 -> 17.0 ms).
   a.row_bins = L.max_n_bins;
+  a.walk_pieces = L.walk_pieces;
   a.order = mcs::Order{L.d_order, L.d_order_begin};
   if (L.tally_agg) {
     if (L.lcg.m == 63) return launch_history_m<63, true>(a, L.f32, L.block, L.blocks_per_sm, L.num_sms, s);

@@ -190,26 +190,27 @@ __device__ __forceinline__ int bin_of(const SlabDev& p, const Sink& s, double x)
 // (hi - lo) * (1/|mu|).  The walk starts from x's bin j, goes the way the
 // particle flies and leaves j at the bin of xe, where the next flight starts:
 // no bin is ever looked up.  (At an edge either neighbour will do for j: the
-// piece in the other one has length zero and adds nothing.)  The first piece,
-// to xe or to the first edge, and the last, from the last edge to xe, take an
-// fp64 difference; whole bins take their length from the width table.
-__device__ __forceinline__ void walk64(const SlabDev& p, double x, double xe, bool fwd, double w_fix, const Sink& s,
-                                       int& j) {
-  const int up = fwd ? 1 : 0, dj = fwd ? 1 : -1;
-  double e = edge_of(p, s, j + up);
-  bool last = fwd ? !nn_lt(e, xe) : !nn_lt(xe, e);
-  s.add(j, mcx::llrint_nonneg(__dmul_rn(mcx::abs_bits(__dsub_rn(last ? xe : e, x)), w_fix)));
-  if (last) return;
-  for (;;) {
-    j += dj;
-    const double e2 = edge_of(p, s, j + up);
-    last = fwd ? !nn_lt(e2, xe) : !nn_lt(xe, e2);
-    if (last) break;
-    const double w = s.widths ? s.widths[j] : mcx::abs_bits(__dsub_rn(e2, e));
-    s.add(j, mcx::llrint_nonneg(__dmul_rn(w, w_fix)));
-    e = e2;
-  }
-  s.add(j, mcx::llrint_nonneg(__dmul_rn(mcx::abs_bits(__dsub_rn(xe, e)), w_fix)));
+// piece in the other one has length zero and adds nothing.)  It goes piece by
+// piece, so that a caller can stop between two: walk_first adds the piece to
+// xe or to the first edge, walk_next the next one, to xe or a whole bin with
+// its length from the width table; both return whether pieces are left.
+struct Walk64 {
+  double xe, w;  // the end, and 2^32 / |mu|
+  bool fwd;
+};
+__device__ __forceinline__ bool walk_first(const SlabDev& p, double x, const Walk64& k, const Sink& s, int j) {
+  const double e = edge_of(p, s, j + (k.fwd ? 1 : 0));
+  const bool last = k.fwd ? !nn_lt(e, k.xe) : !nn_lt(k.xe, e);
+  s.add(j, mcx::llrint_nonneg(__dmul_rn(mcx::abs_bits(__dsub_rn(last ? k.xe : e, x)), k.w)));
+  return !last;
+}
+__device__ __forceinline__ bool walk_next(const SlabDev& p, const Walk64& k, const Sink& s, int& j) {
+  j += k.fwd ? 1 : -1;
+  const double e0 = edge_of(p, s, j + (k.fwd ? 0 : 1)), e1 = edge_of(p, s, j + (k.fwd ? 1 : 0));
+  const bool last = k.fwd ? !nn_lt(e1, k.xe) : !nn_lt(k.xe, e1);
+  const double len = !last && s.widths ? s.widths[j] : mcx::abs_bits(__dsub_rn(last ? k.xe : e1, e0));
+  s.add(j, mcx::llrint_nonneg(__dmul_rn(len, k.w)));
+  return !last;
 }
 
 // Exact llrint((double)v * 2^32) for a finite float v >= 0 (scaling by 2^32
@@ -269,22 +270,27 @@ __device__ __forceinline__ int bin_of_pair(const SlabDev& p, float h, float l) {
   return j;
 }
 
-// walk64's counterpart: from the pair (xh + xl) in bin j to (eh + el).
-__device__ __forceinline__ void walk32(const SlabDev& p, float xh, float xl, float eh, float el, bool fwd, float w_mu,
-                                       const Sink& s, int& j) {
-  const int up = fwd ? 1 : 0, dj = fwd ? 1 : -1;
-  for (;;) {
-    const float e = slab_edge_f(p, j + up);
-    // (eh, el) lies beyond the edge?
-    const bool last = fwd ? !(eh > e || (eh == e && el > 0.0f)) : !(eh < e || (eh == e && el < 0.0f));
-    const float th = last ? eh : e, tl = last ? el : 0.0f;
-    const float d = __fadd_rn(__fsub_rn(th, xh), __fsub_rn(tl, xl)), len = fwd ? d : -d;
-    if (len > 0.0f) s.add(j, fix32_from_float(__fmul_rn(len, w_mu)));
-    if (last) break;
-    xh = e;
-    xl = 0.0f;
-    j += dj;
-  }
+// The fp32 walk, to the pair (eh + el) with weight w = 1 / |mu|.
+struct Walk32 {
+  float eh, el, w;
+  bool fwd;
+};
+__device__ __forceinline__ bool walk_piece(const SlabDev& p, float xh, float xl, const Walk32& k, const Sink& s, int j) {
+  const float e = slab_edge_f(p, j + (k.fwd ? 1 : 0));
+  // the end lies beyond the edge?
+  const bool last = k.fwd ? !(k.eh > e || (k.eh == e && k.el > 0.0f)) : !(k.eh < e || (k.eh == e && k.el < 0.0f));
+  const float th = last ? k.eh : e, tl = last ? k.el : 0.0f;
+  const float d = __fadd_rn(__fsub_rn(th, xh), __fsub_rn(tl, xl)), len = k.fwd ? d : -d;
+  if (len > 0.0f) s.add(j, fix32_from_float(__fmul_rn(len, k.w)));
+  return !last;
+}
+__device__ __forceinline__ bool walk_first(const SlabDev& p, float xh, float xl, const Walk32& k, const Sink& s,
+                                           int j) {
+  return walk_piece(p, xh, xl, k, s, j);
+}
+__device__ __forceinline__ bool walk_next(const SlabDev& p, const Walk32& k, const Sink& s, int& j) {
+  j += k.fwd ? 1 : -1;
+  return walk_piece(p, slab_edge_f(p, j + (k.fwd ? 0 : 1)), 0.0f, k, s, j);
 }
 
 __device__ __forceinline__ void point32(const SlabDev& p, float x, float d, const Sink& s) {
@@ -464,20 +470,29 @@ __device__ __forceinline__ bool leaves64(const SlabDev& p, long long mb, double 
   return (mb > 0 && !nn_lt(xn, p.L)) || (mb < 0 && __double_as_longlong(xn) <= 0);
 }
 
-// The tally of that flight, from x's bin j (left at the bin of xn): the track
-// from x to xn, to the face it leaves through, or (mu = 0) the whole distance
-// d in the bin holding x.  Every kind of flight ends in the one call of the
-// bin walk, with its end chosen first, so that the lanes of a warp whose
-// flights differ in kind still walk the bins together.
-__device__ __forceinline__ void tally64(const SlabDev& p, double x, double xn, double mu, double d, double w_mu,
-                                        int outcome, const Sink& s, int& j) {
+// The tally of that flight, from x's bin j: the track from x to xn, to the
+// face it leaves through, or (mu = 0) the whole distance d in the bin holding
+// x.  Every kind of flight ends in the one walk, with its end chosen first, so
+// that the lanes of a warp whose flights differ in kind still walk the bins
+// together.  begin_tally adds the first piece and returns whether walk_next
+// has more (which leaves j at the bin of xn); tally64 adds them all.
+__device__ __forceinline__ bool begin_tally(const SlabDev& p, double x, double xn, double mu, double d, double w_mu,
+                                            int outcome, const Sink& s, int& j, Walk64& k) {
   const long long mb = __double_as_longlong(mu);
   if (outcome == kCollide && mb == 0) {
     s.add(bin_of(p, s, x), mcx::fix32_nonneg(d));
-    return;
+    return false;
   }
-  const double xe = outcome == kLeakHi ? p.L : (outcome == kLeakLo ? 0.0 : xn);
-  walk64(p, x, xe, mb > 0, w_mu, s, j);
+  k.xe = outcome == kLeakHi ? p.L : (outcome == kLeakLo ? 0.0 : xn);
+  k.w = w_mu;
+  k.fwd = mb > 0;
+  return walk_first(p, x, k, s, j);
+}
+__device__ __forceinline__ void tally64(const SlabDev& p, double x, double xn, double mu, double d, double w_mu,
+                                        int outcome, const Sink& s, int& j) {
+  Walk64 k;
+  if (begin_tally(p, x, xn, mu, d, w_mu, outcome, s, j, k))
+    while (walk_next(p, k, s, j)) {}
 }
 
 // The fp32 path's position step: xn + xnlo = (xf + xlo) + d muf, with pr =
@@ -529,20 +544,35 @@ __device__ __forceinline__ int advance32(const SlabDev& p, float xf, float xlo, 
   return leak_hi ? kLeakHi : (leak_lo ? kLeakLo : kCollide);
 }
 
-// tally64's counterpart for the fp32 path, on position pairs.  A pair's
-// last rounding can move a flight of next to no length backwards; its bin is
-// then looked up again.
+// Their counterparts for the fp32 path, on position pairs.  A pair's last
+// rounding can move a flight of next to no length backwards; its bin is then
+// looked up again.
+__device__ __forceinline__ bool begin_tally(const SlabDev& p, float xf, float xlo, float xn, float xnlo, float muf,
+                                            float d, float wf, int outcome, const Sink& s, int& j, Walk32& k) {
+  if (outcome == kCollide && muf == 0.0f) {
+    point32(p, xf, d, s);
+    return false;
+  }
+  k.eh = xn;
+  k.el = xnlo;
+  if (outcome == kLeakHi) { k.eh = p.L_f; k.el = 0.0f; }
+  else if (outcome == kLeakLo) { k.eh = 0.0f; k.el = 0.0f; }
+  k.w = wf;
+  k.fwd = muf > 0.0f;
+  const bool more = walk_first(p, xf, xlo, k, s, j);
+  const bool less = xn < xf || (xn == xf && xnlo < xlo), beyond = xn > xf || (xn == xf && xnlo > xlo);
+  if (outcome == kCollide && (k.fwd ? less : beyond)) j = bin_of_pair(p, xn, xnlo);
+  return more;
+}
 __device__ __forceinline__ void tally32(const SlabDev& p, float xf, float xlo, float xn, float xnlo, float muf,
                                         float d, float wf, int outcome, const Sink& s, int& j) {
-  if (outcome == kCollide && muf == 0.0f) { point32(p, xf, d, s); return; }
-  float eh = xn, el = xnlo;
-  if (outcome == kLeakHi) { eh = p.L_f; el = 0.0f; }
-  else if (outcome == kLeakLo) { eh = 0.0f; el = 0.0f; }
-  const bool fwd = muf > 0.0f;
-  walk32(p, xf, xlo, eh, el, fwd, wf, s, j);
-  const bool less = xn < xf || (xn == xf && xnlo < xlo), more = xn > xf || (xn == xf && xnlo > xlo);
-  if (outcome == kCollide && (fwd ? less : more)) j = bin_of_pair(p, xn, xnlo);
+  Walk32 k;
+  if (begin_tally(p, xf, xlo, xn, xnlo, muf, d, wf, outcome, s, j, k))
+    while (walk_next(p, k, s, j)) {}
 }
+
+template <bool F32> struct WalkOf { using type = Walk64; };
+template <> struct WalkOf<true> { using type = Walk32; };
 
 // The bin of the particle's position, where none is known from a flight.
 template <bool F32>
@@ -596,9 +626,11 @@ __device__ __forceinline__ int slab_collide(const SlabDev& p, Rng<M>& r, const m
 // not the event comes to use them: the two chains of integer operations
 // (the logarithm, the reciprocal) are independent and fill each other's
 // latencies.  x moves on by the draws the event takes.
+// The tally gets its first piece; `more` says whether k has others, without
+// which q.j is not yet the particle's bin.
 template <int M, bool F32>
 __device__ __forceinline__ int slab_event(const SlabDev& p, uint64_t& x, const mcd::Lcg& l, SlabParticle& q,
-                                          const Sink& s) {
+                                          const Sink& s, typename WalkOf<F32>::type& k, bool& more) {
   const uint64_t x1 = mcd::lcg_step(x, l.g, l.c), x2 = mcd::lcg_step(x1, l.g, l.c), x3 = mcd::lcg_step(x2, l.g, l.c);
   const uint64_t n = mcd::u53<M>(x1, l.m);
   SlabParticle nq = q;
@@ -608,15 +640,16 @@ __device__ __forceinline__ int slab_event(const SlabDev& p, uint64_t& x, const m
     asm volatile("" : "+d"(nq.mu), "+d"(nq.w_mu));  // not moved to its use after the tally
     const double d = __dmul_rn(mclog::neglog1m_n(n), p.inv_st);
     f = advance64(p, q.x, q.mu, __dmul_rn(d, q.mu), nq.x);
-    tally64(p, q.x, nq.x, q.mu, d, q.w_mu, f, s, nq.j);
+    more = begin_tally(p, q.x, nq.x, q.mu, d, q.w_mu, f, s, nq.j, k);
   } else {
     asm volatile("" : "+f"(nq.muf), "+f"(nq.wf));
     const float d = flight_f32(n) * p.inv_st_f;
     const float pr = __fmul_rn(d, q.muf);
     const float pe = __fmaf_rn(d, q.muf, -pr);
     f = advance32(p, q.xf, q.xlo, q.muf, pr, pe, [n] { return n; }, nq.xf, nq.xlo);
-    tally32(p, q.xf, q.xlo, nq.xf, nq.xlo, q.muf, d, q.wf, f, s, nq.j);
+    more = begin_tally(p, q.xf, q.xlo, nq.xf, nq.xlo, q.muf, d, q.wf, f, s, nq.j, k);
   }
+  q.j = nq.j;
   if (f != kCollide) {
     x = x1;
     return f;

@@ -22,6 +22,7 @@ struct SlabLaunch {
   uint32_t smem_slots;         // 0 = global atomics; else slots staged in smem
   uint32_t single_n_bins;      // n_bins of the problem when n_problems == 1
   uint32_t max_n_bins = 0;     // the most bins of any problem
+  uint32_t walk_pieces = 2;    // slab_walk_pieces
   const void* d_tables = nullptr;  // per-problem edge and width tables (nullable; see slab_prep)
   bool f32;
   int block, blocks_per_sm, num_sms;
@@ -53,6 +54,7 @@ inline void slab_order_ptrs(void* d_order, uint32_t n, const uint32_t** order, c
   *begin = reinterpret_cast<const uint64_t*>(*order + ((n + 1u) & ~1u));
 }
 uint64_t slab_table_doubles(const mc_problem* src, uint32_t n);
+uint32_t slab_walk_pieces(const mc_problem* src, uint32_t n);
 int slab_history_launch(const SlabLaunch& L, cudaStream_t s);
 
 // Event-based schedule (slab_event.cu): bank of `cap` particles in d_bank
