@@ -400,6 +400,11 @@ MC_API int mc_ctx_create(mc_ctx** out, int device) {
     delete c;
     return st;
   }
+  // (without it tallies are read into pageable memory)
+  if (cudaMallocHost(&c->h_read, (mci::kReadSlots + MC_NCOUNT) * sizeof(uint64_t)) != cudaSuccess) {
+    cudaGetLastError();
+    c->h_read = nullptr;
+  }
   *out = c;
   return MC_OK;
 }
@@ -554,7 +559,7 @@ int run_slab_graph(mc_ctx* ctx, const mc_lcg* lcg, const mc_problem* problems, u
                         tally->d_hist_draws};
   key = fnv(key, ptrs, sizeof ptrs);
   key = fnv(key, cfg, sizeof *cfg);
-  key = fnv(key, &ctx->limits, sizeof ctx->limits);  // the lock bound is a kernel argument
+  key = fnv(key, &ctx->limits, sizeof ctx->limits);  // they change the launch's arguments
   key = fnv(key, lcg, sizeof *lcg);
   key = fnv(key, &n_problems, sizeof n_problems);
   key = fnv(key, &bytes, sizeof bytes);
@@ -928,11 +933,12 @@ MC_API int mc_tally_read(mc_ctx* ctx, const mc_problem* problems, uint32_t probl
   std::vector<uint64_t> cnt(MC_NCOUNT);
   // A small tally comes back through page-locked memory of the context: a copy
   // into pageable memory waits for the stream by itself and is staged by the
-  // driver, 10 us each (10^4 histories run and read: 78 -> 67 us).
+  // driver, 10 us each (10^4 histories run and read: 78 -> 67 us).  A thread
+  // that finds another one reading does without.
   int64_t* bins_to = raw.data();
   uint64_t* cnt_to = cnt.data();
-  if (slots <= mci::kReadSlots) {
-    if (!ctx->h_read) MC_TRY_CUDA(cudaMallocHost(&ctx->h_read, (mci::kReadSlots + MC_NCOUNT) * sizeof(uint64_t)));
+  std::unique_lock<std::mutex> reading(ctx->read_lock, std::defer_lock);
+  if (ctx->h_read && slots <= mci::kReadSlots && reading.try_lock()) {
     cnt_to = ctx->h_read;
     bins_to = reinterpret_cast<int64_t*>(ctx->h_read + MC_NCOUNT);
   }

@@ -4,6 +4,7 @@
 
 #include <cstdint>
 #include <cstdio>
+#include <mutex>
 #include <string>
 #include <unordered_map>
 #include <vector>
@@ -104,8 +105,10 @@ struct mc_ctx {
   // Event-based schedule: particle bank and a pinned completion flag.
   mci::DeviceBuf bank;
   unsigned int* h_done = nullptr;
-  // mc_tally_read: pinned counts and slots of a small tally.
+  // mc_tally_read: pinned counts and slots of a small tally, of one reader at
+  // a time.
   uint64_t* h_read = nullptr;
+  std::mutex read_lock;
   // Box transport: two banks of split children and a pinned count.
   mci::DeviceBuf children;
   unsigned long long* h_count = nullptr;

@@ -26,7 +26,7 @@ struct SlabLaunch {
   const void* d_tables = nullptr;  // per-problem edge and width tables (nullable; see slab_prep)
   bool f32;
   int block, blocks_per_sm, num_sms;
-  uint32_t pool_lock_attempts = 1u << 20;  // compaction-pool lock (mc_limits)
+  uint32_t pool_lock_attempts = 1u << 20;  // 0: no cooperative tail (mc_limits)
   // processing order of several problems (slab_prep's d_order area; null: id order)
   const uint32_t* d_order = nullptr;
   const uint64_t* d_order_begin = nullptr;
