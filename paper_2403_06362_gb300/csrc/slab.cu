@@ -611,6 +611,16 @@ constexpr uint32_t kMaxRowBins = 256;  // of a warp's row cache (2 KiB)
 // fp32 10.9 ms against 10.6, fp64 17.3 against 15.0).
 constexpr uint32_t kIdle = 16;
 
+// Lanes still walking for which a warp makes another piece of its tallies in
+// the same pass.  A tally in shared memory is a single problem's, or small:
+// one, and slab_walk_pieces the limit (with 8 lanes 300 000 histories of 9
+// flights took 260 us instead of 253).  Otherwise problems of many kinds share
+// the warps and no number of pieces suits all: no limit but 8 lanes (256
+// problems, against two pieces: fp32 8.72 -> 8.55 ms, fp64 13.1 -> 12.4 ms; 4,
+// 6 and 12 lanes within 2 %).
+template <bool SMEM> constexpr int kWalkMin = SMEM ? 1 : 8;
+constexpr uint32_t kWalkNoLimit = ~0u;
+
 // The ticket positions of one problem: begin + id for its history id.
 struct Span {
   uint64_t begin;
@@ -828,11 +838,11 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
         outcome = mcs::slab_event<M, F32>(*P, x, l, q, sink, wk, walking);
       }
     }
-    // The other pieces of the tallies, walk_pieces per lane at most: a lane
-    // whose flight crosses more bins goes on in the next pass, while the others
-    // take their next event.
+    // The other pieces of the tallies, walk_pieces per lane at most and, after
+    // the first, only for kWalkMin lanes together: a lane whose flight crosses
+    // more bins goes on in the next pass, while the others take their next event.
     for (uint32_t i = 0; i < a.walk_pieces; ++i) {
-      if (__ballot_sync(kFull, walking) == 0u) break;
+      if (__popc(__ballot_sync(kFull, walking)) < (i == 0u ? 1 : kWalkMin<SMEM>)) break;
       if (walking) walking = mcs::walk_next(*P, wk, sink, q.j);
     }
     if (alive && !walking && outcome != mcs::kContinue) {
@@ -1046,10 +1056,11 @@ uint64_t slab_table_doubles(const mc_problem* src, uint32_t n) {
   return t;
 }
 
-// Pieces per pass from the edges an average flight crosses, (1/2) bins per
-// mean free path (averaged over the histories): as many as most flights need.
-// slab_long (1/2): 1 / 2 / 3 / all of them 141 / 148 / 159 / 163 ms; 256
-// problems (1.0), fp32: 9.4 / 8.7 / 9.0 / 10.0 ms.
+// Pieces per pass of a run whose tally is in shared memory, from the edges an
+// average flight crosses, (1/2) bins per mean free path (averaged over the
+// histories): as many as most flights need.  slab_long (1/2): 1 / 2 / 3 / all
+// of them 141 / 148 / 159 / 163 ms; 300 000 histories of 9 flights (1.1): 264 /
+// 257 / 269 us with 1 / 2 / 3.
 uint32_t slab_walk_pieces(const mc_problem* src, uint32_t n) {
   double bins = 0.0, paths = 0.0;
   for (uint32_t i = 0; i < n; ++i) {
@@ -1108,7 +1119,7 @@ int slab_history_launch(const SlabLaunch& L, cudaStream_t s) {
   // problems in one order, and their atomics met at a few lines of L2 (256
   // problems: fp32 16.6 -> 11.0 ms, fp64 21.2 -> 17.0 ms).
   a.row_bins = L.max_n_bins;
-  a.walk_pieces = L.walk_pieces;
+  a.walk_pieces = L.smem_slots != 0u ? L.walk_pieces : kWalkNoLimit;
   a.order = mcs::Order{L.d_order, L.d_order_begin};
   if (L.tally_agg) {
     if (L.lcg.m == 63) return launch_history_m<63, true>(a, L.f32, L.block, L.blocks_per_sm, L.num_sms, s);
