@@ -875,10 +875,11 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
   }
 }
 
-// The kernel in two register budgets.  The fp32 flight fits 64 registers
-// (four blocks of 256 per SM); the fp64 flight spills there, and runs faster
-// with 80 and three blocks per SM (slab_long 240 -> 215 ms, batched 23.4 ->
-// 20.6 ms; the fp32 kernel at 80 measured batched 18.0 -> 19.8 ms).  Both
+// The kernel in two register budgets.  The fp32 flight fits 64 registers but
+// for a few spills (four blocks of 256 per SM; at 80, 256 problems took a
+// tenth longer); the fp64 flight runs fastest with 80 and three blocks per SM
+// (slab_long 156 ms, against 166 / 159 / 180 at 64 / 72 / 96, before the bin
+// walk was split: 141 ms since).  Both
 // accept blocks of up to 512 threads.
 template <int M, bool F32, bool SMEM, bool AGG>
 __global__ void __launch_bounds__(512, 2) slab_history_kernel_f32(const RunArgs a) {
@@ -892,7 +893,7 @@ __global__ void __maxnreg__(80) slab_history_kernel_f64(const RunArgs a) {
 // A run of at most a few warps per SM waits for its longest histories, not for
 // issue slots: registers to interleave an event's chains are worth more than
 // warps that are not there (10^4 histories, fp64: 53 us a call at 96 registers
-// and more against 59 at 80).
+// and more against 59 at 80; with one launch to set up, 38).
 template <int M, bool F32, bool SMEM, bool AGG>
 __global__ void __maxnreg__(128) slab_history_kernel_few(const RunArgs a) {
   slab_history_body<M, F32, SMEM, AGG>(a);
@@ -1104,7 +1105,8 @@ int slab_history_launch(const SlabLaunch& L, cudaStream_t s) {
   // carry a history, with four event records per thread in fp64 and two in
   // fp32 (a power of two).  slab_long, 10^6 histories: fp64 154 ms, against 164
   // with half the threads and 157 with two records; fp32 107 ms, against 114
-  // with four records; without the tail 244 and 160 ms.
+  // with four records; without the tail 244 and 160 ms.  (Before the bin walk was
+  // split; 141 and 106 ms since.)  coop_after:
   // passes after which what is left counts as long (16: 298 us instead of 292
   // for 300 000 histories of 9 flights, 4: 329; long chains do not care)
   a.coop_after = 32u;
