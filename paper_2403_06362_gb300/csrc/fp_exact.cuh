@@ -16,6 +16,7 @@
 // One fp64 addition that saves many integer instructions is the better trade
 // where that unit is not the bound:
 //   two_u_minus_1  2u - 1 for a draw u = n 2^-53 (exact: (2n - 2^53) 2^-53)
+//   llrint_add     llrint(v) by an addition of 2^52
 // All of them compile for host and device; the host copies let tests compare
 // them with the host's IEEE arithmetic.
 #pragma once
@@ -211,6 +212,14 @@ __host__ __device__ __forceinline__ long long llrint_nonneg(double v) {
   const uint64_t q = m >> sh, rem = m << (64 - sh);  // rem: the bits shifted out, at the top
   const uint64_t half = 1ull << 63;
   return (long long)(q + ((rem > half || (rem == half && (q & 1ull))) ? 1ull : 0ull));
+}
+
+// The same by the rounding of v + 2^52, whose low bits are the integer, for v <
+// 2^51; above, from the bits.
+__device__ __forceinline__ long long llrint_add(double v) {
+  if ((uint32_t)(raw_bits(v) >> 52) < 1023u + 51u)
+    return (long long)(raw_bits(__dadd_rn(v, 4503599627370496.0)) & ((1ull << 52) - 1ull));
+  return llrint_nonneg(v);
 }
 
 // Order key of a non-NaN double: a < b  <=>  okey(a) < okey(b); -0 and +0

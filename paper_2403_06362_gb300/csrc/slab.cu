@@ -538,7 +538,7 @@ __device__ __forceinline__ void coop_tally(const CoopHist& H, const SlabDev& p, 
       return;
     }
     const double xe = f == mcs::kLeakHi ? p.L : (f == mcs::kLeakLo ? 0.0 : dval(rec[0]));
-    const mcs::Walk64 k{xe, w, !mcs::nn_lt(xe, x)};
+    const mcs::Walk64<true> k{xe, w, !mcs::nn_lt(xe, x)};
     if (mcs::walk_first(p, x, k, sk, j))
       while (mcs::walk_next(p, k, sk, j)) {}
   } else {

@@ -194,22 +194,33 @@ __device__ __forceinline__ int bin_of(const SlabDev& p, const Sink& s, double x)
 // piece, so that a caller can stop between two: walk_first adds the piece to
 // xe or to the first edge, walk_next the next one, to xe or a whole bin with
 // its length from the width table; both return whether pieces are left.
+// ADD: a piece is rounded by an addition instead of from its bits, one fp64
+// instruction for some 15 integer ones.  The history kernel is bound by issue
+// (slab_long 141 -> 137 ms, 300 000 histories of 9 flights 253 -> 243 us); the
+// event schedule waits for its bank and its latency grows (97.8 -> 100.3 ms).
+template <bool ADD>
 struct Walk64 {
   double xe, w;  // the end, and 2^32 / |mu|
   bool fwd;
 };
-__device__ __forceinline__ bool walk_first(const SlabDev& p, double x, const Walk64& k, const Sink& s, int j) {
+template <bool ADD>
+__device__ __forceinline__ long long walk_fix(double v) {
+  return ADD ? mcx::llrint_add(v) : mcx::llrint_nonneg(v);
+}
+template <bool ADD>
+__device__ __forceinline__ bool walk_first(const SlabDev& p, double x, const Walk64<ADD>& k, const Sink& s, int j) {
   const double e = edge_of(p, s, j + (k.fwd ? 1 : 0));
   const bool last = k.fwd ? !nn_lt(e, k.xe) : !nn_lt(k.xe, e);
-  s.add(j, mcx::llrint_nonneg(__dmul_rn(mcx::abs_bits(__dsub_rn(last ? k.xe : e, x)), k.w)));
+  s.add(j, walk_fix<ADD>(__dmul_rn(mcx::abs_bits(__dsub_rn(last ? k.xe : e, x)), k.w)));
   return !last;
 }
-__device__ __forceinline__ bool walk_next(const SlabDev& p, const Walk64& k, const Sink& s, int& j) {
+template <bool ADD>
+__device__ __forceinline__ bool walk_next(const SlabDev& p, const Walk64<ADD>& k, const Sink& s, int& j) {
   j += k.fwd ? 1 : -1;
   const double e0 = edge_of(p, s, j + (k.fwd ? 0 : 1)), e1 = edge_of(p, s, j + (k.fwd ? 1 : 0));
   const bool last = k.fwd ? !nn_lt(e1, k.xe) : !nn_lt(k.xe, e1);
   const double len = !last && s.widths ? s.widths[j] : mcx::abs_bits(__dsub_rn(last ? k.xe : e1, e0));
-  s.add(j, mcx::llrint_nonneg(__dmul_rn(len, k.w)));
+  s.add(j, walk_fix<ADD>(__dmul_rn(len, k.w)));
   return !last;
 }
 
@@ -476,8 +487,9 @@ __device__ __forceinline__ bool leaves64(const SlabDev& p, long long mb, double 
 // that the lanes of a warp whose flights differ in kind still walk the bins
 // together.  begin_tally adds the first piece and returns whether walk_next
 // has more (which leaves j at the bin of xn); tally64 adds them all.
+template <bool ADD>
 __device__ __forceinline__ bool begin_tally(const SlabDev& p, double x, double xn, double mu, double d, double w_mu,
-                                            int outcome, const Sink& s, int& j, Walk64& k) {
+                                            int outcome, const Sink& s, int& j, Walk64<ADD>& k) {
   const long long mb = __double_as_longlong(mu);
   if (outcome == kCollide && mb == 0) {
     s.add(bin_of(p, s, x), mcx::fix32_nonneg(d));
@@ -490,7 +502,7 @@ __device__ __forceinline__ bool begin_tally(const SlabDev& p, double x, double x
 }
 __device__ __forceinline__ void tally64(const SlabDev& p, double x, double xn, double mu, double d, double w_mu,
                                         int outcome, const Sink& s, int& j) {
-  Walk64 k;
+  Walk64<false> k;
   if (begin_tally(p, x, xn, mu, d, w_mu, outcome, s, j, k))
     while (walk_next(p, k, s, j)) {}
 }
@@ -571,7 +583,7 @@ __device__ __forceinline__ void tally32(const SlabDev& p, float xf, float xlo, f
     while (walk_next(p, k, s, j)) {}
 }
 
-template <bool F32> struct WalkOf { using type = Walk64; };
+template <bool F32> struct WalkOf { using type = Walk64<true>; };
 template <> struct WalkOf<true> { using type = Walk32; };
 
 // The bin of the particle's position, where none is known from a flight.
