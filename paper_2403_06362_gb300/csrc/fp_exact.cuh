@@ -7,6 +7,7 @@
 // that unit, so every fp64 step whose exact result can be assembled from
 // integer operations is moved off it:
 //   floor_nonneg   floor(t) for 0 <= t < 2^63
+//   floor_small    floor(t) for 0 <= t < 2^20
 //   abs_le         |x| <= h for h >= 0
 //   recip_rn       1/y correctly rounded (IEEE round to nearest even)
 //   sqrt_rn        sqrt(x) correctly rounded
@@ -199,6 +200,12 @@ __host__ __device__ __forceinline__ double recip_normal(double y) {
   const uint64_t q = recip_mantissa((b & ((1ull << 52) - 1ull)) | (1ull << 52));  // in [2^52, 2^53]
   const uint32_t E = (uint32_t)(b >> 52) & 0x7FFu;
   return from_bits((b & (1ull << 63)) + ((uint64_t)(2044u - E) << 52) + q);
+}
+
+// floor(t) for 0 <= t < 2^20, from the high word alone.
+__host__ __device__ __forceinline__ uint32_t floor_small(double t) {
+  const uint32_t h = (uint32_t)(raw_bits(t) >> 32), sh = 1043u - (h >> 20);
+  return ((h & 0xfffffu) | 0x100000u) >> (sh < 31u ? sh : 31u);
 }
 
 // llrint(v) (round half to even) for 0 <= v < 2^62, from the bits.

@@ -110,10 +110,10 @@ constexpr int kShareMin = 8;
 // of their warp that still hold some -- a stream depends on its seed alone,
 // so who follows it changes nothing.  (Stride: the family shares one stream
 // in depth-first order, so its secondaries stay with their lane.)  Against
-// one record per secondary, all in memory, and no sharing: 58.0 -> 40.4 ms for
+// one record per secondary, all in memory, and no sharing: 58.0 -> 40.4 ms (37.9 since) for
 // 3 * 10^7 sources (29.7 -> 16.7 warp instructions per flight at 12.2 -> 20.7
 // lanes; 52.0 ms without the sharing), 3.4 -> 0.5 ms for 5000.  Hash at 64
-// registers (40.4 ms; 46.6 at 84), stride at 72 (15.5 ms for 6 * 10^6; 15.9).
+// registers (37.9 ms; at 84 a seventh slower), stride at 72 (14.3 ms for 6 * 10^6).
 template <int M, bool HASH, bool AGG>
 __global__ void __launch_bounds__(256, HASH ? 4 : 1) pulse_kernel(const PulseArgs a) {
   __shared__ mcd::Affine tab[64];
@@ -253,7 +253,9 @@ __global__ void __launch_bounds__(256, HASH ? 4 : 1) pulse_kernel(const PulseArg
         } else {
           const double xn = x + d * mu;
           if (mcx::abs_le(xn, P.x_half)) {
-            const uint64_t jf = mcx::floor_nonneg(tn);
+            // (t_end is at most 10^6.  The short form: stride 14.5 -> 14.3 ms; hash at
+            // its 64 registers 37.9 -> 39.1 ms)
+            const uint64_t jf = HASH ? mcx::floor_nonneg(tn) : mcx::floor_small(tn);
             const uint32_t j = jf < P.n_time_bins ? (uint32_t)jf : P.n_time_bins - 1;
             unsigned long long* const slot = a.tally + P.tally_offset + (uint64_t)grp * P.n_time_bins + j;
             if constexpr (AGG) mcd::warp_agg_add(slot, (unsigned long long)P.unit);
