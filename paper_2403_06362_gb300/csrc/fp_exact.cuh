@@ -223,9 +223,9 @@ __host__ __device__ __forceinline__ long long llrint_nonneg(double v) {
 
 // The same by the rounding of v + 2^52, whose low bits are the integer, for v <
 // 2^51; above, from the bits.
-__device__ __forceinline__ long long llrint_add(double v) {
+__host__ __device__ __forceinline__ long long llrint_add(double v) {
   if ((uint32_t)(raw_bits(v) >> 52) < 1023u + 51u)
-    return (long long)(raw_bits(__dadd_rn(v, 4503599627370496.0)) & ((1ull << 52) - 1ull));
+    return (long long)(raw_bits(v + 4503599627370496.0) & ((1ull << 52) - 1ull));
   return llrint_nonneg(v);
 }
 
