@@ -169,8 +169,8 @@ MC_API int mc_lcg_draw(mc_ctx* ctx, const mc_lcg* lcg, const mc_seed_spec* seed,
  *             host uint64_t[n_streams], in/out without a seed.
  *   h_digest  nullable host uint64_t[n_streams].  At least one of h_states
  *             and h_digest is required.
- * The range is processed in slices of at most 2^20 streams through two device
- * slots owned by the context (32 MiB, allocated on the first call): the draw
+ * The range is processed in slices of at most 2^22 streams through two device
+ * slots owned by the context (128 MiB, allocated on the first call): the draw
  * kernel of one slice runs on `stream` while a private copy stream returns
  * the previous slice.  Page-locked host buffers (cudaHostAlloc) let the
  * copies overlap the kernels; pageable ones work, serialised.  The call

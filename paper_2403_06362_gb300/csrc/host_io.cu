@@ -9,23 +9,30 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 
 #include "internal.h"
 
 namespace {
 
-constexpr uint64_t kSlice = 1ull << 20;     // streams per slice at most (8 MiB per array)
-constexpr uint64_t kMinSlice = 1ull << 17;  // and at least
+constexpr uint64_t kSlice = 1ull << 22;     // streams per slice at most (32 MiB per array)
+constexpr uint64_t kMinSlice = 1ull << 17;  // and at least, where there is more than one
 
-// A quarter of the range, so that all but the first slice's kernel runs behind
-// a copy; a slice costs some 5 us of its own, so not more of them than that
-// until a slice is long against it.  (64 draws: 3 * 10^6 streams in slices of
-// up to 2^22 took 361 us, an 80 us kernel and then the copy, now 312; in
-// sixteenths 341.  8 * 10^6 streams 805, now 744.)
-uint64_t slice_of(uint64_t n) {
-  const uint64_t s = (n / 4 + 31) & ~(uint64_t)31;
-  return std::min(kSlice, std::max(kMinSlice, s));
+// In S slices all but the first one's kernel, 1/S of the launch's time K = n
+// draws / (2.4 * 10^12 / s), runs behind a copy, and each slice costs some c = 3
+// us of its own (two events, a launch, two copies): K / S + c S is least at S =
+// sqrt(K / c).  (64 draws: 3 * 10^6 streams in one slice 360 us, in four 312, in
+// five 307, in sixteen 341; 8 * 10^6 in two 808, in eight 747.  16 draws: 8 * 10^5
+// streams in one slice 99-102 us, in four 110.)  Beyond some 200 draws the kernel is longer than
+// the copy and wants slices that fill the GPU several times over.
+uint64_t slice_of(uint64_t n, uint32_t draws) {
+  if (draws > 128u) return kSlice;
+  const double parts = std::sqrt((double)n * draws / 7.2e6);
+  const uint64_t s = std::max<uint64_t>(1, (uint64_t)(parts + 0.5));
+  if (s == 1) return kSlice;
+  const uint64_t slice = ((n + s - 1) / s + 31) & ~(uint64_t)31;
+  return std::min(kSlice, std::max(kMinSlice, slice));
 }
 
 int io_setup(mc_ctx* ctx) {
@@ -62,7 +69,7 @@ extern "C" MC_API int mc_lcg_draw_host(mc_ctx* ctx, const mc_lcg* lcg, const mc_
   if (st != MC_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
   uint64_t* base = static_cast<uint64_t*>(ctx->host_io.ptr);
-  const uint64_t slice = slice_of(n_streams), nslices = (n_streams + slice - 1) / slice;
+  const uint64_t slice = slice_of(n_streams, draws), nslices = (n_streams + slice - 1) / slice;
   for (uint64_t j = 0; j < nslices; ++j) {
     const int k = (int)(j & 1u);
     const uint64_t lo = j * slice, cnt = std::min<uint64_t>(slice, n_streams - lo);
