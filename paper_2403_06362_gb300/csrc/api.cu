@@ -81,22 +81,20 @@ namespace {
 constexpr size_t kTicketOff = 0;     // unsigned long long ticket
 constexpr size_t kScratchBytes = 256;
 
-// Slab records are followed, 256-byte aligned, by every problem's bin edge
-// and width tables (filled on the device by slab_prep).
-// The tables are followed, 256-byte aligned, by the processing order of a
-// launch of several problems (also filled by slab_prep).
-size_t slab_tables_offset(uint32_t n) { return ((size_t)n * mci::slab_dev_size() + 255u) & ~(size_t)255u; }
-size_t slab_order_offset(const mc_problem* problems, uint32_t n) {
-  return (slab_tables_offset(n) + (size_t)mci::slab_table_doubles(problems, n) * sizeof(double) + 255u) &
-         ~(size_t)255u;
+// Slab records are followed, 256-byte aligned, by the processing order of a
+// launch of several problems, and that, 256-byte aligned, by every problem's
+// bin edge and width tables (both filled on the device by slab_prep).  The
+// addresses of order and tables depend on the number of problems alone: a
+// captured launch holds them.
+size_t slab_order_offset(uint32_t n) { return ((size_t)n * mci::slab_dev_size() + 255u) & ~(size_t)255u; }
+size_t slab_tables_offset(uint32_t n) {
+  return (slab_order_offset(n) + mci::slab_order_bytes(n) + 255u) & ~(size_t)255u;
 }
 size_t slab_stage_bytes(const mc_problem* problems, uint32_t n) {
-  return slab_order_offset(problems, n) + mci::slab_order_bytes(n);
+  return slab_tables_offset(n) + (size_t)mci::slab_table_doubles(problems, n) * sizeof(double);
 }
 void* slab_tables_of(mc_ctx* ctx, uint32_t n) { return static_cast<char*>(ctx->problems.ptr) + slab_tables_offset(n); }
-void* slab_order_of(mc_ctx* ctx, const mc_problem* problems, uint32_t n) {
-  return static_cast<char*>(ctx->problems.ptr) + slab_order_offset(problems, n);
-}
+void* slab_order_of(mc_ctx* ctx, uint32_t n) { return static_cast<char*>(ctx->problems.ptr) + slab_order_offset(n); }
 
 // Host half of staging: waits until the pinned buffer is free, sizes the
 // buffers and writes the problem records into pinned memory.
@@ -163,8 +161,7 @@ int stage_problems(mc_ctx* ctx, const mc_problem* problems, uint32_t n, cudaStre
   MC_TRY_CUDA(cudaEventRecord(*ev, s));
   st = pulse ? mci::pulse_prep(ctx->problems.ptr, s)
              : (box ? mci::box_prep(ctx->problems.ptr, n, s)
-                    : mci::slab_prep(ctx->problems.ptr, n, s, slab_tables_of(ctx, n),
-                                     slab_order_of(ctx, problems, n)));
+                    : mci::slab_prep(ctx->problems.ptr, n, s, slab_tables_of(ctx, n), slab_order_of(ctx, n)));
   if (st != MC_OK) return st;
   ctx->staged_image->swap(img);
   ctx->staged_kind = kind;
@@ -517,7 +514,7 @@ int make_slab_launch(mc_ctx* ctx, const mc_lcg* lcg, const mc_problem* problems,
   // A launch of all the histories of 2..kMaxOrderedProblems problems takes
   // them in the order the prep kernel ranked (longest expected chains first).
   if (n_problems >= 2 && n_problems <= mci::kMaxOrderedProblems && rb == 0 && re == total_histories(problems, n_problems))
-    mci::slab_order_ptrs(slab_order_of(ctx, problems, n_problems), n_problems, &L.d_order, &L.d_order_begin);
+    mci::slab_order_ptrs(slab_order_of(ctx, n_problems), n_problems, &L.d_order, &L.d_order_begin);
   L.chunk = cfg->chunk ? cfg->chunk : mci::slab_default_chunk(re - rb, ctx->num_sms);
   L.range_begin = rb;
   L.total = re - rb;
@@ -574,6 +571,9 @@ int run_slab_graph(mc_ctx* ctx, const mc_lcg* lcg, const mc_problem* problems, u
   key = fnv(key, &L.single_n_bins, sizeof L.single_n_bins);
   key = fnv(key, &L.max_n_bins, sizeof L.max_n_bins);
   key = fnv(key, &L.walk_pieces, sizeof L.walk_pieces);
+  // and so is whether the histories are taken in the ranked order (a range
+  // that ends where the problems do) or by id
+  key = fnv(key, &L.d_order, sizeof L.d_order);
   if (!ctx->graphs) ctx->graphs = new mci::GraphCache();
   auto it = ctx->graphs->m.find(key);
   cudaGraphExec_t exec = nullptr;
@@ -589,8 +589,7 @@ int run_slab_graph(mc_ctx* ctx, const mc_lcg* lcg, const mc_problem* problems, u
     cudaGraph_t g = nullptr;
     MC_TRY_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed));
     cudaMemcpyAsync(ctx->problems.ptr, ctx->h_problems, bytes, cudaMemcpyHostToDevice, cs);
-    mci::slab_prep(ctx->problems.ptr, n_problems, cs, slab_tables_of(ctx, n_problems),
-                   slab_order_of(ctx, problems, n_problems));
+    mci::slab_prep(ctx->problems.ptr, n_problems, cs, slab_tables_of(ctx, n_problems), slab_order_of(ctx, n_problems));
     if (!cfg->accumulate) {
       cudaMemsetAsync(tally->d_bins, 0, tally->n_slots * sizeof(int64_t), cs);
       cudaMemsetAsync(tally->d_counts, 0, (size_t)n_problems * MC_NCOUNT * sizeof(uint64_t), cs);
@@ -630,8 +629,8 @@ int transport_run_impl(mc_ctx* ctx, const mc_lcg* lcg, const mc_problem* problem
     if (st != MC_OK) return st;
     // (one problem of up to 3071 bins has its tables in shared memory)
     void* const tables = n_problems == 1 && problems[0].n_bins < 3072u ? nullptr : slab_tables_of(ctx, n_problems);
-    st = mci::slab_init(problems, n_problems, ctx->problems.ptr, tables,
-                        slab_order_of(ctx, problems, n_problems), tally, !cfg->accumulate, ticket, s);
+    st = mci::slab_init(problems, n_problems, ctx->problems.ptr, tables, slab_order_of(ctx, n_problems), tally,
+                        !cfg->accumulate, ticket, s);
     if (st != MC_OK) return st;
   } else {
     st = stage_problems(ctx, problems, n_problems, s);
