@@ -244,8 +244,10 @@ static __device__ __noinline__ long long fix32_any(float v) {
 // For v < 2^22 on the fp32 pipe, without branches: adding 2^23 rounded down
 // leaves floor(v) in the low bits; the fraction (exact) gives its next 16
 // bits the same way, and the last 16 by an addition rounded to nearest even,
-// whose parity is that of the whole.  (A fraction has at most 24 bits, so
-// the last step never carries out of its 16.)
+// whose parity is that of the whole.  The last 16 can round up to 2^16 (v =
+// 2^-16 - 2^-40): the low word is a sum, which carries that into the bits
+// above.  It cannot carry out of the low word: that takes a fraction of 33
+// leading ones, and a fraction has at most 24 bits.
 __device__ __forceinline__ long long fix32_from_float(float v) {
   if (v >= 4194304.0f) return fix32_any(v);
   constexpr float kM = 8388608.0f;  // 2^23, bit pattern 0x4b000000
