@@ -403,15 +403,16 @@ MC_API int mc_log1m_device(const double* d_u, double* d_out, uint64_t n, int whi
 
 /* Diagnostics of the fp64 steps the transport computes on the integer pipes
  * (no counterpart in the paper): mc_recip_rn(y) is 1/y rounded to nearest
- * even, exactly as IEEE division: a table of 2^63/F (F the left end of the
- * mantissa's cell among 1024, the flight logarithm's table), 1/(1 + r)
- * through r^5 by Horner's rule on non-negative fixed point, an exact
- * remainder check and the rounding; IEEE division for zero, subnormal or
- * huge operands (host evaluation of the device code);
+ * even, exactly as IEEE division: an fp32 reciprocal of the mantissa, two
+ * correction terms in fixed point, an exact remainder check and the rounding;
+ * IEEE division for zero, subnormal or huge operands (host evaluation of the
+ * device code, but for the fp32 estimate it starts from);
  * mc_recip_rn_device writes d_out[i] = 1/d_y[i] with it (which = 0) or with
- * the CUDA division (which = 1); mc_two_u_minus_1(n) is 2u - 1 for the
- * uniform u = n 2^-53 (n < 2^53; 0 otherwise).  Errors: MC_ERR_ARG,
- * MC_ERR_CUDA. */
+ * the CUDA division (which = 1); mc_sqrt_rn_device writes d_out[i] =
+ * sqrt(d_x[i]) for positive normal d_x[i] with the transport's integer square
+ * root (which = 0) or with CUDA's sqrt (which = 1); mc_two_u_minus_1(n) is
+ * 2u - 1 for the uniform u = n 2^-53 (n < 2^53; 0 otherwise).  Errors:
+ * MC_ERR_ARG, MC_ERR_CUDA. */
 MC_API double mc_recip_rn(double y);
 MC_API double mc_two_u_minus_1(uint64_t n);
 /* llrint(v) for 0 <= v < 2^62; a < b for non-NaN doubles (1 or 0); RN(j h)
@@ -420,6 +421,7 @@ MC_API long long mc_llrint_nonneg(double v);
 MC_API int mc_d_lt(double a, double b);
 MC_API double mc_mul_small(uint32_t j, double h);
 MC_API int mc_recip_rn_device(const double* d_y, double* d_out, uint64_t n, int which, void* stream);
+MC_API int mc_sqrt_rn_device(const double* d_x, double* d_out, uint64_t n, int which, void* stream);
 
 /* Section 5 normality procedure on host data x[n_batches][n_points]: the
  * normalised deviations z = (x - mean)/sd per point (sd with n-1) and the

@@ -123,7 +123,7 @@ def mc_recip_rn(y: float) -> float:
 
 
 def mc_two_u_minus_1(n: int) -> float:
-    """2u - 1 for u = n 2^-53, assembled from integer operations (host evaluation)."""
+    """2u - 1 for u = n 2^-53, as the transport forms it (host evaluation)."""
     return float(lib().mc_two_u_minus_1(int(n)))
 
 
@@ -136,6 +136,12 @@ def mc_recip_rn_device(d_y, d_out, which=0, stream=None):
     """d_out = 1/d_y on the device: which 0 = the integer-pipe reciprocal,
     1 = the CUDA division (fp64 tensors of equal length)."""
     return _ffi.check(lib().mc_recip_rn_device(_ptr(d_y), _ptr(d_out), d_y.numel(), which, _stream(stream)))
+
+
+def mc_sqrt_rn_device(d_x, d_out, which=0, stream=None):
+    """d_out = sqrt(d_x) on the device for positive normal d_x: which 0 = the
+    integer-pipe square root, 1 = CUDA's sqrt (fp64 tensors of equal length)."""
+    return _ffi.check(lib().mc_sqrt_rn_device(_ptr(d_x), _ptr(d_out), d_x.numel(), which, _stream(stream)))
 
 
 def mc_seed_hash(ctx, lcg, parent_seed, key_begin, count, d_states, stream=None):

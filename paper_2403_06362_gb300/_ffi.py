@@ -34,7 +34,7 @@ EXPORTED = [
     "mc_lcg_draw", "mc_transport_run", "mc_tally_read", "mc_hash64", "mc_normality",
     "mc_transport_run_static", "mc_autotune", "mc_log1m", "mc_log1m_device", "mc_recip_rn",
     "mc_two_u_minus_1", "mc_recip_rn_device", "mc_llrint_nonneg", "mc_d_lt", "mc_mul_small",
-    "mc_ctx_set_limits", "mc_ctx_get_limits", "mc_lcg_draw_host",
+    "mc_ctx_set_limits", "mc_ctx_get_limits", "mc_lcg_draw_host", "mc_sqrt_rn_device",
 ]
 
 
@@ -138,6 +138,7 @@ def _load():
         "mc_recip_rn": (dbl, [dbl]),
         "mc_two_u_minus_1": (dbl, [u64]),
         "mc_recip_rn_device": (i32, [P, P, u64, i32, P]),
+        "mc_sqrt_rn_device": (i32, [P, P, u64, i32, P]),
         "mc_llrint_nonneg": (C.c_longlong, [dbl]),
         "mc_d_lt": (i32, [dbl, dbl]),
         "mc_mul_small": (dbl, [u32, dbl]),
