@@ -24,8 +24,10 @@ constexpr uint64_t kMinSlice = 1ull << 17;  // and at least, where there is more
 // us of its own (two events, a launch, two copies): K / S + c S is least at S =
 // sqrt(K / c).  (64 draws: 3 * 10^6 streams in one slice 360 us, in four 312, in
 // five 307, in sixteen 341; 8 * 10^6 in two 808, in eight 747.  16 draws: 8 * 10^5
-// streams in one slice 99-102 us, in four 110.)  Beyond some 200 draws the kernel is longer than
-// the copy and wants slices that fill the GPU several times over.
+// streams in one slice 99-102 us, in four 110.  128 draws: 10^6 streams in one
+// slice 168 us, in four 144; 5 * 10^6 in two 669, in nine 527.)  Above 128
+// draws slices have not been measured: one slice up to 2^22 streams, whose
+// kernel takes longer than its copy (10^6 streams of 600 draws 390 us).
 uint64_t slice_of(uint64_t n, uint32_t draws) {
   if (draws > 128u) return kSlice;
   const double parts = std::sqrt((double)n * draws / 7.2e6);
@@ -33,6 +35,14 @@ uint64_t slice_of(uint64_t n, uint32_t draws) {
   if (s == 1) return kSlice;
   const uint64_t slice = ((n + s - 1) / s + 31) & ~(uint64_t)31;
   return std::min(kSlice, std::max(kMinSlice, slice));
+}
+
+// Whether copies of a host buffer run beside kernels.
+bool page_locked(const void* p) {
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) == cudaSuccess) return a.type == cudaMemoryTypeHost;
+  cudaGetLastError();
+  return false;
 }
 
 int io_setup(mc_ctx* ctx) {
@@ -69,7 +79,11 @@ extern "C" MC_API int mc_lcg_draw_host(mc_ctx* ctx, const mc_lcg* lcg, const mc_
   if (st != MC_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
   uint64_t* base = static_cast<uint64_t*>(ctx->host_io.ptr);
-  const uint64_t slice = slice_of(n_streams, draws), nslices = (n_streams + slice - 1) / slice;
+  uint64_t slice = slice_of(n_streams, draws);
+  // Copies of pageable memory hold the host up, so slices only add their own
+  // cost (10^6 streams of 64 draws: three slices 195 us, one 151).
+  if (slice < n_streams && ((h_states && !page_locked(h_states)) || (h_digest && !page_locked(h_digest)))) slice = kSlice;
+  const uint64_t nslices = (n_streams + slice - 1) / slice;
   for (uint64_t j = 0; j < nslices; ++j) {
     const int k = (int)(j & 1u);
     const uint64_t lo = j * slice, cnt = std::min<uint64_t>(slice, n_streams - lo);
