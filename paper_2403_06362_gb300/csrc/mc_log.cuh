@@ -171,13 +171,13 @@ __host__ __device__ __forceinline__ W96 sub96(W96 a, W96 b) {
 }
 
 // a 2^-scale as the nearest double (round half to even) for
-// 2^82 <= a < 2^96, without branches.  Defined for every a (sh is 0..32 then),
-// but what it returns outside that range means nothing.
+// 2^82 <= a < 2^96, without branches.  Defined for every a (sh is 0..32 then:
+// hence the mask), but what it returns outside that range means nothing.
 __host__ __device__ __forceinline__ double w96_to_double(W96 a, int scale) {
   const int top = 95 - (int)clz32_(a.w2);  // 82..95
   const uint32_t sh = (uint32_t)(top - 63);  // 19..32
   const uint32_t mh = fsr32_(a.w1, a.w2, sh), ml = fsr32_(a.w0, a.w1, sh);  // bits sh..sh+63, leading 1 at the top
-  const uint32_t sticky = fsr32_(0u, a.w0, sh) != 0u ? 1u : 0u;  // any of the bits below sh
+  const uint32_t sticky = (a.w0 << ((32u - sh) & 31u)) != 0u ? 1u : 0u;  // any of the bits below sh
   const uint64_t m53 = (((uint64_t)mh << 32) | ml) >> 11;
   // the 11 bits below the last, with the sticky bit: up above a half, and at
   // a half when the last bit is odd
