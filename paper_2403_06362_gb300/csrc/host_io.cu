@@ -18,6 +18,7 @@ namespace {
 
 constexpr uint64_t kSlice = 1ull << 22;     // streams per slice at most (32 MiB per array)
 constexpr uint64_t kMinSlice = 1ull << 17;  // and at least, where there is more than one
+constexpr uint64_t kMinGiven = 1ull << 19;  // streams whose states come from the host: fewer go in one slice
 
 // In S slices all but the first one's kernel, 1/S of the launch's time K = n
 // draws / (2.4 * 10^12 / s), runs behind a copy, and each slice costs some c = 3
@@ -27,9 +28,12 @@ constexpr uint64_t kMinSlice = 1ull << 17;  // and at least, where there is more
 // streams in one slice 99-102 us, in four 110.  128 draws: 10^6 streams in one
 // slice 168 us, in four 144; 5 * 10^6 in two 669, in nine 527.)  Above 128
 // draws slices have not been measured: one slice up to 2^22 streams, whose
-// kernel takes longer than its copy (10^6 streams of 600 draws 390 us).
-uint64_t slice_of(uint64_t n, uint32_t draws) {
-  if (draws > 128u) return kSlice;
+// kernel takes longer than its copy (10^6 streams of 600 draws 390 us).  Given
+// states are copied in before each slice's kernel, so their slices cost more: 2 *
+// 10^5 of 128 draws take 91 us in one slice and 95 in two (alone 106 and 135), 4 *
+// 10^5 of 64 the same either way, 10^6 of 33 247 and 229.
+uint64_t slice_of(uint64_t n, uint32_t draws, bool given) {
+  if (draws > 128u || (given && n < kMinGiven)) return kSlice;
   const double parts = std::sqrt((double)n * draws / 7.2e6);
   const uint64_t s = std::max<uint64_t>(1, (uint64_t)(parts + 0.5));
   if (s == 1) return kSlice;
@@ -79,7 +83,7 @@ extern "C" MC_API int mc_lcg_draw_host(mc_ctx* ctx, const mc_lcg* lcg, const mc_
   if (st != MC_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
   uint64_t* base = static_cast<uint64_t*>(ctx->host_io.ptr);
-  uint64_t slice = slice_of(n_streams, draws);
+  uint64_t slice = slice_of(n_streams, draws, !seed);
   // Copies of pageable memory hold the host up, so slices only add their own
   // cost (10^6 streams of 64 draws: three slices 195 us, one 151).
   if (slice < n_streams && ((h_states && !page_locked(h_states)) || (h_digest && !page_locked(h_digest)))) slice = kSlice;

@@ -29,3 +29,19 @@ def test_matches_the_device_call(n, draws, pinned_states, pinned_digest, load):
         mc.mc_lcg_draw_host(ctx, lcg, spec, 9, None, n, draws, only)
         assert torch.equal(only, dg.cpu())
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [2**19 - 1, 2**19])
+def test_given_states_around_the_size_that_is_cut(n):
+    import torch
+
+    import paper_2403_06362_gb300 as mc
+
+    ctx, lcg = mc.Context(0), mc.make_lcg()
+    given = torch.arange(n, dtype=torch.int64) * 7919 + 5
+    st, dg = given.cuda(), torch.empty(n, dtype=torch.int64, device="cuda")
+    mc.mc_lcg_draw(ctx, lcg, None, 0, st, n, 100, None, dg)
+    h_st, h_dg = given.pin_memory(), torch.zeros(n, dtype=torch.int64, pin_memory=True)
+    mc.mc_lcg_draw_host(ctx, lcg, None, 0, h_st, n, 100, h_dg)
+    assert torch.equal(h_st, st.cpu()) and torch.equal(h_dg, dg.cpu())
+    ctx.close()
