@@ -611,14 +611,21 @@ constexpr uint32_t kMaxRowBins = 256;  // of a warp's row cache (2 KiB)
 // fp32 10.9 ms against 10.6, fp64 17.3 against 15.0).
 constexpr uint32_t kIdle = 16;
 
-// Lanes still walking for which a warp makes another piece of its tallies in
-// the same pass.  A tally in shared memory is a single problem's, or small:
-// one, and slab_walk_pieces the limit (with 8 lanes 300 000 histories of 9
-// flights took 260 us instead of 253).  Otherwise problems of many kinds share
-// the warps and no number of pieces suits all: no limit but 8 lanes (256
-// problems, against two pieces: fp32 8.72 -> 8.55 ms, fp64 13.1 -> 12.4 ms; 4,
-// 6 and 12 lanes within 2 %).
-template <bool SMEM> constexpr int kWalkMin = SMEM ? 1 : 8;
+// How many lanes still walking make a warp add another piece of its tallies in
+// the same pass, where `live` lanes carry a history and no other can begin one
+// (32 while there is work left).  A tally in shared memory is a single
+// problem's, or small: one lane, and slab_walk_pieces the limit (with 8 lanes
+// 300 000 histories of 9 flights took 260 us instead of 253).  Otherwise
+// problems of many kinds share the warps and no number of pieces suits all: no
+// limit but 8 lanes (256 problems, against two pieces: fp32 8.72 -> 8.55 ms,
+// fp64 13.1 -> 12.4 ms; 4, 6 and 12 lanes within 2 %), or all that are left:
+// while every one of them walks, none waits for the next pass (5000 histories
+// at 100 bins per mean free path: 1.91 s with a pass for each piece then, now
+// 1.21; 1.54 before passes were split, 1.25 going on for half of them).
+template <bool SMEM>
+__device__ __forceinline__ int walk_least(int live) {
+  return SMEM ? 1 : min(8, live);
+}
 constexpr uint32_t kWalkNoLimit = ~0u;
 
 // The ticket positions of one problem: begin + id for its history id.
@@ -839,10 +846,12 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
       }
     }
     // The other pieces of the tallies, walk_pieces per lane at most and, after
-    // the first, only for kWalkMin lanes together: a lane whose flight crosses
-    // more bins goes on in the next pass, while the others take their next event.
+    // the first, only for so many lanes together (walk_least): a lane whose
+    // flight crosses more bins goes on in the next pass, while the others take
+    // their next event.
+    const int least = walk_least<SMEM>(more ? 32 : __popc(~dead));
     for (uint32_t i = 0; i < a.walk_pieces; ++i) {
-      if (__popc(__ballot_sync(kFull, walking)) < (i == 0u ? 1 : kWalkMin<SMEM>)) break;
+      if (__popc(__ballot_sync(kFull, walking)) < (i == 0u ? 1 : least)) break;
       if (walking) walking = mcs::walk_next(*P, wk, sink, q.j);
     }
     if (alive && !walking && outcome != mcs::kContinue) {
