@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
+#include <type_traits>
 
 #include "internal.h"
 #include "mc_log.cuh"
@@ -76,13 +77,15 @@ __global__ void pulse_prep_kernel(PulseDev* p) {
 // Collisions, absorptions and the rest follow from them: a flight ends at the
 // census or collides, a collision scatters or absorbs.  Event caps, dropped
 // secondaries and exceedances go to the block's counters in shared memory.
+// N: on 32 bits they are flushed now and then; 64 bits never need it.
+template <typename N>
 struct PulseCounts {
-  uint32_t src, flights, census, scat, children;
+  N src, flights, census, scat, children;
   uint64_t draws, maxd;
   __device__ void flush(unsigned long long* c) {
     if (src) atomicAdd(c + MC_C_SOURCE, (unsigned long long)src);
     if (flights) atomicAdd(c + MC_C_FLIGHTS, (unsigned long long)flights);
-    const uint32_t coll = flights - census;
+    const N coll = flights - census;
     if (coll) atomicAdd(c + MC_C_COLLISIONS, (unsigned long long)coll);
     if (coll != scat) atomicAdd(c + MC_C_ABSORPTIONS, (unsigned long long)(coll - scat));
     if (scat) atomicAdd(c + MC_C_SCATTERS, (unsigned long long)scat);
@@ -90,7 +93,7 @@ struct PulseCounts {
     if (children) atomicAdd(c + MC_C_CHILDREN, (unsigned long long)children);
     if (draws) atomicAdd(c + MC_C_DRAWS, (unsigned long long)draws);
     if (maxd) atomicMax(c + MC_C_MAX_DRAWS, (unsigned long long)maxd);
-    src = flights = census = scat = children = 0u;
+    src = flights = census = scat = children = 0;
     draws = maxd = 0ull;
   }
 };
@@ -110,10 +113,14 @@ constexpr int kShareMin = 8;
 // of their warp that still hold some -- a stream depends on its seed alone,
 // so who follows it changes nothing.  (Stride: the family shares one stream
 // in depth-first order, so its secondaries stay with their lane.)  Against
-// one record per secondary, all in memory, and no sharing: 58.0 -> 40.4 ms (37.9 since) for
+// one record per secondary, all in memory, and no sharing: 58.0 -> 40.4 ms for
 // 3 * 10^7 sources (29.7 -> 16.7 warp instructions per flight at 12.2 -> 20.7
-// lanes; 52.0 ms without the sharing), 3.4 -> 0.5 ms for 5000.  Hash at 64
-// registers (37.9 ms; at 84 a seventh slower), stride at 72 (14.3 ms for 6 * 10^6).
+// lanes; 52.0 ms without the sharing), 3.4 -> 0.5 ms for 5000; 37.9 ms with
+// 2u - 1 by a subtraction.  Hash at 64 registers (at 84 a seventh slower).
+// Stride runs wait for a family's one chain of events until many lanes carry
+// one: a scattered particle draws its direction in place, and the row's place
+// is kept with 64-bit counts that need no flush (5000 sources 4.32 -> 3.86 ms,
+// 6 * 10^6 13.8 -> 13.0 at 80 registers; 4.09 and 13.4 held at 72).
 template <int M, bool HASH, bool AGG>
 __global__ void __launch_bounds__(256, HASH ? 4 : 1) pulse_kernel(const PulseArgs a) {
   __shared__ mcd::Affine tab[64];
@@ -135,6 +142,7 @@ __global__ void __launch_bounds__(256, HASH ? 4 : 1) pulse_kernel(const PulseArg
   // stack_depth entries on, round the end (at most pend - left, so they fit)
   uint32_t lo = 0, sp = 0;
   auto entry = [&](uint32_t k) {
+    if constexpr (!HASH) return my_stack + (uint64_t)k * nthreads;  // lo stays 0
     const uint32_t i = lo + k;
     return my_stack + (uint64_t)(i >= a.stack_depth ? i - a.stack_depth : i) * nthreads;
   };
@@ -145,11 +153,12 @@ __global__ void __launch_bounds__(256, HASH ? 4 : 1) pulse_kernel(const PulseArg
   uint32_t left = 0, pend = 0;
   uint64_t pool_next = 0, pool_end = 0;
   bool more = true, alive = false, primary = false;
-  PulseCounts lc{};
+  PulseCounts<std::conditional_t<HASH, uint32_t, uint64_t>> lc{};
   mcs::Rng<M> r{0ull, 0ull};
   double x = 0.0, t = 0.0, mu = 0.0;
   uint64_t gi = 0, events = 0;
   uint32_t grp = 0;
+  unsigned long long* row = nullptr;  // stride: the family's tally row
   const uint64_t total = a.ovf_in ? min((uint64_t)*a.ovf_in_count, a.ovf_cap) : a.total;
 
   for (;;) {
@@ -185,6 +194,7 @@ __global__ void __launch_bounds__(256, HASH ? 4 : 1) pulse_kernel(const PulseArg
             ++lc.src;
           }
           mu = mcx::two_u_minus_1(r.next_n(l));
+          if constexpr (!HASH) row = a.tally + P.tally_offset + (uint64_t)grp * P.n_time_bins;
           events = 0;
           alive = true;
         }
@@ -257,7 +267,8 @@ __global__ void __launch_bounds__(256, HASH ? 4 : 1) pulse_kernel(const PulseArg
             // its 64 registers 37.9 -> 39.1 ms)
             const uint64_t jf = HASH ? mcx::floor_nonneg(tn) : mcx::floor_small(tn);
             const uint32_t j = jf < P.n_time_bins ? (uint32_t)jf : P.n_time_bins - 1;
-            unsigned long long* const slot = a.tally + P.tally_offset + (uint64_t)grp * P.n_time_bins + j;
+            unsigned long long* const slot =
+                HASH ? a.tally + P.tally_offset + (uint64_t)grp * P.n_time_bins + j : row + j;
             if constexpr (AGG) mcd::warp_agg_add(slot, (unsigned long long)P.unit);
             else atomicAdd(slot, (unsigned long long)P.unit);
           }
@@ -297,7 +308,10 @@ __global__ void __launch_bounds__(256, HASH ? 4 : 1) pulse_kernel(const PulseArg
                 }
               }
             }
-            redraw = true;
+            // its new direction: below, on the code path a new particle shares
+            // (hash), or here, one branch sooner (stride)
+            if constexpr (HASH) redraw = true;
+            else mu = mcx::two_u_minus_1(r.next_n(l));
           } else {
             ended = true;
           }
@@ -331,7 +345,7 @@ __global__ void __launch_bounds__(256, HASH ? 4 : 1) pulse_kernel(const PulseArg
           }
         }
         redraw = alive;
-        if (lc.flights > (1u << 24)) lc.flush(a.counts);  // (up to 63 secondaries each)
+        if (HASH && lc.flights > (1u << 24)) lc.flush(a.counts);  // (up to 63 secondaries each)
       }
     }
     if constexpr (HASH) {
@@ -348,8 +362,7 @@ __global__ void __launch_bounds__(256, HASH ? 4 : 1) pulse_kernel(const PulseArg
         }
       }
     }
-    // one code path draws the direction of a scattered and of a new particle
-    // (the same draw, in the same stream order, as drawing it in place)
+    // the direction of a new particle and (hash) of a scattered one
     if (redraw) mu = mcx::two_u_minus_1(r.next_n(l));
   }
   // the lanes' counts, summed over the warp (they share a cache line)
