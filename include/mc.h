@@ -320,7 +320,15 @@ typedef struct {
  * The call enqueues work on `stream` and returns; the device status word
  * is checked by mc_tally_read.  Errors: MC_ERR_ARG (bad problem: L, sigma_t
  * <= 0, c outside [0,1], n_bins or n_batches 0, slots outside the tally),
- * MC_ERR_CUDA. */
+ * MC_ERR_CUDA.
+ * Capture: the history schedule of slab problems (use_graph 0), once a call of
+ * the same shape has made the context's buffers large enough.  A call of at
+ * most 16 problems and 2^19 tally slots carries its problems in the captured
+ * launch; one of more needs the problems of the context's last call to be its
+ * own at every replay.  The graph holds the context's buffers: it is replayed
+ * only while no later call needed larger ones, and not beside other calls under
+ * the context.  Calls that wait for the device (box, hash-seeded pulse, event
+ * schedule) cannot be captured. */
 MC_API int mc_transport_run(mc_ctx* ctx, const mc_lcg* lcg, const mc_problem* problems,
                             uint32_t n_problems, const mc_run_config* config, const mc_tally* tally,
                             void* stream);

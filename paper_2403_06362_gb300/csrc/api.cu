@@ -131,7 +131,7 @@ int stage_problems(mc_ctx* ctx, const mc_problem* problems, uint32_t n, cudaStre
   const size_t dev_bytes = (pulse || box) ? bytes : slab_stage_bytes(problems, n);
   // Fill a host image first: if it equals the image last uploaded, the
   // device copy (base fields and the derived ones the prep kernel computes
-  // from them) is still current.
+  // from them) is still current, unless a caller's graph may have rewritten it.
   const int kind = pulse ? MC_GEOM_PULSE : (box ? MC_GEOM_BOX : MC_GEOM_SLAB);
   if (!ctx->fill_scratch) ctx->fill_scratch = new std::vector<unsigned char>();
   if (!ctx->staged_image) ctx->staged_image = new std::vector<unsigned char>();
@@ -140,7 +140,7 @@ int stage_problems(mc_ctx* ctx, const mc_problem* problems, uint32_t n, cudaStre
   if (pulse) mci::pulse_fill_host(problems, img.data());
   else if (box) mci::box_fill_host(problems, n, img.data());
   else mci::slab_fill_host(problems, n, img.data());
-  if (kind == ctx->staged_kind && n == ctx->staged_n && ctx->problems.bytes >= dev_bytes &&
+  if (!ctx->replayed && kind == ctx->staged_kind && n == ctx->staged_n && ctx->problems.bytes >= dev_bytes &&
       *ctx->staged_image == img)
     return MC_OK;
   cudaEvent_t* ev = &ctx->staged;
@@ -625,6 +625,10 @@ int transport_run_impl(mc_ctx* ctx, const mc_lcg* lcg, const mc_problem* problem
   if (problems[0].geometry == MC_GEOM_SLAB && n_problems <= mci::kInitProblems &&
       tally->n_slots <= mci::kInitSlots) {
     ctx->staged_kind = -1;  // these records do not pass through the staging image
+    // Captured, every replay writes them again, at a time this context does not see.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();  // (the launch reports it)
+    else if (capture != cudaStreamCaptureStatusNone) ctx->replayed = true;
     st = ctx->problems.reserve(slab_stage_bytes(problems, n_problems));
     if (st != MC_OK) return st;
     // (one problem of up to 3071 bins has its tables in shared memory)

@@ -102,6 +102,7 @@ struct mc_ctx {
   std::vector<unsigned char>* fill_scratch = nullptr;
   int staged_kind = -1;
   uint32_t staged_n = 0;
+  bool replayed = false;  // a caller's graph holds a run that writes records: they may change at any time
   // Event-based schedule: particle bank and a pinned completion flag.
   mci::DeviceBuf bank;
   unsigned int* h_done = nullptr;
