@@ -611,21 +611,23 @@ constexpr uint32_t kMaxRowBins = 256;  // of a warp's row cache (2 KiB)
 // fp32 10.9 ms against 10.6, fp64 17.3 against 15.0).
 constexpr uint32_t kIdle = 16;
 
-// How many lanes still walking make a warp add another piece of its tallies in
-// the same pass, where `live` lanes carry a history and no other can begin one
-// (32 while there is work left).  A tally in shared memory is a single
-// problem's, or small: one lane, and slab_walk_pieces the limit (with 8 lanes
-// 300 000 histories of 9 flights took 260 us instead of 253).  Otherwise
-// problems of many kinds share the warps and no number of pieces suits all: no
-// limit but 8 lanes (256 problems, against two pieces: fp32 8.72 -> 8.55 ms,
-// fp64 13.1 -> 12.4 ms; 4, 6 and 12 lanes within 2 %), or all that are left:
-// while every one of them walks, none waits for the next pass (5000 histories
-// at 100 bins per mean free path: 1.91 s with a pass for each piece then, now
-// 1.21; 1.54 before passes were split, 1.25 going on for half of them).
-template <bool SMEM>
-__device__ __forceinline__ int walk_least(int live) {
-  return SMEM ? 1 : min(8, live);
-}
+// Lanes still walking for which a warp adds another piece of its tallies in
+// the same pass.  A tally in shared memory is a single problem's, or small:
+// one lane, and slab_walk_pieces the limit (with 8 lanes 300 000 histories of 9
+// flights took 260 us instead of 253).  Otherwise problems of many kinds share
+// the warps and no number of pieces suits all: no limit but 8 lanes (256
+// problems, against two pieces: fp32 8.72 -> 8.55 ms, fp64 13.1 -> 12.4 ms; 4,
+// 6 and 12 lanes within 2 %).
+template <bool SMEM> constexpr int kWalkMin = SMEM ? 1 : 8;
+// Once the work has run out, all lanes that are left are enough as well: while
+// every one of them walks, none waits for the next pass.  Blocks of one warp
+// run so for long, without a cooperative tail (5000 histories at 100 bins per
+// mean free path: 1.91 s with a pass for each piece then, 1.21 now; 1.54
+// before passes were split, 1.25 going on for half of the lanes).  The kernel
+// of small runs has the registers for it; those of 64 and 80 do without, whose
+// long histories go to the tail (there it cost 256 problems 1 %: 8.54 -> 8.63
+// ms), but for generic widths and warp-aggregated tallies, which have no other.
+template <int M, bool SMEM, bool AGG, bool FEW> constexpr bool kWalkLast = !SMEM && (FEW || M != 63 || AGG);
 constexpr uint32_t kWalkNoLimit = ~0u;
 
 // The ticket positions of one problem: begin + id for its history id.
@@ -647,8 +649,9 @@ __device__ __forceinline__ void flush_row(unsigned long long* global_row, uint32
   __syncwarp();
 }
 
-template <int M, bool F32, bool SMEM, bool AGG>
+template <int M, bool F32, bool SMEM, bool AGG, bool FEW>
 __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
+  constexpr bool LAST = kWalkLast<M, SMEM, AGG, FEW>;
   extern __shared__ unsigned long long s_dyn[];
   unsigned long long* const s_tally = s_dyn;
   __shared__ mcd::Affine tab[64];
@@ -846,12 +849,12 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
       }
     }
     // The other pieces of the tallies, walk_pieces per lane at most and, after
-    // the first, only for so many lanes together (walk_least): a lane whose
-    // flight crosses more bins goes on in the next pass, while the others take
-    // their next event.
-    const int least = walk_least<SMEM>(more ? 32 : __popc(~dead));
+    // the first, only for kWalkMin lanes together (LAST: or all that are left):
+    // a lane whose flight crosses more bins goes on in the next pass, while the
+    // others take their next event.
     for (uint32_t i = 0; i < a.walk_pieces; ++i) {
-      if (__popc(__ballot_sync(kFull, walking)) < (i == 0u ? 1 : least)) break;
+      const unsigned on = __ballot_sync(kFull, walking);
+      if (__popc(on) < (i == 0u ? 1 : kWalkMin<SMEM>) && (!LAST || more || on == 0u || (on | dead) != kFull)) break;
       if (walking) walking = mcs::walk_next(*P, wk, sink, q.j);
     }
     if (alive && !walking && outcome != mcs::kContinue) {
@@ -892,11 +895,11 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
 // accept blocks of up to 512 threads.
 template <int M, bool F32, bool SMEM, bool AGG>
 __global__ void __launch_bounds__(512, 2) slab_history_kernel_f32(const RunArgs a) {
-  slab_history_body<M, F32, SMEM, AGG>(a);
+  slab_history_body<M, F32, SMEM, AGG, false>(a);
 }
 template <int M, bool F32, bool SMEM, bool AGG>
 __global__ void __maxnreg__(80) slab_history_kernel_f64(const RunArgs a) {
-  slab_history_body<M, F32, SMEM, AGG>(a);
+  slab_history_body<M, F32, SMEM, AGG, false>(a);
 }
 
 // A run of at most a few warps per SM waits for its longest histories, not for
@@ -905,7 +908,7 @@ __global__ void __maxnreg__(80) slab_history_kernel_f64(const RunArgs a) {
 // and more against 59 at 80; with one launch to set up, 38).
 template <int M, bool F32, bool SMEM, bool AGG>
 __global__ void __maxnreg__(128) slab_history_kernel_few(const RunArgs a) {
-  slab_history_body<M, F32, SMEM, AGG>(a);
+  slab_history_body<M, F32, SMEM, AGG, true>(a);
 }
 
 constexpr uint64_t kFewThreads = 128;  // per SM, at most, for the kernel of small runs
