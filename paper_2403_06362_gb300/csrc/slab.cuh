@@ -477,12 +477,6 @@ __device__ __forceinline__ int advance64(const SlabDev& p, double x, double mu, 
   return kCollide;
 }
 
-// advance64's face tests alone: whether xn, the end of a flight with
-// direction bits mb, lies outside the slab.
-__device__ __forceinline__ bool leaves64(const SlabDev& p, long long mb, double xn) {
-  return (mb > 0 && !nn_lt(xn, p.L)) || (mb < 0 && __double_as_longlong(xn) <= 0);
-}
-
 // The tally of that flight, from x's bin j: the track from x to xn, to the
 // face it leaves through, or (mu = 0) the whole distance d in the bin holding
 // x.  Every kind of flight ends in the one walk, with its end chosen first, so
