@@ -65,7 +65,7 @@ INST_PER_FLIGHT = {
     "slab_small_fp64": 1292, "slab_small_fp32": 1143, "slab_long_fp64": 655, "slab_long_fp32": 560,
     "batched_fp64": 796, "batched_fp32": 665, "box_fp64": 1604, "box_fp32": 915,
     "box_fp64_event": 2053, "box_fp32_event": 1165,
-    "pulse_hash": 369, "pulse_stride": 337, "pulse_census": 496,
+    "pulse_hash": 369, "pulse_stride": 303, "pulse_census": 496,
 }
 # Bytes each flight of an event schedule moves through its particle bank: the
 # particle's fields read and written once per iteration (slab: x, mu, w, the

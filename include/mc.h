@@ -71,7 +71,8 @@ typedef struct {
  * tickets, the status word, the device copy of the problem list and the
  * particle banks of the event-based schedule.  Create it once, outside any
  * timed or captured region; it allocates device memory.  A context may be
- * used from one host thread at a time. */
+ * used from one host thread at a time, but for mc_tally_read: several threads
+ * may read tallies that no other work writes. */
 typedef struct mc_ctx mc_ctx;
 
 /* Creates a context on `device` (the device is made current).  *out is set
@@ -94,7 +95,11 @@ MC_API void mc_ctx_destroy(mc_ctx* ctx);
  *   box_generations     generations of weight-window children the host
  *                       follows before MC_ERR_TIMEOUT (default 10000).
  *   pulse_generations   generations of overflowed pulse secondaries (hash
- *                       modes) before MC_ERR_TIMEOUT (default 100000).
+ *                       modes) before MC_ERR_TIMEOUT (default 100000).  How
+ *                       many a run needs can differ from run to run: which
+ *                       secondaries overflow depends on which lanes shared a
+ *                       family.  It is never more than with every family on
+ *                       its own lane.
  *   event_iterations    iterations of the event-based schedules (slab, and
  *                       box per generation) before MC_ERR_TIMEOUT; rounded
  *                       up to whole batches of iterations.  UINT64_MAX (the
@@ -284,7 +289,8 @@ typedef struct {
     uint64_t range_end;     /* concatenated problems; end 0 = all                 */
     uint32_t stack_depth;   /* pulse problem: pending secondaries a lane keeps    */
                             /* (1..256, 0 = 256); in hash modes the rest wait in  */
-                            /* a device overflow bank processed after the launch  */
+                            /* a device overflow bank (2^20 per generation; beyond */
+                            /* it MC_C_DROPPED) processed after the launch        */
                             /* (their streams depend only on their seeds, Eq. 5); */
                             /* stride mode counts them in MC_C_DROPPED            */
     uint32_t tally_atomics; /* history-schedule kernels (slab, box, pulse, census  */

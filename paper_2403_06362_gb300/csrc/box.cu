@@ -110,15 +110,18 @@ template <typename T> constexpr int kWalkSteps = sizeof(T) == 4 ? 5 : 4;
 constexpr uint32_t kCountProbs = 16;  // problems whose counters a block keeps in shared memory
 
 // fp32: bound by integer issue (80 % of the slots, at 15.7 lanes per
-// instruction); fp64: by the fp64 unit (66 % busy at 17 lanes).  Each pass of the loop takes every live lane through the same
-// phases -- refill, direction, flight, tally -- so that source and collision
-// share one copy of the direction's code, a refill waits until some lanes
-// need one, and a flight whose track crosses many voxels does not hold its
-// warp.  Particle, walk and axis state are scalars in registers (no local
-// memory); a particle's counts go to its block's counters in shared memory
-// when it ends.  Four blocks per SM in fp32 (64 registers: 16.3 ms for 10^7
-// histories, 17.4 with three, 17.7 with five; 31.7 before the phases), three
-// in fp64 (80: 13.1 ms for 3 * 10^6, 45.7 before; four were 1 % slower).
+// instruction); fp64: by the fp64 unit (66 % busy at 17 lanes).  Each pass of
+// the loop takes every live lane through the same phases -- refill, direction,
+// flight, tally -- so that source and collision share one copy of the
+// direction's code, a refill waits until some lanes need one, and a flight
+// whose track crosses many voxels does not hold its warp.  Particle, walk and
+// axis state are scalars, none of them indexed (fp32 spills some 80 bytes at
+// its 64 registers; in fp64 the rare call of surface_exact takes a copy of the
+// particle through a 96-byte frame); a particle's counts go to its block's
+// counters in shared memory when it ends.  Four blocks per SM in fp32 (64
+// registers: 16.3 ms for 10^7 histories, 17.4 with three, 17.7 with five; 31.7
+// before the phases), three in fp64 (80: 13.0 ms for 3 * 10^6, 45.7 before; four
+// were 1 % slower).
 template <int M, typename T, bool AGG, bool ONE>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) box_history_kernel(const BoxArgs a) {
   __shared__ mcd::Affine tab[64];

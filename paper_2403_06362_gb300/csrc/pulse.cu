@@ -4,13 +4,16 @@
 // flux averaged over [-x_half, x_half] in unit time bins, tallied per
 // (repetition, batch).
 //
-// History-based: a lane follows one source particle and its whole family of
-// secondaries depth-first.  Secondaries wait on a per-lane last-in first-out
-// stack (thread-local memory).  In hash mode each secondary owns a stream
-// seeded on demand by S_c = hash(k, S_p) (Section 4, Eq. 5), so no lane ever
-// coordinates with another; in stride mode the family shares the source
-// particle's stream, which fixes the depth-first order the secondaries are
-// drawn in -- the sequential bookkeeping the paper's hashing removes.
+// History-based: a lane follows one source particle and its family of
+// secondaries depth-first.  Those that wait are records on the lane's stack in
+// device memory.  In hash mode each secondary owns a stream seeded on demand by
+// S_c = hash(k, S_p) (Section 4, Eq. 5), so a record holds all secondaries of a
+// collision, the newest record stays in registers, and when the sources have run
+// out, lanes with nothing left take the oldest record of a lane of their warp:
+// who follows a secondary changes no result.  In stride mode the family shares
+// the source particle's stream, which fixes the depth-first order the
+// secondaries are drawn in -- the sequential bookkeeping the paper's hashing
+// removes -- and its records hold one each and stay with their lane.
 // The fp64 arithmetic is rounded once per operation (--fmad=false).
 #include <cuda_runtime.h>
 

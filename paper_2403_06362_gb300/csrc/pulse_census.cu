@@ -16,10 +16,10 @@
 // nondeterministic -- changes no result: tallies and counters are
 // bit-identical to the sequential definition.
 //
-// The host enqueues the phases back to back (each launch reads the size of
-// its input bank from device memory); it waits only to read how many
-// secondaries overflowed the lane stacks in a phase, and launches the
-// generations of those before the phase's control.
+// Each launch reads the size of its input bank from device memory.  After
+// each the host waits to read how many secondaries overflowed the lane stacks
+// (nearly always none) and launches the generations of those before the
+// phase's control.
 // The fp64 arithmetic is rounded once per operation (--fmad=false).
 #include <cuda_runtime.h>
 

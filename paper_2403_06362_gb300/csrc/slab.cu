@@ -890,9 +890,9 @@ __device__ __forceinline__ void slab_history_body(const RunArgs& a) {
 // The kernel in two register budgets.  The fp32 flight fits 64 registers but
 // for a few spills (four blocks of 256 per SM; at 80, 256 problems took a
 // tenth longer); the fp64 flight runs fastest with 80 and three blocks per SM
-// (slab_long 156 ms, against 166 / 159 / 180 at 64 / 72 / 96, before the bin
-// walk was split: 141 ms since).  Both
-// accept blocks of up to 512 threads.
+// (slab_long at 64 / 72 / 80 / 96 registers 166 / 159 / 156 / 180 ms when each was
+// tried, before the bin walk was split; 136 ms at 80 as it is).  Both accept
+// blocks of up to 512 threads.
 template <int M, bool F32, bool SMEM, bool AGG>
 __global__ void __launch_bounds__(512, 2) slab_history_kernel_f32(const RunArgs a) {
   slab_history_body<M, F32, SMEM, AGG, false>(a);
@@ -1115,12 +1115,12 @@ int slab_history_launch(const SlabLaunch& L, cudaStream_t s) {
   a.min_grab = L.n_problems == 1 ? 8u : a.chunk;
   // The cooperative tail takes over when a quarter of a block's threads still
   // carry a history, with four event records per thread in fp64 and two in
-  // fp32 (a power of two).  slab_long, 10^6 histories: fp64 154 ms, against 164
-  // with half the threads and 157 with two records; fp32 107 ms, against 114
-  // with four records; without the tail 244 and 160 ms.  (Before the bin walk was
-  // split; 141 and 106 ms since.)  coop_after:
-  // passes after which what is left counts as long (16: 298 us instead of 292
-  // for 300 000 histories of 9 flights, 4: 329; long chains do not care)
+  // fp32 (a power of two).  slab_long, 10^6 histories, when each was tried,
+  // before the bin walk was split: fp64 154 ms, against 164 with half the threads
+  // and 157 with two records; fp32 107 ms, against 114 with four records; without
+  // the tail 244 and 160 ms.  (As it is 136 and 107 ms.)  coop_after: passes after
+  // which what is left counts as long (16: 298 us instead of 292 for 300 000
+  // histories of 9 flights, 4: 329; long chains do not care)
   a.coop_after = 32u;
   if (L.pool_lock_attempts != 0u && L.block >= 64) {
     a.coop_slots = 128u;
