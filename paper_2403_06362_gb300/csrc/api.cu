@@ -123,26 +123,37 @@ int stage_host(mc_ctx* ctx, const mc_problem* problems, uint32_t n, size_t* byte
   return MC_OK;
 }
 
+// Fills the host image of a call's records (fill_scratch) and says whether it
+// equals the image last uploaded: the device copy (base fields, and the derived
+// ones, order and tables that the prep kernels compute from them) is then still
+// current, unless a caller's graph may have rewritten it.
+bool records_current(mc_ctx* ctx, const mc_problem* problems, uint32_t n, int kind, size_t bytes, size_t dev_bytes) {
+  if (!ctx->fill_scratch) ctx->fill_scratch = new std::vector<unsigned char>();
+  if (!ctx->staged_image) ctx->staged_image = new std::vector<unsigned char>();
+  std::vector<unsigned char>& img = *ctx->fill_scratch;
+  img.assign(bytes, 0);
+  if (kind == MC_GEOM_PULSE) mci::pulse_fill_host(problems, img.data());
+  else if (kind == MC_GEOM_BOX) mci::box_fill_host(problems, n, img.data());
+  else mci::slab_fill_host(problems, n, img.data());
+  return !ctx->replayed && kind == ctx->staged_kind && n == ctx->staged_n && ctx->problems.bytes >= dev_bytes &&
+         *ctx->staged_image == img;
+}
+
+// The image that records_current filled is the device's from here on.
+void records_uploaded(mc_ctx* ctx, int kind, uint32_t n) {
+  ctx->staged_image->swap(*ctx->fill_scratch);
+  ctx->staged_kind = kind;
+  ctx->staged_n = n;
+}
+
 int stage_problems(mc_ctx* ctx, const mc_problem* problems, uint32_t n, cudaStream_t s) {
   const bool box = problems[0].geometry == MC_GEOM_BOX;
   const bool pulse = problems[0].geometry == MC_GEOM_PULSE;
   const size_t bytes = pulse ? mci::pulse_dev_size()
                              : (size_t)n * (box ? mci::box_dev_size() : mci::slab_dev_size());
   const size_t dev_bytes = (pulse || box) ? bytes : slab_stage_bytes(problems, n);
-  // Fill a host image first: if it equals the image last uploaded, the
-  // device copy (base fields and the derived ones the prep kernel computes
-  // from them) is still current, unless a caller's graph may have rewritten it.
   const int kind = pulse ? MC_GEOM_PULSE : (box ? MC_GEOM_BOX : MC_GEOM_SLAB);
-  if (!ctx->fill_scratch) ctx->fill_scratch = new std::vector<unsigned char>();
-  if (!ctx->staged_image) ctx->staged_image = new std::vector<unsigned char>();
-  std::vector<unsigned char>& img = *ctx->fill_scratch;
-  img.assign(bytes, 0);
-  if (pulse) mci::pulse_fill_host(problems, img.data());
-  else if (box) mci::box_fill_host(problems, n, img.data());
-  else mci::slab_fill_host(problems, n, img.data());
-  if (!ctx->replayed && kind == ctx->staged_kind && n == ctx->staged_n && ctx->problems.bytes >= dev_bytes &&
-      *ctx->staged_image == img)
-    return MC_OK;
+  if (records_current(ctx, problems, n, kind, bytes, dev_bytes)) return MC_OK;
   cudaEvent_t* ev = &ctx->staged;
   if (*ev) MC_TRY_CUDA(cudaEventSynchronize(*ev));
   if (bytes > ctx->h_problems_bytes) {
@@ -155,7 +166,7 @@ int stage_problems(mc_ctx* ctx, const mc_problem* problems, uint32_t n, cudaStre
   ctx->staged_kind = -1;  // until the upload below is enqueued
   int st = ctx->problems.reserve(dev_bytes);
   if (st != MC_OK) return st;
-  std::memcpy(ctx->h_problems, img.data(), bytes);
+  std::memcpy(ctx->h_problems, ctx->fill_scratch->data(), bytes);
   MC_TRY_CUDA(cudaMemcpyAsync(ctx->problems.ptr, ctx->h_problems, bytes, cudaMemcpyHostToDevice, s));
   if (!*ev) MC_TRY_CUDA(cudaEventCreateWithFlags(ev, cudaEventDisableTiming));
   MC_TRY_CUDA(cudaEventRecord(*ev, s));
@@ -163,9 +174,7 @@ int stage_problems(mc_ctx* ctx, const mc_problem* problems, uint32_t n, cudaStre
              : (box ? mci::box_prep(ctx->problems.ptr, n, s)
                     : mci::slab_prep(ctx->problems.ptr, n, s, slab_tables_of(ctx, n), slab_order_of(ctx, n)));
   if (st != MC_OK) return st;
-  ctx->staged_image->swap(img);
-  ctx->staged_kind = kind;
-  ctx->staged_n = n;
+  records_uploaded(ctx, kind, n);
   return MC_OK;
 }
 
@@ -622,23 +631,34 @@ int transport_run_impl(mc_ctx* ctx, const mc_lcg* lcg, const mc_problem* problem
     return run_slab_graph(ctx, lcg, problems, n_problems, cfg, tally, rb, re, s);
 
   auto* ticket = reinterpret_cast<unsigned long long*>(static_cast<char*>(ctx->scratch.ptr) + kTicketOff);
-  if (problems[0].geometry == MC_GEOM_SLAB && n_problems <= mci::kInitProblems &&
-      tally->n_slots <= mci::kInitSlots) {
-    ctx->staged_kind = -1;  // these records do not pass through the staging image
-    // Captured, every replay writes them again, at a time this context does not see.
+  const bool few = problems[0].geometry == MC_GEOM_SLAB && n_problems <= mci::kInitProblems &&
+                   tally->n_slots <= mci::kInitSlots;
+  bool ready = false;
+  if (few) {
+    // Captured, the records go with the graph: every replay writes them again,
+    // at a time this context does not see.
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();  // (the launch reports it)
     else if (capture != cudaStreamCaptureStatusNone) ctx->replayed = true;
-    st = ctx->problems.reserve(slab_stage_bytes(problems, n_problems));
-    if (st != MC_OK) return st;
-    // (one problem of up to 3071 bins has its tables in shared memory)
-    void* const tables = n_problems == 1 && problems[0].n_bins < 3072u ? nullptr : slab_tables_of(ctx, n_problems);
-    st = mci::slab_init(problems, n_problems, ctx->problems.ptr, tables, slab_order_of(ctx, n_problems), tally,
-                        !cfg->accumulate, ticket, s);
-    if (st != MC_OK) return st;
+    const size_t dev_bytes = slab_stage_bytes(problems, n_problems);
+    ready = records_current(ctx, problems, n_problems, MC_GEOM_SLAB, n_problems * mci::slab_dev_size(), dev_bytes);
+    if (!ready) {
+      ctx->staged_kind = -1;  // until the launch below is enqueued
+      st = ctx->problems.reserve(dev_bytes);
+      if (st != MC_OK) return st;
+      // (one problem of up to 3071 bins has its tables in shared memory)
+      void* const tables = n_problems == 1 && problems[0].n_bins < 3072u ? nullptr : slab_tables_of(ctx, n_problems);
+      st = mci::slab_init(ctx->fill_scratch->data(), n_problems, ctx->problems.ptr, tables,
+                          slab_order_of(ctx, n_problems), tally, !cfg->accumulate, ticket, s);
+      if (st != MC_OK) return st;
+      records_uploaded(ctx, MC_GEOM_SLAB, n_problems);
+    }
   } else {
     st = stage_problems(ctx, problems, n_problems, s);
     if (st != MC_OK) return st;
+    ready = true;
+  }
+  if (ready) {  // (slab_init zeroes these too)
     if (!cfg->accumulate) {
       MC_TRY_CUDA(cudaMemsetAsync(tally->d_bins, 0, tally->n_slots * sizeof(int64_t), s));
       MC_TRY_CUDA(cudaMemsetAsync(tally->d_counts, 0, (size_t)n_problems * MC_NCOUNT * sizeof(uint64_t), s));

@@ -1045,10 +1045,10 @@ int slab_prep(void* d_probs, uint32_t n, cudaStream_t s, void* d_tables, void* d
   return cuda_status(cudaGetLastError(), "slab_tables_kernel launch");
 }
 
-int slab_init(const mc_problem* src, uint32_t n, void* d_probs, void* d_tables, void* d_order, const mc_tally* tally,
+int slab_init(const void* records, uint32_t n, void* d_probs, void* d_tables, void* d_order, const mc_tally* tally,
               bool zero, unsigned long long* d_ticket, cudaStream_t s) {
   InitArgs a;
-  slab_fill_host(src, n, a.src);
+  std::memcpy(a.src, records, n * sizeof(SlabDev));
   a.n = n;
   a.dst = static_cast<SlabDev*>(d_probs);
   a.order = n >= 2 ? static_cast<uint32_t*>(d_order) : nullptr;

@@ -43,10 +43,11 @@ void slab_fill_host(const mc_problem* src, uint32_t n, void* dst);
 constexpr uint32_t kMaxOrderedProblems = 4096;
 int slab_prep(void* d_probs, uint32_t n, cudaStream_t s, void* d_tables = nullptr, void* d_order = nullptr);
 // Records, tables, order (both nullable), the ticket and, with `zero`, the
-// tally's zeros of a call with at most kInitProblems problems, in one launch.
+// tally's zeros of a call with at most kInitProblems problems, in one launch,
+// from the records as slab_fill_host has them.
 constexpr uint32_t kInitProblems = 16;
 constexpr uint64_t kInitSlots = 1u << 19;  // of the tally, at most (more: a memset does as well)
-int slab_init(const mc_problem* src, uint32_t n, void* d_probs, void* d_tables, void* d_order, const mc_tally* tally,
+int slab_init(const void* records, uint32_t n, void* d_probs, void* d_tables, void* d_order, const mc_tally* tally,
               bool zero, unsigned long long* d_ticket, cudaStream_t s);
 inline size_t slab_order_bytes(uint32_t n) { return (size_t)((n + 1u) & ~1u) * 4u + (size_t)(n + 1u) * 8u; }
 inline void slab_order_ptrs(void* d_order, uint32_t n, const uint32_t** order, const uint64_t** begin) {
